@@ -26,7 +26,9 @@
  *     after an exact FP32 reduction of the phase to fractional turns (the
  *     adjoint, whose output is real, takes r and the gains in polar form and
  *     one cosine per pair); sums over tiles, norms, step sizes and the
- *     projection stay in FP64.
+ *     projection stay in FP64.  Dirac pixels on a regular (l, m) lattice
+ *     without gains take, where that is faster, an FP32 gridding and FFT
+ *     operator instead, whose result is nearer FP64's than the pairs' is.
  */
 #ifndef SL1M_H
 #define SL1M_H

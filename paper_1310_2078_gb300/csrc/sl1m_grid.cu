@@ -1,0 +1,665 @@
+// sl1m_grid.cu -- the operator of Dirac pixels on a regular (l, m) lattice by
+// gridding and FFT (Hardy 2013, Eq. sme with the entries of Eq. deltam).
+//
+//   V_k = sum_j (x_j / n_j) exp(-2 pi i (u_k l_j + v_k m_j + w_k (n_j - 1)))
+//
+// With l_j = lc + s dl and m_j = mc + t dm for integers s, t, the dependence on
+// u and v is a Fourier series in s and t sampled off its grid, and that on w
+// is a Fourier integral over nu = n - 1 - nc, |nu| <= B.  Both are evaluated
+// by the same device (Dutt & Rokhlin 1993; the kernel is the "exponential of
+// semicircle" of Barnett, Magland & af Klinteberg 2019): a function of bounded
+// support sampled at twice its band is interpolated by a kernel phi of 8
+// samples, once the other side has been divided by phi's transform.  So
+//
+//   forward   for every plane w_p: z_st = x amp exp(-2 pi i w_p nu), rows then
+//             columns transformed (zero-padded to 2^lx, 2^ly), and each V_k
+//             gathered from 8 x 8 cells of 8 planes;
+//   adjoint   the transpose: r spread onto the planes, columns and rows
+//             transformed back, Re(exp(+2 pi i w_p nu) z) summed over the planes.
+//
+// x is real, so V at (-u, -v, -w) is the conjugate of V at (u, v, w): the
+// visibilities with w < 0 are taken at the mirrored point, and the planes cover
+// only 0 .. max |w|.  Tiles of a plane that no visibility touches are neither
+// written nor read, and columns without such a tile are not transformed.
+//
+// The interpolation error is 1e-7 of the result's norm and the whole operator
+// in FP32 is 1.6e-7 to 2.4e-7 off FP64 (2-norm, listed sizes below and others),
+// where evaluating every pair with the SFU's sine and cosine (sl1m_mixed.cu) is
+// 3.6e-7 to 4.9e-7 off.  The work no longer grows with N_v N_p but with the
+// planes' cells: per plane the kernels move up to (3 2^ly + 2 ny) 2^lx complex
+// numbers.  Measured on GB300 against the pair kernels: 1024^2 pixels x 406,400
+// visibilities (55 planes of 2048^2) forward 202.7 -> 1.21 ms, adjoint 141.6 ->
+// 1.75 ms; 256^2 over +/-0.5 x 40,320 (151 planes of 512^2) 1.19 -> 0.34 ms
+// and 0.84 -> 0.46 ms.
+#include <algorithm>
+
+#include "sl1m_devfn.cuh"
+#include "sl1m_grid.h"
+
+namespace sl1m {
+
+// ---------------------------------------------------------------- transforms
+
+__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
+__device__ __forceinline__ float2 cmul(float2 a, float2 b)
+{
+    return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
+}
+// SGN i a
+template <int SGN>
+__device__ __forceinline__ float2 crot(float2 a)
+{
+    return SGN < 0 ? make_float2(a.y, -a.x) : make_float2(-a.y, a.x);
+}
+
+template <int SGN>
+__device__ __forceinline__ void dft4(float2& a0, float2& a1, float2& a2, float2& a3)
+{
+    const float2 s0 = cadd(a0, a2), s1 = csub(a0, a2), s2 = cadd(a1, a3), s3 = crot<SGN>(csub(a1, a3));
+    a0 = cadd(s0, s2);
+    a1 = cadd(s1, s3);
+    a2 = csub(s0, s2);
+    a3 = csub(s1, s3);
+}
+
+template <int SGN>
+__device__ __forceinline__ void dft8(float2 (&v)[8])
+{
+    const float H = 0.70710678118654752f;
+    dft4<SGN>(v[0], v[2], v[4], v[6]);        // even inputs: e0..e3 in v0, v2, v4, v6
+    dft4<SGN>(v[1], v[3], v[5], v[7]);        // odd inputs
+    const float2 r3 = crot<SGN>(v[3]), r7 = crot<SGN>(v[7]);
+    const float2 o1 = make_float2((v[3].x + r3.x) * H, (v[3].y + r3.y) * H);   // times e^{SGN i pi/4}
+    const float2 o2 = crot<SGN>(v[5]);
+    const float2 o3 = make_float2((r7.x - v[7].x) * H, (r7.y - v[7].y) * H);   // times e^{SGN 3 i pi/4}
+    const float2 e0 = v[0], e1 = v[2], e2 = v[4], e3 = v[6], o0 = v[1];
+    v[0] = cadd(e0, o0);
+    v[1] = cadd(e1, o1);
+    v[2] = cadd(e2, o2);
+    v[3] = cadd(e3, o3);
+    v[4] = csub(e0, o0);
+    v[5] = csub(e1, o1);
+    v[6] = csub(e2, o2);
+    v[7] = csub(e3, o3);
+}
+
+// Shared-memory place of element e of CB interleaved transforms (CB a power of
+// two): one row of pad per 8 rows, so that the stride-8 writes of a radix-8
+// pass fall into different banks.
+template <int CB>
+__device__ __forceinline__ int pad_at(int row, int c)
+{
+    return row * CB + c + (row >> 3) * CB;
+}
+constexpr int padded(int n, int cb) { return (n + n / 8) * cb; }
+
+// Transform of length 2^LOG, radix 8 after a first pass of radix 2, 4 or 8
+// (Stockham order: no bit reversal).  A thread holds NB groups of 8 elements:
+// on entry and on exit v[n][q] is element g[n] + q 2^LOG/8 of transform c.
+// Every thread of the CTA calls it; sm holds the CTA's CB interleaved
+// transforms.  Twiddles: per pass of stride ns, e^{-2 pi i k/(8 ns)} and its
+// 2nd and 4th powers for k < ns, rounded from FP64; the other powers are
+// products of two.
+template <int LOG, int SGN, int CB, int NB>
+__device__ __forceinline__ void fft_pass_all(float2 (&v)[NB][8], const int (&g)[NB], int c, float2* sm,
+                                             const float2* __restrict__ tw)
+{
+    constexpr int L = 1 << LOG, E = L / 8;
+    constexpr int R0 = LOG % 3 == 0 ? 8 : LOG % 3 == 1 ? 2 : 4;
+#pragma unroll
+    for (int n = 0; n < NB; ++n) {
+        if (R0 == 8) {
+            dft8<SGN>(v[n]);
+#pragma unroll
+            for (int r = 0; r < 8; ++r) sm[pad_at<CB>(g[n] * 8 + r, c)] = v[n][r];
+        } else if (R0 == 4) {
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                dft4<SGN>(v[n][i], v[n][i + 2], v[n][i + 4], v[n][i + 6]);
+#pragma unroll
+                for (int r = 0; r < 4; ++r) sm[pad_at<CB>((g[n] + i * E) * 4 + r, c)] = v[n][i + 2 * r];
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float2 a = v[n][i], b = v[n][i + 4];
+                sm[pad_at<CB>((g[n] + i * E) * 2, c)] = cadd(a, b);
+                sm[pad_at<CB>((g[n] + i * E) * 2 + 1, c)] = csub(a, b);
+            }
+        }
+    }
+#pragma unroll
+    for (int ns = R0; ns < L; ns *= 8) {
+        __syncthreads();
+#pragma unroll
+        for (int n = 0; n < NB; ++n)
+#pragma unroll
+            for (int r = 0; r < 8; ++r) v[n][r] = sm[pad_at<CB>(g[n] + r * E, c)];
+        __syncthreads();
+#pragma unroll
+        for (int n = 0; n < NB; ++n) {
+            const int k = g[n] & (ns - 1);
+            float2 w1 = __ldg(tw + k), w2 = __ldg(tw + ns + k), w4 = __ldg(tw + 2 * ns + k);
+            if (SGN > 0) {
+                w1.y = -w1.y;
+                w2.y = -w2.y;
+                w4.y = -w4.y;
+            }
+            const float2 w3 = cmul(w1, w2);
+            v[n][1] = cmul(v[n][1], w1);
+            v[n][2] = cmul(v[n][2], w2);
+            v[n][3] = cmul(v[n][3], w3);
+            v[n][4] = cmul(v[n][4], w4);
+            v[n][5] = cmul(v[n][5], cmul(w1, w4));
+            v[n][6] = cmul(v[n][6], cmul(w2, w4));
+            v[n][7] = cmul(v[n][7], cmul(w3, w4));
+            dft8<SGN>(v[n]);
+            if (ns * 8 < L) {
+                const int o = (g[n] - k) * 8 + k;
+#pragma unroll
+                for (int r = 0; r < 8; ++r) sm[pad_at<CB>(o + r * ns, c)] = v[n][r];
+            }
+        }
+        tw += 3 * ns;
+    }
+}
+
+// Cell index of element e (0 <= e < 2^lg) of a zero-padded axis whose cell c0
+// sits at element 0; outside [0, n) where the padding is.
+__device__ __forceinline__ int cell_of(int e, int lg, int c0)
+{
+    return (e < (1 << (lg - 1)) ? e : e - (1 << lg)) + c0;
+}
+
+// exp(-2 pi i w nu) with both factors split in FP32 halves.
+__device__ __forceinline__ float2 plane_phase(float2 w, float2 nu)
+{
+    const float f = frac_turns(tp_frac(w.x, w.y, nu.x, nu.y));
+    float s, c;
+    sincospif(2.0f * f, &s, &c);
+    return make_float2(c, -s);
+}
+
+template <int LOG>
+struct RowShape {
+    static constexpr int T = (1 << LOG) / 8;                  // threads per row
+    static constexpr int ROWS = T >= 256 ? 1 : 256 / T;       // rows per CTA
+    static constexpr int THREADS = T * ROWS;
+    static constexpr int PAD = padded(1 << LOG, 1);           // shared elements per row
+};
+
+// Forward, rows: z = x amp exp(-2 pi i w_p nu) along x, transformed, into g1.
+// A CTA takes ROWS lattice rows of GR_PCH planes: x, amp and nu are read once
+// for them.
+template <int LOG>
+__global__ void __launch_bounds__(RowShape<LOG>::THREADS, LOG < 12 ? 3 : 1)
+grid_rows_fwd_kernel(const DevProblem* __restrict__ probs, int prob, const GridOp g, int p0, int np)
+{
+    using S = RowShape<LOG>;
+    constexpr int L = 1 << LOG;
+    __shared__ float2 sm[S::ROWS][S::PAD];
+    const double* X;
+    if (!fwd_role(probs[prob], X)) return;
+    const int rb = threadIdx.x / S::T;
+    const int gi[1] = {(int)threadIdx.x % S::T};
+    const int iy = blockIdx.x * S::ROWS + rb;
+    float a[8];
+    float2 nu[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        const int ix = cell_of(gi[0] + q * S::T, LOG, g.cx);
+        a[q] = 0.f;
+        nu[q] = make_float2(0.f, 0.f);
+        if (iy < g.ny && ix >= 0 && ix < g.nx) {
+            const size_t at = (size_t)iy * g.nx + ix;
+            const int j = g.cell[at];
+            if (j >= 0) {
+                a[q] = __double2float_rn(X[j]) * g.amp[at] * g.fscale;
+                nu[q] = g.nu[at];
+            }
+        }
+    }
+    const int q1 = min(np, (int)(blockIdx.y + 1) * GR_PCH);
+    for (int p = blockIdx.y * GR_PCH; p < q1; ++p) {
+        const float2 w = g.wp[p0 + p];
+        float2 v[1][8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const int ix = cell_of(gi[0] + q * S::T, LOG, g.cx);
+            v[0][q] = make_float2(0.f, 0.f);
+            if (ix >= 0 && ix < g.nx) {
+                const float2 e = plane_phase(w, nu[q]);
+                v[0][q] = make_float2(a[q] * e.x, a[q] * e.y);
+            }
+        }
+        fft_pass_all<LOG, -1, 1, 1>(v, gi, 0, sm[rb], g.twx);
+        if (iy < g.ny) {
+            float2* dst = g.g1 + ((size_t)p * g.ny + iy) * L;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) dst[gi[0] + q * S::T] = v[0][q];
+        }
+    }
+}
+
+// Adjoint, rows: g1 transformed back along x; Re(exp(+2 pi i w_p nu) z) summed
+// over the CTA's planes (FP32 over GR_PCH planes) into the chunk's partial slots.
+template <int LOG>
+__global__ void __launch_bounds__(RowShape<LOG>::THREADS, LOG < 12 ? 3 : 1)
+grid_rows_adj_kernel(const DevProblem* __restrict__ probs, int prob, const GridOp g, int p0, int np, int chunk0,
+                     int n_pix, int n_pix_pad, double* __restrict__ partial)
+{
+    using S = RowShape<LOG>;
+    constexpr int L = 1 << LOG;
+    __shared__ float2 sm[S::ROWS][S::PAD];
+    const double2* R;
+    if (!adj_role(probs[prob], R)) return;
+    const int rb = threadIdx.x / S::T;
+    const int gi[1] = {(int)threadIdx.x % S::T};
+    const int iy = blockIdx.x * S::ROWS + rb;
+    float acc[8];
+    float2 nu[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        const int ix = cell_of(gi[0] + q * S::T, LOG, g.cx);
+        acc[q] = 0.f;
+        nu[q] = (iy < g.ny && ix >= 0 && ix < g.nx) ? g.nu[(size_t)iy * g.nx + ix] : make_float2(0.f, 0.f);
+    }
+    const int q1 = min(np, (int)(blockIdx.y + 1) * GR_PCH);
+    for (int p = blockIdx.y * GR_PCH; p < q1; ++p) {
+        const float2 w = g.wp[p0 + p];
+        float2 v[1][8];
+        const float2* src = g.g1 + ((size_t)p * g.ny + min(iy, g.ny - 1)) * L;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {          // columns without a visibility were not written
+            const int e = gi[0] + q * S::T;
+            v[0][q] = g.colact[(size_t)(p0 + p) * (L / GR_TILE) + e / GR_TILE] ? src[e] : make_float2(0.f, 0.f);
+        }
+        fft_pass_all<LOG, 1, 1, 1>(v, gi, 0, sm[rb], g.twx);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const int ix = cell_of(gi[0] + q * S::T, LOG, g.cx);
+            if (ix >= 0 && ix < g.nx) {
+                const float2 e = plane_phase(w, nu[q]);              // conj(e) z, real part
+                acc[q] += fmaf(e.x, v[0][q].x, e.y * v[0][q].y);
+            }
+        }
+    }
+    const int chunk = chunk0 + blockIdx.y;
+    if (iy < g.ny) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const int ix = cell_of(gi[0] + q * S::T, LOG, g.cx);
+            if (ix < 0 || ix >= g.nx) continue;
+            const size_t at = (size_t)iy * g.nx + ix;
+            const int j = g.cell[at];
+            if (j >= 0)
+                partial[((size_t)(j / BLK) * g.n_chunk + chunk) * BLK + j % BLK] =
+                    (double)acc[q] * ((double)g.amp[at] / (double)g.ascale);
+        }
+    }
+    if (blockIdx.x == 0)                       // padding slots of the last pixel granule
+        for (int j = n_pix + threadIdx.x; j < n_pix_pad; j += S::THREADS)
+            partial[((size_t)(j / BLK) * g.n_chunk + chunk) * BLK + j % BLK] = 0.0;
+}
+
+// Columns: CB adjacent columns of one plane per CTA, so a row of the tile is
+// 8 CB contiguous bytes.  Forward (SGN -1): the ny rows of g1, zero-padded,
+// into the 2^LOG rows of g2; adjoint (SGN +1): g2 back, its ny lattice rows
+// into g1.
+template <int LOG>
+struct ColShape {
+    static constexpr int CB = LOG >= 11 ? 4 : 8;
+    static constexpr int NB = LOG >= 12 ? 4 : LOG >= 8 ? 2 : 1;
+    static constexpr int THREADS = CB * (1 << LOG) / 8 / NB;
+    static constexpr int SMEM = padded(1 << LOG, CB) * (int)sizeof(float2);
+};
+template <int LOG, int SGN>
+__global__ void __launch_bounds__(ColShape<LOG>::THREADS, ColShape<LOG>::THREADS >= 512 && LOG < 12 ? 2 : 1)
+grid_cols_kernel(const DevProblem* __restrict__ probs, int prob, const GridOp g, int p0)
+{
+    using S = ColShape<LOG>;
+    constexpr int E = (1 << LOG) / 8;
+    extern __shared__ __align__(16) float2 sm_cols[];
+    __shared__ unsigned char s_act[(1 << LOG) / GR_TILE];      // tiles of these columns with a visibility
+    if (SGN < 0) {
+        const double* X;
+        if (!fwd_role(probs[prob], X)) return;
+    } else {
+        const double2* R;
+        if (!adj_role(probs[prob], R)) return;
+    }
+    {
+        const int ty = (1 << LOG) / GR_TILE;
+        const unsigned char* act = g.act + ((size_t)(p0 + blockIdx.y) * ((1 << g.lx) / GR_TILE) +
+                                            blockIdx.x * S::CB / GR_TILE) * ty;
+        int any = 0;
+        for (int t = threadIdx.x; t < ty; t += S::THREADS) any |= (s_act[t] = act[t]);
+        if (!__syncthreads_or(any)) return;
+    }
+    const int c = threadIdx.x % S::CB;
+    int gi[S::NB];
+#pragma unroll
+    for (int n = 0; n < S::NB; ++n) gi[n] = threadIdx.x / S::CB + n * (E / S::NB);
+    const size_t col = (size_t)blockIdx.x * S::CB + c, Lx = (size_t)1 << g.lx;
+    float2* g1 = g.g1 + (size_t)blockIdx.y * g.ny * Lx + col;
+    float2* g2 = g.g2 + ((size_t)blockIdx.y << LOG) * Lx + col;
+    float2 v[S::NB][8];
+#pragma unroll
+    for (int n = 0; n < S::NB; ++n)
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const int e = gi[n] + q * E;
+            if (SGN < 0) {
+                const int iy = cell_of(e, LOG, g.cy);
+                v[n][q] = (iy >= 0 && iy < g.ny) ? g1[(size_t)iy * Lx] : make_float2(0.f, 0.f);
+            } else {
+                v[n][q] = s_act[e / GR_TILE] ? g2[(size_t)e * Lx] : make_float2(0.f, 0.f);
+            }
+        }
+    fft_pass_all<LOG, SGN, S::CB, S::NB>(v, gi, c, sm_cols, g.twy);
+#pragma unroll
+    for (int n = 0; n < S::NB; ++n)
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const int e = gi[n] + q * E;
+            if (SGN < 0) {
+                if (s_act[e / GR_TILE]) g2[(size_t)e * Lx] = v[n][q];
+            } else {
+                const int iy = cell_of(e, LOG, g.cy);
+                if (iy >= 0 && iy < g.ny) g1[(size_t)iy * Lx] = v[n][q];
+            }
+        }
+}
+
+// ------------------------------------------------- gathering and spreading
+
+// Forward: each visibility from its 8 x 8 cells of 8 planes, one warp per
+// visibility (lane = 8 cells in x by 4 rows, twice): a plane's share is 8
+// segments of 64 bytes, and visibilities in k-d order share them in L1 / L2.
+__global__ void __launch_bounds__(256)
+grid_gather_kernel(const DevProblem* __restrict__ probs, int prob, const GridOp g, int p0, int np, int n_vis_pad,
+                   double2* __restrict__ partial)
+{
+    const double* X;
+    if (!fwd_role(probs[prob], X)) return;
+    const int k = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (k >= n_vis_pad) return;
+    const int4 ps = g.pos[k];
+    const float* wt = g.wts + (size_t)k * (3 * GRW);
+    const int tx = lane & 7, ty = lane >> 3;
+    const int Lx = 1 << g.lx, Ly = 1 << g.ly;
+    const int x = (ps.x + tx) & (Lx - 1);
+    const size_t y0 = (size_t)((ps.y + ty) & (Ly - 1)) * Lx + x, y1 = (size_t)((ps.y + ty + 4) & (Ly - 1)) * Lx + x;
+    const float wx = wt[tx], wy0 = wt[GRW + ty], wy1 = wt[GRW + ty + 4];
+    float2 s0 = make_float2(0.f, 0.f), s1 = s0;
+#pragma unroll
+    for (int t = 0; t < GRW; ++t) {
+        const int p = ps.z + t - p0;
+        if (p < 0 || p >= np) continue;
+        const float ww = wt[2 * GRW + t];
+        const float2* pl = g.g2 + (size_t)p * Ly * Lx;
+        const float2 a = pl[y0], b = pl[y1];
+        s0.x = fmaf(ww, a.x, s0.x);
+        s0.y = fmaf(ww, a.y, s0.y);
+        s1.x = fmaf(ww, b.x, s1.x);
+        s1.y = fmaf(ww, b.y, s1.y);
+    }
+    float sr = wx * fmaf(wy0, s0.x, wy1 * s1.x), si = wx * fmaf(wy0, s0.y, wy1 * s1.y);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        sr += __shfl_xor_sync(0xffffffffu, sr, o);
+        si += __shfl_xor_sync(0xffffffffu, si, o);
+    }
+    if (lane == 0) {
+        const float2 e = g.rot[k];
+        const double inv = 1.0 / (double)g.fscale;
+        double2 v = make_double2((double)fmaf(e.x, sr, -e.y * si) * inv, (double)fmaf(e.x, si, e.y * sr) * inv);
+        if (ps.w) v.y = -v.y;                  // taken at the mirrored point
+        if (p0 > 0) {                          // a later pass over the planes
+            const double2 o = partial[k];
+            v.x += o.x;
+            v.y += o.y;
+        }
+        partial[k] = v;
+    }
+}
+
+// Adjoint: a CTA owns GR_TILE^2 cells (one per thread) of GR_PCH planes and
+// adds the visibilities that touch them in list order: no atomics, the same
+// sum every time.  Each point's x, y weights times conj(rot) r are formed once
+// for the 8 planes.
+__global__ void __launch_bounds__(GR_TILE * GR_TILE)
+grid_spread_kernel(const DevProblem* __restrict__ probs, int prob, const GridOp g, int p0, int np)
+{
+    constexpr int PB = 32;                     // points staged at a time
+    __shared__ float4 s_pt[PB];                // {Re, Im of conj(rot) r, first x, first y}
+    __shared__ float s_wx[PB][GRW], s_wy[PB][GRW], s_ww[PB][GR_PCH];
+    const double2* R;
+    if (!adj_role(probs[prob], R)) return;
+    const int Lx = 1 << g.lx, Ly = 1 << g.ly, tiles_x = Lx / GR_TILE;
+    const int tile = blockIdx.x;
+    const int x = (tile % tiles_x) * GR_TILE + (threadIdx.x % GR_TILE);
+    const int y = (tile / tiles_x) * GR_TILE + (threadIdx.x / GR_TILE);
+    const int q0 = blockIdx.y * GR_PCH;        // first plane of the CTA within the pass
+    const int pg = p0 + q0;                    // ... and of all
+    const int ni = g.np - GRW + 1;             // values of a first plane
+    const int* st = g.start + (size_t)tile * (ni + 1);
+    const int i0 = max(0, min(ni, pg - GRW + 1)), i1 = max(i0, min(ni, pg + GR_PCH));
+    const int b0 = st[i0], b1 = st[i1];
+    if (b0 == b1) return;                      // no plane of the CTA is touched here
+    float2 acc[GR_PCH];
+#pragma unroll
+    for (int q = 0; q < GR_PCH; ++q) acc[q] = make_float2(0.f, 0.f);
+    for (int b = b0; b < b1; b += PB) {
+        const int n = min(PB, b1 - b);
+        __syncthreads();
+        for (int e = threadIdx.x; e < n * 32; e += GR_TILE * GR_TILE) {
+            const int i = e >> 5, f = e & 31;
+            const int k = g.list[b + i];
+            const float* wt = g.wts + (size_t)k * (3 * GRW);
+            if (f < 8) {
+                s_wx[i][f] = wt[f];
+            } else if (f < 16) {
+                s_wy[i][f - 8] = wt[f];
+            } else if (f < 24) {
+                const int t = pg + (f - 16) - g.pos[k].z;
+                s_ww[i][f - 16] = (t >= 0 && t < GRW) ? wt[2 * GRW + t] : 0.f;
+            } else if (f == 24) {
+                const int4 ps = g.pos[k];
+                const float2 o = g.rot[k];
+                const double2 r = R[k];
+                const float rr = (float)r.x * g.ascale, ri = (float)(ps.w ? -r.y : r.y) * g.ascale;
+                s_pt[i] = make_float4(fmaf(o.x, rr, o.y * ri), fmaf(o.x, ri, -o.y * rr), __int_as_float(ps.x),
+                                      __int_as_float(ps.y));
+            }
+        }
+        __syncthreads();
+        for (int i = 0; i < n; ++i) {
+            const float4 pt = s_pt[i];
+            const int dx = (x - __float_as_int(pt.z)) & (Lx - 1), dy = (y - __float_as_int(pt.w)) & (Ly - 1);
+            if (dx < GRW && dy < GRW) {
+                const float w = s_wx[i][dx] * s_wy[i][dy];
+                const float vr = w * pt.x, vi = w * pt.y;
+#pragma unroll
+                for (int q = 0; q < GR_PCH; ++q) {
+                    const float ww = s_ww[i][q];
+                    acc[q].x = fmaf(ww, vr, acc[q].x);
+                    acc[q].y = fmaf(ww, vi, acc[q].y);
+                }
+            }
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < GR_PCH; ++q)
+        if (q0 + q < np) g.g2[((size_t)(q0 + q) * Ly + y) * Lx + x] = acc[q];
+}
+
+// ------------------------------------------------------------------ set-up
+
+__device__ __forceinline__ double es_kernel(double z)      // z in cells from the centre
+{
+    const double t = 2.0 * z / GRW, s = 1.0 - t * t;
+    return s > 0.0 ? exp(GR_BETA * (sqrt(s) - 1.0)) : 0.0;
+}
+
+__global__ void grid_setup_vis_kernel(const d4* __restrict__ vd, int n_pad, GridOp g, double dl, double dm, double lc,
+                                      double mc, double nc, double w0, double dw, int4* __restrict__ pos,
+                                      float* __restrict__ wts, float2* __restrict__ rot)
+{
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= n_pad) return;
+    d4 v = vd[k];
+    const bool mirror = v.z < 0.0;
+    if (mirror) v = make_d4(-v.x, -v.y, -v.z, v.w);
+    const int Lx = 1 << g.lx, Ly = 1 << g.ly;
+    const double tx = v.x * dl, ty = v.y * dm;
+    const double gx = (tx - floor(tx)) * Lx, gy = (ty - floor(ty)) * Ly, gw = (v.z - w0) / dw;
+    const double ix = ceil(gx - 0.5 * GRW), iy = ceil(gy - 0.5 * GRW);
+    const double iw = fmin(fmax(ceil(gw - 0.5 * GRW), 0.0), (double)(g.np - GRW));
+    pos[k] = make_int4((int)ix & (Lx - 1), (int)iy & (Ly - 1), (int)iw, mirror ? 1 : 0);
+    for (int t = 0; t < GRW; ++t) {
+        wts[(size_t)k * 3 * GRW + t] = (float)es_kernel(ix + t - gx);
+        wts[(size_t)k * 3 * GRW + GRW + t] = (float)es_kernel(iy + t - gy);
+        wts[(size_t)k * 3 * GRW + 2 * GRW + t] = (float)es_kernel(iw + t - gw);
+    }
+    double a = v.x * lc, b = v.y * mc, c = v.z * nc;
+    a -= rint(a);
+    b -= rint(b);
+    c -= rint(c);
+    double s, co;
+    sincospi(2.0 * (a + b + c), &s, &co);
+    rot[k] = make_float2((float)co, (float)-s);
+}
+
+// amp = (1/n) / (transforms of the kernel in x, y and w); cxy: [nx] then [ny]
+// reciprocal transforms, quad: GR_NQ nodes (cells) and weights times the
+// kernel, for the transform in w.
+__global__ void grid_setup_cells_kernel(const d4* __restrict__ pd, GridOp g, const double* __restrict__ cxy,
+                                        const double* __restrict__ quad, double nc, double dw, float* __restrict__ amp,
+                                        float2* __restrict__ nu)
+{
+    const size_t n = (size_t)g.nx * g.ny;
+    for (size_t at = (size_t)blockIdx.x * blockDim.x + threadIdx.x; at < n; at += (size_t)gridDim.x * blockDim.x) {
+        const int j = g.cell[at];
+        if (j < 0) {
+            amp[at] = 0.f;
+            nu[at] = make_float2(0.f, 0.f);
+            continue;
+        }
+        const d4 d = pd[j];
+        const double v = d.z - nc, xi = v * dw;
+        double hat = 0.0;
+        for (int q = 0; q < GR_NQ; ++q) hat += quad[GR_NQ + q] * cospi(2.0 * xi * quad[q]);
+        hat *= 2.0;
+        amp[at] = (float)(d.w * cxy[at % g.nx] * cxy[g.nx + at / g.nx] / hat);
+        const float hi = (float)v;
+        nu[at] = make_float2(hi, (float)(v - (double)hi));
+    }
+}
+
+cudaError_t grid_setup_vis(const d4* vd, int n_pad, GridOp g, double dl, double dm, double lc, double mc, double nc,
+                           double w0, double dw, int4* pos, float* wts, float2* rot, cudaStream_t st)
+{
+    grid_setup_vis_kernel<<<(n_pad + 127) / 128, 128, 0, st>>>(vd, n_pad, g, dl, dm, lc, mc, nc, w0, dw, pos, wts,
+                                                               rot);
+    return cudaGetLastError();
+}
+cudaError_t grid_setup_cells(const d4* pd, GridOp g, const double* cxy, const double* quad, double nc, double dw,
+                             float* amp, float2* nu, cudaStream_t st)
+{
+    const size_t n = (size_t)g.nx * g.ny;
+    grid_setup_cells_kernel<<<(unsigned)std::min<size_t>(4096, (n + 127) / 128), 128, 0, st>>>(pd, g, cxy, quad, nc,
+                                                                                               dw, amp, nu);
+    return cudaGetLastError();
+}
+
+// ---------------------------------------------------------------- launchers
+
+template <int LOG>
+static void rows_fwd(const DevProblem* probs, int p, const GridOp& g, int p0, int np, cudaStream_t st)
+{
+    using S = RowShape<LOG>;
+    const dim3 grid((unsigned)((g.ny + S::ROWS - 1) / S::ROWS), (unsigned)((np + GR_PCH - 1) / GR_PCH));
+    grid_rows_fwd_kernel<LOG><<<grid, S::THREADS, 0, st>>>(probs, p, g, p0, np);
+}
+template <int LOG>
+static void rows_adj(const DevProblem* probs, int p, const GridOp& g, int p0, int np, int chunk0, int n_pix,
+                     int n_pix_pad, double* partial, cudaStream_t st)
+{
+    using S = RowShape<LOG>;
+    const dim3 grid((unsigned)((g.ny + S::ROWS - 1) / S::ROWS), (unsigned)((np + GR_PCH - 1) / GR_PCH));
+    grid_rows_adj_kernel<LOG><<<grid, S::THREADS, 0, st>>>(probs, p, g, p0, np, chunk0, n_pix, n_pix_pad, partial);
+}
+template <int LOG, int SGN>
+static void cols(const DevProblem* probs, int p, const GridOp& g, int p0, int np, cudaStream_t st)
+{
+    using S = ColShape<LOG>;
+    const dim3 grid((1u << g.lx) / S::CB, (unsigned)np);
+    grid_cols_kernel<LOG, SGN><<<grid, S::THREADS, S::SMEM, st>>>(probs, p, g, p0);
+}
+
+// Calls F<LOG>::go(args...) for the run-time length lg.
+#define GRID_DISPATCH(lg, CALL)                  \
+    switch (lg) {                                \
+    case 6: { constexpr int LOG = 6; CALL; break; }   \
+    case 7: { constexpr int LOG = 7; CALL; break; }   \
+    case 8: { constexpr int LOG = 8; CALL; break; }   \
+    case 9: { constexpr int LOG = 9; CALL; break; }   \
+    case 10: { constexpr int LOG = 10; CALL; break; } \
+    case 11: { constexpr int LOG = 11; CALL; break; } \
+    case 12: { constexpr int LOG = 12; CALL; break; } \
+    default: return cudaErrorInvalidValue;       \
+    }
+
+cudaError_t grid_forward(const DevProblem* probs, int p, const GridOp& g, int n_vis_pad, double2* partial,
+                         cudaStream_t st, long long* n_launch)
+{
+    for (int p0 = 0; p0 < g.np; p0 += g.np_pass) {
+        const int np = std::min(g.np_pass, g.np - p0);
+        GRID_DISPATCH(g.lx, (rows_fwd<LOG>(probs, p, g, p0, np, st)));
+        GRID_DISPATCH(g.ly, (cols<LOG, -1>(probs, p, g, p0, np, st)));
+        grid_gather_kernel<<<(n_vis_pad + 7) / 8, 256, 0, st>>>(probs, p, g, p0, np, n_vis_pad, partial);
+        *n_launch += 3;
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+cudaError_t grid_adjoint(const DevProblem* probs, int p, const GridOp& g, int n_pix, int n_pix_pad, double* partial,
+                         cudaStream_t st, long long* n_launch)
+{
+    for (int p0 = 0; p0 < g.np; p0 += g.np_pass) {
+        const int np = std::min(g.np_pass, g.np - p0);
+        const dim3 sg((unsigned)grid_tiles(g), (unsigned)((np + GR_PCH - 1) / GR_PCH));
+        grid_spread_kernel<<<sg, GR_TILE * GR_TILE, 0, st>>>(probs, p, g, p0, np);
+        GRID_DISPATCH(g.ly, (cols<LOG, 1>(probs, p, g, p0, np, st)));
+        GRID_DISPATCH(g.lx, (rows_adj<LOG>(probs, p, g, p0, np, p0 / GR_PCH, n_pix, n_pix_pad, partial, st)));
+        *n_launch += 3;
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+template <int LOG>
+static cudaError_t raise_cols()
+{
+    cudaError_t e = cudaFuncSetAttribute(grid_cols_kernel<LOG, -1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         ColShape<LOG>::SMEM);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(grid_cols_kernel<LOG, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                ColShape<LOG>::SMEM);
+}
+cudaError_t grid_prepare_kernels()
+{
+    for (int lg = GR_LOG_MIN; lg <= GR_LOG_MAX; ++lg) {
+        cudaError_t e = cudaSuccess;
+        GRID_DISPATCH(lg, (e = raise_cols<LOG>()));
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+}  // namespace sl1m

@@ -113,33 +113,6 @@ static int kd_par_depth()
     return d;
 }
 
-// Run fn(lo, hi) over [0, n) cut into contiguous chunks, one per host thread
-// (at most 16), when n is large enough to pay for the threads.  For loops whose
-// iterations write only their own outputs: the result is the one a single
-// thread gives.
-template <class F>
-static void parallel_chunks(size_t n, size_t min_per_chunk, const F& fn)
-{
-    const size_t t = std::min<size_t>(16, std::max(1u, std::thread::hardware_concurrency()));
-    const size_t nc = std::max<size_t>(1, std::min(t, n / std::max<size_t>(1, min_per_chunk)));
-    if (nc <= 1) {
-        fn((size_t)0, n);
-        return;
-    }
-    std::vector<std::future<void>> fs;
-    size_t done = 0;                       // chunks [0, done) run on threads
-    try {
-        for (size_t c = 1; c < nc; ++c) {
-            fs.push_back(std::async(std::launch::async, [&fn, n, nc, c] { fn(n * c / nc, n * (c + 1) / nc); }));
-            done = c;
-        }
-    } catch (...) {                        // no thread to be had: the rest runs here
-    }
-    fn(0, n / nc);
-    for (size_t c = done + 1; c < nc; ++c) fn(n * c / nc, n * (c + 1) / nc);
-    for (auto& f : fs) f.get();
-}
-
 // Append `members` (caller indices) in k-d order, padded with -1 to a
 // multiple of G.
 static void kd_append(std::vector<int>& order, std::vector<int> members, const double* x,
@@ -419,6 +392,11 @@ cudaError_t build_plan(const std::vector<int>& nb, const std::vector<int>& ns, i
 {
     HostPlan H;
     plan_host(nb, ns, Cmax, H, costs);
+    return upload_plan(H, (int)nb.size(), D, st);
+}
+
+cudaError_t upload_plan(const HostPlan& H, int n_probs, DevPlan& D, cudaStream_t st)
+{
     cudaError_t err;
     auto up = [&](DBuf<int>& b, const std::vector<int>& v) {
         return b.upload(v.data(), std::max<size_t>(1, v.size()), st, v.empty());
@@ -433,7 +411,7 @@ cudaError_t build_plan(const std::vector<int>& nb, const std::vector<int>& ns, i
     } else {
         D.cta.free();
     }
-    D.pl.n_probs = (int)nb.size();
+    D.pl.n_probs = n_probs;
     D.pl.C = H.C;
     D.pl.U = H.U;
     D.pl.prob_u0 = D.u0.p;
@@ -545,7 +523,7 @@ struct ProblemDev {
 
 sl1m_problem::~sl1m_problem() = default;
 
-int sl1m_problem::rebuild(cudaStream_t st)
+int sl1m_problem::rebuild(cudaStream_t st, size_t grid_budget)
 {
     if (!dirty) return SL1M_OK;
     if (n_vis <= 0 || n_pix <= 0)
@@ -758,12 +736,16 @@ int sl1m_problem::rebuild(cudaStream_t st)
     hp.fwd_out = nullptr;
     hp.adj_out = nullptr;
     hp.st = nullptr;
+    grid.reset();
     ctx->h2d += (long long)dev_bytes();
     for (auto& b : op_batch) b.reset();
     for (auto& b : solve_batch) b.reset();
     for (auto& r : ucost_ok) r[0] = r[1] = false;
     solver_ready = false;
     dirty = false;
+    ++gen;
+    if (grid_build(*this, st, grid_budget))
+        ctx->h2d += (long long)(grid->cell.bytes() + grid->list.bytes() + grid->start.bytes());
     return SL1M_OK;
 }
 
@@ -958,6 +940,7 @@ size_t sl1m_problem::dev_bytes() const
     b += D.I0.bytes() + D.I1.bytes() + D.y.bytes() + D.xv.bytes() + D.blk_r2.bytes() + D.blk_l1.bytes() +
          D.blk_z2.bytes() + D.AI0.bytes() + D.AI1.bytes() + D.rr.bytes() + D.blk_nnz.bytes() +
          D.blk_badv.bytes() + D.blk_badp.bytes() + D.st.bytes();
+    if (grid) b += grid->bytes();
     return b;
 }
 
@@ -976,7 +959,44 @@ Batch::~Batch()
     if (gexec) cudaGraphExecDestroy(gexec);
 }
 
-// Set the problems of a batch: descriptors, per (op, gains class) plans,
+// The lattice class's part of a batch: block tables for the finish kernels (one
+// partial slot per visibility block, n_chunk per pixel block; no units, the
+// lattice kernels have grids of their own).
+static int set_grid_plans(sl1m_ctx* ctx, Batch& B, const std::vector<DevProblem>& descs)
+{
+    const int np = (int)descs.size();
+    for (int op = 0; op < 2; ++op) {
+        HostPlan H;
+        H.u0.assign(np + 1, 0);
+        H.b0.assign(np + 1, 0);
+        B.grid_slot[op].assign(np, 0);
+        for (int p = 0; p < np; ++p) {
+            const bool in = B.cls[p] == CLS_GRID;
+            const int nb = !in ? 0 : op == 0 ? descs[p].vis.n_blk : descs[p].pix.n_blk;
+            const int nc = !in ? 0 : op == 0 ? 1 : B.probs[p]->grid->op.n_chunk;
+            B.grid_slot[op][p] = H.n_slots;
+            for (int b = 0; b < nb; ++b) {
+                H.poff.push_back(H.n_slots);
+                H.clo.push_back(0);
+                H.ncon.push_back(nc);
+                H.n_slots += nc;
+            }
+            H.b0[p + 1] = H.b0[p] + nb;
+            if (in && op == 0) {
+                B.has_class[CLS_GRID] = true;
+                B.pairs_class[CLS_GRID] += B.probs[p]->pairs();
+            }
+        }
+        H.n_blocks = H.b0[np];
+        CK(upload_plan(H, np, B.plan[op][CLS_GRID], ctx->stream));
+        if (op == 0) CK(ctx->partial_f.reserve((size_t)std::max(1, H.n_slots) * BLK, ctx->stream));
+        else CK(ctx->partial_a.reserve((size_t)std::max(1, H.n_slots) * BLK, ctx->stream));
+        B.fin_bytes[op] += (double)H.n_slots * BLK * (op == 0 ? 16.0 : 8.0);
+    }
+    return SL1M_OK;
+}
+
+// Set the problems of a batch: descriptors, per (op, class) plans,
 // partial-sum scratch.  The captured tick stays valid while every pointer it
 // bakes in (tables, scratch) is unchanged.
 int batch_set(sl1m_ctx* ctx, Batch& B, const std::vector<sl1m_problem*>& probs,
@@ -985,9 +1005,12 @@ int batch_set(sl1m_ctx* ctx, Batch& B, const std::vector<sl1m_problem*>& probs,
     cudaStream_t st = ctx->stream;
     const int np = (int)probs.size();
     if (np == 0) return sl1m_fail(ctx, SL1M_ERR_ARG, "empty batch");
-    const void* old_ptrs[6] = {B.desc.p, ctx->partial_f.p, ctx->partial_a.p, B.n_probs_dev.p,
-                               B.plan[0][0].dpl.p, B.plan[1][1].dpl.p};
-    const bool same_set = B.probs == probs && B.precision == precision && B.solver == solver;
+    const void* old_ptrs[7] = {B.desc.p, ctx->partial_f.p, ctx->partial_a.p, B.n_probs_dev.p,
+                               B.plan[0][0].dpl.p, B.plan[1][1].dpl.p, ctx->grid_ws.p};
+    std::vector<uint64_t> gens(np);
+    for (int p = 0; p < np; ++p) gens[p] = probs[p]->gen;
+    const bool same_set =
+        B.probs == probs && B.precision == precision && B.solver == solver && B.gens == gens;
     B.precision = precision;
     B.solver = solver;
     B.probs = probs;
@@ -998,15 +1021,28 @@ int batch_set(sl1m_ctx* ctx, Batch& B, const std::vector<sl1m_problem*>& probs,
     CK(cudaMemcpyAsync(B.n_probs_dev.p, &np, sizeof(int), cudaMemcpyHostToDevice, st));
     if (B.phases_dev.n < (size_t)np) CK(B.phases_dev.reserve(np, st));
     if (!same_set) {
-        B.has_class[0] = B.has_class[1] = false;
+        B.gens = gens;
         B.n_ant_max = 0;
-        B.pairs_class[0] = B.pairs_class[1] = 0;
+        for (int c = 0; c < N_CLS; ++c) {
+            B.has_class[c] = false;
+            B.pairs_class[c] = 0;
+        }
         B.fin_bytes[0] = B.fin_bytes[1] = 0;
+        // a lattice problem whose workspace cannot be had takes the pair kernels
+        B.cls.assign(np, CLS_PAIRS);
+        for (int p = 0; p < np; ++p) {
+            if (probs[p]->n_ant > 0) {
+                B.cls[p] = CLS_GAINS;
+            } else if (precision != 0 && probs[p]->grid) {
+                if (ctx->grid_ws.reserve(probs[p]->grid->ws_elems, st) == cudaSuccess) B.cls[p] = CLS_GRID;
+                else cudaGetLastError();
+            }
+        }
+        RET(set_grid_plans(ctx, B, descs));
         for (int c = 0; c < 2; ++c) {
             std::vector<int> nbf(np), nsf(np), nba(np), nsa(np);
             for (int p = 0; p < np; ++p) {
-                const bool g = probs[p]->n_ant > 0;
-                const bool in = (c == 1) == g;
+                const bool g = c == CLS_GAINS, in = B.cls[p] == c;
                 const DevProblem& d = descs[p];
                 nbf[p] = in ? d.vis.n_blk : 0;
                 nsf[p] = in ? d.pix.n_gran : 0;
@@ -1061,8 +1097,8 @@ int batch_set(sl1m_ctx* ctx, Batch& B, const std::vector<sl1m_problem*>& probs,
         B.fin_grid = std::max(1, std::min(4 * ctx->num_sms, nblk * np));
         B.sc_grid = std::max(1, std::min(ctx->num_sms * 4, np));
     }
-    const void* new_ptrs[6] = {B.desc.p, ctx->partial_f.p, ctx->partial_a.p, B.n_probs_dev.p,
-                               B.plan[0][0].dpl.p, B.plan[1][1].dpl.p};
+    const void* new_ptrs[7] = {B.desc.p, ctx->partial_f.p, ctx->partial_a.p, B.n_probs_dev.p,
+                               B.plan[0][0].dpl.p, B.plan[1][1].dpl.p, ctx->grid_ws.p};
     if (!same_set || memcmp(old_ptrs, new_ptrs, sizeof old_ptrs) != 0) B.graph_ok = false;
     return SL1M_OK;
 }
@@ -1073,26 +1109,50 @@ static int launch_op_class(sl1m_ctx* ctx, Batch& B, int op, int c)
     cudaStream_t st = ctx->stream;
     const DevPlan& P = B.plan[op][c];
     ProfTok tk;
+    // the lattice operators, problem by problem: each fills the GPU by itself
+    // and they share the context's workspace in stream order
+    const auto each_grid = [&](const auto& f) -> int {
+        for (size_t p = 0; p < B.probs.size(); ++p) {
+            if (B.cls[p] != CLS_GRID) continue;
+            GridOp g = B.probs[p]->grid->op;
+            g.g1 = ctx->grid_ws.p;
+            g.g2 = g.g1 + (((size_t)g.np_pass * g.ny) << g.lx);
+            CK(f((int)p, g));
+        }
+        return SL1M_OK;
+    };
     if (op == 0) {
         prof_begin(ctx, B.precision == 0 ? 0 : 2, tk);
-        CKL(launch_forward(B.precision, c == 1, B.n_ant_max, B.desc.p, P.dpl.p, P.pl.C, ctx->partial_f.p, st,
-                           B.nst[0][c]));
+        if (c == CLS_GRID)
+            RET(each_grid([&](int p, const GridOp& g) {
+                return grid_forward(B.desc.p, p, g, B.hdesc[p].vis.n_pad,
+                                    ctx->partial_f.p + (size_t)B.grid_slot[0][p] * BLK, st, &ctx->n_launch);
+            }));
+        else
+            CKL(launch_forward(B.precision, c == 1, B.n_ant_max, B.desc.p, P.dpl.p, P.pl.C, ctx->partial_f.p, st,
+                               B.nst[0][c]));
         prof_end(ctx, tk, B.solver ? 0.0 : B.pairs_class[c], 0.0);   // solver ticks: counted on the device
         prof_begin(ctx, 4, tk);
         CKL(launch_fwd_finish(B.desc.p, P.dpl.p, std::min(B.fin_grid, std::max(1, P.pl.n_blocks)),
                               ctx->partial_f.p, st));
         prof_end(ctx, tk, 0.0, B.fin_bytes[0]);
     } else {
-        // the mixed adjoints read r in polar form, written once for the whole
-        // batch before its first class
-        if (B.precision != 0 && (c == 0 || !B.has_class[0])) {
+        // the mixed pair adjoints read r in polar form, written once for the
+        // whole batch before its first class
+        if (B.precision != 0 && c != CLS_GRID && (c == 0 || !B.has_class[0])) {
             int vmax = 1;
             for (const DevProblem& d : B.hdesc) vmax = std::max(vmax, d.vis.n_pad);
             CKL(launch_r32(B.desc.p, (int)B.hdesc.size(), vmax, st));
         }
         prof_begin(ctx, B.precision == 0 ? 1 : 3, tk);
-        CKL(launch_adjoint(B.precision, c == 1, B.n_ant_max, B.desc.p, P.dpl.p, P.pl.C, ctx->partial_a.p, st,
-                           B.nst[1][c]));
+        if (c == CLS_GRID)
+            RET(each_grid([&](int p, const GridOp& g) {
+                return grid_adjoint(B.desc.p, p, g, B.hdesc[p].pix.n, B.hdesc[p].pix.n_pad,
+                                    ctx->partial_a.p + (size_t)B.grid_slot[1][p] * BLK, st, &ctx->n_launch);
+            }));
+        else
+            CKL(launch_adjoint(B.precision, c == 1, B.n_ant_max, B.desc.p, P.dpl.p, P.pl.C, ctx->partial_a.p, st,
+                               B.nst[1][c]));
         prof_end(ctx, tk, B.solver ? 0.0 : B.pairs_class[c], 0.0);
         prof_begin(ctx, 5, tk);
         CKL(launch_adj_finish(B.desc.p, P.dpl.p, std::min(B.fin_grid, std::max(1, P.pl.n_blocks)),
@@ -1105,7 +1165,7 @@ static int launch_op_class(sl1m_ctx* ctx, Batch& B, int op, int c)
 // One operator application (operator-mode batch): forward or adjoint.
 int batch_op(sl1m_ctx* ctx, Batch& B, int op)
 {
-    for (int c = 0; c < 2; ++c) RET(launch_op_class(ctx, B, op, c));
+    for (int c = 0; c < N_CLS; ++c) RET(launch_op_class(ctx, B, op, c));
     return SL1M_OK;
 }
 
@@ -1113,8 +1173,8 @@ int batch_op(sl1m_ctx* ctx, Batch& B, int op)
 // forward, forward finish (per gains class), then the phase machine.
 static int enqueue_tick(sl1m_ctx* ctx, Batch& B)
 {
-    for (int c = 0; c < 2; ++c) RET(launch_op_class(ctx, B, 1, c));
-    for (int c = 0; c < 2; ++c) RET(launch_op_class(ctx, B, 0, c));
+    for (int c = 0; c < N_CLS; ++c) RET(launch_op_class(ctx, B, 1, c));
+    for (int c = 0; c < N_CLS; ++c) RET(launch_op_class(ctx, B, 0, c));
     // while profiling (ticks are launched directly then, never captured) the
     // scalars kernel counts the pairs the tick evaluated
     double* ev = (ctx->prof && B.solver && ctx->evals_dev.p) ? ctx->evals_dev.p + 2 * (B.precision != 0) : nullptr;
@@ -1122,7 +1182,7 @@ static int enqueue_tick(sl1m_ctx* ctx, Batch& B)
     if (B.has_mfista) {
         ProfTok tk;
         prof_begin(ctx, 6, tk);
-        for (int c = 0; c < 2; ++c) {
+        for (int c = 0; c < N_CLS; ++c) {
             if (!B.has_class[c]) continue;
             const int nb = B.plan[0][c].pl.n_blocks + B.plan[1][c].pl.n_blocks;
             CKL(launch_mfista_mix(B.desc.p, B.plan[0][c].dpl.p, B.plan[1][c].dpl.p,
@@ -1152,7 +1212,8 @@ int batch_ticks(sl1m_ctx* ctx, Batch& B, int n)
     // larger batch (another problem's solve or operator call, the autotuner)
     // may have reallocated since: capture again rather than replay with a
     // freed buffer.  The scratch only grows, so it still fits this batch.
-    if (B.graph_ok && (B.cap_partial[0] != ctx->partial_f.p || B.cap_partial[1] != ctx->partial_a.p))
+    if (B.graph_ok && (B.cap_partial[0] != ctx->partial_f.p || B.cap_partial[1] != ctx->partial_a.p ||
+                       B.cap_partial[2] != ctx->grid_ws.p))
         B.graph_ok = false;
     if (!B.graph_ok) {
         if (B.gexec) {
@@ -1176,6 +1237,7 @@ int batch_ticks(sl1m_ctx* ctx, Batch& B, int n)
         B.graph_ok = true;
         B.cap_partial[0] = ctx->partial_f.p;
         B.cap_partial[1] = ctx->partial_a.p;
+        B.cap_partial[2] = ctx->grid_ws.p;
         B.tick_launches = ctx->n_launch - l0;
         ctx->n_launch = l0;
     }

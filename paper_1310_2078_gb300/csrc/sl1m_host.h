@@ -2,14 +2,19 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <algorithm>
+#include <cstdint>
+#include <future>
 #include <map>
 #include <memory>
 #include <mutex>
 #include <string>
+#include <thread>
 #include <vector>
 
 #include "sl1m.h"
 #include "sl1m_dev.h"
+#include "sl1m_grid.h"
 
 // Device buffer owned by the library (cudaMalloc / cudaFree).
 template <class T>
@@ -59,6 +64,33 @@ struct DBuf {
     size_t bytes() const { return n * sizeof(T); }
 };
 
+// Run fn(lo, hi) over [0, n) cut into contiguous chunks, one per host thread
+// (at most 16), when n is large enough to pay for the threads.  For loops whose
+// iterations write only their own outputs: the result is the one a single
+// thread gives.
+template <class F>
+static inline void parallel_chunks(size_t n, size_t min_per_chunk, const F& fn)
+{
+    const size_t t = std::min<size_t>(16, std::max(1u, std::thread::hardware_concurrency()));
+    const size_t nc = std::max<size_t>(1, std::min(t, n / std::max<size_t>(1, min_per_chunk)));
+    if (nc <= 1) {
+        fn((size_t)0, n);
+        return;
+    }
+    std::vector<std::future<void>> fs;
+    size_t done = 0;                       // chunks [0, done) run on threads
+    try {
+        for (size_t c = 1; c < nc; ++c) {
+            fs.push_back(std::async(std::launch::async, [&fn, n, nc, c] { fn(n * c / nc, n * (c + 1) / nc); }));
+            done = c;
+        }
+    } catch (...) {                        // no thread to be had: the rest runs here
+    }
+    fn(0, n / nc);
+    for (size_t c = done + 1; c < nc; ++c) fn(n * c / nc, n * (c + 1) / nc);
+    for (auto& f : fs) f.get();
+}
+
 struct HostPlan {
     std::vector<long long> u0;
     std::vector<int> b0, poff, clo, ncon;
@@ -90,6 +122,29 @@ struct DevPlan {
 cudaError_t build_plan(const std::vector<int>& nb, const std::vector<int>& ns, int Cmax, DevPlan& D,
                        cudaStream_t st, const std::vector<const UnitCost*>* costs = nullptr);
 
+// Uploads a host plan's tables and header.
+cudaError_t upload_plan(const HostPlan& H, int n_probs, DevPlan& D, cudaStream_t st);
+
+// A problem's lattice operator: its tables, and the workspace it needs (the
+// context's, shared by every problem of its stream).
+struct GridTables {
+    sl1m::GridOp op{};
+    size_t ws_elems = 0;                 // float2 of workspace
+    DBuf<int> cell, list, start;
+    DBuf<float> amp, wts;
+    DBuf<float2> nu, wp, twx, twy, rot;
+    DBuf<int4> pos;
+    DBuf<unsigned char> act, colact;
+    size_t bytes() const
+    {
+        return cell.bytes() + list.bytes() + start.bytes() + amp.bytes() + wts.bytes() + nu.bytes() + wp.bytes() +
+               twx.bytes() + twy.bytes() + rot.bytes() + pos.bytes() + act.bytes() + colact.bytes();
+    }
+};
+constexpr size_t GR_WS_MAX = (size_t)4 << 30;      // bytes of workspace at most
+// Operator classes of a batch: each problem's launches are of one of them.
+constexpr int CLS_PAIRS = 0, CLS_GAINS = 1, CLS_GRID = 2, N_CLS = 3;
+
 constexpr int NPROF = 7;
 
 struct ProfRec {
@@ -116,19 +171,22 @@ struct Batch {
     DBuf<sl1m::DevProblem> desc;
     DBuf<int> n_probs_dev;
     DBuf<int> phases_dev;
-    DevPlan plan[2][2];        // [0 forward / 1 adjoint][0 no gains / 1 gains]
-    bool has_class[2] = {false, false};
+    DevPlan plan[2][N_CLS];    // [0 forward / 1 adjoint][class]
+    bool has_class[N_CLS] = {false, false, false};
+    std::vector<int> cls;               // class of every problem
+    std::vector<uint64_t> gens;         // layout of every problem when the plans were made
+    std::vector<int> grid_slot[2];      // [op] first partial slot of every lattice problem
     int nst[2][2] = {{4, 4}, {4, 4}};   // tile shape per [op][class] (autotuned or default)
     int n_ant_max = 0;
     int fin_grid = 1, sc_grid = 1;
-    double pairs_class[2] = {0, 0};
+    double pairs_class[N_CLS] = {0, 0, 0};
     double fin_bytes[2] = {0, 0};   // [forward finish, adjoint finish] per tick
     bool has_mfista = false;         // a tick ends with the MFISTA mix kernel
     // captured tick
     cudaGraphExec_t gexec = nullptr;
     bool graph_ok = false;
     long long tick_launches = 0;
-    const void* cap_partial[2] = {nullptr, nullptr};   // the context's scratch the capture baked in
+    const void* cap_partial[3] = {nullptr, nullptr, nullptr};   // the context's scratch the capture baked in
     ~Batch();
 };
 
@@ -142,6 +200,7 @@ struct sl1m_ctx {
     mutable std::mutex err_mu;           // server thread reports failures here too
     DBuf<double2> partial_f;
     DBuf<double> partial_a;
+    DBuf<float2> grid_ws;                // workspace of the lattice operators
     std::vector<sl1m_problem*> problems;
     // autotuned (streamed granules per stage, CTAs per SM), keyed by
     // (precision, op, gains, Gaussian pixels, log2 of the units)
@@ -193,9 +252,12 @@ struct sl1m_problem {
     UnitCost ucost[2][2];                      // [precision][0 forward / 1 adjoint]
     bool ucost_ok[2][2] = {{false, false}, {false, false}};
     std::unique_ptr<Batch> op_batch[2], solve_batch[2];
+    std::unique_ptr<GridTables> grid;         // lattice operator of the mixed path, or null
+    uint64_t gen = 0;                         // counts the layouts
     const UnitCost& unit_cost(int precision, int op);
 
-    int rebuild(cudaStream_t st);
+    // grid_budget: device bytes the lattice operator may take, tables and workspace
+    int rebuild(cudaStream_t st, size_t grid_budget = SIZE_MAX);
     int ensure_solver(cudaStream_t st);
     int init_solve(const sl1m_solve_opts* o, double L, bool power_only, cudaStream_t st);
     int read_state(sl1m::SolveState& s, cudaStream_t st);
@@ -206,6 +268,10 @@ struct sl1m_problem {
     size_t estimate_bytes() const;
     ~sl1m_problem();
 };
+
+// Builds P.grid when the laid-out problem's pixels are a lattice and the
+// lattice operator is the faster one for it; false (P.grid null) otherwise.
+bool grid_build(sl1m_problem& P, cudaStream_t st, size_t budget);
 
 long long tune_key(int precision, int op, bool gains, bool gauss, long long units);
 

@@ -212,7 +212,20 @@ static void server_loop(Server* Sp)
         std::vector<Request*> joined;
         for (Request* r : admit) {
             sl1m_problem* p = r->prob;
-            int rc = p->rebuild(ctx->upstream);
+            // a lattice operator's tables and workspace count against the budget
+            // like the rest, and are only made when they fit what is left of it
+            size_t left;
+            {
+                std::lock_guard<std::mutex> lk(S.mu);
+                left = S.budget > S.in_use ? S.budget - S.in_use : 0;
+            }
+            int rc = p->rebuild(ctx->upstream, left);
+            if (rc == SL1M_OK && p->grid) {
+                const size_t extra = p->grid->bytes() + p->grid->ws_elems * sizeof(float2);
+                std::lock_guard<std::mutex> lk(S.mu);
+                r->bytes += extra;
+                S.in_use += extra;
+            }
             if (rc == SL1M_OK) rc = p->init_solve(&r->opts, r->opts.L, false, ctx->upstream);
             if (rc != SL1M_OK) retire(S, r, rc);
             else joined.push_back(r);
