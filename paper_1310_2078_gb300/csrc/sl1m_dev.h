@@ -54,6 +54,7 @@ constexpr int BT_P = BT_CH + 1;       // its padded row (rows start in different
 constexpr int BLK_GRAN = 8;           // owned granules per CTA (one per warp)
 constexpr int BLK = G * BLK_GRAN;     // owned elements per CTA block
 constexpr int NTHREADS = 256;         // 8 warps
+constexpr int FP64_SUB = G;           // the FP64 kernels' units per streamed granule
 constexpr int MAX_PROBS = 1024;       // problems per batched launch
 
 enum Kind : int { DIRAC = 0, PARAXIAL = 1, WIDE = 2 };
@@ -150,6 +151,7 @@ struct DevProblem {
     const float4* vgabs;      // [vis.n_pad] {u, v, -2 w, u^2 + v^2} in FP32 (the adjoint's Gaussian terms)
     float2* r32;              // [vis.n_pad] the mixed adjoint's input residual in polar form,
                               // {|r|, arg r in turns} in FP32 (r32_kernel)
+    double2* r64;             // [vis.n_pad] the FP64 adjoint's, {arg r in 1/2048 turns, |r|} (r64_kernel)
     const float2* gpol32;     // [pix.n_gran][gain_rows(n_ant)][GP] {|G|, arg G in turns} or null
     const double2* gains64;   // [pix.n_pad][n_ant] or null
     int n_ant;

@@ -319,8 +319,9 @@ void plan_host(const std::vector<int>& nb, const std::vector<int>& ns, int Cmax,
             const UnitCost* uc = (*costs)[p];
             const long long up = H.u0[p + 1] - H.u0[p];
             double w = 0.0;
-            if (uc && !uc->unit.empty() && (long long)uc->unit.size() == up) {
+            if (uc && !uc->unit.empty() && (long long)uc->unit.size() * uc->sub == up) {
                 for (float f : uc->unit) w += f;
+                w *= uc->sub;
             } else {
                 w = (uc ? uc->uniform : 1.0) * (double)up;
             }
@@ -338,13 +339,17 @@ void plan_host(const std::vector<int>& nb, const std::vector<int>& ns, int Cmax,
             const UnitCost* uc = (*costs)[p];
             const long long up = H.u0[p + 1] - H.u0[p];
             long long i;
-            if (uc && !uc->unit.empty() && (long long)uc->unit.size() == up) {
+            if (uc && !uc->unit.empty() && (long long)uc->unit.size() * uc->sub == up) {
+                const long long nu = (long long)uc->unit.size();
                 if (pref_of != p) {
-                    pref.assign(up + 1, 0.0);
-                    for (long long k = 0; k < up; ++k) pref[k + 1] = pref[k] + uc->unit[k];
+                    pref.assign(nu + 1, 0.0);
+                    for (long long k = 0; k < nu; ++k) pref[k + 1] = pref[k] + (double)uc->unit[k] * uc->sub;
                     pref_of = p;
                 }
                 i = std::lower_bound(pref.begin(), pref.end(), t - W[p]) - pref.begin();
+                if (uc->sub > 1 && i > 0)        // within the run of equal units that ends there
+                    i = (i - 1) * uc->sub +
+                        (long long)std::ceil((t - W[p] - pref[i - 1]) / uc->unit[std::min(i, nu) - 1] - 1e-9);
             } else {
                 const double w = (uc ? uc->uniform : 1.0);
                 i = (long long)std::ceil((t - W[p]) / w - 1e-9);
@@ -500,6 +505,7 @@ struct ProblemDev {
     DBuf<int2> ant;
     DBuf<float4> vgabs;
     DBuf<float2> r32;
+    DBuf<double2> r64;               // made by the first FP64 call
     DBuf<int> vslot, gnb;
     DBuf<int2> gbl;
     DBuf<double2> V;
@@ -718,6 +724,8 @@ int sl1m_problem::rebuild(cudaStream_t st, size_t grid_budget)
     hp.ant = D.ant.p;
     hp.vgabs = D.vgabs.p;
     hp.r32 = D.r32.p;
+    D.r64.free();
+    hp.r64 = nullptr;
     hp.vslot = n_ant > 0 ? D.vslot.p : nullptr;
     hp.gbl = n_ant > 0 ? D.gbl.p : nullptr;
     hp.gnb = n_ant > 0 ? D.gnb.p : nullptr;
@@ -767,7 +775,10 @@ const UnitCost& sl1m_problem::unit_cost(int precision, int op)
     // measured on GB300 (4 x 128x128 pixels of one kind x 32,000 visibilities):
     // forward 1.53, adjoint 1.60 without gains; 1.34 and 1.45 with gains
     const double gfac = n_ant > 0 ? 2.0 : 1.0;
-    const double gcost = n_ant > 0 ? (op == 0 ? 1.34 : 1.45) : (op == 0 ? 1.53 : 1.60);
+    // (FP64: by the instructions of a pair)
+    const double gcost = precision == 0 ? (op == 0 ? 2.1 : 2.3)
+                         : n_ant > 0    ? (op == 0 ? 1.34 : 1.45)
+                                        : (op == 0 ? 1.53 : 1.60);
     const auto base = [gcost](int kind) { return kind == DIRAC ? 1.0 : gcost; };
     int k0 = gkind_pix.empty() ? 0 : gkind_pix[0];
     bool one_kind = true;
@@ -782,6 +793,7 @@ const UnitCost& sl1m_problem::unit_cost(int precision, int op)
     if (one_kind && !any_exact) return uc;
     const int ng_own = (int)own.size(), ng_str = (int)str.size();
     const int nblk = (ng_own + BLK_GRAN - 1) / BLK_GRAN;
+    uc.sub = stream_units(precision, 1);               // units per streamed granule
     uc.unit.resize((size_t)nblk * ng_str);
     for (int b = 0; b < nblk; ++b) {
         const int w1 = std::min(ng_own, (b + 1) * BLK_GRAN);
@@ -816,6 +828,15 @@ size_t sl1m_problem::estimate_bytes() const
     b += nv * (16 + 8);                            // the adjoint's FP32 Gaussian terms and residual
     b += (nv + np) * 16 * 3;                       // operator scratch
     return b + (1 << 16);
+}
+
+// The polar residual of FP64 adjoints without gains.
+int sl1m_problem::ensure_r64(cudaStream_t st)
+{
+    if (n_ant > 0 || hp.r64) return SL1M_OK;
+    CK(dev->r64.reserve(hp.vis.n_pad, st));
+    hp.r64 = dev->r64.p;
+    return SL1M_OK;
 }
 
 int sl1m_problem::ensure_solver(cudaStream_t st)
@@ -933,7 +954,7 @@ size_t sl1m_problem::dev_bytes() const
     };
     side(D.vis);
     side(D.pix);
-    b += D.ant.bytes() + D.vgabs.bytes() + D.r32.bytes() + D.vslot.bytes() + D.gbl.bytes() + D.gnb.bytes() + D.V.bytes() + D.pgauss.bytes() + D.pgauss64.bytes() + D.gsig.bytes() +
+    b += D.ant.bytes() + D.vgabs.bytes() + D.r32.bytes() + D.r64.bytes() + D.vslot.bytes() + D.gbl.bytes() + D.gnb.bytes() + D.V.bytes() + D.pgauss.bytes() + D.pgauss64.bytes() + D.gsig.bytes() +
          D.gsig64.bytes() + D.gkind.bytes() + D.pghdr.bytes() + D.gpol32.bytes() + D.gains64.bytes();
     b += D.x_user.bytes() + D.x_sorted.bytes() + D.adj_sorted.bytes() + D.img_user.bytes() +
          D.r_user.bytes() + D.r_sorted.bytes() + D.fwd_sorted.bytes() + D.vis_user.bytes();
@@ -1045,9 +1066,9 @@ int batch_set(sl1m_ctx* ctx, Batch& B, const std::vector<sl1m_problem*>& probs,
                 const bool g = c == CLS_GAINS, in = B.cls[p] == c;
                 const DevProblem& d = descs[p];
                 nbf[p] = in ? d.vis.n_blk : 0;
-                nsf[p] = in ? d.pix.n_gran : 0;
+                nsf[p] = in ? stream_units(precision, d.pix.n_gran) : 0;
                 nba[p] = in ? d.pix.n_blk : 0;
-                nsa[p] = in ? d.vis.n_gran : 0;
+                nsa[p] = in ? stream_units(precision, d.vis.n_gran) : 0;
                 if (in) {
                     B.has_class[c] = true;
                     B.pairs_class[c] += probs[p]->pairs();
@@ -1068,7 +1089,7 @@ int batch_set(sl1m_ctx* ctx, Batch& B, const std::vector<sl1m_problem*>& probs,
             const auto ta = ctx->tune.find(tune_key(precision, 1, c == 1, gauss, ua));
             if (tf != ctx->tune.end()) { B.nst[0][c] = tf->second.first; kf = tf->second.second; }
             if (ta != ctx->tune.end()) { B.nst[1][c] = ta->second.first; ka = ta->second.second; }
-            if (precision != 0 && c == 0) {         // no Gaussian pixels: the Dirac-only instances
+            if (precision == 0 || c == 0) {         // no Gaussian pixels: the Dirac-only instances
                 B.nst[0][c] = shape_for(B.nst[0][c], gauss);
                 B.nst[1][c] = shape_for(B.nst[1][c], gauss);
             }
@@ -1143,6 +1164,11 @@ static int launch_op_class(sl1m_ctx* ctx, Batch& B, int op, int c)
             int vmax = 1;
             for (const DevProblem& d : B.hdesc) vmax = std::max(vmax, d.vis.n_pad);
             CKL(launch_r32(B.desc.p, (int)B.hdesc.size(), vmax, st));
+        }
+        if (B.precision == 0 && c == CLS_PAIRS) {
+            int vmax = 1;
+            for (const DevProblem& d : B.hdesc) vmax = std::max(vmax, d.vis.n_pad);
+            CKL(launch_r64(B.desc.p, (int)B.hdesc.size(), vmax, st));
         }
         prof_begin(ctx, B.precision == 0 ? 1 : 3, tk);
         if (c == CLS_GRID)
@@ -1280,6 +1306,7 @@ static int op_prepare(sl1m_problem* prob, int precision, Batch** out)
     RET(prob->rebuild(ctx->stream));
     auto& B = prob->op_batch[precision];
     if (!B) B = std::make_unique<Batch>();
+    if (precision == SL1M_FP64) RET(prob->ensure_r64(ctx->stream));
     ProblemDev& D = *prob->dev;
     CK(D.x_sorted.reserve(prob->hp.pix.n_pad, ctx->stream));
     CK(D.fwd_sorted.reserve(prob->hp.vis.n_pad, ctx->stream));
@@ -1303,6 +1330,7 @@ static int run_single(sl1m_problem* prob, int precision, int max_ticks, SolveSta
     sl1m_ctx* ctx = prob->ctx;
     auto& B = prob->solve_batch[precision];
     if (!B) B = std::make_unique<Batch>();
+    if (precision == SL1M_FP64) RET(prob->ensure_r64(ctx->stream));
     const DevProblem d = prob->solver_desc();
     if (B->probs.empty() || memcmp(&B->hdesc[0], &d, sizeof d) != 0)
         RET(batch_set(ctx, *B, {prob}, {d}, precision, true));
@@ -1362,7 +1390,8 @@ int sl1m_create(sl1m_ctx** out, int device, void* cuda_stream)
         }
         c->own_stream = true;
     }
-    if (cudaStreamCreateWithFlags(&c->upstream, cudaStreamNonBlocking) != cudaSuccess) {
+    if (cudaStreamCreateWithFlags(&c->upstream, cudaStreamNonBlocking) != cudaSuccess ||
+        fp64_init_tables(c->stream) != cudaSuccess) {
         delete c;
         return SL1M_ERR_CUDA;
     }
@@ -1751,7 +1780,7 @@ int sl1m_autotune(sl1m_problem* prob, int precision, int32_t* nst_out, int32_t* 
     int rc = SL1M_OK;
     for (int op = 0; op < 2 && rc == SL1M_OK; ++op) {
         const std::vector<int> nb = {op == 0 ? d.vis.n_blk : d.pix.n_blk};
-        const std::vector<int> ns = {op == 0 ? d.pix.n_gran : d.vis.n_gran};
+        const std::vector<int> ns = {stream_units(precision, op == 0 ? d.pix.n_gran : d.vis.n_gran)};
         const std::vector<const UnitCost*> uc = {&prob->unit_cost(precision, op)};
         const long long units = (long long)nb[0] * ns[0];
         // stage 1: streamed granules per stage x CTAs per SM; stage 2: at the
@@ -1844,7 +1873,8 @@ int sl1m_set_tile_shape(sl1m_problem* prob, int precision, int op, int nst, int 
         return sl1m_fail(ctx, SL1M_ERR_ARG, "with gains or in FP64 only the CTAs per SM can be set");
     RET(prob->rebuild(ctx->stream));
     const DevProblem& d = prob->hp;
-    const long long units = op == 0 ? (long long)d.vis.n_blk * d.pix.n_gran : (long long)d.pix.n_blk * d.vis.n_gran;
+    const long long units = (long long)(op == 0 ? d.vis.n_blk : d.pix.n_blk) *
+                            stream_units(precision, op == 0 ? d.pix.n_gran : d.vis.n_gran);
     const int code = shape_code(nst, npoly);
     const int occ = occupancy((precision == SL1M_FP64 ? 0 : 2) + op, gains, std::max(1, prob->n_ant), code);
     if (ctas_per_sm > occ)

@@ -100,9 +100,10 @@ struct HostPlan {
 };
 
 // Relative cost of the units of one problem in a plan: a constant per unit,
-// or one value per unit (block-major, streamed granule minor).
+// or one value per `sub` units (block-major, streamed granule minor).
 struct UnitCost {
     double uniform = 1.0;
+    int sub = 1;
     std::vector<float> unit;
 };
 
@@ -258,6 +259,7 @@ struct sl1m_problem {
 
     // grid_budget: device bytes the lattice operator may take, tables and workspace
     int rebuild(cudaStream_t st, size_t grid_budget = SIZE_MAX);
+    int ensure_r64(cudaStream_t st);
     int ensure_solver(cudaStream_t st);
     int init_solve(const sl1m_solve_opts* o, double L, bool power_only, cudaStream_t st);
     int read_state(sl1m::SolveState& s, cudaStream_t st);

@@ -31,6 +31,13 @@ cudaError_t launch_adjoint(int precision, bool gains, int n_ant, const DevProble
 // which: 0 fwd fp64, 1 adj fp64, 2 fwd mixed, 3 adj mixed
 int occupancy(int which, bool gains, int n_ant, int nst = NST_DEFAULT);
 int fwd_smem_bytes(int n_ant, bool gains, int nst);
+// Before an FP64 adjoint without gains: r64, likewise in FP64.
+cudaError_t launch_r64(const DevProblem* probs, int n_probs, int max_vis_pad, cudaStream_t st);
+// The FP64 kernels' tables on the current device; called by every new context.
+cudaError_t fp64_init_tables(cudaStream_t st);
+// Streamed granules as the plans count them: the FP64 kernels' units
+// stream one element, FP64_SUB per granule.
+constexpr int stream_units(int precision, int n_gran) { return precision == 0 ? n_gran * FP64_SUB : n_gran; }
 // Before a mixed adjoint: each problem's input residual in polar form, {|r|,
 // arg r in turns} in FP32 (r32).
 cudaError_t launch_r32(const DevProblem* probs, int n_probs, int max_vis_pad, cudaStream_t st);

@@ -110,7 +110,7 @@ extern "C" int sl1m_forward_noalloc(sl1m_problem* prob, const double* x_dev, dou
     // work split of this single problem (host tables)
     HostPlan H;
     const int which = precision == SL1M_FP64 ? 0 : 2;
-    plan_host({lay.vis.n_blk}, {lay.pix.n_gran}, ctx->num_sms * occupancy(which, gains, std::max(1, prob->n_ant)), H);
+    plan_host({lay.vis.n_blk}, {stream_units(precision == SL1M_FP64 ? 0 : 1, lay.pix.n_gran)}, ctx->num_sms * occupancy(which, gains, std::max(1, prob->n_ant)), H);
     // carve the static scratch
     size_t off = 0;
     auto take = [&](size_t bytes) {

@@ -226,6 +226,7 @@ static void server_loop(Server* Sp)
                 r->bytes += extra;
                 S.in_use += extra;
             }
+            if (rc == SL1M_OK && S.precision == SL1M_FP64) rc = p->ensure_r64(ctx->upstream);
             if (rc == SL1M_OK) rc = p->init_solve(&r->opts, r->opts.L, false, ctx->upstream);
             if (rc != SL1M_OK) retire(S, r, rc);
             else joined.push_back(r);
