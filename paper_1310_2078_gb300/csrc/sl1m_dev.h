@@ -54,6 +54,7 @@ constexpr int BT_P = BT_CH + 1;       // its padded row (rows start in different
 constexpr int BLK_GRAN = 8;           // owned granules per CTA (one per warp)
 constexpr int BLK = G * BLK_GRAN;     // owned elements per CTA block
 constexpr int NTHREADS = 256;         // 8 warps
+constexpr double R64_TURN = 2048.0;  // units of arg r in r64 per turn (the FP64 kernels' phase unit)
 constexpr int FP64_SUB = G;           // the FP64 kernels' units per streamed granule
 constexpr int MAX_PROBS = 1024;       // problems per batched launch
 
@@ -126,12 +127,12 @@ struct SolveBufs {
     double* xv;          // power-iteration vector [pix.n_pad]
     double2* AI[2];      // A I_k ping-pong [vis.n_pad]
     double2* r;          // W (A y - V), or W A x in the power iteration [vis.n_pad]
-    double* blk_r2;      // [vis.n_blk] per-block sum W|A I - V|^2
-    double* blk_l1;      // [pix.n_blk] per-block sum I
-    double* blk_z2;      // [pix.n_blk] per-block sum z^2 (power)
-    int* blk_nnz;        // [pix.n_blk]
-    int* blk_badv;       // [vis.n_blk] non-finite flags
-    int* blk_badp;       // [pix.n_blk] non-finite flags
+    double* blk_r2;      // [vis.n_gran] per-granule sum W|A I - V|^2
+    double* blk_l1;      // [pix.n_gran] per-granule sum I
+    double* blk_z2;      // [pix.n_gran] per-granule sum z^2 (power)
+    int* blk_nnz;        // [pix.n_gran]
+    int* blk_badv;       // [vis.n_gran] non-finite flags
+    int* blk_badp;       // [pix.n_gran] non-finite flags
 };
 
 struct DevProblem {
@@ -150,8 +151,8 @@ struct DevProblem {
     const float4* pghdr;      // [pix.n_gran][4] centre hi, centre lo, extent, {sigma, kind, 0, 0}
     const float4* vgabs;      // [vis.n_pad] {u, v, -2 w, u^2 + v^2} in FP32 (the adjoint's Gaussian terms)
     float2* r32;              // [vis.n_pad] the mixed adjoint's input residual in polar form,
-                              // {|r|, arg r in turns} in FP32 (r32_kernel)
-    double2* r64;             // [vis.n_pad] the FP64 adjoint's, {arg r in 1/2048 turns, |r|} (r64_kernel)
+                              // {|r|, arg r in turns} in FP32
+    double2* r64;             // [vis.n_pad] the FP64 adjoint's, {arg r in 1/R64_TURN turns, |r|}
     const float2* gpol32;     // [pix.n_gran][gain_rows(n_ant)][GP] {|G|, arg G in turns} or null
     const double2* gains64;   // [pix.n_pad][n_ant] or null
     int n_ant;
@@ -199,6 +200,7 @@ struct Plan {
                                   // or null: CTA c takes [c U / C, (c+1) U / C)
     int n_blocks;
     int n_slots;
+    int blk_el;                   // elements per owned block and partial slot
 };
 
 // Unit range [u, u_end) of CTA c.

@@ -32,7 +32,7 @@
 
 namespace sl1m {
 
-constexpr int CIRC = 2048;                 // table points of the circle, and of [1, 2) for 2^x
+constexpr int CIRC = (int)R64_TURN;                 // table points of the circle, and of [1, 2) for 2^x
 static_assert(FP64_SUB == G, "a unit streams one element");
 
 // e^{2 pi i k / CIRC} and 2^(k / CIRC), filled once per device (fp64_init_tables).
@@ -424,25 +424,6 @@ adj_fp64_kernel(const DevProblem* __restrict__ probs, const Plan* __restrict__ p
         }
         u += g1 - g0;
     }
-}
-
-// r64 = the FP64 adjoint's input residual in polar form {arg r in 1/CIRC turns,
-// |r|}, for every problem that takes part (blockIdx.y = problem).
-__global__ void r64_kernel(const DevProblem* __restrict__ probs)
-{
-    const DevProblem& P = probs[blockIdx.y];
-    const double2* R;
-    if (!adj_role(P, R) || P.n_ant > 0) return;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < P.vis.n_pad; i += gridDim.x * blockDim.x) {
-        const double2 v = R[i];
-        P.r64[i] = make_double2(atan2(v.y, v.x) * (0.15915494309189533577 * CIRC), hypot(v.x, v.y));
-    }
-}
-cudaError_t launch_r64(const DevProblem* probs, int n_probs, int max_vis_pad, cudaStream_t st)
-{
-    const int nb = (max_vis_pad + 127) / 128;
-    r64_kernel<<<dim3((unsigned)(nb < 1 ? 1 : nb > 1024 ? 1024 : nb), (unsigned)n_probs), 128, 0, st>>>(probs);
-    return cudaGetLastError();
 }
 
 // ------------------------------------------------------------- launchers

@@ -392,15 +392,15 @@ void plan_host(const std::vector<int>& nb, const std::vector<int>& ns, int Cmax,
 
 // Build a stream-K plan over problems with owned blocks nb[p] and streamed
 // granules ns[p]; C CTAs at most.  Uploads the tables.
-cudaError_t build_plan(const std::vector<int>& nb, const std::vector<int>& ns, int Cmax,
+cudaError_t build_plan(const std::vector<int>& nb, const std::vector<int>& ns, int Cmax, int own_gran,
                        DevPlan& D, cudaStream_t st, const std::vector<const UnitCost*>* costs)
 {
     HostPlan H;
     plan_host(nb, ns, Cmax, H, costs);
-    return upload_plan(H, (int)nb.size(), D, st);
+    return upload_plan(H, (int)nb.size(), own_gran * G, D, st);
 }
 
-cudaError_t upload_plan(const HostPlan& H, int n_probs, DevPlan& D, cudaStream_t st)
+cudaError_t upload_plan(const HostPlan& H, int n_probs, int blk_el, DevPlan& D, cudaStream_t st)
 {
     cudaError_t err;
     auto up = [&](DBuf<int>& b, const std::vector<int>& v) {
@@ -427,6 +427,7 @@ cudaError_t upload_plan(const HostPlan& H, int n_probs, DevPlan& D, cudaStream_t
     D.pl.cta_u0 = H.cta_u0.empty() ? nullptr : D.cta.p;
     D.pl.n_blocks = H.n_blocks;
     D.pl.n_slots = H.n_slots;
+    D.pl.blk_el = blk_el;
     return D.dpl.upload(&D.pl, 1, st);
 }
 
@@ -792,19 +793,19 @@ const UnitCost& sl1m_problem::unit_cost(int precision, int op)
     uc.uniform = base(k0) * gfac;
     if (one_kind && !any_exact) return uc;
     const int ng_own = (int)own.size(), ng_str = (int)str.size();
-    const int nblk = (ng_own + BLK_GRAN - 1) / BLK_GRAN;
+    const int bg = own_granules(precision, op, n_ant > 0), nblk = own_blocks(precision, op, n_ant > 0, ng_own);
     uc.sub = stream_units(precision, 1);               // units per streamed granule
     uc.unit.resize((size_t)nblk * ng_str);
     for (int b = 0; b < nblk; ++b) {
-        const int w1 = std::min(ng_own, (b + 1) * BLK_GRAN);
+        const int w1 = std::min(ng_own, (b + 1) * bg);
         double kb = 1.0;
         if (op == 1)
-            for (int w = b * BLK_GRAN; w < w1; ++w) kb = std::max(kb, base(gkind_pix[w]));
+            for (int w = b * bg; w < w1; ++w) kb = std::max(kb, base(gkind_pix[w]));
         for (int g = 0; g < ng_str; ++g) {
             bool ex = false;
             if (any_exact) {
                 const float4 s4 = str[g];
-                for (int w = b * BLK_GRAN; w < w1 && !ex; ++w)
+                for (int w = b * bg; w < w1 && !ex; ++w)
                     ex = own[w].x * s4.x + own[w].y * s4.y + own[w].z * s4.z > D_MAX;
             }
             const double kbase = op == 0 ? base(gkind_pix[g]) : kb;
@@ -846,12 +847,12 @@ int sl1m_problem::ensure_solver(cudaStream_t st)
     const size_t np = hp.pix.n_pad, nv = hp.vis.n_pad;
     CK(D.I0.alloc(np)); CK(D.I1.alloc(np)); CK(D.y.alloc(np)); CK(D.xv.alloc(np));
     CK(D.AI0.alloc(nv)); CK(D.AI1.alloc(nv)); CK(D.rr.alloc(nv));
-    CK(D.blk_r2.alloc(std::max(1, hp.vis.n_blk)));
-    CK(D.blk_badv.alloc(std::max(1, hp.vis.n_blk)));
-    CK(D.blk_l1.alloc(std::max(1, hp.pix.n_blk)));
-    CK(D.blk_z2.alloc(std::max(1, hp.pix.n_blk)));
-    CK(D.blk_nnz.alloc(std::max(1, hp.pix.n_blk)));
-    CK(D.blk_badp.alloc(std::max(1, hp.pix.n_blk)));
+    CK(D.blk_r2.alloc(std::max(1, hp.vis.n_gran)));
+    CK(D.blk_badv.alloc(std::max(1, hp.vis.n_gran)));
+    CK(D.blk_l1.alloc(std::max(1, hp.pix.n_gran)));
+    CK(D.blk_z2.alloc(std::max(1, hp.pix.n_gran)));
+    CK(D.blk_nnz.alloc(std::max(1, hp.pix.n_gran)));
+    CK(D.blk_badp.alloc(std::max(1, hp.pix.n_gran)));
     CK(D.st.alloc(1));
     SolveBufs b;
     b.I[0] = D.I0.p; b.I[1] = D.I1.p; b.y = D.y.p; b.xv = D.xv.p;
@@ -859,8 +860,8 @@ int sl1m_problem::ensure_solver(cudaStream_t st)
     b.blk_r2 = D.blk_r2.p; b.blk_l1 = D.blk_l1.p; b.blk_z2 = D.blk_z2.p;
     b.blk_nnz = D.blk_nnz.p; b.blk_badv = D.blk_badv.p; b.blk_badp = D.blk_badp.p;
     hbufs = b;
-    CK(cudaMemsetAsync(D.blk_badp.p, 0, sizeof(int) * std::max(1, hp.pix.n_blk), st));
-    CK(cudaMemsetAsync(D.blk_badv.p, 0, sizeof(int) * std::max(1, hp.vis.n_blk), st));
+    CK(cudaMemsetAsync(D.blk_badp.p, 0, sizeof(int) * std::max(1, hp.pix.n_gran), st));
+    CK(cudaMemsetAsync(D.blk_badv.p, 0, sizeof(int) * std::max(1, hp.vis.n_gran), st));
     solver_ready = true;
     return SL1M_OK;
 }
@@ -1009,7 +1010,7 @@ static int set_grid_plans(sl1m_ctx* ctx, Batch& B, const std::vector<DevProblem>
             }
         }
         H.n_blocks = H.b0[np];
-        CK(upload_plan(H, np, B.plan[op][CLS_GRID], ctx->stream));
+        CK(upload_plan(H, np, BLK, B.plan[op][CLS_GRID], ctx->stream));
         if (op == 0) CK(ctx->partial_f.reserve((size_t)std::max(1, H.n_slots) * BLK, ctx->stream));
         else CK(ctx->partial_a.reserve((size_t)std::max(1, H.n_slots) * BLK, ctx->stream));
         B.fin_bytes[op] += (double)H.n_slots * BLK * (op == 0 ? 16.0 : 8.0);
@@ -1059,15 +1060,16 @@ int batch_set(sl1m_ctx* ctx, Batch& B, const std::vector<sl1m_problem*>& probs,
                 else cudaGetLastError();
             }
         }
-        RET(set_grid_plans(ctx, B, descs));
+        if (std::count(B.cls.begin(), B.cls.end(), CLS_GRID)) RET(set_grid_plans(ctx, B, descs));
         for (int c = 0; c < 2; ++c) {
+            if (!std::count(B.cls.begin(), B.cls.end(), c)) continue;
             std::vector<int> nbf(np), nsf(np), nba(np), nsa(np);
             for (int p = 0; p < np; ++p) {
                 const bool g = c == CLS_GAINS, in = B.cls[p] == c;
                 const DevProblem& d = descs[p];
                 nbf[p] = in ? d.vis.n_blk : 0;
                 nsf[p] = in ? stream_units(precision, d.pix.n_gran) : 0;
-                nba[p] = in ? d.pix.n_blk : 0;
+                nba[p] = in ? own_blocks(precision, 1, g, d.pix.n_gran) : 0;
                 nsa[p] = in ? stream_units(precision, d.vis.n_gran) : 0;
                 if (in) {
                     B.has_class[c] = true;
@@ -1102,20 +1104,19 @@ int batch_set(sl1m_ctx* ctx, Batch& B, const std::vector<sl1m_problem*>& probs,
                 cf[p] = &probs[p]->unit_cost(precision == 0 ? 0 : 1, 0);
                 ca[p] = &probs[p]->unit_cost(precision == 0 ? 0 : 1, 1);
             }
-            CK(build_plan(nbf, nsf, ctx->num_sms * kf, B.plan[0][c], st, &cf));
-            CK(build_plan(nba, nsa, ctx->num_sms * ka, B.plan[1][c], st, &ca));
-            CK(ctx->partial_f.reserve((size_t)std::max(1, B.plan[0][c].pl.n_slots) * BLK, st));
-            CK(ctx->partial_a.reserve((size_t)std::max(1, B.plan[1][c].pl.n_slots) * BLK, st));
-            B.fin_bytes[0] += (double)B.plan[0][c].pl.n_slots * BLK * 16.0;
-            B.fin_bytes[1] += (double)B.plan[1][c].pl.n_slots * BLK * 8.0;
+            const int oga = own_granules(precision, 1, c == CLS_GAINS);
+            CK(build_plan(nbf, nsf, ctx->num_sms * kf, BLK_GRAN, B.plan[0][c], st, &cf));
+            CK(build_plan(nba, nsa, ctx->num_sms * ka, oga, B.plan[1][c], st, &ca));
+            const Plan &pf = B.plan[0][c].pl, &pa = B.plan[1][c].pl;
+            CK(ctx->partial_f.reserve((size_t)std::max(1, pf.n_slots) * pf.blk_el, st));
+            CK(ctx->partial_a.reserve((size_t)std::max(1, pa.n_slots) * pa.blk_el, st));
+            B.fin_bytes[0] += (double)pf.n_slots * pf.blk_el * 16.0;
+            B.fin_bytes[1] += (double)pa.n_slots * pa.blk_el * 8.0;
         }
-        int nblk = 0;
         for (int p = 0; p < np; ++p) {
-            nblk = std::max({nblk, descs[p].vis.n_blk, descs[p].pix.n_blk});
             B.fin_bytes[0] += descs[p].vis.n_pad * (solver ? 16.0 * 5 + 32 : 48.0);
             B.fin_bytes[1] += descs[p].pix.n_pad * (solver ? 8.0 * 5 + 4 : 8.0);
         }
-        B.fin_grid = std::max(1, std::min(4 * ctx->num_sms, nblk * np));
         B.sc_grid = std::max(1, std::min(ctx->num_sms * 4, np));
     }
     const void* new_ptrs[7] = {B.desc.p, ctx->partial_f.p, ctx->partial_a.p, B.n_probs_dev.p,
@@ -1124,7 +1125,15 @@ int batch_set(sl1m_ctx* ctx, Batch& B, const std::vector<sl1m_problem*>& probs,
     return SL1M_OK;
 }
 
-static int launch_op_class(sl1m_ctx* ctx, Batch& B, int op, int c)
+// The polar form of r that the adjoint of a class reads (sl1m_kernels.h).
+static int polar_of(int precision, int c)
+{
+    if (c == CLS_GRID) return 0;
+    return precision != 0 ? 1 : c == CLS_GAINS ? 0 : 2;
+}
+
+// user_out: the result of an operator call, in the caller's order (null in a tick).
+static int launch_op_class(sl1m_ctx* ctx, Batch& B, int op, int c, double* user_out)
 {
     if (!B.has_class[c]) return SL1M_OK;
     cudaStream_t st = ctx->stream;
@@ -1154,22 +1163,10 @@ static int launch_op_class(sl1m_ctx* ctx, Batch& B, int op, int c)
                                B.nst[0][c]));
         prof_end(ctx, tk, B.solver ? 0.0 : B.pairs_class[c], 0.0);   // solver ticks: counted on the device
         prof_begin(ctx, 4, tk);
-        CKL(launch_fwd_finish(B.desc.p, P.dpl.p, std::min(B.fin_grid, std::max(1, P.pl.n_blocks)),
-                              ctx->partial_f.p, st));
+        CKL(launch_fwd_finish(B.desc.p, P.dpl.p, P.pl, ctx->num_sms, ctx->partial_f.p, polar_of(B.precision, c),
+                              (double2*)user_out, st));
         prof_end(ctx, tk, 0.0, B.fin_bytes[0]);
     } else {
-        // the mixed pair adjoints read r in polar form, written once for the
-        // whole batch before its first class
-        if (B.precision != 0 && c != CLS_GRID && (c == 0 || !B.has_class[0])) {
-            int vmax = 1;
-            for (const DevProblem& d : B.hdesc) vmax = std::max(vmax, d.vis.n_pad);
-            CKL(launch_r32(B.desc.p, (int)B.hdesc.size(), vmax, st));
-        }
-        if (B.precision == 0 && c == CLS_PAIRS) {
-            int vmax = 1;
-            for (const DevProblem& d : B.hdesc) vmax = std::max(vmax, d.vis.n_pad);
-            CKL(launch_r64(B.desc.p, (int)B.hdesc.size(), vmax, st));
-        }
         prof_begin(ctx, B.precision == 0 ? 1 : 3, tk);
         if (c == CLS_GRID)
             RET(each_grid([&](int p, const GridOp& g) {
@@ -1181,17 +1178,17 @@ static int launch_op_class(sl1m_ctx* ctx, Batch& B, int op, int c)
                                B.nst[1][c]));
         prof_end(ctx, tk, B.solver ? 0.0 : B.pairs_class[c], 0.0);
         prof_begin(ctx, 5, tk);
-        CKL(launch_adj_finish(B.desc.p, P.dpl.p, std::min(B.fin_grid, std::max(1, P.pl.n_blocks)),
-                              ctx->partial_a.p, st));
+        CKL(launch_adj_finish(B.desc.p, P.dpl.p, P.pl, ctx->num_sms, ctx->partial_a.p, user_out, st));
         prof_end(ctx, tk, 0.0, B.fin_bytes[1]);
     }
     return SL1M_OK;
 }
 
-// One operator application (operator-mode batch): forward or adjoint.
-int batch_op(sl1m_ctx* ctx, Batch& B, int op)
+// One operator application (operator-mode batch): forward or adjoint, into
+// user_out in the caller's order (null: the batch's own array).
+int batch_op(sl1m_ctx* ctx, Batch& B, int op, double* user_out)
 {
-    for (int c = 0; c < N_CLS; ++c) RET(launch_op_class(ctx, B, op, c));
+    for (int c = 0; c < N_CLS; ++c) RET(launch_op_class(ctx, B, op, c, user_out));
     return SL1M_OK;
 }
 
@@ -1199,8 +1196,8 @@ int batch_op(sl1m_ctx* ctx, Batch& B, int op)
 // forward, forward finish (per gains class), then the phase machine.
 static int enqueue_tick(sl1m_ctx* ctx, Batch& B)
 {
-    for (int c = 0; c < N_CLS; ++c) RET(launch_op_class(ctx, B, 1, c));
-    for (int c = 0; c < N_CLS; ++c) RET(launch_op_class(ctx, B, 0, c));
+    for (int c = 0; c < N_CLS; ++c) RET(launch_op_class(ctx, B, 1, c, nullptr));
+    for (int c = 0; c < N_CLS; ++c) RET(launch_op_class(ctx, B, 0, c, nullptr));
     // while profiling (ticks are launched directly then, never captured) the
     // scalars kernel counts the pairs the tick evaluated
     double* ev = (ctx->prof && B.solver && ctx->evals_dev.p) ? ctx->evals_dev.p + 2 * (B.precision != 0) : nullptr;
@@ -1212,7 +1209,7 @@ static int enqueue_tick(sl1m_ctx* ctx, Batch& B)
             if (!B.has_class[c]) continue;
             const int nb = B.plan[0][c].pl.n_blocks + B.plan[1][c].pl.n_blocks;
             CKL(launch_mfista_mix(B.desc.p, B.plan[0][c].dpl.p, B.plan[1][c].dpl.p,
-                                  std::min(B.fin_grid, std::max(1, nb)), ctx->stream));
+                                  std::min(4 * ctx->num_sms, std::max(1, nb)), polar_of(B.precision, c), ctx->stream));
         }
         prof_end(ctx, tk, 0.0, 0.0);
     }
@@ -1597,10 +1594,7 @@ int sl1m_forward_dev(sl1m_problem* prob, const double* x_dev, double* vis_out_de
     RET(op_prepare(prob, precision, &B));
     ProblemDev& D = *prob->dev;
     CKL(launch_gather_real(x_dev, D.x_sorted.p, prob->hp.pix.orig, prob->hp.pix.n_pad, 1.0, ctx->stream));
-    RET(batch_op(ctx, *B, 0));
-    CKL(launch_scatter_cplx(D.fwd_sorted.p, (double2*)vis_out_dev, prob->hp.vis.orig, prob->hp.vis.n_pad,
-                            ctx->stream));
-    return SL1M_OK;
+    return batch_op(ctx, *B, 0, vis_out_dev);
 }
 
 int sl1m_adjoint_dev(sl1m_problem* prob, const double* r_dev, double* img_out_dev, int precision)
@@ -1614,11 +1608,9 @@ int sl1m_adjoint_dev(sl1m_problem* prob, const double* r_dev, double* img_out_de
     Batch* B;
     RET(op_prepare(prob, precision, &B));
     ProblemDev& D = *prob->dev;
-    CKL(launch_gather_cplx((const double2*)r_dev, D.r_sorted.p, prob->hp.vis.orig, prob->hp.vis.n_pad,
-                           ctx->stream));
-    RET(batch_op(ctx, *B, 1));
-    CKL(launch_scatter_real(D.adj_sorted.p, img_out_dev, prob->hp.pix.orig, prob->hp.pix.n_pad, ctx->stream));
-    return SL1M_OK;
+    CKL(launch_gather_resid((const double2*)r_dev, B->desc.p, prob->hp.vis.n_pad, polar_of(B->precision, B->cls[0]),
+                            D.r_sorted.p, ctx->stream));
+    return batch_op(ctx, *B, 1, img_out_dev);
 }
 
 int sl1m_forward(sl1m_problem* prob, const double* x, double* vis_out, int precision)
@@ -1681,10 +1673,9 @@ int sl1m_dirty_image(sl1m_problem* prob, int precision, double* img_out, double*
     RET(op_prepare(prob, precision, &B));
     ProblemDev& D = *prob->dev;
     cudaStream_t st = ctx->stream;
-    CKL(launch_weighted_vis(prob->hp.V, prob->hp.vis.d, D.r_sorted.p, prob->hp.vis.n_pad, st));
-    RET(batch_op(ctx, *B, 1));
     CK(D.img_user.reserve(prob->n_pix, st));
-    CKL(launch_scatter_real(D.adj_sorted.p, D.img_user.p, prob->hp.pix.orig, prob->hp.pix.n_pad, st));
+    CKL(launch_weighted_vis(B->desc.p, prob->hp.vis.n_pad, polar_of(B->precision, B->cls[0]), D.r_sorted.p, st));
+    RET(batch_op(ctx, *B, 1, D.img_user.p));
     std::vector<double> img(prob->n_pix);
     CK(cudaMemcpyAsync(img.data(), D.img_user.p, sizeof(double) * prob->n_pix, cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
@@ -1779,7 +1770,7 @@ int sl1m_autotune(sl1m_problem* prob, int precision, int32_t* nst_out, int32_t* 
     CK(cudaEventCreate(&e1));
     int rc = SL1M_OK;
     for (int op = 0; op < 2 && rc == SL1M_OK; ++op) {
-        const std::vector<int> nb = {op == 0 ? d.vis.n_blk : d.pix.n_blk};
+        const std::vector<int> nb = {own_blocks(precision, op, gains, op == 0 ? d.vis.n_gran : d.pix.n_gran)};
         const std::vector<int> ns = {stream_units(precision, op == 0 ? d.pix.n_gran : d.vis.n_gran)};
         const std::vector<const UnitCost*> uc = {&prob->unit_cost(precision, op)};
         const long long units = (long long)nb[0] * ns[0];
@@ -1793,8 +1784,8 @@ int sl1m_autotune(sl1m_problem* prob, int precision, int32_t* nst_out, int32_t* 
         const auto time_shape = [&](int code, int k) -> float {
             if (mixed_plain) code = shape_for(code, prob->has_gauss);
             DevPlan P;
-            if (build_plan(nb, ns, ctx->num_sms * k, P, st, &uc) != cudaSuccess) { rc = SL1M_ERR_CUDA; return 0.f; }
-            const size_t need = (size_t)std::max(1, P.pl.n_slots) * BLK;
+            if (build_plan(nb, ns, ctx->num_sms * k, own_granules(precision, op, gains), P, st, &uc) != cudaSuccess) { rc = SL1M_ERR_CUDA; return 0.f; }
+            const size_t need = (size_t)std::max(1, P.pl.n_slots) * P.pl.blk_el;
             if ((op == 0 ? ctx->partial_f.reserve(need, st) : ctx->partial_a.reserve(need, st)) != cudaSuccess) {
                 rc = SL1M_ERR_OOM;
                 return 0.f;
@@ -1804,7 +1795,7 @@ int sl1m_autotune(sl1m_problem* prob, int precision, int32_t* nst_out, int32_t* 
             // forward left in L2, and shapes are ranked as a solve runs them
             float ms = 0.f;
             for (int rep = 0; rep < 4; ++rep) {
-                const int rb = batch_op(ctx, *Bop, 1 - op);
+                const int rb = batch_op(ctx, *Bop, 1 - op, nullptr);
                 if (rb != SL1M_OK) { rc = rb; return 0.f; }
                 cudaEventRecord(e0, st);
                 cudaError_t e = op == 0 ? launch_forward(precision, gains, prob->n_ant, Bop->desc.p, P.dpl.p, P.pl.C,
@@ -1873,7 +1864,7 @@ int sl1m_set_tile_shape(sl1m_problem* prob, int precision, int op, int nst, int 
         return sl1m_fail(ctx, SL1M_ERR_ARG, "with gains or in FP64 only the CTAs per SM can be set");
     RET(prob->rebuild(ctx->stream));
     const DevProblem& d = prob->hp;
-    const long long units = (long long)(op == 0 ? d.vis.n_blk : d.pix.n_blk) *
+    const long long units = (long long)own_blocks(precision, op, gains, op == 0 ? d.vis.n_gran : d.pix.n_gran) *
                             stream_units(precision, op == 0 ? d.pix.n_gran : d.vis.n_gran);
     const int code = shape_code(nst, npoly);
     const int occ = occupancy((precision == SL1M_FP64 ? 0 : 2) + op, gains, std::max(1, prob->n_ant), code);

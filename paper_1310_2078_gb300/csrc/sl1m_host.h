@@ -120,11 +120,11 @@ struct DevPlan {
     DBuf<long long> cta;
     DBuf<sl1m::Plan> dpl;     // device header
 };
-cudaError_t build_plan(const std::vector<int>& nb, const std::vector<int>& ns, int Cmax, DevPlan& D,
+cudaError_t build_plan(const std::vector<int>& nb, const std::vector<int>& ns, int Cmax, int own_gran, DevPlan& D,
                        cudaStream_t st, const std::vector<const UnitCost*>* costs = nullptr);
 
 // Uploads a host plan's tables and header.
-cudaError_t upload_plan(const HostPlan& H, int n_probs, DevPlan& D, cudaStream_t st);
+cudaError_t upload_plan(const HostPlan& H, int n_probs, int blk_el, DevPlan& D, cudaStream_t st);
 
 // A problem's lattice operator: its tables, and the workspace it needs (the
 // context's, shared by every problem of its stream).
@@ -179,7 +179,7 @@ struct Batch {
     std::vector<int> grid_slot[2];      // [op] first partial slot of every lattice problem
     int nst[2][2] = {{4, 4}, {4, 4}};   // tile shape per [op][class] (autotuned or default)
     int n_ant_max = 0;
-    int fin_grid = 1, sc_grid = 1;
+    int sc_grid = 1;
     double pairs_class[N_CLS] = {0, 0, 0};
     double fin_bytes[2] = {0, 0};   // [forward finish, adjoint finish] per tick
     bool has_mfista = false;         // a tick ends with the MFISTA mix kernel
@@ -280,7 +280,7 @@ long long tune_key(int precision, int op, bool gains, bool gauss, long long unit
 // batches (sl1m_host.cpp)
 int batch_set(sl1m_ctx* ctx, Batch& B, const std::vector<sl1m_problem*>& probs,
               const std::vector<sl1m::DevProblem>& descs, int precision, bool solver);
-int batch_op(sl1m_ctx* ctx, Batch& B, int op);
+int batch_op(sl1m_ctx* ctx, Batch& B, int op, double* user_out);
 int batch_ticks(sl1m_ctx* ctx, Batch& B, int n);
 int batch_phases(sl1m_ctx* ctx, Batch& B, std::vector<int>& out);
 

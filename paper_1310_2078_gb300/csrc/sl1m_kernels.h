@@ -31,16 +31,26 @@ cudaError_t launch_adjoint(int precision, bool gains, int n_ant, const DevProble
 // which: 0 fwd fp64, 1 adj fp64, 2 fwd mixed, 3 adj mixed
 int occupancy(int which, bool gains, int n_ant, int nst = NST_DEFAULT);
 int fwd_smem_bytes(int n_ant, bool gains, int nst);
-// Before an FP64 adjoint without gains: r64, likewise in FP64.
-cudaError_t launch_r64(const DevProblem* probs, int n_probs, int max_vis_pad, cudaStream_t st);
 // The FP64 kernels' tables on the current device; called by every new context.
 cudaError_t fp64_init_tables(cudaStream_t st);
+// Owned granules per block of a plan.  A CTA of the mixed gains adjoint works on
+// one pixel granule at a time with all its warps, so its blocks are granules:
+// a CTA's range is then a long run of visibility granules for its 8 warps,
+// where 8 granules x a short run left some of them idle on small problems.
+constexpr int own_granules(int precision, int op, bool gains)
+{
+    return precision != 0 && op == 1 && gains ? 1 : BLK_GRAN;
+}
+constexpr int own_blocks(int precision, int op, bool gains, int n_gran)
+{
+    return (n_gran + own_granules(precision, op, gains) - 1) / own_granules(precision, op, gains);
+}
 // Streamed granules as the plans count them: the FP64 kernels' units
 // stream one element, FP64_SUB per granule.
 constexpr int stream_units(int precision, int n_gran) { return precision == 0 ? n_gran * FP64_SUB : n_gran; }
-// Before a mixed adjoint: each problem's input residual in polar form, {|r|,
-// arg r in turns} in FP32 (r32).
-cudaError_t launch_r32(const DevProblem* probs, int n_probs, int max_vis_pad, cudaStream_t st);
+// The adjoints without FP64 gains read r in polar form too, {|r|, arg r in turns}
+// in FP32 (r32) or {arg r in 1/R64_TURN turns, |r|} in FP64 (r64).  Whatever writes r
+// writes it: `polar` below is 0 (the lattice operator, FP64 gains), 1 r32 or 2 r64.
 // The mixed gains kernels' bounded waits for their bulk copies set a device
 // flag when they give up; read it into *host_flag (asynchronously on st: valid
 // after the stream is synchronised) and clear it.
@@ -55,19 +65,22 @@ unsigned long long wait_limit_ns();
 // solver kernels (sl1m_solver.cu)
 cudaError_t launch_gather_real(const double* src, double* dst, const int* orig, int n_pad,
                                double scale, cudaStream_t st);
-cudaError_t launch_gather_cplx(const double2* src, double2* dst, const int* orig, int n_pad,
-                               cudaStream_t st);
+// P: the problem's descriptor on the device.
+cudaError_t launch_gather_resid(const double2* src, const DevProblem* P, int n_pad, int polar, double2* dst,
+                                cudaStream_t st);
 cudaError_t launch_scatter_real(const double* src, double* dst, const int* orig, int n_pad,
                                 cudaStream_t st);
 cudaError_t launch_scatter_cplx(const double2* src, double2* dst, const int* orig, int n_pad,
                                 cudaStream_t st);
 cudaError_t launch_fill_valid(double* dst, const int* orig, int n_pad, double val, cudaStream_t st);
-cudaError_t launch_weighted_vis(const double2* V, const d4* vd, double2* r, int n_pad, cudaStream_t st);
-cudaError_t launch_fwd_finish(const DevProblem* probs, const Plan* plp, int grid, const double2* partial,
-                              cudaStream_t st);
-cudaError_t launch_adj_finish(const DevProblem* probs, const Plan* plp, int grid, const double* partial,
-                              cudaStream_t st);
-cudaError_t launch_mfista_mix(const DevProblem* probs, const Plan* fplp, const Plan* aplp, int grid,
+cudaError_t launch_weighted_vis(const DevProblem* P, int n_pad, int polar, double2* r, cudaStream_t st);
+// pl: host copy of the plan's header.  user_out: where an operator call's result
+// goes, in the caller's order (null: the descriptor's array, in the library's).
+cudaError_t launch_fwd_finish(const DevProblem* probs, const Plan* plp, const Plan& pl, int num_sms,
+                              const double2* partial, int polar, double2* user_out, cudaStream_t st);
+cudaError_t launch_adj_finish(const DevProblem* probs, const Plan* plp, const Plan& pl, int num_sms,
+                              const double* partial, double* user_out, cudaStream_t st);
+cudaError_t launch_mfista_mix(const DevProblem* probs, const Plan* fplp, const Plan* aplp, int grid, int polar,
                               cudaStream_t st);
 // evals (may be null): [0] += pairs the forward and [1] += pairs the adjoint
 // evaluated in this tick, summed over the problems that took part.

@@ -546,7 +546,7 @@ fwd_mixed_kernel(const DevProblem* __restrict__ probs, const Plan* __restrict__ 
 // The adjoint's output is real (the image is real: its gradient is Re A^H r),
 // and for one pair Re(conj(A_kj) r_k) = |A_kj| |r_k| cos(theta_kj + arg r_k)
 // with theta_kj = -arg A_kj: a cosine alone, not a sine and a cosine.
-// r32_kernel writes r in polar form {|r|, arg r in turns}; when a stage is
+// Whatever writes r writes it in polar form too, {|r|, arg r in turns}; when a stage is
 // derived, arg r_k is added to the visibility's B term (so theta + arg r
 // costs nothing per pair) and |r_k| rides in the same record (Gaussian
 // owners: log2 |r'_k| inside the amplitude's exponent).
@@ -654,7 +654,7 @@ __device__ __forceinline__ float4 adj_gauss_record(float b, float2 rp, const flo
 // Adjoint stage buffers in dynamic shared memory: two of them, each holding
 // NSA streamed visibility granules as they sit in HBM -- offsets, offset
 // residuals, the Gaussian form {u, v, -2 w, u^2 + v^2}, the residual r in
-// polar form (written by r32_kernel just before the launch) and the granule
+// polar form and the granule
 // centres and extents -- filled by bulk (TMA) copies on one mbarrier per
 // buffer; the copies of stage s + 1 are issued when stage s starts.
 template <int NSA>
@@ -952,14 +952,14 @@ __device__ __forceinline__ void adjg_gauss_tile(const float4* __restrict__ s_off
 // warp derives what its tiles read, then at once copies its following granule
 // into the freed slice, so the copy runs under the tiles.  No CTA barrier
 // inside the run.  For each owned granule the 8 warp sums are added in warp
-// order (deterministic).
+// order (deterministic).  A unit is one pixel granule x one visibility granule.
 struct AdjRaw {                                   // one warp's slice, bytes
     static constexpr int OFF = 0, LO = 1024, HI = 2048, R = 3072, ANT = 3584, CEN = 4096;
     static constexpr int BYTES = CEN + 48;        // a multiple of 16
 };
 
 // Lane 0: copy visibility granule g of P into a warp's raw slice (r: the
-// polar residual r32_kernel wrote).
+// residual in polar form).
 __device__ __forceinline__ void adj_raw_load(unsigned char* raw, const DevProblem& P, int g, unsigned long long* bar)
 {
     const size_t e = (size_t)g * G;
@@ -1023,107 +1023,103 @@ adj_mixed_gains_kernel(const DevProblem* __restrict__ probs, const Plan* __restr
             continue;
         }
         const int upb = P.vis.n_gran;
-        const int blk = (int)(loc / upb);
+        const int pgi = (int)(loc / upb);
         const int g0 = (int)(loc % upb);
         const int g1 = (int)min((long long)upb, (long long)g0 + (u_end - u));
         const int gtab_n = gain_rows(P.n_ant) * GP;      // float2 per granule table
-        const int gb = pl.prob_b0[p] + blk;
-        double* dst = partial + (size_t)slot_of(pl, gb) * BLK;
-        for (int og = 0; og < BLK_GRAN; ++og) {
-            const int pgi = blk * BLK_GRAN + og;
-            if (pgi >= P.pix.n_gran) break;                  // uniform over the CTA
-            __syncthreads();                                 // s_gain / s_red free again
-            if (threadIdx.x == 0 && !fault) {
-                fence_proxy_async_smem();                    // the table's last readers are done
-                bulk_load(s_gain, P.gpol32 + (size_t)pgi * gtab_n, (unsigned)gtab_n * (unsigned)sizeof(float2),
-                          &s_gbar);
-            }
-            if (lane == 0 && !fault && g0 + warp < g1) adj_raw_load(raw, P, g0 + warp, &s_wbar[warp]);
-            const float4 ch = P.pix.cen_hi[pgi], cl = P.pix.cen_lo[pgi], ext = P.pix.ext[pgi];
-            const int kind = P.gkind[pgi];
-            const float sigma = P.gsig[pgi];
-            const bool gauss = (kind != DIRAC), par = (kind == PARAXIAL);
-            const int e0 = pgi * G + lane;
-            const int eidx[2] = {e0, e0 + 32};
-            const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
-            float4 xh[2], dx[2], pgd[2] = {z4, z4};
+        const int gb = pl.prob_b0[p] + pgi;              // a block is one pixel granule (own_granules)
+        double* dst = partial + (size_t)slot_of(pl, gb) * G;
+        __syncthreads();                                 // s_gain / s_red free again
+        if (threadIdx.x == 0 && !fault) {
+            fence_proxy_async_smem();                    // the table's last readers are done
+            bulk_load(s_gain, P.gpol32 + (size_t)pgi * gtab_n, (unsigned)gtab_n * (unsigned)sizeof(float2),
+                      &s_gbar);
+        }
+        if (lane == 0 && !fault && g0 + warp < g1) adj_raw_load(raw, P, g0 + warp, &s_wbar[warp]);
+        const float4 ch = P.pix.cen_hi[pgi], cl = P.pix.cen_lo[pgi], ext = P.pix.ext[pgi];
+        const int kind = P.gkind[pgi];
+        const float sigma = P.gsig[pgi];
+        const bool gauss = (kind != DIRAC), par = (kind == PARAXIAL);
+        const int e0 = pgi * G + lane;
+        const int eidx[2] = {e0, e0 + 32};
+        const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
+        float4 xh[2], dx[2], pgd[2] = {z4, z4};
 #pragma unroll
-            for (int r = 0; r < 2; ++r) {
-                xh[r] = P.pix.hi[eidx[r]];
-                dx[r] = to_rad(P.pix.off[eidx[r]]);
-                if (gauss) pgd[r] = pix_for_gauss(P.pgauss[eidx[r]]);
-            }
-            const SmemGain sg{s_gain, lane};
-            mbar_wait(&s_gbar, gpar, fault);
-            gpar ^= 1u;
-            double tot[2] = {0.0, 0.0};
-            for (int g = g0 + warp; g < g1; g += BLK_GRAN) {
-                mbar_wait(&s_wbar[warp], wpar, fault);
-                wpar ^= 1u;
-                // derive this granule's records for the tiles
+        for (int r = 0; r < 2; ++r) {
+            xh[r] = P.pix.hi[eidx[r]];
+            dx[r] = to_rad(P.pix.off[eidx[r]]);
+            if (gauss) pgd[r] = pix_for_gauss(P.pgauss[eidx[r]]);
+        }
+        const SmemGain sg{s_gain, lane};
+        mbar_wait(&s_gbar, gpar, fault);
+        gpar ^= 1u;
+        double tot[2] = {0.0, 0.0};
+        for (int g = g0 + warp; g < g1; g += BLK_GRAN) {
+            mbar_wait(&s_wbar[warp], wpar, fault);
+            wpar ^= 1u;
+            // derive this granule's records for the tiles
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int k = lane + 32 * h;
-                    float4 o = raw_off[k];
-                    const int2 ab = raw_ant[k];
-                    const float key = __int_as_float(ab.x << 16 | ab.y);   // the pair (adjg_next_run)
-                    const float b = frac_dot3(ch, cl, o, raw_lo[k]) + odd_turn(k);   // turns
-                    const float2 rp = raw_r[k];                             // {|r|, arg r in turns}
-                    float4 kr;
-                    if (gauss) {
-                        const float4 va = vis_for_gauss(raw_hi[k]);
-                        const float4 rec = adj_gauss_record(b, rp, va, sigma);   // {B', gamr, k1, k0'}
-                        o.w = rec.x;
-                        s_va[warp][k] = make_float4(va.x, va.y, va.z, rec.y);
-                        kr = make_float4(key, rec.w, rec.z, 0.f);
-                    } else {
-                        o.w = frac_turns(b + rp.y) * TWO_PI_F;
-                        kr = make_float4(key, rp.x, 0.f, 0.f);
-                    }
-                    s_off[warp][k] = o;
-                    s_kr[warp][k] = kr;
+            for (int h = 0; h < 2; ++h) {
+                const int k = lane + 32 * h;
+                float4 o = raw_off[k];
+                const int2 ab = raw_ant[k];
+                const float key = __int_as_float(ab.x << 16 | ab.y);   // the pair (adjg_next_run)
+                const float b = frac_dot3(ch, cl, o, raw_lo[k]) + odd_turn(k);   // turns
+                const float2 rp = raw_r[k];                             // {|r|, arg r in turns}
+                float4 kr;
+                if (gauss) {
+                    const float4 va = vis_for_gauss(raw_hi[k]);
+                    const float4 rec = adj_gauss_record(b, rp, va, sigma);   // {B', gamr, k1, k0'}
+                    o.w = rec.x;
+                    s_va[warp][k] = make_float4(va.x, va.y, va.z, rec.y);
+                    kr = make_float4(key, rec.w, rec.z, 0.f);
+                } else {
+                    o.w = frac_turns(b + rp.y) * TWO_PI_F;
+                    kr = make_float4(key, rp.x, 0.f, 0.f);
                 }
-                const float4 yc_h = raw_cen[0], yc_l = raw_cen[1], yext = raw_cen[2];
-                __syncwarp();                                 // the slice is read: refill it
-                if (lane == 0 && !fault && g + BLK_GRAN < g1) adj_raw_load(raw, P, g + BLK_GRAN, &s_wbar[warp]);
-                const bool exact = dot3(ext, yext) > D_MAX;
-                float Ct[2];                          // the tile's centre term C, turns
+                s_off[warp][k] = o;
+                s_kr[warp][k] = kr;
+            }
+            const float4 yc_h = raw_cen[0], yc_l = raw_cen[1], yext = raw_cen[2];
+            __syncwarp();                                 // the slice is read: refill it
+            if (lane == 0 && !fault && g + BLK_GRAN < g1) adj_raw_load(raw, P, g + BLK_GRAN, &s_wbar[warp]);
+            const bool exact = dot3(ext, yext) > D_MAX;
+            float Ct[2];                          // the tile's centre term C, turns
 #pragma unroll
-                for (int r = 0; r < 2; ++r) Ct[r] = frac_dot3(xh[r], P.pix.lo[eidx[r]], yc_h, yc_l);
-                const float4* g_lo = P.vis.offlo + (size_t)g * G;   // exact tiles only (rare)
-                float acc[2] = {0.f, 0.f};
-                if (!gauss) {
-                    if (exact) {
-                        const float4 dxt[2] = {P.pix.off[eidx[0]], P.pix.off[eidx[1]]},
-                                     dxl[2] = {P.pix.offlo[eidx[0]], P.pix.offlo[eidx[1]]};
-                        adjg_dirac_tile<true>(s_off[warp], g_lo, s_kr[warp], sg, Ct, dxt, dxl, acc);
-                    } else {
-                        adjg_dirac_tile<false>(s_off[warp], g_lo, s_kr[warp], sg, Ct, dx, dx, acc);
-                    }
-                } else if (exact) {
+            for (int r = 0; r < 2; ++r) Ct[r] = frac_dot3(xh[r], P.pix.lo[eidx[r]], yc_h, yc_l);
+            const float4* g_lo = P.vis.offlo + (size_t)g * G;   // exact tiles only (rare)
+            float acc[2] = {0.f, 0.f};
+            if (!gauss) {
+                if (exact) {
                     const float4 dxt[2] = {P.pix.off[eidx[0]], P.pix.off[eidx[1]]},
                                  dxl[2] = {P.pix.offlo[eidx[0]], P.pix.offlo[eidx[1]]};
-                    if (par) adjg_gauss_tile<true, true>(s_off[warp], g_lo, s_va[warp], s_kr[warp], sg, Ct, dxt, dxl, pgd, acc);
-                    else adjg_gauss_tile<true, false>(s_off[warp], g_lo, s_va[warp], s_kr[warp], sg, Ct, dxt, dxl, pgd, acc);
-                } else if (par) {
-                    adjg_gauss_tile<false, true>(s_off[warp], g_lo, s_va[warp], s_kr[warp], sg, Ct, dx, dx, pgd, acc);
+                    adjg_dirac_tile<true>(s_off[warp], g_lo, s_kr[warp], sg, Ct, dxt, dxl, acc);
                 } else {
-                    adjg_gauss_tile<false, false>(s_off[warp], g_lo, s_va[warp], s_kr[warp], sg, Ct, dx, dx, pgd, acc);
+                    adjg_dirac_tile<false>(s_off[warp], g_lo, s_kr[warp], sg, Ct, dx, dx, acc);
                 }
-#pragma unroll
-                for (int r = 0; r < 2; ++r) tot[r] += (double)acc[r];
-                __syncwarp();                                 // s_off ... of this warp free again
+            } else if (exact) {
+                const float4 dxt[2] = {P.pix.off[eidx[0]], P.pix.off[eidx[1]]},
+                             dxl[2] = {P.pix.offlo[eidx[0]], P.pix.offlo[eidx[1]]};
+                if (par) adjg_gauss_tile<true, true>(s_off[warp], g_lo, s_va[warp], s_kr[warp], sg, Ct, dxt, dxl, pgd, acc);
+                else adjg_gauss_tile<true, false>(s_off[warp], g_lo, s_va[warp], s_kr[warp], sg, Ct, dxt, dxl, pgd, acc);
+            } else if (par) {
+                adjg_gauss_tile<false, true>(s_off[warp], g_lo, s_va[warp], s_kr[warp], sg, Ct, dx, dx, pgd, acc);
+            } else {
+                adjg_gauss_tile<false, false>(s_off[warp], g_lo, s_va[warp], s_kr[warp], sg, Ct, dx, dx, pgd, acc);
             }
 #pragma unroll
-            for (int r = 0; r < 2; ++r) s_red[warp][lane + 32 * r] = tot[r];
-            __syncthreads();
-            if (warp == 0) {
+            for (int r = 0; r < 2; ++r) tot[r] += (double)acc[r];
+            __syncwarp();                                 // s_off ... of this warp free again
+        }
 #pragma unroll
-                for (int r = 0; r < 2; ++r) {
-                    double t = 0.0;
-                    for (int w = 0; w < BLK_GRAN; ++w) t += s_red[w][lane + 32 * r];
-                    dst[og * G + lane + 32 * r] = t * P.pix.d[eidx[r]].w;
-                }
+        for (int r = 0; r < 2; ++r) s_red[warp][lane + 32 * r] = tot[r];
+        __syncthreads();
+        if (warp == 0) {
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                double t = 0.0;
+                for (int w = 0; w < BLK_GRAN; ++w) t += s_red[w][lane + 32 * r];
+                dst[lane + 32 * r] = t * P.pix.d[eidx[r]].w;
             }
         }
         u += g1 - g0;
@@ -1157,27 +1153,6 @@ int adj_gains_smem_bytes(int n_ant) { return BLK_GRAN * AdjRaw::BYTES + gains_ta
 static int adj_stage_bytes_of(int nst)
 {
     return 2 * (nst <= 2 ? AdjStage<2>::BYTES : AdjStage<4>::BYTES);
-}
-
-// r32 = the mixed adjoint's input residual in polar form, {|r|, arg r in
-// turns}, for every problem of the batch that takes part in the coming adjoint
-// (blockIdx.y = problem).  Modulus and argument are taken in FP64 and rounded
-// once to FP32 (arg r to 3e-8 turn).
-__global__ void r32_kernel(const DevProblem* __restrict__ probs)
-{
-    const DevProblem& P = probs[blockIdx.y];
-    const double2* R;
-    if (!adj_role(P, R) || !P.r32) return;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < P.vis.n_pad; i += gridDim.x * blockDim.x) {
-        const double2 v = R[i];
-        P.r32[i] = make_float2((float)hypot(v.x, v.y), (float)(atan2(v.y, v.x) * 0.15915494309189535));
-    }
-}
-cudaError_t launch_r32(const DevProblem* probs, int n_probs, int max_vis_pad, cudaStream_t st)
-{
-    const dim3 grid((unsigned)std::max(1, std::min(1024, (max_vis_pad + 255) / 256)), (unsigned)n_probs);
-    r32_kernel<<<grid, 256, 0, st>>>(probs);
-    return cudaGetLastError();
 }
 
 cudaError_t wait_fault_read(unsigned* host_flag, cudaStream_t st)

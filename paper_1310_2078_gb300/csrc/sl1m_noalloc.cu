@@ -151,6 +151,7 @@ extern "C" int sl1m_forward_noalloc(sl1m_problem* prob, const double* x_dev, dou
     pl.blk_ncon = d_ncon;
     pl.n_blocks = H.n_blocks;
     pl.n_slots = H.n_slots;
+    pl.blk_el = BLK;
     const size_t head = (size_t)((unsigned char*)d_x - base);     // descriptor .. tables
     std::vector<unsigned char> img(head, 0);
     auto put = [&](void* at, const void* src, size_t bytes) {
@@ -179,7 +180,7 @@ extern "C" int sl1m_forward_noalloc(sl1m_problem* prob, const double* x_dev, dou
     // launch, so nothing in the scratch needs clearing
     CKN(launch_gather_real(x_dev, d_x, lay.pix.orig, lay.pix.n_pad, 1.0, st));
     CKN(launch_forward(precision == SL1M_FP64 ? 0 : 1, gains, prob->n_ant, d_desc, d_plan, H.C, d_part, st));
-    CKN(launch_fwd_finish(d_desc, d_plan, std::max(1, std::min(H.n_blocks, 4 * ctx->num_sms)), d_part, st));
+    CKN(launch_fwd_finish(d_desc, d_plan, pl, ctx->num_sms, d_part, 0, nullptr, st));
     CKN(launch_scatter_cplx(d_out, (double2*)vis_out_dev, lay.vis.orig, lay.vis.n_pad, st));
 #undef CKN
     ctx->n_launch += 4;
