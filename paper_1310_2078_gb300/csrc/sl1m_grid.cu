@@ -63,12 +63,26 @@ __device__ __forceinline__ void dft4(float2& a0, float2& a1, float2& a2, float2&
     a3 = csub(s1, s3);
 }
 
+// Half-zero inputs: with the cells at elements [0, L/4) and [3L/4, L) of a
+// transform (2^lx >= 2 nx, the origin in the middle), elements q = 2..5 of the 8
+// that a thread holds are zero, and of its outputs only q = 0, 1, 6, 7 are cells.
+
+// dft4 and dft8 with the middle inputs (a1, a2; v2..v5) zero.
 template <int SGN>
-__device__ __forceinline__ void dft8(float2 (&v)[8])
+__device__ __forceinline__ void dft4_outer(float2& a0, float2& a1, float2& a2, float2& a3)
+{
+    const float2 p = a0, q = a3, r = crot<SGN>(q);
+    a0 = cadd(p, q);
+    a1 = csub(p, r);
+    a2 = csub(p, q);
+    a3 = cadd(p, r);
+}
+
+// The last step of dft8 from the transforms e of the even and o of the odd inputs.
+template <int SGN, bool POUT>
+__device__ __forceinline__ void dft8_join(float2 (&v)[8])
 {
     const float H = 0.70710678118654752f;
-    dft4<SGN>(v[0], v[2], v[4], v[6]);        // even inputs: e0..e3 in v0, v2, v4, v6
-    dft4<SGN>(v[1], v[3], v[5], v[7]);        // odd inputs
     const float2 r3 = crot<SGN>(v[3]), r7 = crot<SGN>(v[7]);
     const float2 o1 = make_float2((v[3].x + r3.x) * H, (v[3].y + r3.y) * H);   // times e^{SGN i pi/4}
     const float2 o2 = crot<SGN>(v[5]);
@@ -76,56 +90,88 @@ __device__ __forceinline__ void dft8(float2 (&v)[8])
     const float2 e0 = v[0], e1 = v[2], e2 = v[4], e3 = v[6], o0 = v[1];
     v[0] = cadd(e0, o0);
     v[1] = cadd(e1, o1);
-    v[2] = cadd(e2, o2);
-    v[3] = cadd(e3, o3);
-    v[4] = csub(e0, o0);
-    v[5] = csub(e1, o1);
+    if (!POUT) {
+        v[2] = cadd(e2, o2);
+        v[3] = cadd(e3, o3);
+        v[4] = csub(e0, o0);
+        v[5] = csub(e1, o1);
+    }
     v[6] = csub(e2, o2);
     v[7] = csub(e3, o3);
 }
-
-// Shared-memory place of element e of CB interleaved transforms (CB a power of
-// two): one row of pad per 8 rows, so that the stride-8 writes of a radix-8
-// pass fall into different banks.
-template <int CB>
-__device__ __forceinline__ int pad_at(int row, int c)
+template <int SGN, bool PIN, bool POUT>
+__device__ __forceinline__ void dft8(float2 (&v)[8])
 {
-    return row * CB + c + (row >> 3) * CB;
+    if (PIN) {
+        dft4_outer<SGN>(v[0], v[2], v[4], v[6]);
+        dft4_outer<SGN>(v[1], v[3], v[5], v[7]);
+    } else {
+        dft4<SGN>(v[0], v[2], v[4], v[6]);    // even inputs: e0..e3 in v0, v2, v4, v6
+        dft4<SGN>(v[1], v[3], v[5], v[7]);    // odd inputs
+    }
+    dft8_join<SGN, POUT>(v);
 }
-constexpr int padded(int n, int cb) { return (n + n / 8) * cb; }
+
+// Shared-memory place of element i = e CB + c (element e of transform c of CB
+// interleaved ones): its low four bits (the 16 float2 that one wavefront of
+// shared memory holds) are XORed with bits of its next three, chosen so that the
+// 16 lanes of a half warp hit 16 different places in every access pattern of
+// the passes below: strides of 1, 2, 4 and 8 elements, and runs of 2, 4 or 8
+// elements 16, 32 or 64 apart.  (A pad of one element per 8 instead cost the
+// unit-stride reads a second wavefront: the rows kernel kept L1 82% busy.)  The
+// map is linear over GF(2): place(e | d) = place(e) ^ place(d) for e and d
+// without common bits, and d is always a constant.
+template <int CB>
+__host__ __device__ __forceinline__ constexpr int place(int i)
+{
+    const int r0 = (i >> 4) & 1, r1 = (i >> 5) & 1, r2 = (i >> 6) & 1;
+    return i ^ (CB == 1   ? (r0 | (r0 ^ r1) << 1 | r2 << 2 | (r1 ^ r2) << 3)
+                : CB == 4 ? (r1 << 2 | (r0 ^ r2) << 3)
+                          : (r0 ^ r1 ^ r2) << 3);
+}
+template <int CB>
+__device__ __forceinline__ float2& elem(float2* sm, int at, int d)     // at = place(e CB + c)
+{
+    const int pd = place<CB>(d * CB);
+    return sm[(at ^ (pd & 15)) + (pd & ~15)];
+}
 
 // Transform of length 2^LOG, radix 8 after a first pass of radix 2, 4 or 8
 // (Stockham order: no bit reversal).  A thread holds NB groups of 8 elements:
-// on entry and on exit v[n][q] is element g[n] + q 2^LOG/8 of transform c.
+// on entry and on exit v[n][q] is element g[n] + q 2^LOG/8 of its transform.
 // Every thread of the CTA calls it; sm holds the CTA's CB interleaved
-// transforms.  Twiddles: per pass of stride ns, e^{-2 pi i k/(8 ns)} and its
-// 2nd and 4th powers for k < ns, rounded from FP64; the other powers are
-// products of two.
-template <int LOG, int SGN, int CB, int NB>
-__device__ __forceinline__ void fft_pass_all(float2 (&v)[NB][8], const int (&g)[NB], int c, float2* sm,
+// transforms, c is this thread's.  PP: sm is two buffers of PP elements used in
+// turn (one barrier per exchange instead of two); sm is left at the next one to
+// write.  PIN: half-zero input, POUT: only the cells are wanted (above).
+// Twiddles: per pass of stride ns, e^{-2 pi i k/(8 ns)} and its 2nd and 4th
+// powers for k < ns, rounded from FP64; the other powers are products of two.
+template <int LOG, int SGN, int CB, int NB, bool PIN, bool POUT, int PP>
+__device__ __forceinline__ void fft_pass_all(float2 (&v)[NB][8], const int (&g)[NB], int c, float2*& sm, int& par,
                                              const float2* __restrict__ tw)
 {
     constexpr int L = 1 << LOG, E = L / 8;
     constexpr int R0 = LOG % 3 == 0 ? 8 : LOG % 3 == 1 ? 2 : 4;
 #pragma unroll
     for (int n = 0; n < NB; ++n) {
+        const int at = place<CB>(g[n] * R0 * CB + c);
         if (R0 == 8) {
-            dft8<SGN>(v[n]);
+            dft8<SGN, PIN, false>(v[n]);
 #pragma unroll
-            for (int r = 0; r < 8; ++r) sm[pad_at<CB>(g[n] * 8 + r, c)] = v[n][r];
+            for (int r = 0; r < 8; ++r) elem<CB>(sm, at, r) = v[n][r];
         } else if (R0 == 4) {
 #pragma unroll
             for (int i = 0; i < 2; ++i) {
-                dft4<SGN>(v[n][i], v[n][i + 2], v[n][i + 4], v[n][i + 6]);
+                if (PIN) dft4_outer<SGN>(v[n][i], v[n][i + 2], v[n][i + 4], v[n][i + 6]);
+                else dft4<SGN>(v[n][i], v[n][i + 2], v[n][i + 4], v[n][i + 6]);
 #pragma unroll
-                for (int r = 0; r < 4; ++r) sm[pad_at<CB>((g[n] + i * E) * 4 + r, c)] = v[n][i + 2 * r];
+                for (int r = 0; r < 4; ++r) elem<CB>(sm, at, i * E * 4 + r) = v[n][i + 2 * r];
             }
         } else {
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const float2 a = v[n][i], b = v[n][i + 4];
-                sm[pad_at<CB>((g[n] + i * E) * 2, c)] = cadd(a, b);
-                sm[pad_at<CB>((g[n] + i * E) * 2 + 1, c)] = csub(a, b);
+                elem<CB>(sm, at, i * E * 2) = !PIN ? cadd(a, b) : i < 2 ? a : b;
+                elem<CB>(sm, at, i * E * 2 + 1) = !PIN ? csub(a, b) : i < 2 ? a : make_float2(-b.x, -b.y);
             }
         }
     }
@@ -133,10 +179,17 @@ __device__ __forceinline__ void fft_pass_all(float2 (&v)[NB][8], const int (&g)[
     for (int ns = R0; ns < L; ns *= 8) {
         __syncthreads();
 #pragma unroll
-        for (int n = 0; n < NB; ++n)
+        for (int n = 0; n < NB; ++n) {
+            const int at = place<CB>(g[n] * CB + c);
 #pragma unroll
-            for (int r = 0; r < 8; ++r) v[n][r] = sm[pad_at<CB>(g[n] + r * E, c)];
-        __syncthreads();
+            for (int r = 0; r < 8; ++r) v[n][r] = elem<CB>(sm, at, r * E);
+        }
+        if (PP) {
+            sm += par ? -PP : PP;
+            par ^= 1;
+        } else {
+            __syncthreads();
+        }
 #pragma unroll
         for (int n = 0; n < NB; ++n) {
             const int k = g[n] & (ns - 1);
@@ -154,16 +207,21 @@ __device__ __forceinline__ void fft_pass_all(float2 (&v)[NB][8], const int (&g)[
             v[n][5] = cmul(v[n][5], cmul(w1, w4));
             v[n][6] = cmul(v[n][6], cmul(w2, w4));
             v[n][7] = cmul(v[n][7], cmul(w3, w4));
-            dft8<SGN>(v[n]);
             if (ns * 8 < L) {
-                const int o = (g[n] - k) * 8 + k;
+                dft8<SGN, false, false>(v[n]);
+                const int at = place<CB>(((g[n] - k) * 8 + k) * CB + c);
 #pragma unroll
-                for (int r = 0; r < 8; ++r) sm[pad_at<CB>(o + r * ns, c)] = v[n][r];
+                for (int r = 0; r < 8; ++r) elem<CB>(sm, at, r * ns) = v[n][r];
+            } else {
+                dft8<SGN, false, POUT>(v[n]);
             }
         }
         tw += 3 * ns;
     }
 }
+
+// The elements q of a thread's 8 that are cells.
+__device__ __forceinline__ constexpr int cell_q(int i) { return i < 2 ? i : i + 4; }
 
 // Cell index of element e (0 <= e < 2^lg) of a zero-padded axis whose cell c0
 // sits at element 0; outside [0, n) where the padding is.
@@ -186,7 +244,8 @@ struct RowShape {
     static constexpr int T = (1 << LOG) / 8;                  // threads per row
     static constexpr int ROWS = T >= 256 ? 1 : 256 / T;       // rows per CTA
     static constexpr int THREADS = T * ROWS;
-    static constexpr int PAD = padded(1 << LOG, 1);           // shared elements per row
+    static constexpr int BUF = ROWS << LOG;                   // shared elements of one buffer
+    static constexpr int SMEM = 2 * BUF * (int)sizeof(float2);
 };
 
 // Forward, rows: z = x amp exp(-2 pi i w_p nu) along x, transformed, into g1.
@@ -198,42 +257,40 @@ grid_rows_fwd_kernel(const DevProblem* __restrict__ probs, int prob, const GridO
 {
     using S = RowShape<LOG>;
     constexpr int L = 1 << LOG;
-    __shared__ float2 sm[S::ROWS][S::PAD];
+    extern __shared__ __align__(16) float2 sm_rows[];         // two buffers of BUF
     const double* X;
     if (!fwd_role(probs[prob], X)) return;
     const int rb = threadIdx.x / S::T;
     const int gi[1] = {(int)threadIdx.x % S::T};
     const int iy = blockIdx.x * S::ROWS + rb;
-    float a[8];
-    float2 nu[8];
+    float a[4];
+    float2 nu[4];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-        const int ix = cell_of(gi[0] + q * S::T, LOG, g.cx);
-        a[q] = 0.f;
-        nu[q] = make_float2(0.f, 0.f);
+    for (int i = 0; i < 4; ++i) {
+        const int ix = cell_of(gi[0] + cell_q(i) * S::T, LOG, g.cx);
+        a[i] = 0.f;
+        nu[i] = make_float2(0.f, 0.f);
         if (iy < g.ny && ix >= 0 && ix < g.nx) {
             const size_t at = (size_t)iy * g.nx + ix;
             const int j = g.cell[at];
             if (j >= 0) {
-                a[q] = __double2float_rn(X[j]) * g.amp[at] * g.fscale;
-                nu[q] = g.nu[at];
+                a[i] = __double2float_rn(X[j]) * g.amp[at] * g.fscale;
+                nu[i] = g.nu[at];
             }
         }
     }
+    float2* smr = sm_rows + rb * L;
+    int par = 0;
     const int q1 = min(np, (int)(blockIdx.y + 1) * GR_PCH);
     for (int p = blockIdx.y * GR_PCH; p < q1; ++p) {
         const float2 w = g.wp[p0 + p];
         float2 v[1][8];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const int ix = cell_of(gi[0] + q * S::T, LOG, g.cx);
-            v[0][q] = make_float2(0.f, 0.f);
-            if (ix >= 0 && ix < g.nx) {
-                const float2 e = plane_phase(w, nu[q]);
-                v[0][q] = make_float2(a[q] * e.x, a[q] * e.y);
-            }
+        for (int i = 0; i < 4; ++i) {
+            const float2 e = plane_phase(w, nu[i]);
+            v[0][cell_q(i)] = make_float2(a[i] * e.x, a[i] * e.y);
         }
-        fft_pass_all<LOG, -1, 1, 1>(v, gi, 0, sm[rb], g.twx);
+        fft_pass_all<LOG, -1, 1, 1, true, false, S::BUF>(v, gi, 0, smr, par, g.twx);
         if (iy < g.ny) {
             float2* dst = g.g1 + ((size_t)p * g.ny + iy) * L;
 #pragma unroll
@@ -251,51 +308,51 @@ grid_rows_adj_kernel(const DevProblem* __restrict__ probs, int prob, const GridO
 {
     using S = RowShape<LOG>;
     constexpr int L = 1 << LOG;
-    __shared__ float2 sm[S::ROWS][S::PAD];
+    extern __shared__ __align__(16) float2 sm_rows[];         // two buffers of BUF
     const double2* R;
     if (!adj_role(probs[prob], R)) return;
     const int rb = threadIdx.x / S::T;
     const int gi[1] = {(int)threadIdx.x % S::T};
     const int iy = blockIdx.x * S::ROWS + rb;
-    float acc[8];
-    float2 nu[8];
+    float acc[4];
+    float2 nu[4];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-        const int ix = cell_of(gi[0] + q * S::T, LOG, g.cx);
-        acc[q] = 0.f;
-        nu[q] = (iy < g.ny && ix >= 0 && ix < g.nx) ? g.nu[(size_t)iy * g.nx + ix] : make_float2(0.f, 0.f);
+    for (int i = 0; i < 4; ++i) {
+        const int ix = cell_of(gi[0] + cell_q(i) * S::T, LOG, g.cx);
+        acc[i] = 0.f;
+        nu[i] = (iy < g.ny && ix >= 0 && ix < g.nx) ? g.nu[(size_t)iy * g.nx + ix] : make_float2(0.f, 0.f);
     }
+    float2* smr = sm_rows + rb * L;
+    int par = 0;
     const int q1 = min(np, (int)(blockIdx.y + 1) * GR_PCH);
     for (int p = blockIdx.y * GR_PCH; p < q1; ++p) {
         const float2 w = g.wp[p0 + p];
         float2 v[1][8];
         const float2* src = g.g1 + ((size_t)p * g.ny + min(iy, g.ny - 1)) * L;
+        const unsigned char* act = g.colact + (size_t)(p0 + p) * (L / GR_TILE);
 #pragma unroll
         for (int q = 0; q < 8; ++q) {          // columns without a visibility were not written
             const int e = gi[0] + q * S::T;
-            v[0][q] = g.colact[(size_t)(p0 + p) * (L / GR_TILE) + e / GR_TILE] ? src[e] : make_float2(0.f, 0.f);
+            v[0][q] = act[e / GR_TILE] ? src[e] : make_float2(0.f, 0.f);
         }
-        fft_pass_all<LOG, 1, 1, 1>(v, gi, 0, sm[rb], g.twx);
+        fft_pass_all<LOG, 1, 1, 1, false, true, S::BUF>(v, gi, 0, smr, par, g.twx);
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const int ix = cell_of(gi[0] + q * S::T, LOG, g.cx);
-            if (ix >= 0 && ix < g.nx) {
-                const float2 e = plane_phase(w, nu[q]);              // conj(e) z, real part
-                acc[q] += fmaf(e.x, v[0][q].x, e.y * v[0][q].y);
-            }
+        for (int i = 0; i < 4; ++i) {
+            const float2 e = plane_phase(w, nu[i]);                  // conj(e) z, real part
+            acc[i] += fmaf(e.x, v[0][cell_q(i)].x, e.y * v[0][cell_q(i)].y);
         }
     }
     const int chunk = chunk0 + blockIdx.y;
     if (iy < g.ny) {
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const int ix = cell_of(gi[0] + q * S::T, LOG, g.cx);
+        for (int i = 0; i < 4; ++i) {
+            const int ix = cell_of(gi[0] + cell_q(i) * S::T, LOG, g.cx);
             if (ix < 0 || ix >= g.nx) continue;
             const size_t at = (size_t)iy * g.nx + ix;
             const int j = g.cell[at];
             if (j >= 0)
                 partial[((size_t)(j / BLK) * g.n_chunk + chunk) * BLK + j % BLK] =
-                    (double)acc[q] * ((double)g.amp[at] / (double)g.ascale);
+                    (double)acc[i] * ((double)g.amp[at] / (double)g.ascale);
         }
     }
     if (blockIdx.x == 0)                       // padding slots of the last pixel granule
@@ -312,7 +369,7 @@ struct ColShape {
     static constexpr int CB = LOG >= 11 ? 4 : 8;
     static constexpr int NB = LOG >= 12 ? 4 : LOG >= 8 ? 2 : 1;
     static constexpr int THREADS = CB * (1 << LOG) / 8 / NB;
-    static constexpr int SMEM = padded(1 << LOG, CB) * (int)sizeof(float2);
+    static constexpr int SMEM = CB * (1 << LOG) * (int)sizeof(float2);
 };
 template <int LOG, int SGN>
 __global__ void __launch_bounds__(ColShape<LOG>::THREADS, ColShape<LOG>::THREADS >= 512 && LOG < 12 ? 2 : 1)
@@ -350,14 +407,16 @@ grid_cols_kernel(const DevProblem* __restrict__ probs, int prob, const GridOp g,
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
             const int e = gi[n] + q * E;
-            if (SGN < 0) {
+            if (SGN > 0) {
+                v[n][q] = s_act[e / GR_TILE] ? g2[(size_t)e * Lx] : make_float2(0.f, 0.f);
+            } else if (q < 2 || q > 5) {
                 const int iy = cell_of(e, LOG, g.cy);
                 v[n][q] = (iy >= 0 && iy < g.ny) ? g1[(size_t)iy * Lx] : make_float2(0.f, 0.f);
-            } else {
-                v[n][q] = s_act[e / GR_TILE] ? g2[(size_t)e * Lx] : make_float2(0.f, 0.f);
             }
         }
-    fft_pass_all<LOG, SGN, S::CB, S::NB>(v, gi, c, sm_cols, g.twy);
+    float2* sm = sm_cols;
+    int par = 0;
+    fft_pass_all<LOG, SGN, S::CB, S::NB, (SGN < 0), (SGN > 0), 0>(v, gi, c, sm, par, g.twy);
 #pragma unroll
     for (int n = 0; n < S::NB; ++n)
 #pragma unroll
@@ -365,7 +424,7 @@ grid_cols_kernel(const DevProblem* __restrict__ probs, int prob, const GridOp g,
             const int e = gi[n] + q * E;
             if (SGN < 0) {
                 if (s_act[e / GR_TILE]) g2[(size_t)e * Lx] = v[n][q];
-            } else {
+            } else if (q < 2 || q > 5) {
                 const int iy = cell_of(e, LOG, g.cy);
                 if (iy >= 0 && iy < g.ny) g1[(size_t)iy * Lx] = v[n][q];
             }
@@ -376,34 +435,51 @@ grid_cols_kernel(const DevProblem* __restrict__ probs, int prob, const GridOp g,
 
 // Forward: each visibility from its 8 x 8 cells of 8 planes, one warp per
 // visibility (lane = 8 cells in x by 4 rows, twice): a plane's share is 8
-// segments of 64 bytes, and visibilities in k-d order share them in L1 / L2.
-__global__ void __launch_bounds__(256)
+// segments of 64 bytes.  Visibilities are taken by tile and first plane, so the
+// warps of a CTA find each other's cells in L1.  ALL: one pass holds every
+// plane, so the 16 loads of a lane need no test and are in flight together.
+template <bool ALL>
+__global__ void __launch_bounds__(256, 4)
 grid_gather_kernel(const DevProblem* __restrict__ probs, int prob, const GridOp g, int p0, int np, int n_vis_pad,
                    double2* __restrict__ partial)
 {
     const double* X;
     if (!fwd_role(probs[prob], X)) return;
-    const int k = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (k >= n_vis_pad) return;
+    const int i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (i >= n_vis_pad) return;
+    const int k = g.order[i];
     const int4 ps = g.pos[k];
+    if (!ALL && (ps.z >= p0 + np || ps.z + GRW <= p0) && p0 > 0) return;     // nothing to add
     const float* wt = g.wts + (size_t)k * (3 * GRW);
     const int tx = lane & 7, ty = lane >> 3;
     const int Lx = 1 << g.lx, Ly = 1 << g.ly;
     const int x = (ps.x + tx) & (Lx - 1);
     const size_t y0 = (size_t)((ps.y + ty) & (Ly - 1)) * Lx + x, y1 = (size_t)((ps.y + ty + 4) & (Ly - 1)) * Lx + x;
+    const size_t plane = (size_t)Ly * Lx;
+    const float2* pl = g.g2 + (size_t)(ALL ? ps.z : 0) * plane;
+    float2 a[GRW], b[GRW];
+#pragma unroll
+    for (int t = 0; t < GRW; ++t) {
+        if (ALL) {
+            a[t] = pl[t * plane + y0];
+            b[t] = pl[t * plane + y1];
+        } else {
+            const int p = ps.z + t - p0;
+            const bool in = p >= 0 && p < np;
+            a[t] = in ? pl[p * plane + y0] : make_float2(0.f, 0.f);
+            b[t] = in ? pl[p * plane + y1] : make_float2(0.f, 0.f);
+        }
+    }
     const float wx = wt[tx], wy0 = wt[GRW + ty], wy1 = wt[GRW + ty + 4];
+    const float4 wa = *reinterpret_cast<const float4*>(wt + 2 * GRW), wb = *reinterpret_cast<const float4*>(wt + 2 * GRW + 4);
+    const float ww[GRW] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
     float2 s0 = make_float2(0.f, 0.f), s1 = s0;
 #pragma unroll
     for (int t = 0; t < GRW; ++t) {
-        const int p = ps.z + t - p0;
-        if (p < 0 || p >= np) continue;
-        const float ww = wt[2 * GRW + t];
-        const float2* pl = g.g2 + (size_t)p * Ly * Lx;
-        const float2 a = pl[y0], b = pl[y1];
-        s0.x = fmaf(ww, a.x, s0.x);
-        s0.y = fmaf(ww, a.y, s0.y);
-        s1.x = fmaf(ww, b.x, s1.x);
-        s1.y = fmaf(ww, b.y, s1.y);
+        s0.x = fmaf(ww[t], a[t].x, s0.x);
+        s0.y = fmaf(ww[t], a[t].y, s0.y);
+        s1.x = fmaf(ww[t], b[t].x, s1.x);
+        s1.y = fmaf(ww[t], b[t].y, s1.y);
     }
     float sr = wx * fmaf(wy0, s0.x, wy1 * s1.x), si = wx * fmaf(wy0, s0.y, wy1 * s1.y);
 #pragma unroll
@@ -416,7 +492,7 @@ grid_gather_kernel(const DevProblem* __restrict__ probs, int prob, const GridOp 
         const double inv = 1.0 / (double)g.fscale;
         double2 v = make_double2((double)fmaf(e.x, sr, -e.y * si) * inv, (double)fmaf(e.x, si, e.y * sr) * inv);
         if (ps.w) v.y = -v.y;                  // taken at the mirrored point
-        if (p0 > 0) {                          // a later pass over the planes
+        if (!ALL && p0 > 0) {                  // a later pass over the planes
             const double2 o = partial[k];
             v.x += o.x;
             v.y += o.y;
@@ -425,74 +501,111 @@ grid_gather_kernel(const DevProblem* __restrict__ probs, int prob, const GridOp 
     }
 }
 
-// Adjoint: a CTA owns GR_TILE^2 cells (one per thread) of GR_PCH planes and
-// adds the visibilities that touch them in list order: no atomics, the same
-// sum every time.  Each point's x, y weights times conj(rot) r are formed once
-// for the 8 planes.
-__global__ void __launch_bounds__(GR_TILE * GR_TILE)
-grid_spread_kernel(const DevProblem* __restrict__ probs, int prob, const GridOp g, int p0, int np)
+// Adjoint: a CTA owns the GR_TILE^2 cells (one per thread) of a tile and walks
+// the visibilities that touch it in the order of their first plane, with a ring
+// of 8 accumulators per cell, the planes the current point reaches: once the
+// points move on to a later first plane, the planes left behind are complete
+// and are written.  So every point is visited once per tile, no atomics are
+// needed and the sums are the same every time.  A warp (8 x 4 cells) visits
+// only the points that meet it.  Points are staged 32 at a time, the next ones
+// loaded while the current ones are added (a CTA has few, and each is two
+// dependent loads away).  blockIdx.y cuts the planes into segments of
+// seg_planes; a point that reaches into two segments is visited in both.
+__global__ void __launch_bounds__(GR_TILE * GR_TILE, 4)
+grid_spread_kernel(const DevProblem* __restrict__ probs, int prob, const GridOp g, int p0, int np, int seg_planes)
 {
-    constexpr int PB = 32;                     // points staged at a time
-    __shared__ float4 s_pt[PB];                // {Re, Im of conj(rot) r, first x, first y}
-    __shared__ float s_wx[PB][GRW], s_wy[PB][GRW], s_ww[PB][GR_PCH];
+    constexpr int PB = 32;                     // points staged at a time, by 8 threads each
+    __shared__ float4 s_pt[2][PB];             // {Re, Im of conj(rot) r, first x, first y}
+    __shared__ __align__(16) float s_wx[2][PB][GRW], s_wy[2][PB][GRW], s_ww[2][PB][GRW];
+    __shared__ int s_ip[2][PB];
     const double2* R;
     if (!adj_role(probs[prob], R)) return;
     const int Lx = 1 << g.lx, Ly = 1 << g.ly, tiles_x = Lx / GR_TILE;
     const int tile = blockIdx.x;
-    const int x = (tile % tiles_x) * GR_TILE + (threadIdx.x % GR_TILE);
-    const int y = (tile / tiles_x) * GR_TILE + (threadIdx.x / GR_TILE);
-    const int q0 = blockIdx.y * GR_PCH;        // first plane of the CTA within the pass
-    const int pg = p0 + q0;                    // ... and of all
+    const int ta = p0 + blockIdx.y * seg_planes, tb = min(ta + seg_planes, p0 + np);   // planes [ta, tb)
     const int ni = g.np - GRW + 1;             // values of a first plane
     const int* st = g.start + (size_t)tile * (ni + 1);
-    const int i0 = max(0, min(ni, pg - GRW + 1)), i1 = max(i0, min(ni, pg + GR_PCH));
-    const int b0 = st[i0], b1 = st[i1];
-    if (b0 == b1) return;                      // no plane of the CTA is touched here
-    float2 acc[GR_PCH];
-#pragma unroll
-    for (int q = 0; q < GR_PCH; ++q) acc[q] = make_float2(0.f, 0.f);
-    for (int b = b0; b < b1; b += PB) {
-        const int n = min(PB, b1 - b);
-        __syncthreads();
-        for (int e = threadIdx.x; e < n * 32; e += GR_TILE * GR_TILE) {
-            const int i = e >> 5, f = e & 31;
-            const int k = g.list[b + i];
-            const float* wt = g.wts + (size_t)k * (3 * GRW);
-            if (f < 8) {
-                s_wx[i][f] = wt[f];
-            } else if (f < 16) {
-                s_wy[i][f - 8] = wt[f];
-            } else if (f < 24) {
-                const int t = pg + (f - 16) - g.pos[k].z;
-                s_ww[i][f - 16] = (t >= 0 && t < GRW) ? wt[2 * GRW + t] : 0.f;
-            } else if (f == 24) {
-                const int4 ps = g.pos[k];
-                const float2 o = g.rot[k];
-                const double2 r = R[k];
-                const float rr = (float)r.x * g.ascale, ri = (float)(ps.w ? -r.y : r.y) * g.ascale;
-                s_pt[i] = make_float4(fmaf(o.x, rr, o.y * ri), fmaf(o.x, ri, -o.y * rr), __int_as_float(ps.x),
-                                      __int_as_float(ps.y));
-            }
+    const int b0 = st[max(0, min(ni, ta - GRW + 1))], b1 = st[max(0, min(ni, tb))];
+    if (b0 >= b1) return;                      // no plane of the segment is touched here
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int wx0 = (tile % tiles_x) * GR_TILE + (warp & 1) * 8, wy0 = (tile / tiles_x) * GR_TILE + (warp >> 1) * 4;
+    const int x = wx0 + (lane & 7), y = wy0 + (lane >> 3);
+    const size_t plane = (size_t)Ly * Lx;
+    float2* const cell = g.g2 + (size_t)y * Lx + x;
+    const unsigned char* act = g.act + ((size_t)(tile % tiles_x)) * (Ly / GR_TILE) + tile / tiles_x;
+    const size_t act_plane = (size_t)tiles_x * (Ly / GR_TILE);
+    // this thread's part of the staging: point si, weights sf of each axis
+    const int si = threadIdx.x >> 3, sf = threadIdx.x & 7;
+    float lwx = 0.f, lwy = 0.f, lww = 0.f;
+    float4 lpt = make_float4(0.f, 0.f, 0.f, 0.f);
+    int lip = 0;
+    const auto fetch = [&](int b) {
+        if (b + si >= b1) return;
+        const int k = g.list[b + si];
+        const float* wt = g.wts + (size_t)k * (3 * GRW);
+        lwx = wt[sf];
+        lwy = wt[GRW + sf];
+        lww = wt[2 * GRW + sf];
+        if (sf == 0) {
+            const int4 ps = g.pos[k];
+            const float2 o = g.rot[k];
+            const double2 r = R[k];
+            const float rr = (float)r.x * g.ascale, ri = (float)(ps.w ? -r.y : r.y) * g.ascale;
+            lpt = make_float4(fmaf(o.x, rr, o.y * ri), fmaf(o.x, ri, -o.y * rr), __int_as_float(ps.x),
+                              __int_as_float(ps.y));
+            lip = ps.z;
         }
-        __syncthreads();
-        for (int i = 0; i < n; ++i) {
-            const float4 pt = s_pt[i];
+    };
+    float2 acc[GRW];
+#pragma unroll
+    for (int q = 0; q < GRW; ++q) acc[q] = make_float2(0.f, 0.f);
+    int cur = max(0, ta - GRW + 1);            // acc[q] is plane cur + q
+    // planes [cur, to) are complete
+    const auto advance = [&](int to) {
+        for (; cur < to; ++cur) {
+            if (cur >= ta && cur < tb && act[cur * act_plane]) cell[(size_t)(cur - p0) * plane] = acc[0];
+#pragma unroll
+            for (int q = 0; q + 1 < GRW; ++q) acc[q] = acc[q + 1];
+            acc[GRW - 1] = make_float2(0.f, 0.f);
+        }
+    };
+    fetch(b0);
+    int buf = 0;
+    for (int b = b0; b < b1; b += PB, buf ^= 1) {
+        const int n = min(PB, b1 - b);
+        s_wx[buf][si][sf] = lwx;
+        s_wy[buf][si][sf] = lwy;
+        s_ww[buf][si][sf] = lww;
+        if (sf == 0) {
+            s_pt[buf][si] = lpt;
+            s_ip[buf][si] = lip;
+        }
+        __syncthreads();                       // (the other buffer's readers are done, too)
+        fetch(b + PB);
+        // the staged points whose 8 x 8 cells meet the warp's (lane = point)
+        const float4 pl = s_pt[buf][lane];
+        const int ox = (__float_as_int(pl.z) - wx0 + GRW - 1) & (Lx - 1), oy = (__float_as_int(pl.w) - wy0 + GRW - 1) & (Ly - 1);
+        unsigned todo = __ballot_sync(0xffffffffu, lane < n && ox < 8 + GRW - 1 && oy < 4 + GRW - 1);
+        for (; todo; todo &= todo - 1) {
+            const int i = __ffs(todo) - 1;
+            const float4 pt = s_pt[buf][i];
+            advance(s_ip[buf][i]);
             const int dx = (x - __float_as_int(pt.z)) & (Lx - 1), dy = (y - __float_as_int(pt.w)) & (Ly - 1);
             if (dx < GRW && dy < GRW) {
-                const float w = s_wx[i][dx] * s_wy[i][dy];
+                const float w = s_wx[buf][i][dx] * s_wy[buf][i][dy];
                 const float vr = w * pt.x, vi = w * pt.y;
+                const float4 wa = *reinterpret_cast<const float4*>(s_ww[buf][i]);
+                const float4 wb = *reinterpret_cast<const float4*>(s_ww[buf][i] + 4);
+                const float ww[GRW] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
 #pragma unroll
-                for (int q = 0; q < GR_PCH; ++q) {
-                    const float ww = s_ww[i][q];
-                    acc[q].x = fmaf(ww, vr, acc[q].x);
-                    acc[q].y = fmaf(ww, vi, acc[q].y);
+                for (int q = 0; q < GRW; ++q) {
+                    acc[q].x = fmaf(ww[q], vr, acc[q].x);
+                    acc[q].y = fmaf(ww[q], vi, acc[q].y);
                 }
             }
         }
     }
-#pragma unroll
-    for (int q = 0; q < GR_PCH; ++q)
-        if (q0 + q < np) g.g2[((size_t)(q0 + q) * Ly + y) * Lx + x] = acc[q];
+    advance(tb);
 }
 
 // ------------------------------------------------------------------ set-up
@@ -581,7 +694,7 @@ static void rows_fwd(const DevProblem* probs, int p, const GridOp& g, int p0, in
 {
     using S = RowShape<LOG>;
     const dim3 grid((unsigned)((g.ny + S::ROWS - 1) / S::ROWS), (unsigned)((np + GR_PCH - 1) / GR_PCH));
-    grid_rows_fwd_kernel<LOG><<<grid, S::THREADS, 0, st>>>(probs, p, g, p0, np);
+    grid_rows_fwd_kernel<LOG><<<grid, S::THREADS, S::SMEM, st>>>(probs, p, g, p0, np);
 }
 template <int LOG>
 static void rows_adj(const DevProblem* probs, int p, const GridOp& g, int p0, int np, int chunk0, int n_pix,
@@ -589,7 +702,7 @@ static void rows_adj(const DevProblem* probs, int p, const GridOp& g, int p0, in
 {
     using S = RowShape<LOG>;
     const dim3 grid((unsigned)((g.ny + S::ROWS - 1) / S::ROWS), (unsigned)((np + GR_PCH - 1) / GR_PCH));
-    grid_rows_adj_kernel<LOG><<<grid, S::THREADS, 0, st>>>(probs, p, g, p0, np, chunk0, n_pix, n_pix_pad, partial);
+    grid_rows_adj_kernel<LOG><<<grid, S::THREADS, S::SMEM, st>>>(probs, p, g, p0, np, chunk0, n_pix, n_pix_pad, partial);
 }
 template <int LOG, int SGN>
 static void cols(const DevProblem* probs, int p, const GridOp& g, int p0, int np, cudaStream_t st)
@@ -619,7 +732,10 @@ cudaError_t grid_forward(const DevProblem* probs, int p, const GridOp& g, int n_
         const int np = std::min(g.np_pass, g.np - p0);
         GRID_DISPATCH(g.lx, (rows_fwd<LOG>(probs, p, g, p0, np, st)));
         GRID_DISPATCH(g.ly, (cols<LOG, -1>(probs, p, g, p0, np, st)));
-        grid_gather_kernel<<<(n_vis_pad + 7) / 8, 256, 0, st>>>(probs, p, g, p0, np, n_vis_pad, partial);
+        if (g.np_pass >= g.np)
+            grid_gather_kernel<true><<<(n_vis_pad + 7) / 8, 256, 0, st>>>(probs, p, g, p0, np, n_vis_pad, partial);
+        else
+            grid_gather_kernel<false><<<(n_vis_pad + 7) / 8, 256, 0, st>>>(probs, p, g, p0, np, n_vis_pad, partial);
         *n_launch += 3;
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
@@ -632,8 +748,11 @@ cudaError_t grid_adjoint(const DevProblem* probs, int p, const GridOp& g, int n_
 {
     for (int p0 = 0; p0 < g.np; p0 += g.np_pass) {
         const int np = std::min(g.np_pass, g.np - p0);
-        const dim3 sg((unsigned)grid_tiles(g), (unsigned)((np + GR_PCH - 1) / GR_PCH));
-        grid_spread_kernel<<<sg, GR_TILE * GR_TILE, 0, st>>>(probs, p, g, p0, np);
+        // segments of planes: enough CTAs for a few waves, no fewer planes than 32
+        const int tiles = grid_tiles(g), nseg = std::max(1, std::min((np + 31) / 32, 4096 / tiles));
+        const int seg = (np + nseg - 1) / nseg;
+        const dim3 sg((unsigned)tiles, (unsigned)((np + seg - 1) / seg));
+        grid_spread_kernel<<<sg, GR_TILE * GR_TILE, 0, st>>>(probs, p, g, p0, np, seg);
         GRID_DISPATCH(g.ly, (cols<LOG, 1>(probs, p, g, p0, np, st)));
         GRID_DISPATCH(g.lx, (rows_adj<LOG>(probs, p, g, p0, np, p0 / GR_PCH, n_pix, n_pix_pad, partial, st)));
         *n_launch += 3;
@@ -644,19 +763,25 @@ cudaError_t grid_adjoint(const DevProblem* probs, int p, const GridOp& g, int n_
 }
 
 template <int LOG>
-static cudaError_t raise_cols()
+static cudaError_t raise_limits()
 {
     cudaError_t e = cudaFuncSetAttribute(grid_cols_kernel<LOG, -1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          ColShape<LOG>::SMEM);
     if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(grid_cols_kernel<LOG, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                ColShape<LOG>::SMEM);
+    e = cudaFuncSetAttribute(grid_cols_kernel<LOG, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             ColShape<LOG>::SMEM);
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(grid_rows_fwd_kernel<LOG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             RowShape<LOG>::SMEM);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(grid_rows_adj_kernel<LOG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                RowShape<LOG>::SMEM);
 }
 cudaError_t grid_prepare_kernels()
 {
     for (int lg = GR_LOG_MIN; lg <= GR_LOG_MAX; ++lg) {
         cudaError_t e = cudaSuccess;
-        GRID_DISPATCH(lg, (e = raise_cols<LOG>()));
+        GRID_DISPATCH(lg, (e = raise_limits<LOG>()));
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;

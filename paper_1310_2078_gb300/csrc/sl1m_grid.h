@@ -9,7 +9,7 @@ namespace sl1m {
 
 constexpr int GRW = 8;          // gridding kernel width: cells per axis, and planes in w
 constexpr int GR_TILE = 16;     // the adjoint spreads onto tiles of GR_TILE^2 cells
-constexpr int GR_PCH = 8;       // planes a CTA of the row and spreading kernels takes
+constexpr int GR_PCH = 8;       // planes a CTA of the row kernels takes
 constexpr int GR_LOG_MIN = 6, GR_LOG_MAX = 12;   // FFT lengths 64 .. 4096
 // The exponential-of-semicircle kernel phi(z) = exp(GR_BETA (sqrt(1 - (2z/GRW)^2) - 1)).
 constexpr double GR_BETA = 2.30 * GRW;
@@ -33,6 +33,7 @@ struct GridOp {
     const int4* pos;            // [vis.n_pad] first cell x, y (wrapped), first plane, 1 if mirrored
     const float* wts;           // [vis.n_pad][3 GRW] kernel weights in x, y, w
     const float2* rot;          // [vis.n_pad] exp(-2 pi i (u lc + v mc + w nc))
+    const int* order;           // [vis.n_pad] the visibilities by tile and first plane
     const int* list;            // visibilities touching each tile, by first plane
     const int* start;           // [tiles][np - GRW + 2] list offsets
     const unsigned char* act;   // [np][tiles in x][tiles in y] 1 where a visibility touches the plane's tile

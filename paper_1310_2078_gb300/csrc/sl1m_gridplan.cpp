@@ -174,7 +174,7 @@ bool grid_build(sl1m_problem& P, cudaStream_t st, size_t budget)
     T->ws_elems = grid_plane_elems(g) * g.np_pass;
     const size_t nv = P.hp.vis.n_pad, cells = (size_t)g.nx * g.ny;
     const int tiles = grid_tiles(g), ni = g.np - GRW + 1;
-    const size_t tab = cells * 16 + nv * (16 + 12 * GRW + 8 + 16) + (size_t)tiles * (ni * 5 + 44);
+    const size_t tab = cells * 16 + nv * (16 + 12 * GRW + 8 + 20) + (size_t)tiles * (ni * 5 + 44);
     if (tab + T->ws_elems * sizeof(float2) > std::min(budget, free_b / 2)) return false;
     // powers of two that keep a coherent sum of the largest inputs in range
     const auto p2 = [](double n) { return (float)std::exp2(-std::ceil(std::log2(std::max(1.0, n)))); };
@@ -235,7 +235,7 @@ bool grid_build(sl1m_problem& P, cudaStream_t st, size_t budget)
     }
     // visibilities per tile (at most two tiles per axis), by first plane, in the
     // library's order: a counting sort
-    std::vector<int> start, list;
+    std::vector<int> start, list, order;
     if (ok) {
         const int txn = (1 << g.lx) / GR_TILE, mx = (1 << g.lx) - 1, my = (1 << g.ly) - 1;
         start.assign((size_t)tiles * (ni + 1) + 1, 0);
@@ -254,6 +254,15 @@ bool grid_build(sl1m_problem& P, cudaStream_t st, size_t budget)
         list.resize(std::max(1, start.back()));
         std::vector<int> fill(start.begin(), start.end() - 1);
         each([&](size_t k, size_t at) { list[fill[at]++] = (int)k; });
+        // each visibility once, at its first tile; then the padding slots
+        order.reserve(nv);
+        for (int t = 0; t < tiles; ++t)
+            for (int i = start[(size_t)t * (ni + 1)]; i < start[(size_t)(t + 1) * (ni + 1)]; ++i) {
+                const int4 q = pos[list[i]];
+                if ((q.y / GR_TILE) * txn + q.x / GR_TILE == t) order.push_back(list[i]);
+            }
+        for (size_t k = 0; k < nv; ++k)
+            if (P.vis_orig[k] < 0) order.push_back((int)k);
         // which tiles of each plane have a visibility
         const int tyn = (1 << g.ly) / GR_TILE;
         std::vector<unsigned char> act((size_t)g.np * tiles, 0), colact((size_t)g.np * txn, 0);
@@ -268,6 +277,7 @@ bool grid_build(sl1m_problem& P, cudaStream_t st, size_t budget)
             }
         ok = T->start.upload(start.data(), start.size(), st) == cudaSuccess &&
              T->list.upload(list.data(), list.size(), st) == cudaSuccess &&
+             T->order.upload(order.data(), order.size(), st) == cudaSuccess &&
              T->act.upload(act.data(), act.size(), st) == cudaSuccess &&
              T->colact.upload(colact.data(), colact.size(), st) == cudaSuccess;
     }
@@ -280,6 +290,7 @@ bool grid_build(sl1m_problem& P, cudaStream_t st, size_t budget)
     g.pos = T->pos.p;
     g.wts = T->wts.p;
     g.rot = T->rot.p;
+    g.order = T->order.p;
     g.list = T->list.p;
     g.start = T->start.p;
     g.act = T->act.p;

@@ -131,14 +131,14 @@ cudaError_t upload_plan(const HostPlan& H, int n_probs, int blk_el, DevPlan& D, 
 struct GridTables {
     sl1m::GridOp op{};
     size_t ws_elems = 0;                 // float2 of workspace
-    DBuf<int> cell, list, start;
+    DBuf<int> cell, list, start, order;
     DBuf<float> amp, wts;
     DBuf<float2> nu, wp, twx, twy, rot;
     DBuf<int4> pos;
     DBuf<unsigned char> act, colact;
     size_t bytes() const
     {
-        return cell.bytes() + list.bytes() + start.bytes() + amp.bytes() + wts.bytes() + nu.bytes() + wp.bytes() +
+        return cell.bytes() + order.bytes() + list.bytes() + start.bytes() + amp.bytes() + wts.bytes() + nu.bytes() + wp.bytes() +
                twx.bytes() + twy.bytes() + rot.bytes() + pos.bytes() + act.bytes() + colact.bytes();
     }
 };
