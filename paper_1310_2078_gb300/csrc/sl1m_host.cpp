@@ -69,11 +69,12 @@ static inline float f32lo(double x) { return (float)(x - (double)(float)x); }
 // split are independent (disjoint ranges of idx), so down to `par_depth`
 // levels the left half runs on a thread of its own: the same operations on
 // the same ranges, so the same order as one thread gives.
+// leaf: elements per granule (fewer than G where an element stands for several).
 static void kd_rec(std::vector<int>& idx, size_t lo, size_t hi, const double* x, const double* y,
-                   size_t stride, int par_depth)
+                   size_t stride, int par_depth, size_t leaf = G)
 {
     const size_t n = hi - lo;
-    if (n <= (size_t)G) return;
+    if (n <= leaf) return;
     double x0 = 1e300, x1 = -1e300, y0 = 1e300, y1 = -1e300;
     for (size_t i = lo; i < hi; ++i) {
         const double a = x[(size_t)idx[i] * stride], b = y[(size_t)idx[i] * stride];
@@ -81,8 +82,8 @@ static void kd_rec(std::vector<int>& idx, size_t lo, size_t hi, const double* x,
         y0 = std::min(y0, b); y1 = std::max(y1, b);
     }
     const double* key = (x1 - x0 >= y1 - y0) ? x : y;
-    const size_t ng = (n + G - 1) / G;
-    const size_t left = (ng / 2) * G;
+    const size_t ng = (n + leaf - 1) / leaf;
+    const size_t left = (ng / 2) * leaf;
     std::nth_element(idx.begin() + lo, idx.begin() + lo + left, idx.begin() + hi,
                      [&](int a, int b) {
                          const double ka = key[(size_t)a * stride], kb = key[(size_t)b * stride];
@@ -91,15 +92,15 @@ static void kd_rec(std::vector<int>& idx, size_t lo, size_t hi, const double* x,
     if (par_depth > 0 && n >= (size_t)1 << 16) {
         std::future<void> f;
         try {
-            f = std::async(std::launch::async, [&] { kd_rec(idx, lo, lo + left, x, y, stride, par_depth - 1); });
+            f = std::async(std::launch::async, [&] { kd_rec(idx, lo, lo + left, x, y, stride, par_depth - 1, leaf); });
         } catch (...) {                    // no thread to be had: the left half runs here
-            kd_rec(idx, lo, lo + left, x, y, stride, 0);
+            kd_rec(idx, lo, lo + left, x, y, stride, 0, leaf);
         }
-        kd_rec(idx, lo + left, hi, x, y, stride, par_depth - 1);
+        kd_rec(idx, lo + left, hi, x, y, stride, par_depth - 1, leaf);
         if (f.valid()) f.get();
     } else {
-        kd_rec(idx, lo, lo + left, x, y, stride, 0);
-        kd_rec(idx, lo + left, hi, x, y, stride, 0);
+        kd_rec(idx, lo, lo + left, x, y, stride, 0, leaf);
+        kd_rec(idx, lo + left, hi, x, y, stride, 0, leaf);
     }
 }
 
@@ -182,6 +183,81 @@ static void sort_baselines(std::vector<int>& order, const std::vector<int>& ant)
             const long long ky = (long long)ant[2 * y] << 32 | (unsigned)ant[2 * y + 1];
             return kx < ky;
         });
+}
+
+// With gains: an order of the visibilities in which a granule holds few antenna
+// pairs.  Every pair's visibilities are cut, in the caller's order (time, as a
+// rule), into runs of s; granules are 64 / s runs that are neighbours in (u, v)
+// (k-d order of the runs' centres).  What is left over of each pair follows in
+// point order.  keys: the pair of every visibility.
+static std::vector<int> order_by_runs(const std::vector<long long>& keys, const double* uvw, int s)
+{
+    const size_t n = keys.size();
+    std::vector<int> by(n);
+    for (size_t k = 0; k < n; ++k) by[k] = (int)k;
+    std::stable_sort(by.begin(), by.end(), [&](int a, int b) { return keys[a] < keys[b]; });
+    std::vector<int> first, rest;               // first member of every run, in `by`
+    std::vector<double> centre;                 // (u, v) of every run
+    for (size_t i = 0, j; i < n; i = j) {
+        for (j = i; j < n && keys[by[j]] == keys[by[i]]; ++j) {}
+        size_t at = i;
+        for (; at + s <= j; at += s) {
+            double u = 0, v = 0;
+            for (int t = 0; t < s; ++t) {
+                u += uvw[3 * (size_t)by[at + t]];
+                v += uvw[3 * (size_t)by[at + t] + 1];
+            }
+            first.push_back((int)at);
+            centre.push_back(u / s);
+            centre.push_back(v / s);
+        }
+        rest.insert(rest.end(), by.begin() + at, by.begin() + j);
+    }
+    std::vector<int> runs(first.size()), order;
+    for (size_t r = 0; r < runs.size(); ++r) runs[r] = (int)r;
+    if (!runs.empty()) kd_rec(runs, 0, runs.size(), centre.data(), centre.data() + 1, 2, kd_par_depth(), G / s);
+    order.reserve(n + 2 * G);
+    for (int r : runs) order.insert(order.end(), by.begin() + first[r], by.begin() + first[r] + s);
+    while (order.size() % G) order.push_back(-1);
+    if (!rest.empty()) kd_append(order, std::move(rest), uvw, uvw + 1, 3);
+    return order;
+}
+
+// Relative cost of the gains kernels' tiles over all granules of an order: a
+// pair takes about 15 instructions (three times that on the exact phase path),
+// and every distinct antenna pair of a granule about 28 per streamed pixel
+// (the pair table); a granule with more than NB_MAX pairs takes gathers, about
+// 10 more a pair.
+static double gains_order_cost(const std::vector<int>& order, const std::vector<long long>& keys, const double* uvw,
+                               const std::vector<float4>& pext)
+{
+    const size_t ng = order.size() / G, step = (pext.size() + 255) / 256;
+    std::vector<double> cost(ng, 0.0);
+    parallel_chunks(ng, 64, [&](size_t g0, size_t g1) {
+        std::vector<long long> ks;
+        for (size_t g = g0; g < g1; ++g) {
+            double mn[3] = {1e300, 1e300, 1e300}, mx[3] = {-1e300, -1e300, -1e300};
+            ks.clear();
+            for (size_t i = g * G; i < (g + 1) * G; ++i) {
+                const int o = order[i];
+                if (o < 0) continue;
+                ks.push_back(keys[o]);
+                for (int a = 0; a < 3; ++a) {
+                    mn[a] = std::min(mn[a], uvw[3 * (size_t)o + a]);
+                    mx[a] = std::max(mx[a], uvw[3 * (size_t)o + a]);
+                }
+            }
+            std::sort(ks.begin(), ks.end());
+            const int nb = (int)(std::unique(ks.begin(), ks.end()) - ks.begin());
+            int n_ex = 0, n = 0;
+            for (size_t p = 0; p < pext.size(); p += step, ++n)
+                n_ex += 0.5 * ((mx[0] - mn[0]) * pext[p].x + (mx[1] - mn[1]) * pext[p].y + (mx[2] - mn[2]) * pext[p].z) > D_MAX;
+            cost[g] = G * (15.0 + 30.0 * n_ex / std::max(1, n)) + (nb <= NB_MAX ? 28.0 * nb : 10.0 * G);
+        }
+    });
+    double t = 0;
+    for (double c : cost) t += c;
+    return t;
 }
 
 // An allocator whose resize() leaves new elements of a trivial type
@@ -667,6 +743,25 @@ int sl1m_problem::rebuild(cudaStream_t st, size_t grid_budget)
         for (int64_t k = 0; k < n_vis; ++k) members[k] = (int)k;
         std::vector<int> order;
         kd_append(order, std::move(members), uvw.data(), uvw.data() + 1, 3);
+        if (n_ant > 0) {
+            // the cheapest of the point order and of runs of 16, 8 and 4 samples
+            // of a pair (tried while the mean pair has that many)
+            std::vector<long long> keys(n_vis), distinct;
+            for (int64_t k = 0; k < n_vis; ++k) keys[k] = (long long)ant[2 * k] * n_ant + ant[2 * k + 1];
+            distinct = keys;
+            std::sort(distinct.begin(), distinct.end());
+            const double per = (double)n_vis / (double)(std::unique(distinct.begin(), distinct.end()) - distinct.begin());
+            double best = gains_order_cost(order, keys, uvw.data(), gext_pix);
+            for (int s = 16; s >= 4; s /= 2) {
+                if (per < 0.75 * s) continue;
+                std::vector<int> o = order_by_runs(keys, uvw.data(), s);
+                const double c = gains_order_cost(o, keys, uvw.data(), gext_pix);
+                if (c < best) {
+                    best = c;
+                    order.swap(o);
+                }
+            }
+        }
         group_by_exact_share(order, uvw.data(), gext_pix);
         if (n_ant > 0) sort_baselines(order, ant);
         std::vector<d4> xyz(n_vis);
