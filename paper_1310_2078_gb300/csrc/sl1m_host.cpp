@@ -572,6 +572,11 @@ sl1m_ctx::~sl1m_ctx()
     drain_profile();
     for (auto e : ev_pool) cudaEventDestroy(e);
     if (upstream) cudaStreamDestroy(upstream);
+    for (auto s : side)
+        if (s) cudaStreamDestroy(s);
+    for (auto e : ev_join)
+        if (e) cudaEventDestroy(e);
+    if (ev_fork) cudaEventDestroy(ev_fork);
     if (own_stream && stream) cudaStreamDestroy(stream);
 }
 
@@ -1106,8 +1111,8 @@ static int set_grid_plans(sl1m_ctx* ctx, Batch& B, const std::vector<DevProblem>
         }
         H.n_blocks = H.b0[np];
         CK(upload_plan(H, np, BLK, B.plan[op][CLS_GRID], ctx->stream));
-        if (op == 0) CK(ctx->partial_f.reserve((size_t)std::max(1, H.n_slots) * BLK, ctx->stream));
-        else CK(ctx->partial_a.reserve((size_t)std::max(1, H.n_slots) * BLK, ctx->stream));
+        if (op == 0) CK(ctx->partial_f[CLS_GRID].reserve((size_t)std::max(1, H.n_slots) * BLK, ctx->stream));
+        else CK(ctx->partial_a[CLS_GRID].reserve((size_t)std::max(1, H.n_slots) * BLK, ctx->stream));
         B.fin_bytes[op] += (double)H.n_slots * BLK * (op == 0 ? 16.0 : 8.0);
     }
     return SL1M_OK;
@@ -1122,8 +1127,12 @@ int batch_set(sl1m_ctx* ctx, Batch& B, const std::vector<sl1m_problem*>& probs,
     cudaStream_t st = ctx->stream;
     const int np = (int)probs.size();
     if (np == 0) return sl1m_fail(ctx, SL1M_ERR_ARG, "empty batch");
-    const void* old_ptrs[7] = {B.desc.p, ctx->partial_f.p, ctx->partial_a.p, B.n_probs_dev.p,
-                               B.plan[0][0].dpl.p, B.plan[1][1].dpl.p, ctx->grid_ws.p};
+    const auto baked = [&] {
+        std::vector<const void*> v = ctx->scratch();
+        v.insert(v.end(), {B.desc.p, B.n_probs_dev.p, B.plan[0][0].dpl.p, B.plan[1][1].dpl.p});
+        return v;
+    };
+    const std::vector<const void*> old_ptrs = baked();
     std::vector<uint64_t> gens(np);
     for (int p = 0; p < np; ++p) gens[p] = probs[p]->gen;
     const bool same_set =
@@ -1203,8 +1212,8 @@ int batch_set(sl1m_ctx* ctx, Batch& B, const std::vector<sl1m_problem*>& probs,
             CK(build_plan(nbf, nsf, ctx->num_sms * kf, BLK_GRAN, B.plan[0][c], st, &cf));
             CK(build_plan(nba, nsa, ctx->num_sms * ka, oga, B.plan[1][c], st, &ca));
             const Plan &pf = B.plan[0][c].pl, &pa = B.plan[1][c].pl;
-            CK(ctx->partial_f.reserve((size_t)std::max(1, pf.n_slots) * pf.blk_el, st));
-            CK(ctx->partial_a.reserve((size_t)std::max(1, pa.n_slots) * pa.blk_el, st));
+            CK(ctx->partial_f[c].reserve((size_t)std::max(1, pf.n_slots) * pf.blk_el, st));
+            CK(ctx->partial_a[c].reserve((size_t)std::max(1, pa.n_slots) * pa.blk_el, st));
             B.fin_bytes[0] += (double)pf.n_slots * pf.blk_el * 16.0;
             B.fin_bytes[1] += (double)pa.n_slots * pa.blk_el * 8.0;
         }
@@ -1214,9 +1223,7 @@ int batch_set(sl1m_ctx* ctx, Batch& B, const std::vector<sl1m_problem*>& probs,
         }
         B.sc_grid = std::max(1, std::min(ctx->num_sms * 4, np));
     }
-    const void* new_ptrs[7] = {B.desc.p, ctx->partial_f.p, ctx->partial_a.p, B.n_probs_dev.p,
-                               B.plan[0][0].dpl.p, B.plan[1][1].dpl.p, ctx->grid_ws.p};
-    if (!same_set || memcmp(old_ptrs, new_ptrs, sizeof old_ptrs) != 0) B.graph_ok = false;
+    if (!same_set || old_ptrs != baked()) B.graph_ok = false;
     return SL1M_OK;
 }
 
@@ -1228,10 +1235,9 @@ static int polar_of(int precision, int c)
 }
 
 // user_out: the result of an operator call, in the caller's order (null in a tick).
-static int launch_op_class(sl1m_ctx* ctx, Batch& B, int op, int c, double* user_out)
+static int launch_op_class(sl1m_ctx* ctx, Batch& B, int op, int c, double* user_out, cudaStream_t st)
 {
     if (!B.has_class[c]) return SL1M_OK;
-    cudaStream_t st = ctx->stream;
     const DevPlan& P = B.plan[op][c];
     ProfTok tk;
     // the lattice operators, problem by problem: each fills the GPU by itself
@@ -1251,14 +1257,14 @@ static int launch_op_class(sl1m_ctx* ctx, Batch& B, int op, int c, double* user_
         if (c == CLS_GRID)
             RET(each_grid([&](int p, const GridOp& g) {
                 return grid_forward(B.desc.p, p, g, B.hdesc[p].vis.n_pad,
-                                    ctx->partial_f.p + (size_t)B.grid_slot[0][p] * BLK, st, &ctx->n_launch);
+                                    ctx->partial_f[c].p + (size_t)B.grid_slot[0][p] * BLK, st, &ctx->n_launch);
             }));
         else
-            CKL(launch_forward(B.precision, c == 1, B.n_ant_max, B.desc.p, P.dpl.p, P.pl.C, ctx->partial_f.p, st,
+            CKL(launch_forward(B.precision, c == 1, B.n_ant_max, B.desc.p, P.dpl.p, P.pl.C, ctx->partial_f[c].p, st,
                                B.nst[0][c]));
         prof_end(ctx, tk, B.solver ? 0.0 : B.pairs_class[c], 0.0);   // solver ticks: counted on the device
         prof_begin(ctx, 4, tk);
-        CKL(launch_fwd_finish(B.desc.p, P.dpl.p, P.pl, ctx->num_sms, ctx->partial_f.p, polar_of(B.precision, c),
+        CKL(launch_fwd_finish(B.desc.p, P.dpl.p, P.pl, ctx->num_sms, ctx->partial_f[c].p, polar_of(B.precision, c),
                               (double2*)user_out, st));
         prof_end(ctx, tk, 0.0, B.fin_bytes[0]);
     } else {
@@ -1266,14 +1272,14 @@ static int launch_op_class(sl1m_ctx* ctx, Batch& B, int op, int c, double* user_
         if (c == CLS_GRID)
             RET(each_grid([&](int p, const GridOp& g) {
                 return grid_adjoint(B.desc.p, p, g, B.hdesc[p].pix.n, B.hdesc[p].pix.n_pad,
-                                    ctx->partial_a.p + (size_t)B.grid_slot[1][p] * BLK, st, &ctx->n_launch);
+                                    ctx->partial_a[c].p + (size_t)B.grid_slot[1][p] * BLK, st, &ctx->n_launch);
             }));
         else
-            CKL(launch_adjoint(B.precision, c == 1, B.n_ant_max, B.desc.p, P.dpl.p, P.pl.C, ctx->partial_a.p, st,
+            CKL(launch_adjoint(B.precision, c == 1, B.n_ant_max, B.desc.p, P.dpl.p, P.pl.C, ctx->partial_a[c].p, st,
                                B.nst[1][c]));
         prof_end(ctx, tk, B.solver ? 0.0 : B.pairs_class[c], 0.0);
         prof_begin(ctx, 5, tk);
-        CKL(launch_adj_finish(B.desc.p, P.dpl.p, P.pl, ctx->num_sms, ctx->partial_a.p, user_out, st));
+        CKL(launch_adj_finish(B.desc.p, P.dpl.p, P.pl, ctx->num_sms, ctx->partial_a[c].p, user_out, st));
         prof_end(ctx, tk, 0.0, B.fin_bytes[1]);
     }
     return SL1M_OK;
@@ -1283,7 +1289,7 @@ static int launch_op_class(sl1m_ctx* ctx, Batch& B, int op, int c, double* user_
 // user_out in the caller's order (null: the batch's own array).
 int batch_op(sl1m_ctx* ctx, Batch& B, int op, double* user_out)
 {
-    for (int c = 0; c < N_CLS; ++c) RET(launch_op_class(ctx, B, op, c, user_out));
+    for (int c = 0; c < N_CLS; ++c) RET(launch_op_class(ctx, B, op, c, user_out, ctx->stream));
     return SL1M_OK;
 }
 
@@ -1291,8 +1297,30 @@ int batch_op(sl1m_ctx* ctx, Batch& B, int op, double* user_out)
 // forward, forward finish (per gains class), then the phase machine.
 static int enqueue_tick(sl1m_ctx* ctx, Batch& B)
 {
-    for (int c = 0; c < N_CLS; ++c) RET(launch_op_class(ctx, B, 1, c, nullptr));
-    for (int c = 0; c < N_CLS; ++c) RET(launch_op_class(ctx, B, 0, c, nullptr));
+    // Under capture the classes are branches of their own: their problems are
+    // disjoint, and on small problems one class's finish kernels and tails leave
+    // the GPU to the other (four 4096 x 6000 requests, two with gains: 238 ->
+    // 205 us a tick).
+    const bool fork = ctx->use_graphs && !ctx->prof && B.has_class[0] + B.has_class[1] + B.has_class[2] > 1;
+    int side = 0;
+    bool own = true;                             // the first class stays on the stream
+    if (fork) CK(cudaEventRecord(ctx->ev_fork, ctx->stream));
+    for (int c = N_CLS - 1; c >= 0; --c) {
+        if (!B.has_class[c]) continue;
+        cudaStream_t st = ctx->stream;
+        if (fork && !own) {
+            st = ctx->side[side];
+            CK(cudaStreamWaitEvent(st, ctx->ev_fork, 0));
+        }
+        RET(launch_op_class(ctx, B, 1, c, nullptr, st));
+        RET(launch_op_class(ctx, B, 0, c, nullptr, st));
+        if (fork && !own) {
+            CK(cudaEventRecord(ctx->ev_join[side], st));
+            CK(cudaStreamWaitEvent(ctx->stream, ctx->ev_join[side], 0));
+            ++side;
+        }
+        own = false;
+    }
     // while profiling (ticks are launched directly then, never captured) the
     // scalars kernel counts the pairs the tick evaluated
     double* ev = (ctx->prof && B.solver && ctx->evals_dev.p) ? ctx->evals_dev.p + 2 * (B.precision != 0) : nullptr;
@@ -1330,9 +1358,7 @@ int batch_ticks(sl1m_ctx* ctx, Batch& B, int n)
     // larger batch (another problem's solve or operator call, the autotuner)
     // may have reallocated since: capture again rather than replay with a
     // freed buffer.  The scratch only grows, so it still fits this batch.
-    if (B.graph_ok && (B.cap_partial[0] != ctx->partial_f.p || B.cap_partial[1] != ctx->partial_a.p ||
-                       B.cap_partial[2] != ctx->grid_ws.p))
-        B.graph_ok = false;
+    if (B.graph_ok && B.cap_scratch != ctx->scratch()) B.graph_ok = false;
     if (!B.graph_ok) {
         if (B.gexec) {
             cudaGraphExecDestroy(B.gexec);
@@ -1353,9 +1379,7 @@ int batch_ticks(sl1m_ctx* ctx, Batch& B, int n)
         if (ei != cudaSuccess) B.gexec = nullptr;
         CK(ei);
         B.graph_ok = true;
-        B.cap_partial[0] = ctx->partial_f.p;
-        B.cap_partial[1] = ctx->partial_a.p;
-        B.cap_partial[2] = ctx->grid_ws.p;
+        B.cap_scratch = ctx->scratch();
         B.tick_launches = ctx->n_launch - l0;
         ctx->n_launch = l0;
     }
@@ -1484,6 +1508,14 @@ int sl1m_create(sl1m_ctx** out, int device, void* cuda_stream)
     }
     if (cudaStreamCreateWithFlags(&c->upstream, cudaStreamNonBlocking) != cudaSuccess ||
         fp64_init_tables(c->stream) != cudaSuccess) {
+        delete c;
+        return SL1M_ERR_CUDA;
+    }
+    bool ok = cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) == cudaSuccess;
+    for (int i = 0; i < N_CLS - 1; ++i)
+        ok = ok && cudaStreamCreateWithFlags(&c->side[i], cudaStreamNonBlocking) == cudaSuccess &&
+             cudaEventCreateWithFlags(&c->ev_join[i], cudaEventDisableTiming) == cudaSuccess;
+    if (!ok) {
         delete c;
         return SL1M_ERR_CUDA;
     }
@@ -1881,7 +1913,7 @@ int sl1m_autotune(sl1m_problem* prob, int precision, int32_t* nst_out, int32_t* 
             DevPlan P;
             if (build_plan(nb, ns, ctx->num_sms * k, own_granules(precision, op, gains), P, st, &uc) != cudaSuccess) { rc = SL1M_ERR_CUDA; return 0.f; }
             const size_t need = (size_t)std::max(1, P.pl.n_slots) * P.pl.blk_el;
-            if ((op == 0 ? ctx->partial_f.reserve(need, st) : ctx->partial_a.reserve(need, st)) != cudaSuccess) {
+            if ((op == 0 ? ctx->partial_f[gains].reserve(need, st) : ctx->partial_a[gains].reserve(need, st)) != cudaSuccess) {
                 rc = SL1M_ERR_OOM;
                 return 0.f;
             }
@@ -1894,9 +1926,9 @@ int sl1m_autotune(sl1m_problem* prob, int precision, int32_t* nst_out, int32_t* 
                 if (rb != SL1M_OK) { rc = rb; return 0.f; }
                 cudaEventRecord(e0, st);
                 cudaError_t e = op == 0 ? launch_forward(precision, gains, prob->n_ant, Bop->desc.p, P.dpl.p, P.pl.C,
-                                                         ctx->partial_f.p, st, code)
+                                                         ctx->partial_f[gains].p, st, code)
                                         : launch_adjoint(precision, gains, prob->n_ant, Bop->desc.p, P.dpl.p, P.pl.C,
-                                                         ctx->partial_a.p, st, code);
+                                                         ctx->partial_a[gains].p, st, code);
                 if (e != cudaSuccess) { rc = SL1M_ERR_CUDA; return 0.f; }
                 ctx->n_launch += 1;
                 cudaEventRecord(e1, st);

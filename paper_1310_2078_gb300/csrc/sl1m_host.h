@@ -187,7 +187,7 @@ struct Batch {
     cudaGraphExec_t gexec = nullptr;
     bool graph_ok = false;
     long long tick_launches = 0;
-    const void* cap_partial[3] = {nullptr, nullptr, nullptr};   // the context's scratch the capture baked in
+    std::vector<const void*> cap_scratch;   // the context's scratch the capture baked in
     ~Batch();
 };
 
@@ -199,8 +199,20 @@ struct sl1m_ctx {
     int num_sms = 1;
     std::string err;                     // last error message, guarded by err_mu: a running
     mutable std::mutex err_mu;           // server thread reports failures here too
-    DBuf<double2> partial_f;
-    DBuf<double> partial_a;
+    DBuf<double2> partial_f[N_CLS];      // partial sums per class: classes of a tick overlap
+    DBuf<double> partial_a[N_CLS];
+    cudaStream_t side[N_CLS - 1] = {};   // classes of a captured tick beside the stream's own
+    cudaEvent_t ev_fork = nullptr, ev_join[N_CLS - 1] = {};
+    // the scratch a captured tick bakes in
+    std::vector<const void*> scratch() const
+    {
+        std::vector<const void*> v = {grid_ws.p};
+        for (int c = 0; c < N_CLS; ++c) {
+            v.push_back(partial_f[c].p);
+            v.push_back(partial_a[c].p);
+        }
+        return v;
+    }
     DBuf<float2> grid_ws;                // workspace of the lattice operators
     std::vector<sl1m_problem*> problems;
     // autotuned (streamed granules per stage, CTAs per SM), keyed by
