@@ -148,6 +148,8 @@ struct DevProblem {
     const float* gsig;        // [pix.n_gran] sigma per pixel granule (FP32 path)
     const double* gsig64;     // [pix.n_gran] sigma per pixel granule (FP64 path)
     const int* gkind;         // [pix.n_gran] kind per pixel granule
+    const int* gclass;        // gains: [pix.n_gran] the granule's scale in gcls, -1 if none, or null
+    const float4* gcls;       // gains: [scales][vis.n_pad] constants of (visibility, Gaussian scale), or null
     const float4* pghdr;      // [pix.n_gran][4] centre hi, centre lo, extent, {sigma, kind, 0, 0}
     const float4* vgabs;      // [vis.n_pad] {u, v, -2 w, u^2 + v^2} in FP32 (the adjoint's Gaussian terms)
     float2* r32;              // [vis.n_pad] the mixed adjoint's input residual in polar form,

@@ -585,7 +585,9 @@ sl1m_ctx::~sl1m_ctx()
 struct ProblemDev {
     DevSide vis, pix;
     DBuf<int2> ant;
-    DBuf<float4> vgabs;
+    DBuf<float4> vgabs, gcls;
+    DBuf<int> gclass;
+    DBuf<double> gcls_sigma;
     DBuf<float2> r32;
     DBuf<double2> r64;               // made by the first FP64 call
     DBuf<int> vslot, gnb;
@@ -714,6 +716,7 @@ int sl1m_problem::rebuild(cudaStream_t st, size_t grid_budget)
         }
         CK(D.pghdr.upload(hdr.data(), hdr.size(), st));
         gkind_pix = gk;
+        gsig_pix = gs64;
         pix_orig = H.orig;
         if (n_ant > 0) {
             // FP32 in polar form {|G|, arg G in turns} (modulus and argument
@@ -822,6 +825,27 @@ int sl1m_problem::rebuild(cudaStream_t st, size_t grid_budget)
             D.gnb.free();
         }
     }
+    // the gains adjoint's constants per (visibility, Gaussian scale), for few scales
+    D.gcls.free();
+    D.gclass.free();
+    if (n_ant > 0 && has_gauss) {
+        std::vector<double> scales;
+        std::vector<int> cl(hp.pix.n_gran, -1);
+        for (int g = 0; g < hp.pix.n_gran && scales.size() <= GCLS_MAX; ++g) {
+            if (gkind_pix[g] == DIRAC) continue;
+            const auto at = std::find(scales.begin(), scales.end(), gsig_pix[g]);
+            cl[g] = (int)(at - scales.begin());
+            if (at == scales.end()) scales.push_back(gsig_pix[g]);
+        }
+        if (scales.size() <= GCLS_MAX) {
+            CK(D.gcls.alloc(scales.size() * (size_t)hp.vis.n_pad));
+            CK(D.gclass.upload(cl.data(), cl.size(), st));
+            CK(D.gcls_sigma.upload(scales.data(), scales.size(), st));
+            CK(launch_gauss_class(hp.vis.d, hp.vis.n_pad, D.gcls_sigma.p, (int)scales.size(), D.gcls.p, st));
+        }
+    }
+    hp.gcls = D.gcls.p;
+    hp.gclass = D.gclass.p;
     hp.ant = D.ant.p;
     hp.vgabs = D.vgabs.p;
     hp.r32 = D.r32.p;
@@ -1055,7 +1079,7 @@ size_t sl1m_problem::dev_bytes() const
     };
     side(D.vis);
     side(D.pix);
-    b += D.ant.bytes() + D.vgabs.bytes() + D.r32.bytes() + D.r64.bytes() + D.vslot.bytes() + D.gbl.bytes() + D.gnb.bytes() + D.V.bytes() + D.pgauss.bytes() + D.pgauss64.bytes() + D.gsig.bytes() +
+    b += D.ant.bytes() + D.vgabs.bytes() + D.gcls.bytes() + D.gclass.bytes() + D.r32.bytes() + D.r64.bytes() + D.vslot.bytes() + D.gbl.bytes() + D.gnb.bytes() + D.V.bytes() + D.pgauss.bytes() + D.pgauss64.bytes() + D.gsig.bytes() +
          D.gsig64.bytes() + D.gkind.bytes() + D.pghdr.bytes() + D.gpol32.bytes() + D.gains64.bytes();
     b += D.x_user.bytes() + D.x_sorted.bytes() + D.adj_sorted.bytes() + D.img_user.bytes() +
          D.r_user.bytes() + D.r_sorted.bytes() + D.fwd_sorted.bytes() + D.vis_user.bytes();

@@ -262,6 +262,7 @@ struct sl1m_problem {
     int algo = 0;                              // solver of the last init_solve (0 FISTA, 1 MFISTA)
     std::vector<float4> gext_vis, gext_pix;   // granule extents (host copies)
     std::vector<int> gkind_pix;               // pixel granule kinds
+    std::vector<double> gsig_pix;             // and scales
     UnitCost ucost[2][2];                      // [precision][0 forward / 1 adjoint]
     bool ucost_ok[2][2] = {{false, false}, {false, false}};
     std::unique_ptr<Batch> op_batch[2], solve_batch[2];

@@ -839,10 +839,18 @@ adj_mixed_kernel(const DevProblem* __restrict__ probs, const Plan* __restrict__ 
 // Phi = C + psi_b - psi_a, theta = 2 pi (B + D) (+ the Gaussian terms): rho_k
 // sits in the record's B term, Phi is formed once per run from the gains in
 // polar form, and M multiplies the run's sum z at the run's end.
-// Per record k: off = {du, dv, dw, B + rho (radians)}, kr = {pair key a << 16
-// | b, |r| (Dirac owners) or k0 + log2 |r'| (Gaussian owners), k1, 0};
-// Gaussian owners also read va = {u, v, -2 w, gam in radians}, the amplitude
-// times |r'| being 2^(k1 t + k0') with t = u l + v m - w r^2/2.
+// Per record k, Dirac owners: off = {du, dv, dw, B + rho (radians)}, kr = {pair
+// key a << 16 | b, |r|}.  Gaussian owners: the phase and the exponent of the
+// amplitude are linear in the owned pixel's offsets y = (dl, dm, dn, q), q = r^2/2
+// - qc from its granule's centre (with t = u l + v m - w r^2/2 = tc + u dl + v dm
+// - w q), so the record holds their coefficients, off = {p1, p2, p3, p4} (radians)
+// and va = {e1, e2, e4, k0''}, kr = {key, B''}, everything at the centre (gam tc,
+// k1 tc, the constant phase, log2 |r'|) folded into B'' and k0'': 7 FFMA a pair
+// instead of 3 + 3 + 1 + 1 for the offset phase, t, gam t and k1 t.
+//
+// AL4: every run of the granule starts at a multiple of 4 (orders by runs of a
+// pair's samples make that the usual case), so the pair is looked up once per 4
+// visibilities instead of at each.
 
 // The run held in z, of magnitude M, into acc: acc += M z.
 __device__ __forceinline__ void adjg_flush(const float (&M)[2], float (&z)[2], float (&acc)[2])
@@ -875,22 +883,22 @@ __device__ __forceinline__ void adjg_next_run(int key, int& cur, const GF& gain,
     }
 }
 
-template <bool EXACT, class GF>
+template <bool EXACT, bool AL4, class GF>
 __device__ __forceinline__ void adjg_dirac_tile(const float4* __restrict__ s_off, const float4* __restrict__ g_lo,
-                                                const float4* __restrict__ s_kr, const GF& gain,
+                                                const float2* __restrict__ s_kr, const GF& gain,
                                                 const float (&Ct)[2], const float4 (&dx)[2],
                                                 const float4 (&dxl)[2], float (&acc)[2])
 {
     int cur = -1;
     float M[2] = {0.f, 0.f}, Phi[2] = {0.f, 0.f}, z[2] = {0.f, 0.f};
-#pragma unroll 1
+#pragma unroll(AL4 ? 2 : 1)
     for (int k0 = 0; k0 < G; k0 += 4)
 #pragma unroll
     for (int kk = 0; kk < 4; ++kk) {
         const int k = k0 + kk;
         const float4 o = s_off[k];
-        const float2 kr = *reinterpret_cast<const float2*>(s_kr + k);   // {key, |r|}
-        adjg_next_run<EXACT>(__float_as_int(kr.x), cur, gain, Ct, M, Phi, z, acc);
+        const float2 kr = s_kr[k];             // {key, |r|}
+        if (!AL4 || kk == 0) adjg_next_run<EXACT>(__float_as_int(kr.x), cur, gain, Ct, M, Phi, z, acc);
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
             float ph;                              // radians
@@ -902,44 +910,69 @@ __device__ __forceinline__ void adjg_dirac_tile(const float4* __restrict__ s_off
     adjg_flush(M, z, acc);                      // the last run
 }
 
-template <bool EXACT, bool PAR, class GF>
-__device__ __forceinline__ void adjg_gauss_tile(const float4* __restrict__ s_off, const float4* __restrict__ g_lo,
-                                                const float4* __restrict__ s_va, const float4* __restrict__ s_kr,
-                                                const GF& gain, const float (&Ct)[2],
-                                                const float4 (&dx)[2], const float4 (&dxl)[2],
-                                                const float4 (&pgd)[2], float (&acc)[2])
+// g_off, g_lo, dx, dxl (EXACT): the offsets of either side and their residuals
+// in turns, the coefficients then leave the product of the offsets out.
+template <bool EXACT, bool AL4, class GF>
+__device__ __forceinline__ void adjg_gauss_tile(const float4* __restrict__ s_p, const float4* __restrict__ s_e,
+                                                const float2* __restrict__ s_kr, const float4* __restrict__ g_off,
+                                                const float4* __restrict__ g_lo, const GF& gain,
+                                                const float (&Ct)[2], const float4 (&y)[2],
+                                                const float4 (&dx)[2], const float4 (&dxl)[2], float (&acc)[2])
 {
     int cur = -1;
     float M[2] = {0.f, 0.f}, Phi[2] = {0.f, 0.f}, z[2] = {0.f, 0.f};
 #pragma unroll 1
-    for (int k0 = 0; k0 < G; k0 += 2)
+    for (int k0 = 0; k0 < G; k0 += 4)
 #pragma unroll
-    for (int kk = 0; kk < 2; ++kk) {
+    for (int kk = 0; kk < 4; ++kk) {
         const int k = k0 + kk;
-        const float4 o = s_off[k];
-        const float4 va = s_va[k];                 // {u, v, -2 w, gam (radians)}
-        const float4 kr = s_kr[k];                 // {key, k0', k1, 0}
-        adjg_next_run<EXACT>(__float_as_int(kr.x), cur, gain, Ct, M, Phi, z, acc);
+        const float4 p = s_p[k], e = s_e[k];
+        const float2 kr = s_kr[k];                 // {key, B'' (radians)}
+        if (!AL4 || kk == 0) adjg_next_run<EXACT>(__float_as_int(kr.x), cur, gain, Ct, M, Phi, z, acc);
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
-            // pgd = {l, m, r^2/4, pi nu}: t = u l + v m - w r^2/2
-            const float t = fmaf(va.x, pgd[r].x, fmaf(va.y, pgd[r].y, va.z * pgd[r].z));
-            float ph;                              // radians
-            if (EXACT) {
-                ph = (o.w * INV_TWO_PI_F + Phi[r]) + frac_dot3(dx[r], dxl[r], o, g_lo[k]);
-                ph = fmaf(-va.w * INV_TWO_PI_F, t, ph);
-                if (PAR) ph = fmaf(va.z, pgd[r].w * INV_TWO_PI_F, ph);   // -w nu, turns
-                ph = frac_turns(ph) * TWO_PI_F;
-            } else {
-                ph = fmaf(dx[r].z, o.z, fmaf(dx[r].y, o.y, fmaf(dx[r].x, o.x, o.w + Phi[r])));
-                ph = fmaf(-va.w, t, ph);
-                if (PAR) ph = fmaf(va.z, pgd[r].w, ph);                  // -2 pi w nu
-            }
-            const float amp = ex2_approx(fmaf(kr.z, t, kr.y));        // |r'| e^{Re(qc)}
-            z[r] = fmaf(kk ? -amp : amp, __cosf(ph), z[r]);             // odd k: -cos(theta + pi)
+            float ph = EXACT ? 0.f : kr.y + Phi[r];    // radians
+            ph = fmaf(p.w, y[r].w, fmaf(p.z, y[r].z, fmaf(p.y, y[r].y, fmaf(p.x, y[r].x, ph))));
+            if (EXACT)
+                ph = frac_turns(fmaf(ph + kr.y, INV_TWO_PI_F, Phi[r]) + frac_dot3(dx[r], dxl[r], g_off[k], g_lo[k])) * TWO_PI_F;
+            const float amp = ex2_approx(fmaf(e.z, y[r].w, fmaf(e.y, y[r].y, fmaf(e.x, y[r].x, e.w))));   // |r'| e^{Re(qc)}
+            z[r] = fmaf((kk & 1) ? -amp : amp, __cosf(ph), z[r]);      // odd k: -cos(theta + pi)
         }
     }
     adjg_flush(M, z, acc);                      // the last run
+}
+
+// What a streamed visibility's record takes of a Gaussian scale: {gam (radians
+// per turn of t), k1, k0 + log2 sqrt(id), cphase - atan(beta) / 2 pi in turns}, the
+// last two with r' = id (1 - i beta) r, |r'| = |r| sqrt(id), arg r' = arg r -
+// atan(beta).
+__device__ __forceinline__ float4 gauss_class(const float4 uvw, float sigma)
+{
+    const GaussConst gc = gauss_const(uvw.x, uvw.y, uvw.z, sigma);
+    return make_float4(gc.gamr, gc.k1, gc.k0 - 0.5f * __log2f(fmaf(gc.beta, gc.beta, 1.0f)),
+                       frac_turns(fmaf(-atanf(gc.beta), INV_TWO_PI_F, gc.cphase)));
+}
+
+// The same for every visibility and each of the problem's scales, in FP64: made
+// once per layout when there are few scales (gcls[class][vis.n_pad]).
+__global__ void gauss_class_kernel(const d4* __restrict__ vd, int n_pad, const double* __restrict__ sigma,
+                                   float4* __restrict__ gcls)
+{
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= n_pad) return;
+    const d4 v = vd[k];
+    const double s2 = sigma[blockIdx.y] * sigma[blockIdx.y], beta = v.z * s2, id = 1.0 / (1.0 + beta * beta);
+    const double coef = -3.14159265358979324 * 1.44269504088896341 * s2 * id, uv2 = v.x * v.x + v.y * v.y;
+    double ph = 0.5 * id * beta * s2 * uv2 - atan(beta) * 0.15915494309189534;
+    ph -= rint(ph);
+    gcls[(size_t)blockIdx.y * n_pad + k] =
+        make_float4((float)(beta * beta * id * 6.28318530717958648), (float)(-2.0 * coef * v.z),
+                    (float)(coef * uv2 + 0.5 * log2(id)), (float)ph);
+}
+cudaError_t launch_gauss_class(const d4* vd, int n_pad, const double* sigma, int n_cls, float4* gcls, cudaStream_t st)
+{
+    gauss_class_kernel<<<dim3((unsigned)((n_pad + 127) / 128), (unsigned)n_cls), 128, 0, st>>>(vd, n_pad, sigma, gcls);
+    return cudaGetLastError();
 }
 
 // Adjoint with gains.  The CTA's 8 warps share one owned pixel granule at a
@@ -980,9 +1013,10 @@ adj_mixed_gains_kernel(const DevProblem* __restrict__ probs, const Plan* __restr
                        double* __restrict__ partial)
 {
     // per warp, what its tiles read for its current granule
-    __shared__ float4 s_off[BLK_GRAN][G];       // {du, dv, dw, B + arg r (radians)}
-    __shared__ float4 s_kr[BLK_GRAN][G];        // {pair key, |r| or k0 + log2 |r'|, k1, 0}
-    __shared__ float4 s_va[BLK_GRAN][G];        // Gaussian owners: {u, v, -2 w, gam (radians)}
+    // (Dirac / Gaussian owners)
+    __shared__ float4 s_off[BLK_GRAN][G];       // {du, dv, dw, B + arg r (radians)} / {p1, p2, p3, p4}
+    __shared__ float2 s_kr[BLK_GRAN][G];        // {pair key, |r|} / {pair key, B''}
+    __shared__ float4 s_va[BLK_GRAN][G];        // - / {e1, e2, e4, k0''}
     __shared__ double s_red[BLK_GRAN][G];
     __shared__ __align__(8) unsigned long long s_wbar[BLK_GRAN];   // each warp's raw slice
     __shared__ __align__(8) unsigned long long s_gbar;             // the gains table
@@ -1043,12 +1077,16 @@ adj_mixed_gains_kernel(const DevProblem* __restrict__ probs, const Plan* __restr
         const int e0 = pgi * G + lane;
         const int eidx[2] = {e0, e0 + 32};
         const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
-        float4 xh[2], dx[2], pgd[2] = {z4, z4};
+        float4 xh[2], dx[2], y[2] = {z4, z4};
+        // the granule's centre, which the Gaussian terms are taken from
+        const float qc = 0.5f * fmaf(ch.x, ch.x, ch.y * ch.y), nuc = ch.z + qc;
+        const float4* const cls = gauss && P.gcls && P.gclass[pgi] >= 0 ? P.gcls + (size_t)P.gclass[pgi] * P.vis.n_pad : nullptr;
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
             xh[r] = P.pix.hi[eidx[r]];
-            dx[r] = to_rad(P.pix.off[eidx[r]]);
-            if (gauss) pgd[r] = pix_for_gauss(P.pgauss[eidx[r]]);
+            y[r] = P.pix.off[eidx[r]];
+            dx[r] = to_rad(y[r]);
+            if (gauss) y[r].w = P.pgauss[eidx[r]].z - qc;
         }
         const SmemGain sg{s_gain, lane};
         mbar_wait(&s_gbar, gpar, fault);
@@ -1058,54 +1096,63 @@ adj_mixed_gains_kernel(const DevProblem* __restrict__ probs, const Plan* __restr
             mbar_wait(&s_wbar[warp], wpar, fault);
             wpar ^= 1u;
             // derive this granule's records for the tiles
+            const float4 yc_h = raw_cen[0], yc_l = raw_cen[1], yext = raw_cen[2];
+            const bool exact = dot3(ext, yext) > D_MAX;
+            int keys[2];
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 const int k = lane + 32 * h;
                 float4 o = raw_off[k];
                 const int2 ab = raw_ant[k];
-                const float key = __int_as_float(ab.x << 16 | ab.y);   // the pair (adjg_next_run)
-                const float b = frac_dot3(ch, cl, o, raw_lo[k]) + odd_turn(k);   // turns
+                keys[h] = ab.x << 16 | ab.y;                            // the pair (adjg_next_run)
+                float b = frac_dot3(ch, cl, o, raw_lo[k]) + odd_turn(k);   // turns
                 const float2 rp = raw_r[k];                             // {|r|, arg r in turns}
-                float4 kr;
+                float2 kr = make_float2(__int_as_float(keys[h]), rp.x);
                 if (gauss) {
-                    const float4 va = vis_for_gauss(raw_hi[k]);
-                    const float4 rec = adj_gauss_record(b, rp, va, sigma);   // {B', gamr, k1, k0'}
-                    o.w = rec.x;
-                    s_va[warp][k] = make_float4(va.x, va.y, va.z, rec.y);
-                    kr = make_float4(key, rec.w, rec.z, 0.f);
+                    const float4 x = raw_hi[k];                         // u, v, w
+                    const float4 gc = cls ? cls[g * G + k] : gauss_class(x, sigma);
+                    const float tc = fmaf(x.x, ch.x, fmaf(x.y, ch.y, -x.z * qc));
+                    b = frac_turns(b + gc.w);
+                    b = frac_turns(fmaf(-gc.x * INV_TWO_PI_F, tc, b + rp.y));
+                    if (par) b = frac_turns(fmaf(-x.z, nuc, b));
+                    const float wp = par ? -TWO_PI_F * x.z : 0.f;
+                    o = exact ? z4 : to_rad(o);
+                    s_off[warp][k] = make_float4(fmaf(-gc.x, x.x, o.x), fmaf(-gc.x, x.y, o.y), o.z + wp,
+                                                 fmaf(gc.x, x.z, wp));
+                    s_va[warp][k] = make_float4(gc.y * x.x, gc.y * x.y, -gc.y * x.z, fmaf(gc.y, tc, gc.z) + __log2f(rp.x));
+                    kr.y = b * TWO_PI_F;
                 } else {
                     o.w = frac_turns(b + rp.y) * TWO_PI_F;
-                    kr = make_float4(key, rp.x, 0.f, 0.f);
+                    s_off[warp][k] = o;
                 }
-                s_off[warp][k] = o;
                 s_kr[warp][k] = kr;
             }
-            const float4 yc_h = raw_cen[0], yc_l = raw_cen[1], yext = raw_cen[2];
+            // runs that start off a multiple of 4 (a neighbour's pair differs)
+            bool odd_run = false;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int prev = __shfl_up_sync(0xffffffffu, keys[h], 1);
+                odd_run |= (lane & 3) != 0 && prev != keys[h];
+            }
+            const bool al4 = !__any_sync(0xffffffffu, odd_run);
             __syncwarp();                                 // the slice is read: refill it
             if (lane == 0 && !fault && g + BLK_GRAN < g1) adj_raw_load(raw, P, g + BLK_GRAN, &s_wbar[warp]);
-            const bool exact = dot3(ext, yext) > D_MAX;
             float Ct[2];                          // the tile's centre term C, turns
 #pragma unroll
             for (int r = 0; r < 2; ++r) Ct[r] = frac_dot3(xh[r], P.pix.lo[eidx[r]], yc_h, yc_l);
             const float4* g_lo = P.vis.offlo + (size_t)g * G;   // exact tiles only (rare)
             float acc[2] = {0.f, 0.f};
-            if (!gauss) {
-                if (exact) {
-                    const float4 dxt[2] = {P.pix.off[eidx[0]], P.pix.off[eidx[1]]},
-                                 dxl[2] = {P.pix.offlo[eidx[0]], P.pix.offlo[eidx[1]]};
-                    adjg_dirac_tile<true>(s_off[warp], g_lo, s_kr[warp], sg, Ct, dxt, dxl, acc);
-                } else {
-                    adjg_dirac_tile<false>(s_off[warp], g_lo, s_kr[warp], sg, Ct, dx, dx, acc);
-                }
-            } else if (exact) {
+            if (exact) {
                 const float4 dxt[2] = {P.pix.off[eidx[0]], P.pix.off[eidx[1]]},
                              dxl[2] = {P.pix.offlo[eidx[0]], P.pix.offlo[eidx[1]]};
-                if (par) adjg_gauss_tile<true, true>(s_off[warp], g_lo, s_va[warp], s_kr[warp], sg, Ct, dxt, dxl, pgd, acc);
-                else adjg_gauss_tile<true, false>(s_off[warp], g_lo, s_va[warp], s_kr[warp], sg, Ct, dxt, dxl, pgd, acc);
-            } else if (par) {
-                adjg_gauss_tile<false, true>(s_off[warp], g_lo, s_va[warp], s_kr[warp], sg, Ct, dx, dx, pgd, acc);
+                if (gauss) adjg_gauss_tile<true, false>(s_off[warp], s_va[warp], s_kr[warp], P.vis.off + (size_t)g * G, g_lo, sg, Ct, y, dxt, dxl, acc);
+                else adjg_dirac_tile<true, false>(s_off[warp], g_lo, s_kr[warp], sg, Ct, dxt, dxl, acc);
+            } else if (gauss) {
+                if (al4) adjg_gauss_tile<false, true>(s_off[warp], s_va[warp], s_kr[warp], g_lo, g_lo, sg, Ct, y, dx, dx, acc);
+                else adjg_gauss_tile<false, false>(s_off[warp], s_va[warp], s_kr[warp], g_lo, g_lo, sg, Ct, y, dx, dx, acc);
             } else {
-                adjg_gauss_tile<false, false>(s_off[warp], g_lo, s_va[warp], s_kr[warp], sg, Ct, dx, dx, pgd, acc);
+                if (al4) adjg_dirac_tile<false, true>(s_off[warp], g_lo, s_kr[warp], sg, Ct, dx, dx, acc);
+                else adjg_dirac_tile<false, false>(s_off[warp], g_lo, s_kr[warp], sg, Ct, dx, dx, acc);
             }
 #pragma unroll
             for (int r = 0; r < 2; ++r) tot[r] += (double)acc[r];
