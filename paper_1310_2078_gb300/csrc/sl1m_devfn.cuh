@@ -208,6 +208,20 @@ __device__ __forceinline__ int slot_of(const Plan& pl, int gblk)
     return pl.blk_poff[gblk] + ((int)blockIdx.x - pl.blk_clo[gblk]);
 }
 
+// A 16-byte load that stays where it is written (the compiler may neither hoist
+// it nor keep its result for the next one): for values that cost fewer
+// registers reloaded than held.
+__device__ __forceinline__ float4 reload4(const float4* p)
+{
+    float4 v;
+    asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+    return v;
+}
+
+// r^2/2 at a granule's centre (l, m), as the offsets q (DevProblem::pgoff) are
+// taken from it; the host computes the same.
+__device__ __forceinline__ float centre_q(float l, float m) { return 0.5f * fmaf(l, l, m * m); }
+
 // Constants of one (visibility, Gaussian scale) pair, Eq. samlm4 in split form.
 struct GaussConst {
     float beta, id, gamr, coef;  // beta = w s^2, id = 1/(1+beta^2), gamr = 2 pi beta^2 id

@@ -593,7 +593,7 @@ struct ProblemDev {
     DBuf<int> vslot, gnb;
     DBuf<int2> gbl;
     DBuf<double2> V;
-    DBuf<float4> pgauss;
+    DBuf<float4> pgauss, pgoff;
     DBuf<d4> pgauss64;
     DBuf<float> gsig;
     DBuf<double> gsig64;
@@ -650,6 +650,7 @@ int sl1m_problem::rebuild(cudaStream_t st, size_t grid_budget)
     }
     if (!dev) dev = std::make_unique<ProblemDev>();
     ProblemDev& D = *dev;
+    std::vector<float4> hdr;                   // pixel granule headers
     // ---- pixels: classes of equal (kind, sigma), each in k-d order on (l, m)
     {
         std::vector<std::pair<std::pair<int, double>, int>> cls(n_pix);
@@ -707,14 +708,22 @@ int sl1m_problem::rebuild(cudaStream_t st, size_t grid_budget)
         CK(D.gsig64.upload(gs64.data(), gs64.size(), st));
         CK(D.gkind.upload(gk.data(), gk.size(), st));
         // per pixel granule, as the forward's bulk copies take it
-        std::vector<float4> hdr((size_t)H.n_gran * 4);
+        hdr.resize((size_t)H.n_gran * 4);
+        std::vector<float4> pgo(has_gauss ? H.n_pad : 0);
         for (int g = 0; g < H.n_gran; ++g) {
             hdr[4 * (size_t)g] = H.cen_hi[g];
             hdr[4 * (size_t)g + 1] = H.cen_lo[g];
             hdr[4 * (size_t)g + 2] = H.ext[g];
-            hdr[4 * (size_t)g + 3] = make_float4(gs[g], (float)gk[g], 0.f, 0.f);
+            const double cl = (double)H.cen_hi[g].x + H.cen_lo[g].x, cm = (double)H.cen_hi[g].y + H.cen_lo[g].y,
+                         cn = (double)H.cen_hi[g].z + H.cen_lo[g].z;
+            const float qc = 0.5f * std::fmaf(H.cen_hi[g].x, H.cen_hi[g].x, H.cen_hi[g].y * H.cen_hi[g].y);
+            hdr[4 * (size_t)g + 3] = make_float4(gs[g], (float)gk[g], (float)(cn + 0.5 * (cl * cl + cm * cm)), -1.f);
+            if (has_gauss)
+                for (int t = g * G; t < (g + 1) * G; ++t)
+                    pgo[t] = make_float4(H.off[t].x, H.off[t].y, H.off[t].z, (float)(pg64[t].z - (double)qc));
         }
-        CK(D.pghdr.upload(hdr.data(), hdr.size(), st));
+        D.pgoff.free();
+        if (has_gauss) CK(D.pgoff.upload(pgo.data(), pgo.size(), st));
         gkind_pix = gk;
         gsig_pix = gs64;
         pix_orig = H.orig;
@@ -800,6 +809,7 @@ int sl1m_problem::rebuild(cudaStream_t st, size_t grid_budget)
         vis_orig = H.orig;
         if (n_ant > 0) {
             // each granule's distinct antenna pairs (adjacent after sort_baselines)
+            gpairs_vis.assign(H.n_gran, 0);
             std::vector<int> vslot(H.n_pad, 0), gnb(H.n_gran, 0);
             std::vector<int2> gbl((size_t)H.n_gran * NB_MAX, make_int2(0, 0));
             for (int g = 0; g < H.n_gran; ++g) {
@@ -815,6 +825,8 @@ int sl1m_problem::rebuild(cudaStream_t st, size_t grid_budget)
                     vslot[i] = nb - 1;
                 }
                 gnb[g] = over ? 0 : nb;
+                for (int i = g * G; i < (g + 1) * G; ++i)
+                    gpairs_vis[g] += i == g * G || a[i].x != a[i - 1].x || a[i].y != a[i - 1].y;
             }
             CK(D.vslot.upload(vslot.data(), vslot.size(), st));
             CK(D.gbl.upload(gbl.data(), gbl.size(), st));
@@ -825,10 +837,11 @@ int sl1m_problem::rebuild(cudaStream_t st, size_t grid_budget)
             D.gnb.free();
         }
     }
-    // the gains adjoint's constants per (visibility, Gaussian scale), for few scales
+    // constants per (visibility, Gaussian scale), for few scales; the pixel
+    // granules' headers name the scale too
     D.gcls.free();
     D.gclass.free();
-    if (n_ant > 0 && has_gauss) {
+    if (has_gauss) {
         std::vector<double> scales;
         std::vector<int> cl(hp.pix.n_gran, -1);
         for (int g = 0; g < hp.pix.n_gran && scales.size() <= GCLS_MAX; ++g) {
@@ -842,8 +855,10 @@ int sl1m_problem::rebuild(cudaStream_t st, size_t grid_budget)
             CK(D.gclass.upload(cl.data(), cl.size(), st));
             CK(D.gcls_sigma.upload(scales.data(), scales.size(), st));
             CK(launch_gauss_class(hp.vis.d, hp.vis.n_pad, D.gcls_sigma.p, (int)scales.size(), D.gcls.p, st));
+            for (int g = 0; g < hp.pix.n_gran; ++g) hdr[4 * (size_t)g + 3].w = (float)cl[g];
         }
     }
+    CK(D.pghdr.upload(hdr.data(), hdr.size(), st));
     hp.gcls = D.gcls.p;
     hp.gclass = D.gclass.p;
     hp.ant = D.ant.p;
@@ -856,6 +871,7 @@ int sl1m_problem::rebuild(cudaStream_t st, size_t grid_budget)
     hp.gnb = n_ant > 0 ? D.gnb.p : nullptr;
     hp.V = D.V.p;
     hp.pgauss = D.pgauss.p;
+    hp.pgoff = has_gauss ? D.pgoff.p : D.pgauss.p;
     hp.pgauss64 = D.pgauss64.p;
     hp.gsig = D.gsig.p;
     hp.gsig64 = D.gsig64.p;
@@ -885,7 +901,7 @@ int sl1m_problem::rebuild(cudaStream_t st, size_t grid_budget)
 double sl1m_problem::pairs() const { return (double)n_vis * (double)n_pix; }
 
 // Relative cost of the units (owned block x streamed granule) of one operator:
-// a Gaussian pixel granule costs 1.34 to 1.60 times a Dirac one (measured, see
+// a Gaussian pixel granule costs 1.42 to 1.80 times a Dirac one (measured, see
 // below), a tile taking the exact phase path 3x, and gains 2x (gains problems
 // run in launches of their own, so that factor only orders work across the
 // two classes).  A block's 8 warps meet at each shared-memory stage, so a unit
@@ -898,12 +914,12 @@ const UnitCost& sl1m_problem::unit_cost(int precision, int op)
     uc.unit.clear();
     // cost of a Gaussian pair relative to a Dirac pair of the same launch,
     // measured on GB300 (4 x 128x128 pixels of one kind x 32,000 visibilities):
-    // forward 1.53, adjoint 1.60 without gains; 1.34 and 1.45 with gains
+    // forward 1.45, adjoint 1.80 without gains; 1.42 and 1.50 with gains
     const double gfac = n_ant > 0 ? 2.0 : 1.0;
     // (FP64: by the instructions of a pair)
     const double gcost = precision == 0 ? (op == 0 ? 2.1 : 2.3)
-                         : n_ant > 0    ? (op == 0 ? 1.34 : 1.45)
-                                        : (op == 0 ? 1.53 : 1.60);
+                         : n_ant > 0    ? (op == 0 ? 1.42 : 1.50)
+                                        : (op == 0 ? 1.45 : 1.80);
     const auto base = [gcost](int kind) { return kind == DIRAC ? 1.0 : gcost; };
     int k0 = gkind_pix.empty() ? 0 : gkind_pix[0];
     bool one_kind = true;
@@ -914,15 +930,25 @@ const UnitCost& sl1m_problem::unit_cost(int precision, int op)
     for (const float4& e : own) { mo.x = std::max(mo.x, e.x); mo.y = std::max(mo.y, e.y); mo.z = std::max(mo.z, e.z); }
     for (const float4& e : str) { ms.x = std::max(ms.x, e.x); ms.y = std::max(ms.y, e.y); ms.z = std::max(ms.z, e.z); }
     const bool any_exact = precision == 1 && (mo.x * ms.x + mo.y * ms.y + mo.z * ms.z) > D_MAX;
+    // gains: a tile's own cost of the antenna pairs of its visibility granule, in
+    // units of its pairs' (instructions of a tile of 64 x 64: forward 2,414 + 70 per
+    // pair table row, or 640 more with gathers; adjoint 2,180 + 30 per run)
+    const bool by_pairs = n_ant > 0 && precision == 1 && !gpairs_vis.empty();
+    const auto pair_cost = [&](int g) {
+        const int nb = gpairs_vis[g];
+        return op == 0 ? (nb <= NB_MAX ? 70.0 * nb : 640.0 * 2) / 2414.0 : 30.0 * nb / 2180.0;
+    };
     uc.uniform = base(k0) * gfac;
-    if (one_kind && !any_exact) return uc;
+    if (one_kind && !any_exact && !by_pairs) return uc;
     const int ng_own = (int)own.size(), ng_str = (int)str.size();
     const int bg = own_granules(precision, op, n_ant > 0), nblk = own_blocks(precision, op, n_ant > 0, ng_own);
     uc.sub = stream_units(precision, 1);               // units per streamed granule
     uc.unit.resize((size_t)nblk * ng_str);
     for (int b = 0; b < nblk; ++b) {
         const int w1 = std::min(ng_own, (b + 1) * bg);
-        double kb = 1.0;
+        double kb = 1.0, own_pairs = 0.0;
+        if (op == 0 && by_pairs)
+            for (int w = b * bg; w < w1; ++w) own_pairs = std::max(own_pairs, pair_cost(w));
         if (op == 1)
             for (int w = b * bg; w < w1; ++w) kb = std::max(kb, base(gkind_pix[w]));
         for (int g = 0; g < ng_str; ++g) {
@@ -933,7 +959,8 @@ const UnitCost& sl1m_problem::unit_cost(int precision, int op)
                     ex = own[w].x * s4.x + own[w].y * s4.y + own[w].z * s4.z > D_MAX;
             }
             const double kbase = op == 0 ? base(gkind_pix[g]) : kb;
-            uc.unit[(size_t)b * ng_str + g] = (float)(kbase * (ex ? 3.0 : 1.0) * gfac);
+            uc.unit[(size_t)b * ng_str + g] =
+                (float)((kbase * (ex ? 3.0 : 1.0) + (op == 0 ? own_pairs : by_pairs ? pair_cost(g) : 0.0)) * gfac);
         }
     }
     return uc;
@@ -1079,7 +1106,7 @@ size_t sl1m_problem::dev_bytes() const
     };
     side(D.vis);
     side(D.pix);
-    b += D.ant.bytes() + D.vgabs.bytes() + D.gcls.bytes() + D.gclass.bytes() + D.r32.bytes() + D.r64.bytes() + D.vslot.bytes() + D.gbl.bytes() + D.gnb.bytes() + D.V.bytes() + D.pgauss.bytes() + D.pgauss64.bytes() + D.gsig.bytes() +
+    b += D.ant.bytes() + D.vgabs.bytes() + D.gcls.bytes() + D.gclass.bytes() + D.r32.bytes() + D.r64.bytes() + D.vslot.bytes() + D.gbl.bytes() + D.gnb.bytes() + D.V.bytes() + D.pgauss.bytes() + D.pgoff.bytes() + D.pgauss64.bytes() + D.gsig.bytes() +
          D.gsig64.bytes() + D.gkind.bytes() + D.pghdr.bytes() + D.gpol32.bytes() + D.gains64.bytes();
     b += D.x_user.bytes() + D.x_sorted.bytes() + D.adj_sorted.bytes() + D.img_user.bytes() +
          D.r_user.bytes() + D.r_sorted.bytes() + D.fwd_sorted.bytes() + D.vis_user.bytes();

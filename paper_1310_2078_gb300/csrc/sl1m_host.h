@@ -263,6 +263,7 @@ struct sl1m_problem {
     std::vector<float4> gext_vis, gext_pix;   // granule extents (host copies)
     std::vector<int> gkind_pix;               // pixel granule kinds
     std::vector<double> gsig_pix;             // and scales
+    std::vector<int> gpairs_vis;              // gains: runs of equal antenna pairs per visibility granule
     UnitCost ucost[2][2];                      // [precision][0 forward / 1 adjoint]
     bool ucost_ok[2][2] = {{false, false}, {false, false}};
     std::unique_ptr<Batch> op_batch[2], solve_batch[2];

@@ -51,7 +51,7 @@ constexpr int stream_units(int precision, int n_gran) { return precision == 0 ? 
 // The adjoints without FP64 gains read r in polar form too, {|r|, arg r in turns}
 // in FP32 (r32) or {arg r in 1/R64_TURN turns, |r|} in FP64 (r64).  Whatever writes r
 // writes it: `polar` below is 0 (the lattice operator, FP64 gains), 1 r32 or 2 r64.
-// The gains adjoint's per-visibility constants of up to GCLS_MAX Gaussian scales.
+// Per-visibility constants of up to GCLS_MAX Gaussian scales.
 constexpr int GCLS_MAX = 4;
 cudaError_t launch_gauss_class(const d4* vd, int n_pad, const double* sigma, int n_cls, float4* gcls, cudaStream_t st);
 // The mixed gains kernels' bounded waits for their bulk copies set a device

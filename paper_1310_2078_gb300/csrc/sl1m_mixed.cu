@@ -107,50 +107,100 @@ __device__ __forceinline__ void fwd_dirac_tile(const float4* __restrict__ s_off,
     }
 }
 
-template <bool GAINS, bool EXACT, bool PAR>
+// Constants of a visibility and a Gaussian scale as the tables hold them: {gam
+// (radians per turn of t), k1, k0 + log2 sqrt(id), cphase - atan(beta) / 2 pi in
+// turns}.  The entry's factor id (1 + i beta) is sqrt(id) e^{i atan(beta)}, so the
+// last two take it in.
+__device__ __forceinline__ float4 gauss_class(const float4 uvw, float sigma)
+{
+    const GaussConst gc = gauss_const(uvw.x, uvw.y, uvw.z, sigma);
+    return make_float4(gc.gamr, gc.k1, gc.k0 - 0.5f * __log2f(fmaf(gc.beta, gc.beta, 1.0f)),
+                       frac_turns(fmaf(-atanf(gc.beta), INV_TWO_PI_F, gc.cphase)));
+}
+
+// Gaussian tiles.  Phase and amplitude exponent of a pair are linear in the
+// streamed pixel's offsets y = (dl, dm, dn, q), q = r^2/2 - qc, from its granule's
+// centre (t = u l + v m - w r^2/2 = tc + u dl + v dm - w q), so a lane holds their
+// coefficients for the tile,
+//   phase  p = {2 pi du - gam u, 2 pi dv - gam v, 2 pi dw, gam w} (radians;
+//          paraxial: - 2 pi w on the last two)
+//   exponent e = {k1 u, k1 v, - k1 w, k0 + k1 tc}
+// and what belongs to the centre (gam tc, the constant phase, paraxial w nu_c) is
+// in its C term: 7 FFMA a pair and one 16-byte load, where t, its products and
+// the offset phase took 3 + 3 + 2 and two loads.  EXACT: p without the product
+// of the offsets, which is reduced exactly.
+struct GaussTile {
+    float4 p, e;
+    float beta, id;
+};
+// x = {u, v, w}, dx: its offset (radians; zero when EXACT); yc: the streamed
+// granule's centre, nuc = nu at it.  C (turns) gains the centre's share.  cls:
+// the visibility's constants of the scale (gauss_class, which has the factor id
+// (1 + i beta) in it), or null: formed here, and the factor left to the caller.
+__device__ __forceinline__ GaussTile gauss_tile(const float4 x, const float4 dx, const float4 yc, float nuc, float sigma,
+                                                bool par, const float4* cls, float& C)
+{
+    GaussTile g;
+    float4 k;                                        // gam (radians), k1, k0, constant phase (turns)
+    if (cls) {
+        k = *cls;
+        g.beta = 0.f;
+        g.id = 1.f;
+    } else {
+        const GaussConst gc = gauss_const(x.x, x.y, x.z, sigma);
+        k = make_float4(gc.gamr, gc.k1, gc.k0, gc.cphase);
+        g.beta = gc.beta;
+        g.id = gc.id;
+    }
+    const float qc = centre_q(yc.x, yc.y);
+    const float tc = fmaf(x.x, yc.x, fmaf(x.y, yc.y, -x.z * qc));
+    C = frac_turns(C + k.w);
+    C = frac_turns(fmaf(-k.x * INV_TWO_PI_F, tc, C));
+    if (par) C = frac_turns(fmaf(-x.z, nuc, C));
+    const float wp = par ? -TWO_PI_F * x.z : 0.f;
+    g.p = make_float4(fmaf(-k.x, x.x, dx.x), fmaf(-k.x, x.y, dx.y), dx.z + wp, fmaf(k.x, x.z, wp));
+    g.e = make_float4(k.y * x.x, k.y * x.y, -k.y * x.z, fmaf(k.y, tc, k.z));
+    return g;
+}
+__device__ __forceinline__ float lin4(const float4 a, const float4 y, float s)
+{
+    return fmaf(a.w, y.w, fmaf(a.z, y.z, fmaf(a.y, y.y, fmaf(a.x, y.x, s))));
+}
+__device__ __forceinline__ float lin3(const float4 e, const float4 y, float s)      // {dl, dm, -, q}
+{
+    return fmaf(e.z, y.w, fmaf(e.y, y.y, fmaf(e.x, y.x, s)));
+}
+
+template <bool GAINS, bool EXACT>
 __device__ __forceinline__ void fwd_gauss_tile(const float4* __restrict__ s_off,
                                                const float4* __restrict__ s_lo,
                                                const float4* __restrict__ s_pg,
                                                const float2* __restrict__ sBa,
                                                const float2* __restrict__ s_gain,
-                                               const float4 (&xh)[2], const float4 (&dx)[2],
-                                               const float4 (&dxl)[2], const GaussConst (&gc)[2],
+                                               const GaussTile (&gt)[2], const float4 (&dx)[2],
+                                               const float4 (&dxl)[2],
                                                const int2 (&ant)[2], float (&sr)[2], float (&si)[2])
 {
     const float2* ga_row[2] = {s_gain + ant[0].x * GP, s_gain + ant[1].x * GP};   // GAINS only
     const float2* gb_row[2] = {s_gain + ant[0].y * GP, s_gain + ant[1].y * GP};
 #pragma unroll(GAINS ? 1 : 4)   // the gains variant stays within its registers
     for (int j = 0; j < G; ++j) {
-        const float4 o = s_off[j];
-        const float4 pg = s_pg[j];             // {l, m, r^2/2, nu}
+        const float4 y = s_pg[j];              // {dl, dm, dn, q}
         const float2 ba = sBa[j];
-        const float b = ba.x;
-        const float4 ol = EXACT ? s_lo[j] : o;
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
-            const float uf = xh[r].x, vf = xh[r].y, wf = xh[r].z;
-            const float t = fmaf(uf, pg.x, fmaf(vf, pg.y, -wf * pg.z));
             float2 ga = make_float2(1.f, 0.f), gb = ga;      // gains {|G|, arg G in turns}
             if (GAINS) {
                 ga = ga_row[r][j];
                 gb = gb_row[r][j];
             }
-            float ph;                          // radians
-            if (EXACT) {
-                ph = fmaf(b, INV_TWO_PI_F, frac_dot3(dx[r], dxl[r], o, ol));
-                if (GAINS) ph += gb.y - ga.y;
-                ph = fmaf(-gc[r].gamr * INV_TWO_PI_F, t, ph);
-                if (PAR) ph = fmaf(-wf, pg.w, ph);
-                ph = frac_turns(ph) * TWO_PI_F;
-            } else {
-                const float b0 = GAINS ? fmaf(gb.y - ga.y, TWO_PI_F, b) : b;
-                ph = fmaf(dx[r].z, o.z, fmaf(dx[r].y, o.y, fmaf(dx[r].x, o.x, b0)));
-                ph = fmaf(-gc[r].gamr, t, ph);
-                if (PAR) ph = fmaf(-wf * TWO_PI_F, pg.w, ph);
-            }
+            const float b0 = GAINS ? fmaf(gb.y - ga.y, TWO_PI_F, ba.x) : ba.x;
+            float ph = lin4(gt[r].p, y, b0);                 // radians
+            if (EXACT)
+                ph = frac_turns(fmaf(ph, INV_TWO_PI_F, frac_dot3(dx[r], dxl[r], s_off[j], s_lo[j]))) * TWO_PI_F;
             float sn, cs;
             __sincosf(ph, &sn, &cs);
-            float amp = ba.y * ex2_approx(fmaf(gc[r].k1, t, gc[r].k0));   // (x/n) e^{Re(qc)}
+            float amp = ba.y * ex2_approx(lin3(gt[r].e, y, gt[r].e.w));   // (x/n) e^{Re(qc)}
             if (GAINS) amp *= ga.x * gb.x;
             sr[r] = fmaf(amp, cs, sr[r]);
             si[r] = fmaf(-amp, sn, si[r]);
@@ -160,21 +210,30 @@ __device__ __forceinline__ void fwd_gauss_tile(const float4* __restrict__ s_off,
 
 // ---- forward with gains through the granule's pair table
 // For the nb distinct antenna pairs (a_s, b_s) of the warp's visibility
-// granule and BT_CH pixels j = c0 + jj of the streamed granule, the table
+// granule and a chunk of pixels j = c0 + jj of the streamed granule, the table
 // holds a_j G_{j a_s} conj(G_{j b_s}) e^{-i B_j} (a_j = x_j / n_j) in polar
 // form: T[s][jj] = {B_j - arg (radians, within one turn), |a_j G G|} (Dirac
 // pixels) or {.., log2 |a_j G G|} (Gaussian pixels, for the amplitude's
 // exponent).  A pair then starts its phase from the table entry, needs no B_j
-// of its own, and accumulates with two FFMA.  Rows of BT_P, so the lanes of a
+// of its own, and accumulates with two FFMA.  Rows are padded by one, so the lanes of a
 // half-warp (one pair, consecutive pixels) write distinct banks.  gtab: the
 // gains in polar form {|G|, arg G in turns}.
+// Pixels per chunk: as many of the granule's 64 as the table holds rows for
+// (lch: their log2), since building a chunk is a chain of shared loads, a
+// logarithm and a store that only its 32 entries at a time overlap.
+__device__ __forceinline__ int pair_chunk_log2(int nb)
+{
+    return nb * (64 + 1) <= NB_MAX * BT_P ? 6 : nb * (32 + 1) <= NB_MAX * BT_P ? 5 : 4;
+}
 template <bool LOG>
 __device__ __forceinline__ void build_pair_table(float2* __restrict__ T, const int2* __restrict__ bl, int nb,
                                                  const float2* __restrict__ sBa,
-                                                 const float2* __restrict__ gtab, int c0, int lane)
+                                                 const float2* __restrict__ gtab, int c0, int lch, int lane)
 {
-    for (int e = lane; e < nb * BT_CH; e += 32) {
-        const int s = e / BT_CH, jj = e % BT_CH, j = c0 + jj;
+    const int n = nb << lch, row = (1 << lch) + 1;
+#pragma unroll 3
+    for (int e = lane; e < n; e += 32) {
+        const int s = e >> lch, jj = e & ((1 << lch) - 1), j = c0 + jj;
         const int2 ab = bl[s];
         const float2 ga = gtab[ab.x * GP + j], gb = gtab[ab.y * GP + j];
         const float2 ba = sBa[j];                                    // {B_j (radians), a_j}
@@ -182,7 +241,7 @@ __device__ __forceinline__ void build_pair_table(float2* __restrict__ T, const i
         const float arg = (ga.y - gb.y) + (ba.y < 0.f ? 0.5f : 0.f);
         const float ph = frac_turns(fmaf(ba.x, INV_TWO_PI_F, -arg)) * TWO_PI_F;
         const float m = fabsf(ba.y) * (ga.x * gb.x);
-        T[s * BT_P + jj] = make_float2(ph, LOG ? __log2f(m) : m);   // log2(0) = -inf: amplitude 0
+        T[s * row + jj] = make_float2(ph, LOG ? __log2f(m) : m);   // log2(0) = -inf: amplitude 0
     }
 }
 
@@ -191,16 +250,19 @@ __device__ __forceinline__ void fwd_dirac_tile_pt(const float4* __restrict__ s_o
                                                   const float4* __restrict__ s_lo,
                                                   const float2* __restrict__ sBa,
                                                   const float2* __restrict__ gtab, float2* __restrict__ T,
-                                                  const int2* __restrict__ bl, int nb, const int (&toff)[2],
+                                                  const int2* __restrict__ bl, int nb, int lch, const int (&toff)[2],
                                                   const float4 (&dx)[2], const float4 (&dxl)[2], int lane,
                                                   float (&sr)[2], float (&si)[2])
 {
 #pragma unroll 1
-    for (int c0 = 0; c0 < G; c0 += BT_CH) {
-        build_pair_table<false>(T, bl, nb, sBa, gtab, c0, lane);
+    for (int c0 = 0; c0 < G; c0 += 1 << lch) {
+        build_pair_table<false>(T, bl, nb, sBa, gtab, c0, lch, lane);
         __syncwarp();
-#pragma unroll 8
-        for (int jj = 0; jj < BT_CH; ++jj) {
+#pragma unroll 1
+        for (int j8 = 0; j8 < 1 << lch; j8 += 8)
+#pragma unroll
+        for (int j1 = 0; j1 < 8; ++j1) {
+            const int jj = j8 + j1;
             const int j = c0 + jj;
             const float4 o = s_off[j];
             const float4 ol = EXACT ? s_lo[j] : o;
@@ -220,46 +282,36 @@ __device__ __forceinline__ void fwd_dirac_tile_pt(const float4* __restrict__ s_o
     }
 }
 
-template <bool EXACT, bool PAR>
+template <bool EXACT>
 __device__ __forceinline__ void fwd_gauss_tile_pt(const float4* __restrict__ s_off,
                                                   const float4* __restrict__ s_lo,
                                                   const float4* __restrict__ s_pg,
                                                   const float2* __restrict__ sBa,
                                                   const float2* __restrict__ gtab, float2* __restrict__ T,
-                                                  const int2* __restrict__ bl, int nb, const int (&toff)[2],
-                                                  const float4 (&xh)[2], const float4 (&dx)[2],
-                                                  const float4 (&dxl)[2], const GaussConst (&gc)[2], int lane,
-                                                  float (&sr)[2], float (&si)[2])
+                                                  const int2* __restrict__ bl, int nb, int lch, const int (&toff)[2],
+                                                  const GaussTile (&gt)[2], const float4 (&dx)[2],
+                                                  const float4 (&dxl)[2], int lane, float (&sr)[2], float (&si)[2])
 {
 #pragma unroll 1
-    for (int c0 = 0; c0 < G; c0 += BT_CH) {
-        build_pair_table<true>(T, bl, nb, sBa, gtab, c0, lane);
+    for (int c0 = 0; c0 < G; c0 += 1 << lch) {
+        build_pair_table<true>(T, bl, nb, sBa, gtab, c0, lch, lane);
         __syncwarp();
-#pragma unroll 4
-        for (int jj = 0; jj < BT_CH; ++jj) {
+#pragma unroll 1
+        for (int j4 = 0; j4 < 1 << lch; j4 += 4)
+#pragma unroll
+        for (int j1 = 0; j1 < 4; ++j1) {
+            const int jj = j4 + j1;
             const int j = c0 + jj;
-            const float4 o = s_off[j];
-            const float4 pg = s_pg[j];
-            const float4 ol = EXACT ? s_lo[j] : o;
+            const float4 y = s_pg[j];
 #pragma unroll
             for (int r = 0; r < 2; ++r) {
                 const float2 tv = T[toff[r] + jj];                     // {B - arg, log2 |a g|}
-                const float wf = xh[r].z;
-                const float t = fmaf(xh[r].x, pg.x, fmaf(xh[r].y, pg.y, -wf * pg.z));
-                float ph;
-                if (EXACT) {
-                    ph = fmaf(tv.x, INV_TWO_PI_F, frac_dot3(dx[r], dxl[r], o, ol));
-                    ph = fmaf(-gc[r].gamr * INV_TWO_PI_F, t, ph);
-                    if (PAR) ph = fmaf(-wf, pg.w, ph);
-                    ph = frac_turns(ph) * TWO_PI_F;
-                } else {
-                    ph = fmaf(dx[r].z, o.z, fmaf(dx[r].y, o.y, fmaf(dx[r].x, o.x, tv.x)));
-                    ph = fmaf(-gc[r].gamr, t, ph);
-                    if (PAR) ph = fmaf(-wf * TWO_PI_F, pg.w, ph);
-                }
+                float ph = lin4(gt[r].p, y, tv.x);
+                if (EXACT)
+                    ph = frac_turns(fmaf(ph, INV_TWO_PI_F, frac_dot3(dx[r], dxl[r], s_off[j], s_lo[j]))) * TWO_PI_F;
                 float sn, cs;
                 __sincosf(ph, &sn, &cs);
-                const float amp = ex2_approx(fmaf(gc[r].k1, t, gc[r].k0 + tv.y));   // |a g| e^{Re(qc)}
+                const float amp = ex2_approx(lin3(gt[r].e, y, gt[r].e.w + tv.y));   // |a g| e^{Re(qc)}
                 sr[r] = fmaf(amp, cs, sr[r]);
                 si[r] = fmaf(-amp, sn, si[r]);
             }
@@ -270,8 +322,8 @@ __device__ __forceinline__ void fwd_gauss_tile_pt(const float4* __restrict__ s_o
 
 // Forward stage buffers in dynamic shared memory: two of them, each holding
 // NST streamed pixel granules as they sit in HBM -- offsets {dl, dm, dn, 1/n},
-// offset residuals, Gaussian data {l, m, r^2/2, nu}, x (FP64) and the granule
-// headers {centre hi, centre lo, extent, {sigma, kind}} -- filled by bulk (TMA)
+// offset residuals, Gaussian data {dl, dm, dn, q}, x (FP64) and the granule
+// headers {centre hi, centre lo, extent, {sigma, kind, nu at the centre, scale}} -- filled by bulk (TMA)
 // copies that complete on one mbarrier per buffer.  The copies of stage s + 1
 // are issued when stage s starts, so they land while stage s is computed.
 template <int NST>
@@ -299,7 +351,7 @@ __device__ __forceinline__ void fwd_stage_load(unsigned char* buf, const DevProb
     mbar_arrive_expect(bar, 3 * n4 + n8 + nh);
     bulk_copy(buf + S::OFF, P.pix.off + e, n4, bar);
     bulk_copy(buf + S::LO, P.pix.offlo + e, n4, bar);
-    bulk_copy(buf + S::PG, P.pgauss + e, n4, bar);
+    bulk_copy(buf + S::PG, P.pgoff + e, n4, bar);
     bulk_copy(buf + S::X, X + e, n8, bar);
     bulk_copy(buf + S::HDR, P.pghdr + (size_t)gs * 4, nh, bar);
 }
@@ -381,18 +433,21 @@ fwd_mixed_kernel(const DevProblem* __restrict__ probs, const Plan* __restrict__ 
             ext = P.vis.ext[vg];
 #pragma unroll
             for (int r = 0; r < 2; ++r) {
-                xh[r] = P.vis.hi[e0 + 32 * r];
-                dx[r] = to_rad(P.vis.off[e0 + 32 * r]);
+                if (!GAUSS) {
+                    xh[r] = P.vis.hi[e0 + 32 * r];
+                    dx[r] = to_rad(P.vis.off[e0 + 32 * r]);
+                }
                 if (GAINS) ant[r] = P.ant[e0 + 32 * r];
             }
         }
         double tr[2] = {0.0, 0.0}, ti[2] = {0.0, 0.0};
-        int nb = 0, toff[2] = {0, 0};          // GAINS: pairs in the granule's list (0: gathers)
+        int nb = 0, lch = 4, toff[2] = {0, 0};  // GAINS: pairs in the granule's list (0: gathers)
         if (GAINS) {
             if (vg_ok) nb = P.gnb[vg];
             if (nb > 0) {
+                lch = pair_chunk_log2(nb);
 #pragma unroll
-                for (int r = 0; r < 2; ++r) toff[r] = P.vslot[e0 + 32 * r] * BT_P;
+                for (int r = 0; r < 2; ++r) toff[r] = P.vslot[e0 + 32 * r] * ((1 << lch) + 1);
                 if (lane < nb) s_bl[warp][lane] = P.gbl[(size_t)vg * NB_MAX + lane];
             }
             __syncwarp();
@@ -444,7 +499,7 @@ fwd_mixed_kernel(const DevProblem* __restrict__ probs, const Plan* __restrict__ 
             }
             __syncwarp();
             for (int q = 0; q < ns; ++q) {
-                const float4 meta = s_hdr[4 * q + 3];                    // {sigma, kind, -, -}
+                const float4 meta = s_hdr[4 * q + 3];                    // {sigma, kind, nu at the centre, scale}
                 const int kind = (int)meta.y;
                 const float4 yc_h = s_hdr[4 * q], yc_l = s_hdr[4 * q + 1];
                 const bool exact = dot3(ext, s_hdr[4 * q + 2]) > D_MAX;  // warp-uniform
@@ -454,17 +509,23 @@ fwd_mixed_kernel(const DevProblem* __restrict__ probs, const Plan* __restrict__ 
                 const float2* q_Ba = s_Ba[warp][q];
                 float C[2];
 #pragma unroll
-                for (int r = 0; r < 2; ++r) C[r] = frac_dot3(xh[r], P.vis.lo[e0 + 32 * r], yc_h, yc_l);
+                for (int r = 0; r < 2; ++r) {
+                    if (GAUSS) {                                         // (not held across granules)
+                        xh[r] = reload4(P.vis.hi + e0 + 32 * r);
+                        dx[r] = to_rad(reload4(P.vis.off + e0 + 32 * r));
+                    }
+                    C[r] = frac_dot3(xh[r], P.vis.lo[e0 + 32 * r], yc_h, yc_l);
+                }
                 float sr[2] = {0.f, 0.f}, si[2] = {0.f, 0.f};
                 if (!GAUSS || kind == DIRAC) {
                     if (GAINS && nb > 0) {
                         if (exact) {
                             const float4 dxt[2] = {P.vis.off[e0], P.vis.off[e0 + 32]},
                                          dxl[2] = {P.vis.offlo[e0], P.vis.offlo[e0 + 32]};
-                            fwd_dirac_tile_pt<true>(q_off, q_lo, q_Ba, gtab, s_pt[warp], s_bl[warp], nb, toff, dxt,
+                            fwd_dirac_tile_pt<true>(q_off, q_lo, q_Ba, gtab, s_pt[warp], s_bl[warp], nb, lch, toff, dxt,
                                                     dxl, lane, sr, si);
                         } else {
-                            fwd_dirac_tile_pt<false>(q_off, q_lo, q_Ba, gtab, s_pt[warp], s_bl[warp], nb, toff, dx,
+                            fwd_dirac_tile_pt<false>(q_off, q_lo, q_Ba, gtab, s_pt[warp], s_bl[warp], nb, lch, toff, dx,
                                                      dx, lane, sr, si);
                         }
                     } else if (exact) {
@@ -483,46 +544,32 @@ fwd_mixed_kernel(const DevProblem* __restrict__ probs, const Plan* __restrict__ 
                     }
                 } else {
                     const bool par = (kind == PARAXIAL);
-                    GaussConst gc[2];
+                    GaussTile gt[2];
+                    const int scale = (int)meta.w;                       // -1: no table
+                    const float4* const cls = scale >= 0 ? P.gcls + (size_t)scale * P.vis.n_pad + e0 : nullptr;
 #pragma unroll
-                    for (int r = 0; r < 2; ++r) {
-                        gc[r] = gauss_const(xh[r].x, xh[r].y, xh[r].z, meta.x);
-                        C[r] = frac_turns(C[r] + gc[r].cphase);
-                    }
-                    if (GAINS && nb > 0) {
-                        if (exact) {
-                            const float4 dxt[2] = {P.vis.off[e0], P.vis.off[e0 + 32]},
-                                         dxl[2] = {P.vis.offlo[e0], P.vis.offlo[e0 + 32]};
-                            if (par) fwd_gauss_tile_pt<true, true>(q_off, q_lo, q_pg, q_Ba, gtab, s_pt[warp],
-                                                                   s_bl[warp], nb, toff, xh, dxt, dxl, gc, lane, sr,
-                                                                   si);
-                            else fwd_gauss_tile_pt<true, false>(q_off, q_lo, q_pg, q_Ba, gtab, s_pt[warp],
-                                                                s_bl[warp], nb, toff, xh, dxt, dxl, gc, lane, sr, si);
-                        } else if (par) {
-                            fwd_gauss_tile_pt<false, true>(q_off, q_lo, q_pg, q_Ba, gtab, s_pt[warp], s_bl[warp], nb,
-                                                           toff, xh, dx, dx, gc, lane, sr, si);
-                        } else {
-                            fwd_gauss_tile_pt<false, false>(q_off, q_lo, q_pg, q_Ba, gtab, s_pt[warp], s_bl[warp], nb,
-                                                            toff, xh, dx, dx, gc, lane, sr, si);
-                        }
-                    } else if (exact) {
+                    for (int r = 0; r < 2; ++r)
+                        gt[r] = gauss_tile(xh[r], exact ? z4 : dx[r], yc_h, meta.z, meta.x, par,
+                                           cls ? cls + 32 * r : nullptr, C[r]);
+                    if (exact) {
                         const float4 dxt[2] = {P.vis.off[e0], P.vis.off[e0 + 32]},
                                      dxl[2] = {P.vis.offlo[e0], P.vis.offlo[e0 + 32]};
-                        if (par) fwd_gauss_tile<GAINS, true, true>(q_off, q_lo, q_pg, q_Ba, gtab, xh, dxt, dxl, gc,
-                                                                   ant, sr, si);
-                        else fwd_gauss_tile<GAINS, true, false>(q_off, q_lo, q_pg, q_Ba, gtab, xh, dxt, dxl, gc, ant,
-                                                                sr, si);
-                    } else if (par) {
-                        fwd_gauss_tile<GAINS, false, true>(q_off, q_lo, q_pg, q_Ba, gtab, xh, dx, dx, gc, ant, sr, si);
+                        if (GAINS && nb > 0)
+                            fwd_gauss_tile_pt<true>(q_off, q_lo, q_pg, q_Ba, gtab, s_pt[warp], s_bl[warp], nb, lch, toff, gt,
+                                                    dxt, dxl, lane, sr, si);
+                        else
+                            fwd_gauss_tile<GAINS, true>(q_off, q_lo, q_pg, q_Ba, gtab, gt, dxt, dxl, ant, sr, si);
+                    } else if (GAINS && nb > 0) {
+                        fwd_gauss_tile_pt<false>(q_off, q_lo, q_pg, q_Ba, gtab, s_pt[warp], s_bl[warp], nb, lch, toff, gt,
+                                                 dx, dx, lane, sr, si);
                     } else {
-                        fwd_gauss_tile<GAINS, false, false>(q_off, q_lo, q_pg, q_Ba, gtab, xh, dx, dx, gc, ant, sr,
-                                                            si);
+                        fwd_gauss_tile<GAINS, false>(q_off, q_lo, q_pg, q_Ba, gtab, gt, dx, dx, ant, sr, si);
                     }
 #pragma unroll
                     for (int r = 0; r < 2; ++r) {
                         // S id (1 + i beta), then rotate by exp(-2 pi i C)
-                        const float ar = gc[r].id * fmaf(-gc[r].beta, si[r], sr[r]);
-                        const float ai = gc[r].id * fmaf(gc[r].beta, sr[r], si[r]);
+                        const float ar = gt[r].id * fmaf(-gt[r].beta, si[r], sr[r]);
+                        const float ai = gt[r].id * fmaf(gt[r].beta, sr[r], si[r]);
                         float sn, cs;
                         __sincosf(C[r] * TWO_PI_F, &sn, &cs);
                         tr[r] += (double)fmaf(cs, ar, sn * ai);
@@ -640,15 +687,13 @@ __device__ __forceinline__ void adj_gauss_tile(const float4* __restrict__ s_off,
 // The record of a streamed visibility for a Gaussian owner of scale sigma:
 // r' = id (1 - i beta) r has |r'| = |r| / sqrt(1 + beta^2) and arg r' =
 // arg r - atan(beta) (id > 0).  b: the visibility's B term in turns, with
-// odd_turn's half turn for odd k; rp = {|r|, arg r in turns}; va = {u, v, -2 w,
-// -}.  Returns {B + arg r' (radians), gamr, k1, k0 + log2 |r'|}.
-__device__ __forceinline__ float4 adj_gauss_record(float b, float2 rp, const float4 va, float sigma)
+// odd_turn's half turn for odd k; rp = {|r|, arg r in turns}; gc: gauss_class of the
+// visibility.  Returns {B + arg r' (radians), gamr, k1, k0 + log2 |r'|}.
+__device__ __forceinline__ float4 adj_gauss_record(float b, float2 rp, const float4 gc)
 {
-    const GaussConst gc = gauss_const(va.x, va.y, -0.5f * va.z, sigma);
-    b = frac_turns(b + gc.cphase);
-    b = frac_turns(b + fmaf(-atanf(gc.beta), INV_TWO_PI_F, rp.y));
-    const float lgr = __log2f(rp.x) - 0.5f * __log2f(fmaf(gc.beta, gc.beta, 1.0f));   // -inf when r = 0
-    return make_float4(b * TWO_PI_F, gc.gamr, gc.k1, gc.k0 + lgr);
+    b = frac_turns(b + gc.w);
+    b = frac_turns(b + rp.y);
+    return make_float4(b * TWO_PI_F, gc.x, gc.y, gc.z + __log2f(rp.x));       // log2: -inf when r = 0
 }
 
 // Adjoint stage buffers in dynamic shared memory: two of them, each holding
@@ -778,8 +823,13 @@ adj_mixed_kernel(const DevProblem* __restrict__ probs, const Plan* __restrict__ 
                     const int k = lane + 32 * h;
                     const float b = frac_dot3(ch, cl, b_off[q * G + k], b_lo[q * G + k]) + odd_turn(k);
                     const float2 rp = b_r[q * G + k];
-                    s_rec[warp][q][k] = gauss ? adj_gauss_record(b, rp, b_ga[q * G + k], sigma)
-                                              : make_float4(frac_turns(b + rp.y) * TWO_PI_F, rp.x, 0.f, 0.f);
+                    if (gauss) {
+                        const float4 va = b_ga[q * G + k];                  // {u, v, -2 w, -}
+                        s_rec[warp][q][k] =
+                            adj_gauss_record(b, rp, gauss_class(make_float4(va.x, va.y, -0.5f * va.z, 0.f), sigma));
+                        continue;
+                    }
+                    s_rec[warp][q][k] = make_float4(frac_turns(b + rp.y) * TWO_PI_F, rp.x, 0.f, 0.f);
                 }
             }
             __syncwarp();
@@ -942,17 +992,6 @@ __device__ __forceinline__ void adjg_gauss_tile(const float4* __restrict__ s_p, 
     adjg_flush(M, z, acc);                      // the last run
 }
 
-// What a streamed visibility's record takes of a Gaussian scale: {gam (radians
-// per turn of t), k1, k0 + log2 sqrt(id), cphase - atan(beta) / 2 pi in turns}, the
-// last two with r' = id (1 - i beta) r, |r'| = |r| sqrt(id), arg r' = arg r -
-// atan(beta).
-__device__ __forceinline__ float4 gauss_class(const float4 uvw, float sigma)
-{
-    const GaussConst gc = gauss_const(uvw.x, uvw.y, uvw.z, sigma);
-    return make_float4(gc.gamr, gc.k1, gc.k0 - 0.5f * __log2f(fmaf(gc.beta, gc.beta, 1.0f)),
-                       frac_turns(fmaf(-atanf(gc.beta), INV_TWO_PI_F, gc.cphase)));
-}
-
 // The same for every visibility and each of the problem's scales, in FP64: made
 // once per layout when there are few scales (gcls[class][vis.n_pad]).
 __global__ void gauss_class_kernel(const d4* __restrict__ vd, int n_pad, const double* __restrict__ sigma,
@@ -1079,14 +1118,14 @@ adj_mixed_gains_kernel(const DevProblem* __restrict__ probs, const Plan* __restr
         const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
         float4 xh[2], dx[2], y[2] = {z4, z4};
         // the granule's centre, which the Gaussian terms are taken from
-        const float qc = 0.5f * fmaf(ch.x, ch.x, ch.y * ch.y), nuc = ch.z + qc;
-        const float4* const cls = gauss && P.gcls && P.gclass[pgi] >= 0 ? P.gcls + (size_t)P.gclass[pgi] * P.vis.n_pad : nullptr;
+        const float qc = centre_q(ch.x, ch.y), nuc = P.pghdr[4 * (size_t)pgi + 3].z;
+        const float4* const cls = gauss && P.gclass && P.gclass[pgi] >= 0
+                                      ? P.gcls + (size_t)P.gclass[pgi] * P.vis.n_pad : nullptr;
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
             xh[r] = P.pix.hi[eidx[r]];
-            y[r] = P.pix.off[eidx[r]];
-            dx[r] = to_rad(y[r]);
-            if (gauss) y[r].w = P.pgauss[eidx[r]].z - qc;
+            dx[r] = to_rad(P.pix.off[eidx[r]]);
+            if (gauss) y[r] = P.pgoff[eidx[r]];
         }
         const SmemGain sg{s_gain, lane};
         mbar_wait(&s_gbar, gpar, fault);
