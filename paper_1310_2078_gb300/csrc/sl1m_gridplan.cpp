@@ -115,20 +115,28 @@ std::vector<float2> twiddles(int lg)
 
 }  // namespace
 
-// Seconds a pass of the operator takes, forward and adjoint averaged, the
-// launches that both paths share left out.
-double grid_seconds(const GridOp& g, double n_vis)
+// Seconds of a pass (forward and adjoint averaged) by either operator, fitted to
+// both on GB300 over 64^2 .. 1024^2 pixels x 1,500 .. 100,000 visibilities, fields
+// of +/-0.02 .. +/-0.5 (us, forward / adjoint; pairs and then lattice):
+//   64^2 x 4,000      41 / 38       43 / 87       256^2 +/-0.5 x 5,000   275 / 266    191 / 292
+//   64^2 x 40,000    110 / 87       66 / 230      500^2 x 3,000          399 / 286     76 / 93
+//   128^2 x 5,000     69 / 58       45 / 60       1024^2 +/-0.3 x 3,000 1569 / 1096   482 / 669
+//   200^2 x 60,000  1181 / 843      96 / 127      1024^2 x 100,000     50011 / 34845  252 / 386
+// Lattice: launches, the planes' cells, the visibilities, and the points that a
+// tile's CTA spreads one after the other where there are few tiles.  The lattice
+// is taken where it promises a tenth or more.
+static double grid_seconds(const GridOp& g, double n_vis)
 {
-    return 2.5e-5 + (double)g.np * grid_plane_elems(g) * 8.0 * 2.2 / 3.5e12 + n_vis * 8.0e-10;
+    return 4.2e-5 + 2.8e-12 * (double)g.np * grid_plane_elems(g) + 1.05e-9 * n_vis + 2.7e-7 * n_vis / grid_tiles(g);
 }
-static double pair_seconds(double pairs) { return 1.0e-5 + pairs / 2.4e12; }
+static double pair_seconds(double pairs) { return 2.8e-5 + pairs / 2.4e12; }
 
 bool grid_build(sl1m_problem& P, cudaStream_t st, size_t budget)
 {
     P.grid.reset();
     if (P.n_ant > 0 || P.has_gauss) return false;
     const double pairs = P.pairs();
-    if (pair_seconds(pairs) < 4.0e-5) return false;      // launches, not pairs, decide
+    if (0.9 * pair_seconds(pairs) < 4.2e-5) return false;   // launches, not pairs, decide
     // extents of the visibilities and of n - 1
     double um = 0, vm = 0, w0 = 1e300, w1 = -1e300, n0 = 1e300, n1 = -1e300;
     for (int64_t k = 0; k < P.n_vis; ++k) {
@@ -159,7 +167,7 @@ bool grid_build(sl1m_problem& P, cudaStream_t st, size_t budget)
     const double dw = 0.25 / B, span = (w1 - w0) / dw;
     if (!(span < 1e5)) return false;
     g.np = (int)std::ceil(span) + GRW;
-    if (grid_seconds(g, (double)P.n_vis) > 0.8 * pair_seconds(pairs)) return false;
+    if (grid_seconds(g, (double)P.n_vis) > 0.9 * pair_seconds(pairs)) return false;
     g.cx = g.nx / 2;
     g.cy = g.ny / 2;
     // the workspace holds as many planes as fit GR_WS_MAX bytes and a quarter

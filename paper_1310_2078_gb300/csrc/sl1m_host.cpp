@@ -577,6 +577,7 @@ sl1m_ctx::~sl1m_ctx()
     for (auto e : ev_join)
         if (e) cudaEventDestroy(e);
     if (ev_fork) cudaEventDestroy(ev_fork);
+    if (mail) cudaFreeHost(mail);
     if (own_stream && stream) cudaStreamDestroy(stream);
 }
 
@@ -1075,8 +1076,9 @@ int sl1m_problem::init_solve(const sl1m_solve_opts* o, double L, bool power_only
 
 int sl1m_problem::read_state(SolveState& s, cudaStream_t st)
 {
-    CK(cudaMemcpyAsync(&s, dev->st.p, sizeof s, cudaMemcpyDeviceToHost, st));
+    CK(cudaMemcpyAsync(&ctx->mail->state, dev->st.p, sizeof s, cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
+    s = ctx->mail->state;
     return SL1M_OK;
 }
 
@@ -1459,11 +1461,25 @@ int batch_phases(sl1m_ctx* ctx, Batch& B, std::vector<int>& out)
     out.resize(np);
     CKL(launch_phases(B.desc.p, B.n_probs_dev.p, std::max(1, std::min(64, (np + 127) / 128)), B.phases_dev.p,
                       ctx->stream));
-    CK(cudaMemcpyAsync(out.data(), B.phases_dev.p, sizeof(int) * np, cudaMemcpyDeviceToHost, ctx->stream));
-    unsigned fault = 0;
-    CK(wait_fault_read(&fault, ctx->stream));
+    Mailbox& mail = *ctx->mail;
+    CK(cudaMemcpyAsync(mail.phases, B.phases_dev.p, sizeof(int) * np, cudaMemcpyDeviceToHost, ctx->stream));
+    CK(wait_fault_read(&mail.fault, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
-    return check_wait_fault(ctx, fault);
+    std::copy(mail.phases, mail.phases + np, out.begin());
+    return check_wait_fault(ctx, mail.fault);
+}
+
+// An operator call's result and the fault flag to the host; waits for the stream.
+static int read_result(sl1m_ctx* ctx, void* out, const void* dev, size_t bytes)
+{
+    Mailbox& mail = *ctx->mail;
+    const bool fits = bytes <= sizeof mail.result;
+    CK(wait_fault_read(&mail.fault, ctx->stream));
+    CK(cudaMemcpyAsync(fits ? (void*)mail.result : out, dev, bytes, cudaMemcpyDeviceToHost, ctx->stream));
+    CK(cudaStreamSynchronize(ctx->stream));
+    RET(check_wait_fault(ctx, mail.fault));
+    if (fits) memcpy(out, mail.result, bytes);
+    return SL1M_OK;
 }
 
 // Operator-mode batch of a single problem (cached per precision).
@@ -1562,7 +1578,8 @@ int sl1m_create(sl1m_ctx** out, int device, void* cuda_stream)
         delete c;
         return SL1M_ERR_CUDA;
     }
-    bool ok = cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) == cudaSuccess;
+    bool ok = cudaHostAlloc((void**)&c->mail, sizeof(Mailbox), cudaHostAllocDefault) == cudaSuccess &&
+              cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) == cudaSuccess;
     for (int i = 0; i < N_CLS - 1; ++i)
         ok = ok && cudaStreamCreateWithFlags(&c->side[i], cudaStreamNonBlocking) == cudaSuccess &&
              cudaEventCreateWithFlags(&c->ev_join[i], cudaEventDisableTiming) == cudaSuccess;
@@ -1805,11 +1822,7 @@ int sl1m_forward(sl1m_problem* prob, const double* x, double* vis_out, int preci
     CK(D.vis_user.reserve(prob->n_vis, ctx->stream));
     CK(cudaMemcpyAsync(D.x_user.p, x, sizeof(double) * prob->n_pix, cudaMemcpyHostToDevice, ctx->stream));
     RET(sl1m_forward_dev(prob, D.x_user.p, (double*)D.vis_user.p, precision));
-    CK(cudaMemcpyAsync(vis_out, D.vis_user.p, sizeof(double2) * prob->n_vis, cudaMemcpyDeviceToHost, ctx->stream));
-    unsigned fault = 0;
-    CK(wait_fault_read(&fault, ctx->stream));
-    CK(cudaStreamSynchronize(ctx->stream));
-    RET(check_wait_fault(ctx, fault));
+    RET(read_result(ctx, vis_out, D.vis_user.p, sizeof(double2) * prob->n_vis));
     ctx->h2d += (long long)sizeof(double) * prob->n_pix;
     ctx->d2h += (long long)sizeof(double2) * prob->n_vis;
     return SL1M_OK;
@@ -1829,11 +1842,7 @@ int sl1m_adjoint(sl1m_problem* prob, const double* r, double* img_out, int preci
     CK(D.img_user.reserve(prob->n_pix, ctx->stream));
     CK(cudaMemcpyAsync(D.r_user.p, r, sizeof(double2) * prob->n_vis, cudaMemcpyHostToDevice, ctx->stream));
     RET(sl1m_adjoint_dev(prob, (const double*)D.r_user.p, D.img_user.p, precision));
-    CK(cudaMemcpyAsync(img_out, D.img_user.p, sizeof(double) * prob->n_pix, cudaMemcpyDeviceToHost, ctx->stream));
-    unsigned fault = 0;
-    CK(wait_fault_read(&fault, ctx->stream));
-    CK(cudaStreamSynchronize(ctx->stream));
-    RET(check_wait_fault(ctx, fault));
+    RET(read_result(ctx, img_out, D.img_user.p, sizeof(double) * prob->n_pix));
     ctx->h2d += (long long)sizeof(double2) * prob->n_vis;
     ctx->d2h += (long long)sizeof(double) * prob->n_pix;
     return SL1M_OK;

@@ -191,6 +191,15 @@ struct Batch {
     ~Batch();
 };
 
+// What the host reads back from the device, in pinned memory: copies into it are
+// asynchronous, so a call waits for the stream once and not at each of them.
+struct Mailbox {
+    unsigned fault;                      // the bounded waits' flag
+    sl1m::SolveState state;
+    int phases[sl1m::MAX_PROBS];
+    unsigned char result[256 * 1024];    // an operator call's result, when it fits
+};
+
 struct sl1m_ctx {
     int device = 0;
     cudaStream_t stream = nullptr;
@@ -214,6 +223,7 @@ struct sl1m_ctx {
         return v;
     }
     DBuf<float2> grid_ws;                // workspace of the lattice operators
+    Mailbox* mail = nullptr;             // used by one call (or the server's loop) at a time
     std::vector<sl1m_problem*> problems;
     // autotuned (streamed granules per stage, CTAs per SM), keyed by
     // (precision, op, gains, Gaussian pixels, log2 of the units)
