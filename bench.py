@@ -7,8 +7,11 @@ noise, mixed precision (FP32 operator, FP64 solver scalars).  L is computed
 once by power iteration (untimed); one step = `--iters` FISTA steps (default
 5) at that L through the C ABI's solve call, each one forward and one
 adjoint over all 4.26e11 pixel-visibility pairs, plus the forward of I_0.
-Metric: pixel-visibility pairs evaluated per second by the forward and
-adjoint kernels (pairs/s), whole job.
+Metric: pixel-visibility pairs per second that the forward and adjoint
+products cover (N_v N_p per product; pairs/s), whole job.  The library's pair
+kernels evaluate each of them; on a regular lattice of Dirac pixels, as here,
+its lattice operator (gridding and FFT) computes the same products without
+(`operator` in the line says which one ran, and the roofline is its own).
 
 value   : inputs resident in HBM when the timed region starts; each step
           timed with CUDA events on the library's stream, L2 flushed between
@@ -228,7 +231,7 @@ class ClockSampler:
                 "reasons": sorted(reasons)}
 
 
-KERNEL_SOURCES = ("sl1m_mixed.cu", "sl1m_fp64.cu", "sl1m_devfn.cuh", "sl1m_dev.h", "sl1m_sincos_poly.h")
+KERNEL_SOURCES = ("sl1m_mixed.cu", "sl1m_grid.cu", "sl1m_fp64.cu", "sl1m_devfn.cuh", "sl1m_dev.h", "sl1m_sincos_poly.h")
 
 
 def kernel_source_hash(csrc=None):
@@ -273,6 +276,31 @@ def ncu_traffic(kernel, nst, npoly, ctas, workload):
             if key == (kernel, nst, npoly, ctas, workload, src):
                 return int(m.group(7))
     return None
+
+
+def hbm_peak():
+    """(GB/s, where from): the measured copy bandwidth, else a fallback."""
+    try:
+        with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as f:
+            return float(json.load(f)["hbm_gbs"]), "of measured copy bandwidth"
+    except (OSError, ValueError, KeyError, TypeError):
+        return 6800.0, "of fallback"
+
+
+def lattice_bytes(w):
+    """What one product of the lattice operator moves on workload w: planes in
+    w of 2^lx x 2^ly complex FP32 cells (twice the lattice's sides and more),
+    at Delta w = 1 / (4 B) for |n - 1 - nc| <= B over 0 .. max |w|, and 8 planes
+    for the kernel's width; the row pass writes ny rows, the column pass reads
+    them and writes 2^ly, gathering (spreading) reads (writes) those.  An upper
+    bound: tiles that no visibility touches are left out."""
+    lm, r2 = w.lm, (w.lm ** 2).sum(axis=1)
+    nm1 = -r2 / (1 + np.sqrt(1 - r2))
+    aw = np.abs(w.uvw[:, 2])
+    planes = math.ceil((aw.max() - aw.min()) * 2 * (nm1.max() - nm1.min())) + 8
+    n = [len(np.unique(np.round(lm[:, a], 12))) for a in (0, 1)]
+    lx, ly = (max(64, 1 << (2 * k - 1).bit_length()) for k in n)
+    return {"planes": planes, "cells": [lx, ly], "bytes": planes * lx * (2 * n[1] + 2 * ly) * 8}
 
 
 def sfu_peak(w, op="fwd"):
@@ -659,6 +687,10 @@ def main():
     V = P.forward(w.x_true, sl1m.FP64 if w.n_vis * w.n_pix < 5e9 else sl1m.MIXED) + w.noise
     P.set_vis_data(V)
     lam = w.lambda_frac * P.adjoint(V * (1 if w.weights is None else w.weights), prec).max()
+    # a product takes 3 launches by the pair kernels, more by the lattice operator
+    ctx.counters_reset()
+    P.forward(w.x_true, prec)
+    lattice = prec == sl1m.MIXED and ctx.counters()["launches"] > 3
     if args.shape:                                              # untimed set-up
         sh = [[int(v) for v in part.split(",")] for part in args.shape.split(":")]
         for op in (0, 1):
@@ -666,7 +698,8 @@ def main():
         tuned = {"nst": [sh[0][0], sh[1][0]], "ctas_per_sm": [sh[0][1], sh[1][1]],
                  "npoly": [sh[0][2], sh[1][2]], "source": "--shape"}
     else:
-        tuned = None if args.no_autotune else P.autotune(prec)
+        # (the lattice operator has no tile shapes)
+        tuned = None if args.no_autotune or lattice else P.autotune(prec)
     sfu = ctx.measure_sfu()                                      # untimed: the measured MUFU rate
     flush = torch.empty(2 * L2_BYTES // 4, dtype=torch.float32, device=f"cuda:{dev}")
 
@@ -751,11 +784,25 @@ def main():
     meas = sfu_peak_measured(w, sfu, op_of(dom))
     roofline["peak_measured_sfu"] = meas
     roofline["frac_of_measured_sfu"] = achieved / meas["peak"]
+    if lattice:
+        # bound by the planes' traffic: bytes of a product over its event time
+        by = lattice_bytes(w)
+        hbm, src = hbm_peak()
+        sec = pd["ms"] / 1e3 / worked[dom]
+        roofline = {"bound": "hbm", "kernel": dom + " (lattice: rows, columns, gather / spread)",
+                    "achieved": by["bytes"] / sec / 1e9, "peak": hbm, "unit": "GB/s",
+                    "frac": by["bytes"] / sec / 1e9 / hbm, "peak_basis": src, "planes": by["planes"],
+                    "cells": by["cells"], "bytes_per_launch": by["bytes"], "launches": pd["launches"],
+                    "launches_with_work": worked[dom], "avg_launch_ms": 1e3 * sec, "traffic": None}
     per_kernel = {}
     for k in keys:
         if prof[k]["ms"] <= 0:
             continue
         rate = prof[k]["pairs"] / (prof[k]["ms"] / 1e3) / 1e9
+        if lattice:
+            per_kernel[k] = {"launches": prof[k]["launches"], "launches_with_work": worked[k],
+                             "avg_launch_ms": prof[k]["ms"] / worked[k], "Gpairs_per_s": rate}
+            continue
         pk, _, pk_alt = sfu_peak(w, op_of(k))
         per_kernel[k] = {"launches": prof[k]["launches"], "launches_with_work": worked[k],
                          "avg_launch_ms": prof[k]["ms"] / worked[k], "Gpairs_per_s": rate,
@@ -790,6 +837,7 @@ def main():
                "scaling": "weak", "vs_baseline": None,
                "dtype": "f32+f64" if prec == sl1m.MIXED else "f64", "data": "synthetic",
                "config": bench_config(args, w), "lambda": lam, "tile_shape": tuned,
+               "operator": "lattice" if lattice else "pairs",
                rate_key: rate_val,
                "iters": [s["iters"] for s in stats], "power_iters": stats[-1]["power_iters"],
                "final": {"E": stats[-1]["E"], "resid2": stats[-1]["resid2"],
