@@ -501,6 +501,8 @@ grid_gather_kernel(const DevProblem* __restrict__ probs, int prob, const GridOp 
     }
 }
 
+constexpr int GR_SEG = GR_TILE * GR_TILE;      // planes of a spreading segment at most
+
 // Adjoint: a CTA owns the GR_TILE^2 cells (one per thread) of a tile and walks
 // the visibilities that touch it in the order of their first plane, with a ring
 // of 8 accumulators per cell, the planes the current point reaches: once the
@@ -518,6 +520,7 @@ grid_spread_kernel(const DevProblem* __restrict__ probs, int prob, const GridOp 
     __shared__ float4 s_pt[2][PB];             // {Re, Im of conj(rot) r, first x, first y}
     __shared__ __align__(16) float s_wx[2][PB][GRW], s_wy[2][PB][GRW], s_ww[2][PB][GRW];
     __shared__ int s_ip[2][PB];
+    __shared__ unsigned char s_act[GR_SEG];    // planes of the segment that have to be written
     const double2* R;
     if (!adj_role(probs[prob], R)) return;
     const int Lx = 1 << g.lx, Ly = 1 << g.ly, tiles_x = Lx / GR_TILE;
@@ -532,8 +535,8 @@ grid_spread_kernel(const DevProblem* __restrict__ probs, int prob, const GridOp 
     const int x = wx0 + (lane & 7), y = wy0 + (lane >> 3);
     const size_t plane = (size_t)Ly * Lx;
     float2* const cell = g.g2 + (size_t)y * Lx + x;
-    const unsigned char* act = g.act + ((size_t)(tile % tiles_x)) * (Ly / GR_TILE) + tile / tiles_x;
-    const size_t act_plane = (size_t)tiles_x * (Ly / GR_TILE);
+    if ((int)threadIdx.x < tb - ta)            // (read after the loop's first barrier)
+        s_act[threadIdx.x] = g.act[((size_t)(ta + threadIdx.x) * tiles_x + tile % tiles_x) * (Ly / GR_TILE) + tile / tiles_x];
     // this thread's part of the staging: point si, weights sf of each axis
     const int si = threadIdx.x >> 3, sf = threadIdx.x & 7;
     float lwx = 0.f, lwy = 0.f, lww = 0.f;
@@ -546,28 +549,39 @@ grid_spread_kernel(const DevProblem* __restrict__ probs, int prob, const GridOp 
         lwx = wt[sf];
         lwy = wt[GRW + sf];
         lww = wt[2 * GRW + sf];
+        const int4 ps = g.pos[k];
+        lip = ps.z;
         if (sf == 0) {
-            const int4 ps = g.pos[k];
             const float2 o = g.rot[k];
             const double2 r = R[k];
             const float rr = (float)r.x * g.ascale, ri = (float)(ps.w ? -r.y : r.y) * g.ascale;
             lpt = make_float4(fmaf(o.x, rr, o.y * ri), fmaf(o.x, ri, -o.y * rr), __int_as_float(ps.x),
                               __int_as_float(ps.y));
-            lip = ps.z;
         }
     };
+    // acc[p mod 8] is plane p of [cur, cur + 8); the staged weights in w are
+    // rotated to match, so the ring turns without moving a register
     float2 acc[GRW];
 #pragma unroll
     for (int q = 0; q < GRW; ++q) acc[q] = make_float2(0.f, 0.f);
-    int cur = max(0, ta - GRW + 1);            // acc[q] is plane cur + q
+    int cur = max(0, ta - GRW + 1);
+    const auto put = [&](int p, float2 v) {
+        if (p >= ta && p < tb && s_act[p - ta]) cell[(size_t)(p - p0) * plane] = v;
+    };
     // planes [cur, to) are complete
     const auto advance = [&](int to) {
-        for (; cur < to; ++cur) {
-            if (cur >= ta && cur < tb && act[cur * act_plane]) cell[(size_t)(cur - p0) * plane] = acc[0];
+        if (cur >= to) return;
+        const int n = to - cur;
 #pragma unroll
-            for (int q = 0; q + 1 < GRW; ++q) acc[q] = acc[q + 1];
-            acc[GRW - 1] = make_float2(0.f, 0.f);
+        for (int q = 0; q < GRW; ++q) {
+            const int d = (q - cur) & (GRW - 1);           // acc[q] is plane cur + d
+            if (d < n) {
+                put(cur + d, acc[q]);
+                acc[q] = make_float2(0.f, 0.f);
+            }
         }
+        for (int p = cur + GRW; p < to; ++p) put(p, make_float2(0.f, 0.f));
+        cur = to;
     };
     fetch(b0);
     int buf = 0;
@@ -575,7 +589,7 @@ grid_spread_kernel(const DevProblem* __restrict__ probs, int prob, const GridOp 
         const int n = min(PB, b1 - b);
         s_wx[buf][si][sf] = lwx;
         s_wy[buf][si][sf] = lwy;
-        s_ww[buf][si][sf] = lww;
+        s_ww[buf][si][(sf + lip) & (GRW - 1)] = lww;       // by plane mod 8
         if (sf == 0) {
             s_pt[buf][si] = lpt;
             s_ip[buf][si] = lip;
@@ -749,7 +763,9 @@ cudaError_t grid_adjoint(const DevProblem* probs, int p, const GridOp& g, int n_
     for (int p0 = 0; p0 < g.np; p0 += g.np_pass) {
         const int np = std::min(g.np_pass, g.np - p0);
         // segments of planes: enough CTAs for a few waves, no fewer planes than 32
-        const int tiles = grid_tiles(g), nseg = std::max(1, std::min((np + 31) / 32, 4096 / tiles));
+        // and no more than GR_SEG
+        const int tiles = grid_tiles(g);
+        const int nseg = std::max((np + GR_SEG - 1) / GR_SEG, std::max(1, std::min((np + 31) / 32, 4096 / tiles)));
         const int seg = (np + nseg - 1) / nseg;
         const dim3 sg((unsigned)tiles, (unsigned)((np + seg - 1) / seg));
         grid_spread_kernel<<<sg, GR_TILE * GR_TILE, 0, st>>>(probs, p, g, p0, np, seg);

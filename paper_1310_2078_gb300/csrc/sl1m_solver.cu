@@ -372,6 +372,15 @@ adj_finish_kernel(const DevProblem* __restrict__ probs, const Plan* __restrict__
         const int t = threadIdx.x % S::EL, e = e0 + t;
         const bool in = e < P.pix.n_pad;
         const int poff = pl.blk_poff[gb], ncon = in ? pl.blk_ncon[gb] : 0;
+        // the step's other loads are issued before the partial sums'
+        const int par = mode == FIN_SOLVE && !P.st->algo ? (P.st->k + 1) & 1 : 0;
+        double y0 = 0.0, Io = 0.0;
+        int orig = 0;
+        if (mode == FIN_SOLVE && threadIdx.x < S::EL && in) {
+            y0 = P.b.y[e];
+            Io = P.b.I[par ^ 1][e];
+            orig = P.pix.orig[e];
+        }
         const double s = sum_slots<SL>(partial, pl.blk_el, poff, ncon, i0 + t, sh1);
         double acc = 0.0;
         int cnt = 0, bad = 0;
@@ -388,16 +397,14 @@ adj_finish_kernel(const DevProblem* __restrict__ probs, const Plan* __restrict__
             } else {
                 const SolveState& S2 = *P.st;
                 const double inv_L = 1.0 / S2.L, thr = S2.lambda / S2.L;
-                const double v = B.y[e] - s * inv_L;
+                const double v = y0 - s * inv_L;
                 double In = v > thr ? v - thr : 0.0;
-                if (P.pix.orig[e] < 0) In = 0.0;
+                if (orig < 0) In = 0.0;
                 if (S2.algo) {
                     B.I[1][e] = In;                 // z_k; y is formed by the mix kernel
                 } else {
                     double tn, beta;
                     fista_beta(S2.t, tn, beta);
-                    const int par = (S2.k + 1) & 1;
-                    const double Io = B.I[par ^ 1][e];
                     B.I[par][e] = In;
                     B.y[e] = In + beta * (In - Io);
                 }
