@@ -28,9 +28,10 @@
 // 3.6e-7 to 4.9e-7 off.  The work no longer grows with N_v N_p but with the
 // planes' cells: per plane the kernels move up to (3 2^ly + 2 ny) 2^lx complex
 // numbers.  Measured on GB300 against the pair kernels: 1024^2 pixels x 406,400
-// visibilities (55 planes of 2048^2) forward 202.7 -> 1.21 ms, adjoint 141.6 ->
-// 1.75 ms; 256^2 over +/-0.5 x 40,320 (151 planes of 512^2) 1.19 -> 0.34 ms
-// and 0.84 -> 0.46 ms.
+// visibilities (55 planes of 2048^2) forward 202.9 -> 0.99 ms, adjoint 141.7 ->
+// 1.13 ms; 256^2 over +/-0.5 x 40,320 (273 planes of 512^2) 1.19 -> 0.25 ms and
+// 0.85 -> 0.32 ms.  The planes' traffic alone would take 0.35 ms at paper scale
+// (2.3 GB at the 6.7 TB/s of a copy) and 0.14 ms on the wide field.
 #include <algorithm>
 
 #include "sl1m_devfn.cuh"
@@ -64,10 +65,11 @@ __device__ __forceinline__ void dft4(float2& a0, float2& a1, float2& a2, float2&
 }
 
 // Half-zero inputs: with the cells at elements [0, L/4) and [3L/4, L) of a
-// transform (2^lx >= 2 nx, the origin in the middle), elements q = 2..5 of the 8
-// that a thread holds are zero, and of its outputs only q = 0, 1, 6, 7 are cells.
+// transform (2^lx >= 2 nx, the origin in the middle), the middle half of the P
+// elements that a thread holds are zero, and of its outputs only the outer
+// quarters are cells.  PIN: the inputs are such; POUT: only those outputs are wanted.
 
-// dft4 and dft8 with the middle inputs (a1, a2; v2..v5) zero.
+// dft4 with the middle inputs zero.
 template <int SGN>
 __device__ __forceinline__ void dft4_outer(float2& a0, float2& a1, float2& a2, float2& a3)
 {
@@ -77,57 +79,111 @@ __device__ __forceinline__ void dft4_outer(float2& a0, float2& a1, float2& a2, f
     a2 = csub(p, q);
     a3 = cadd(p, r);
 }
-
-// The last step of dft8 from the transforms e of the even and o of the odd inputs.
-template <int SGN, bool POUT>
-__device__ __forceinline__ void dft8_join(float2 (&v)[8])
+// a e^{SGN 2 pi i M / 16}
+template <int SGN, int M>
+__device__ __forceinline__ float2 rot16(float2 a)
 {
-    const float H = 0.70710678118654752f;
-    const float2 r3 = crot<SGN>(v[3]), r7 = crot<SGN>(v[7]);
-    const float2 o1 = make_float2((v[3].x + r3.x) * H, (v[3].y + r3.y) * H);   // times e^{SGN i pi/4}
-    const float2 o2 = crot<SGN>(v[5]);
-    const float2 o3 = make_float2((r7.x - v[7].x) * H, (r7.y - v[7].y) * H);   // times e^{SGN 3 i pi/4}
-    const float2 e0 = v[0], e1 = v[2], e2 = v[4], e3 = v[6], o0 = v[1];
-    v[0] = cadd(e0, o0);
-    v[1] = cadd(e1, o1);
-    if (!POUT) {
-        v[2] = cadd(e2, o2);
-        v[3] = cadd(e3, o3);
-        v[4] = csub(e0, o0);
-        v[5] = csub(e1, o1);
+    constexpr float H = 0.70710678118654752f, C = 0.92387953251128676f, S = 0.38268343236508977f;
+    if constexpr (M >= 8) {
+        const float2 b = rot16<SGN, M - 8>(a);
+        return make_float2(-b.x, -b.y);
+    } else if constexpr (M >= 4) {
+        return crot<SGN>(rot16<SGN, M - 4>(a));
+    } else if constexpr (M == 0) {
+        return a;
+    } else if constexpr (M == 2) {
+        const float2 b = crot<SGN>(a);
+        return make_float2((a.x + b.x) * H, (a.y + b.y) * H);
+    } else {
+        return cmul(a, make_float2(M == 1 ? C : S, SGN * (M == 1 ? S : C)));
     }
-    v[6] = csub(e2, o2);
-    v[7] = csub(e3, o3);
 }
+
+// Transforms of 8 and 16 elements in place, as 2 x 4 and 4 x 4.
 template <int SGN, bool PIN, bool POUT>
-__device__ __forceinline__ void dft8(float2 (&v)[8])
+__device__ __forceinline__ void dft8(float2& v0, float2& v1, float2& v2, float2& v3, float2& v4, float2& v5,
+                                     float2& v6, float2& v7)
 {
     if (PIN) {
-        dft4_outer<SGN>(v[0], v[2], v[4], v[6]);
-        dft4_outer<SGN>(v[1], v[3], v[5], v[7]);
+        dft4_outer<SGN>(v0, v2, v4, v6);
+        dft4_outer<SGN>(v1, v3, v5, v7);
     } else {
-        dft4<SGN>(v[0], v[2], v[4], v[6]);    // even inputs: e0..e3 in v0, v2, v4, v6
-        dft4<SGN>(v[1], v[3], v[5], v[7]);    // odd inputs
+        dft4<SGN>(v0, v2, v4, v6);            // even inputs: e0..e3 in v0, v2, v4, v6
+        dft4<SGN>(v1, v3, v5, v7);            // odd inputs
     }
-    dft8_join<SGN, POUT>(v);
+    const float2 o0 = v1, o1 = rot16<SGN, 2>(v3), o2 = rot16<SGN, 4>(v5), o3 = rot16<SGN, 6>(v7);
+    const float2 e0 = v0, e1 = v2, e2 = v4, e3 = v6;
+    v0 = cadd(e0, o0);
+    v1 = cadd(e1, o1);
+    if (!POUT) {
+        v2 = cadd(e2, o2);
+        v3 = cadd(e3, o3);
+        v4 = csub(e0, o0);
+        v5 = csub(e1, o1);
+    }
+    v6 = csub(e2, o2);
+    v7 = csub(e3, o3);
+}
+// One second-stage transform of dft16: outputs K, K + 4, K + 8, K + 12.
+template <int SGN, int K, bool POUT>
+__device__ __forceinline__ void dft16_tail(const float2 (&t)[16], float2 (&v)[16])
+{
+    const float2 a0 = t[4 * K], a1 = rot16<SGN, K>(t[4 * K + 1]), a2 = rot16<SGN, 2 * K>(t[4 * K + 2]),
+                 a3 = rot16<SGN, 3 * K>(t[4 * K + 3]);
+    const float2 s0 = cadd(a0, a2), s1 = csub(a0, a2), s2 = cadd(a1, a3), s3 = crot<SGN>(csub(a1, a3));
+    v[K] = cadd(s0, s2);
+    if (!POUT) {
+        v[K + 4] = cadd(s1, s3);
+        v[K + 8] = csub(s0, s2);
+    }
+    v[K + 12] = csub(s1, s3);
+}
+template <int SGN, bool PIN, bool POUT>
+__device__ __forceinline__ void dft16(float2 (&v)[16])
+{
+    float2 t[16];                             // t[4 k + a]: output k of the transform of v[a], v[a + 4], ..
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+        float2 x0 = v[a], x1 = v[a + 4], x2 = v[a + 8], x3 = v[a + 12];
+        if (PIN) dft4_outer<SGN>(x0, x1, x2, x3);
+        else dft4<SGN>(x0, x1, x2, x3);
+        t[a] = x0;
+        t[4 + a] = x1;
+        t[8 + a] = x2;
+        t[12 + a] = x3;
+    }
+    dft16_tail<SGN, 0, POUT>(t, v);
+    dft16_tail<SGN, 1, POUT>(t, v);
+    dft16_tail<SGN, 2, POUT>(t, v);
+    dft16_tail<SGN, 3, POUT>(t, v);
+}
+
+template <int SGN, bool PIN, bool POUT>
+__device__ __forceinline__ void dft_all(float2 (&v)[16])
+{
+    dft16<SGN, PIN, POUT>(v);
+}
+template <int SGN, bool PIN, bool POUT>
+__device__ __forceinline__ void dft_all(float2 (&v)[8])
+{
+    dft8<SGN, PIN, POUT>(v[0], v[1], v[2], v[3], v[4], v[5], v[6], v[7]);
 }
 
 // Shared-memory place of element i = e CB + c (element e of transform c of CB
 // interleaved ones): its low four bits (the 16 float2 that one wavefront of
-// shared memory holds) are XORed with bits of its next three, chosen so that the
-// 16 lanes of a half warp hit 16 different places in every access pattern of
-// the passes below: strides of 1, 2, 4 and 8 elements, and runs of 2, 4 or 8
-// elements 16, 32 or 64 apart.  (A pad of one element per 8 instead cost the
-// unit-stride reads a second wavefront: the rows kernel kept L1 82% busy.)  The
-// map is linear over GF(2): place(e | d) = place(e) ^ place(d) for e and d
-// without common bits, and d is always a constant.
+// shared memory holds) are XORed with its next four, or with sums of them, so
+// that the 16 lanes of a half warp hit 16 different places in every access
+// pattern of the passes below: unit stride, strides of 2, 4, 8 and 16 elements,
+// and runs of 2, 4 or 8 elements 32, 64 or 128 (radix 8: 64) apart.  (A pad of one element
+// per 8 instead cost the unit-stride reads a second wavefront.)  The map is
+// linear over GF(2): place(e | d) = place(e) ^ place(d) for e and d without
+// common bits, and d is always a constant.
 template <int CB>
 __host__ __device__ __forceinline__ constexpr int place(int i)
 {
-    const int r0 = (i >> 4) & 1, r1 = (i >> 5) & 1, r2 = (i >> 6) & 1;
-    return i ^ (CB == 1   ? (r0 | (r0 ^ r1) << 1 | r2 << 2 | (r1 ^ r2) << 3)
-                : CB == 4 ? (r1 << 2 | (r0 ^ r2) << 3)
-                          : (r0 ^ r1 ^ r2) << 3);
+    return i ^ (CB == 1   ? ((i >> 4) ^ ((i >> 3) & 8)) & 15
+                : CB == 4 ? ((i >> 4) ^ (i >> 6)) << 2 & 12
+                          : ((i >> 4) ^ (i >> 5) ^ (i >> 6) ^ (i >> 7)) << 3 & 8);
 }
 template <int CB>
 __device__ __forceinline__ float2& elem(float2* sm, int at, int d)     // at = place(e CB + c)
@@ -136,53 +192,74 @@ __device__ __forceinline__ float2& elem(float2* sm, int at, int d)     // at = p
     return sm[(at ^ (pd & 15)) + (pd & ~15)];
 }
 
-// Transform of length 2^LOG, radix 8 after a first pass of radix 2, 4 or 8
-// (Stockham order: no bit reversal).  A thread holds NB groups of 8 elements:
-// on entry and on exit v[n][q] is element g[n] + q 2^LOG/8 of its transform.
-// Every thread of the CTA calls it; sm holds the CTA's CB interleaved
-// transforms, c is this thread's.  PP: sm is two buffers of PP elements used in
-// turn (one barrier per exchange instead of two); sm is left at the next one to
-// write.  PIN: half-zero input, POUT: only the cells are wanted (above).
-// Twiddles: per pass of stride ns, e^{-2 pi i k/(8 ns)} and its 2nd and 4th
-// powers for k < ns, rounded from FP64; the other powers are products of two.
+template <int LOG>
+struct FftShape {
+    static constexpr int P = grid_radix(LOG), R0 = grid_radix0(LOG);
+};
+
+// Transform of length 2^LOG, radix P = 8 or 16 (grid_radix) after a first pass
+// of radix 2, 4, 8 or 16 (Stockham order: no bit reversal).  A thread holds NB
+// groups of P elements: on entry and on exit vs[n][q] is element gs[n] + q 2^LOG/P
+// of its transform.  Every thread of the CTA calls it; sm holds the CTA's CB
+// interleaved transforms, c is this thread's.  PP: sm is two buffers of PP
+// elements used in turn (one barrier per exchange instead of two); sm is left at
+// the next one to write.  Twiddles: per pass of stride ns, e^{-2 pi i k/(P ns)}
+// and its 2nd, 4th (and 8th) powers for k < ns, rounded from FP64; the others are
+// products of these.
+//
+// The transforms are bound by their exchanges (issue slots and barriers of passes
+// that each move every element through shared memory and back; the memory they
+// stream is a third of the time), so the radix is the one with fewer of them:
+// 2^11 takes 2 with radix 16 and 3 with radix 8.  Radix 16 against 8 at the same
+// threads' load, 55 planes of 2048^2: forward 1.017 -> 0.985 ms, adjoint 1.203 ->
+// 1.129 ms, and a 31-operator solve of 15 planes 10.4 -> 9.8 ms.  2^6 and 2^9 take
+// as many with radix 8 and are faster with it: 273 planes of 512^2 forward 0.25
+// against 0.28 ms, adjoint 0.31 against 0.33 ms.  Also slower: two planes or two
+// columns to a thread as float4 (twice the registers, half the warps: 1.18 -> 1.41
+// ms), and leaving out the forward's writes of columns nobody reads (a test per
+// element; 1.02 against 0.985 ms, although a third less is written).
 template <int LOG, int SGN, int CB, int NB, bool PIN, bool POUT, int PP>
-__device__ __forceinline__ void fft_pass_all(float2 (&v)[NB][8], const int (&g)[NB], int c, float2*& sm, int& par,
-                                             const float2* __restrict__ tw)
+__device__ __forceinline__ void fft_pass_all(float2 (&vs)[NB][FftShape<LOG>::P], const int (&gs)[NB], int c,
+                                             float2*& sm, int& par, const float2* __restrict__ tw)
 {
-    constexpr int L = 1 << LOG, E = L / 8;
-    constexpr int R0 = LOG % 3 == 0 ? 8 : LOG % 3 == 1 ? 2 : 4;
+    constexpr int P = FftShape<LOG>::P, R0 = FftShape<LOG>::R0, L = 1 << LOG, E = L / P;
 #pragma unroll
     for (int n = 0; n < NB; ++n) {
-        const int at = place<CB>(g[n] * R0 * CB + c);
-        if (R0 == 8) {
-            dft8<SGN, PIN, false>(v[n]);
+        float2 (&v)[P] = vs[n];
+        if constexpr (R0 == P) {
+            dft_all<SGN, PIN, false>(v);
+        } else if constexpr (R0 == 8) {
 #pragma unroll
-            for (int r = 0; r < 8; ++r) elem<CB>(sm, at, r) = v[n][r];
-        } else if (R0 == 4) {
+            for (int i = 0; i < 2; ++i)
+                dft8<SGN, PIN, false>(v[i], v[i + 2], v[i + 4], v[i + 6], v[i + 8], v[i + 10], v[i + 12], v[i + 14]);
+        } else if constexpr (R0 == 4) {
 #pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                if (PIN) dft4_outer<SGN>(v[n][i], v[n][i + 2], v[n][i + 4], v[n][i + 6]);
-                else dft4<SGN>(v[n][i], v[n][i + 2], v[n][i + 4], v[n][i + 6]);
-#pragma unroll
-                for (int r = 0; r < 4; ++r) elem<CB>(sm, at, i * E * 4 + r) = v[n][i + 2 * r];
+            for (int i = 0; i < 4; ++i) {
+                if (PIN) dft4_outer<SGN>(v[i], v[i + 4], v[i + 8], v[i + 12]);
+                else dft4<SGN>(v[i], v[i + 4], v[i + 8], v[i + 12]);
             }
         } else {
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const float2 a = v[n][i], b = v[n][i + 4];
-                elem<CB>(sm, at, i * E * 2) = !PIN ? cadd(a, b) : i < 2 ? a : b;
-                elem<CB>(sm, at, i * E * 2 + 1) = !PIN ? csub(a, b) : i < 2 ? a : make_float2(-b.x, -b.y);
+            for (int i = 0; i < 8; ++i) {
+                const float2 a = v[i], b = v[i + 8];
+                v[i] = !PIN ? cadd(a, b) : i < 4 ? a : b;
+                v[i + 8] = !PIN ? csub(a, b) : i < 4 ? a : make_float2(-b.x, -b.y);
             }
         }
+        const int at = place<CB>(gs[n] * R0 * CB + c);        // output r of the i-th transform is v[i + r P/R0]
+#pragma unroll
+        for (int i = 0; i < P / R0; ++i)
+#pragma unroll
+            for (int r = 0; r < R0; ++r) elem<CB>(sm, at, i * E * R0 + r) = v[i + r * (P / R0)];
     }
 #pragma unroll
-    for (int ns = R0; ns < L; ns *= 8) {
+    for (int ns = R0; ns < L; ns *= P) {
         __syncthreads();
 #pragma unroll
         for (int n = 0; n < NB; ++n) {
-            const int at = place<CB>(g[n] * CB + c);
+            const int at = place<CB>(gs[n] * CB + c);
 #pragma unroll
-            for (int r = 0; r < 8; ++r) v[n][r] = elem<CB>(sm, at, r * E);
+            for (int r = 0; r < P; ++r) vs[n][r] = elem<CB>(sm, at, r * E);
         }
         if (PP) {
             sm += par ? -PP : PP;
@@ -192,7 +269,8 @@ __device__ __forceinline__ void fft_pass_all(float2 (&v)[NB][8], const int (&g)[
         }
 #pragma unroll
         for (int n = 0; n < NB; ++n) {
-            const int k = g[n] & (ns - 1);
+            float2 (&v)[P] = vs[n];
+            const int k = gs[n] & (ns - 1);
             float2 w1 = __ldg(tw + k), w2 = __ldg(tw + ns + k), w4 = __ldg(tw + 2 * ns + k);
             if (SGN > 0) {
                 w1.y = -w1.y;
@@ -200,28 +278,45 @@ __device__ __forceinline__ void fft_pass_all(float2 (&v)[NB][8], const int (&g)[
                 w4.y = -w4.y;
             }
             const float2 w3 = cmul(w1, w2);
-            v[n][1] = cmul(v[n][1], w1);
-            v[n][2] = cmul(v[n][2], w2);
-            v[n][3] = cmul(v[n][3], w3);
-            v[n][4] = cmul(v[n][4], w4);
-            v[n][5] = cmul(v[n][5], cmul(w1, w4));
-            v[n][6] = cmul(v[n][6], cmul(w2, w4));
-            v[n][7] = cmul(v[n][7], cmul(w3, w4));
-            if (ns * 8 < L) {
-                dft8<SGN, false, false>(v[n]);
-                const int at = place<CB>(((g[n] - k) * 8 + k) * CB + c);
+            if constexpr (P == 16) {
+                float2 w8 = __ldg(tw + 3 * ns + k);
+                if (SGN > 0) w8.y = -w8.y;
+                const float2 w12 = cmul(w8, w4);
+                v[8] = cmul(v[8], w8);
+                v[9] = cmul(v[9], cmul(w8, w1));
+                v[10] = cmul(v[10], cmul(w8, w2));
+                v[11] = cmul(v[11], cmul(w8, w3));
+                v[12] = cmul(v[12], w12);
+                v[13] = cmul(v[13], cmul(w12, w1));
+                v[14] = cmul(v[14], cmul(w12, w2));
+                v[15] = cmul(v[15], cmul(w12, w3));
+            }
+            v[1] = cmul(v[1], w1);
+            v[2] = cmul(v[2], w2);
+            v[3] = cmul(v[3], w3);
+            v[4] = cmul(v[4], w4);
+            v[5] = cmul(v[5], cmul(w4, w1));
+            v[6] = cmul(v[6], cmul(w4, w2));
+            v[7] = cmul(v[7], cmul(w4, w3));
+            if (ns * P < L) {
+                dft_all<SGN, false, false>(v);
+                const int at = place<CB>(((gs[n] - k) * P + k) * CB + c);
 #pragma unroll
-                for (int r = 0; r < 8; ++r) elem<CB>(sm, at, r * ns) = v[n][r];
+                for (int r = 0; r < P; ++r) elem<CB>(sm, at, r * ns) = v[r];
             } else {
-                dft8<SGN, false, POUT>(v[n]);
+                dft_all<SGN, false, POUT>(v);
             }
         }
-        tw += 3 * ns;
+        tw += (P == 16 ? 4 : 3) * ns;
     }
 }
 
-// The elements q of a thread's 8 that are cells.
-__device__ __forceinline__ constexpr int cell_q(int i) { return i < 2 ? i : i + 4; }
+// The elements q of a thread's P that are cells.
+template <int P>
+__device__ __forceinline__ constexpr int cell_q(int i)
+{
+    return i < P / 4 ? i : i + P / 2;
+}
 
 // Cell index of element e (0 <= e < 2^lg) of a zero-padded axis whose cell c0
 // sits at element 0; outside [0, n) where the padding is.
@@ -241,8 +336,11 @@ __device__ __forceinline__ float2 plane_phase(float2 w, float2 nu)
 
 template <int LOG>
 struct RowShape {
-    static constexpr int T = (1 << LOG) / 8;                  // threads per row
-    static constexpr int ROWS = T >= 256 ? 1 : 256 / T;       // rows per CTA
+    static constexpr int P = grid_radix(LOG);                 // elements per thread
+    static constexpr int T = (1 << LOG) / P;                  // threads per row
+    static constexpr int WIDE = P == 16 ? 128 : 256;
+    static constexpr int ROWS = T >= WIDE ? 1 : WIDE / T;     // rows per CTA
+    static constexpr int CTAS = LOG == 12 ? 2 : P == 16 ? 5 : 3;
     static constexpr int THREADS = T * ROWS;
     static constexpr int BUF = ROWS << LOG;                   // shared elements of one buffer
     static constexpr int SMEM = 2 * BUF * (int)sizeof(float2);
@@ -252,7 +350,7 @@ struct RowShape {
 // A CTA takes ROWS lattice rows of GR_PCH planes: x, amp and nu are read once
 // for them.
 template <int LOG>
-__global__ void __launch_bounds__(RowShape<LOG>::THREADS, LOG < 12 ? 3 : 1)
+__global__ void __launch_bounds__(RowShape<LOG>::THREADS, RowShape<LOG>::CTAS)
 grid_rows_fwd_kernel(const DevProblem* __restrict__ probs, int prob, const GridOp g, int p0, int np)
 {
     using S = RowShape<LOG>;
@@ -263,11 +361,11 @@ grid_rows_fwd_kernel(const DevProblem* __restrict__ probs, int prob, const GridO
     const int rb = threadIdx.x / S::T;
     const int gi[1] = {(int)threadIdx.x % S::T};
     const int iy = blockIdx.x * S::ROWS + rb;
-    float a[4];
-    float2 nu[4];
+    float a[S::P / 2];
+    float2 nu[S::P / 2];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int ix = cell_of(gi[0] + cell_q(i) * S::T, LOG, g.cx);
+    for (int i = 0; i < S::P / 2; ++i) {
+        const int ix = cell_of(gi[0] + cell_q<S::P>(i) * S::T, LOG, g.cx);
         a[i] = 0.f;
         nu[i] = make_float2(0.f, 0.f);
         if (iy < g.ny && ix >= 0 && ix < g.nx) {
@@ -284,17 +382,17 @@ grid_rows_fwd_kernel(const DevProblem* __restrict__ probs, int prob, const GridO
     const int q1 = min(np, (int)(blockIdx.y + 1) * GR_PCH);
     for (int p = blockIdx.y * GR_PCH; p < q1; ++p) {
         const float2 w = g.wp[p0 + p];
-        float2 v[1][8];
+        float2 v[1][S::P];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
+        for (int i = 0; i < S::P / 2; ++i) {
             const float2 e = plane_phase(w, nu[i]);
-            v[0][cell_q(i)] = make_float2(a[i] * e.x, a[i] * e.y);
+            v[0][cell_q<S::P>(i)] = make_float2(a[i] * e.x, a[i] * e.y);
         }
         fft_pass_all<LOG, -1, 1, 1, true, false, S::BUF>(v, gi, 0, smr, par, g.twx);
         if (iy < g.ny) {
             float2* dst = g.g1 + ((size_t)p * g.ny + iy) * L;
 #pragma unroll
-            for (int q = 0; q < 8; ++q) dst[gi[0] + q * S::T] = v[0][q];
+            for (int q = 0; q < S::P; ++q) dst[gi[0] + q * S::T] = v[0][q];
         }
     }
 }
@@ -302,7 +400,7 @@ grid_rows_fwd_kernel(const DevProblem* __restrict__ probs, int prob, const GridO
 // Adjoint, rows: g1 transformed back along x; Re(exp(+2 pi i w_p nu) z) summed
 // over the CTA's planes (FP32 over GR_PCH planes) into the chunk's partial slots.
 template <int LOG>
-__global__ void __launch_bounds__(RowShape<LOG>::THREADS, LOG < 12 ? 3 : 1)
+__global__ void __launch_bounds__(RowShape<LOG>::THREADS, RowShape<LOG>::CTAS)
 grid_rows_adj_kernel(const DevProblem* __restrict__ probs, int prob, const GridOp g, int p0, int np, int chunk0,
                      int n_pix, int n_pix_pad, double* __restrict__ partial)
 {
@@ -314,11 +412,11 @@ grid_rows_adj_kernel(const DevProblem* __restrict__ probs, int prob, const GridO
     const int rb = threadIdx.x / S::T;
     const int gi[1] = {(int)threadIdx.x % S::T};
     const int iy = blockIdx.x * S::ROWS + rb;
-    float acc[4];
-    float2 nu[4];
+    float acc[S::P / 2];
+    float2 nu[S::P / 2];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int ix = cell_of(gi[0] + cell_q(i) * S::T, LOG, g.cx);
+    for (int i = 0; i < S::P / 2; ++i) {
+        const int ix = cell_of(gi[0] + cell_q<S::P>(i) * S::T, LOG, g.cx);
         acc[i] = 0.f;
         nu[i] = (iy < g.ny && ix >= 0 && ix < g.nx) ? g.nu[(size_t)iy * g.nx + ix] : make_float2(0.f, 0.f);
     }
@@ -327,26 +425,26 @@ grid_rows_adj_kernel(const DevProblem* __restrict__ probs, int prob, const GridO
     const int q1 = min(np, (int)(blockIdx.y + 1) * GR_PCH);
     for (int p = blockIdx.y * GR_PCH; p < q1; ++p) {
         const float2 w = g.wp[p0 + p];
-        float2 v[1][8];
+        float2 v[1][S::P];
         const float2* src = g.g1 + ((size_t)p * g.ny + min(iy, g.ny - 1)) * L;
         const unsigned char* act = g.colact + (size_t)(p0 + p) * (L / GR_TILE);
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {          // columns without a visibility were not written
+        for (int q = 0; q < S::P; ++q) {          // columns without a visibility were not written
             const int e = gi[0] + q * S::T;
             v[0][q] = act[e / GR_TILE] ? src[e] : make_float2(0.f, 0.f);
         }
         fft_pass_all<LOG, 1, 1, 1, false, true, S::BUF>(v, gi, 0, smr, par, g.twx);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
+        for (int i = 0; i < S::P / 2; ++i) {
             const float2 e = plane_phase(w, nu[i]);                  // conj(e) z, real part
-            acc[i] += fmaf(e.x, v[0][cell_q(i)].x, e.y * v[0][cell_q(i)].y);
+            acc[i] += fmaf(e.x, v[0][cell_q<S::P>(i)].x, e.y * v[0][cell_q<S::P>(i)].y);
         }
     }
     const int chunk = chunk0 + blockIdx.y;
     if (iy < g.ny) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int ix = cell_of(gi[0] + cell_q(i) * S::T, LOG, g.cx);
+        for (int i = 0; i < S::P / 2; ++i) {
+            const int ix = cell_of(gi[0] + cell_q<S::P>(i) * S::T, LOG, g.cx);
             if (ix < 0 || ix >= g.nx) continue;
             const size_t at = (size_t)iy * g.nx + ix;
             const int j = g.cell[at];
@@ -366,9 +464,10 @@ grid_rows_adj_kernel(const DevProblem* __restrict__ probs, int prob, const GridO
 // into g1.
 template <int LOG>
 struct ColShape {
+    static constexpr int P = grid_radix(LOG);
     static constexpr int CB = LOG >= 11 ? 4 : 8;
-    static constexpr int NB = LOG >= 12 ? 4 : LOG >= 8 ? 2 : 1;
-    static constexpr int THREADS = CB * (1 << LOG) / 8 / NB;
+    static constexpr int NB = 16 / P;                         // 16 elements per thread
+    static constexpr int THREADS = CB * (1 << LOG) / 16;
     static constexpr int SMEM = CB * (1 << LOG) * (int)sizeof(float2);
 };
 template <int LOG, int SGN>
@@ -376,7 +475,7 @@ __global__ void __launch_bounds__(ColShape<LOG>::THREADS, ColShape<LOG>::THREADS
 grid_cols_kernel(const DevProblem* __restrict__ probs, int prob, const GridOp g, int p0)
 {
     using S = ColShape<LOG>;
-    constexpr int E = (1 << LOG) / 8;
+    constexpr int P = S::P, E = (1 << LOG) / P;
     extern __shared__ __align__(16) float2 sm_cols[];
     __shared__ unsigned char s_act[(1 << LOG) / GR_TILE];      // tiles of these columns with a visibility
     if (SGN < 0) {
@@ -401,34 +500,32 @@ grid_cols_kernel(const DevProblem* __restrict__ probs, int prob, const GridOp g,
     const size_t col = (size_t)blockIdx.x * S::CB + c, Lx = (size_t)1 << g.lx;
     float2* g1 = g.g1 + (size_t)blockIdx.y * g.ny * Lx + col;
     float2* g2 = g.g2 + ((size_t)blockIdx.y << LOG) * Lx + col;
-    float2 v[S::NB][8];
+    float2 v[S::NB][P];
 #pragma unroll
-    for (int n = 0; n < S::NB; ++n)
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const int e = gi[n] + q * E;
-            if (SGN > 0) {
-                v[n][q] = s_act[e / GR_TILE] ? g2[(size_t)e * Lx] : make_float2(0.f, 0.f);
-            } else if (q < 2 || q > 5) {
-                const int iy = cell_of(e, LOG, g.cy);
-                v[n][q] = (iy >= 0 && iy < g.ny) ? g1[(size_t)iy * Lx] : make_float2(0.f, 0.f);
-            }
+    for (int i = 0; i < 16; ++i) {
+        const int n = i / P, q = i % P;
+        const int e = gi[n] + q * E;
+        if (SGN > 0) {
+            v[n][q] = s_act[e / GR_TILE] ? g2[(size_t)e * Lx] : make_float2(0.f, 0.f);
+        } else if (q < P / 4 || q >= 3 * P / 4) {
+            const int iy = cell_of(e, LOG, g.cy);
+            v[n][q] = (iy >= 0 && iy < g.ny) ? g1[(size_t)iy * Lx] : make_float2(0.f, 0.f);
         }
+    }
     float2* sm = sm_cols;
     int par = 0;
     fft_pass_all<LOG, SGN, S::CB, S::NB, (SGN < 0), (SGN > 0), 0>(v, gi, c, sm, par, g.twy);
 #pragma unroll
-    for (int n = 0; n < S::NB; ++n)
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const int e = gi[n] + q * E;
-            if (SGN < 0) {
-                if (s_act[e / GR_TILE]) g2[(size_t)e * Lx] = v[n][q];
-            } else if (q < 2 || q > 5) {
-                const int iy = cell_of(e, LOG, g.cy);
-                if (iy >= 0 && iy < g.ny) g1[(size_t)iy * Lx] = v[n][q];
-            }
+    for (int i = 0; i < 16; ++i) {
+        const int n = i / P, q = i % P;
+        const int e = gi[n] + q * E;
+        if (SGN < 0) {
+            if (s_act[e / GR_TILE]) g2[(size_t)e * Lx] = v[n][q];
+        } else if (q < P / 4 || q >= 3 * P / 4) {
+            const int iy = cell_of(e, LOG, g.cy);
+            if (iy >= 0 && iy < g.ny) g1[(size_t)iy * Lx] = v[n][q];
         }
+    }
 }
 
 // ------------------------------------------------- gathering and spreading

@@ -44,11 +44,16 @@ struct GridOp {
 
 inline size_t grid_plane_elems(const GridOp& g) { return ((size_t)g.ny + ((size_t)1 << g.ly)) << g.lx; }
 inline int grid_tiles(const GridOp& g) { return ((1 << g.lx) / GR_TILE) * ((1 << g.ly) / GR_TILE); }
-// float2 entries of the twiddle table of a transform of length 2^lg.
+// Radix of a transform of length 2^lg, and of its first pass: 16 where that saves
+// an exchange over radix 8.
+constexpr int grid_radix(int lg) { return lg == 6 || lg == 9 ? 8 : 16; }
+constexpr int grid_radix0(int lg) { return grid_radix(lg) == 8 ? 8 : lg % 4 ? 1 << (lg % 4) : 16; }
+// float2 entries of its twiddle table.
 inline int grid_tw_elems(int lg)
 {
+    const int radix = grid_radix(lg);
     int n = 0;
-    for (int ns = 1 << (lg % 3 ? lg % 3 : 3); ns < (1 << lg); ns *= 8) n += 3 * ns;
+    for (int ns = grid_radix0(lg); ns < (1 << lg); ns *= radix) n += (radix == 16 ? 4 : 3) * ns;
     return n;
 }
 

@@ -104,10 +104,11 @@ std::vector<float2> twiddles(int lg)
 {
     std::vector<float2> t;
     t.reserve(grid_tw_elems(lg));
-    for (int ns = 1 << (lg % 3 ? lg % 3 : 3); ns < (1 << lg); ns *= 8)
-        for (int m = 1; m <= 4; m *= 2)
+    const int radix = grid_radix(lg);
+    for (int ns = grid_radix0(lg); ns < (1 << lg); ns *= radix)
+        for (int m = 1; m < radix; m *= 2)
             for (int k = 0; k < ns; ++k) {
-                const double a = 2.0 * M_PI * m * k / (8.0 * ns);
+                const double a = 2.0 * M_PI * m * k / ((double)radix * ns);
                 t.push_back(make_float2((float)std::cos(a), (float)-std::sin(a)));
             }
     return t;
@@ -119,9 +120,12 @@ std::vector<float2> twiddles(int lg)
 // both on GB300 over 64^2 .. 1024^2 pixels x 1,500 .. 100,000 visibilities, fields
 // of +/-0.02 .. +/-0.5 (us, forward / adjoint; pairs and then lattice):
 //   64^2 x 4,000      41 / 38       43 / 87       256^2 +/-0.5 x 5,000   275 / 266    191 / 292
-//   64^2 x 40,000    110 / 87       66 / 230      500^2 x 3,000          399 / 286     76 / 93
-//   128^2 x 5,000     69 / 58       45 / 60       1024^2 +/-0.3 x 3,000 1569 / 1096   482 / 669
-//   200^2 x 60,000  1181 / 843      96 / 127      1024^2 x 100,000     50011 / 34845  252 / 386
+//   64^2 x 40,000    110 / 87       66 / 230      500^2 x 3,000          427 / 293     75 / 94
+//   128^2 x 5,000     88 / 68       45 / 54       1024^2 +/-0.3 x 3,000 1609 / 1110   439 / 584
+//   200^2 x 60,000  1185 / 853      98 / 120      1024^2 +/-0.3 x 1,000  629 / 415    291 / 395
+// (the first column's first two rows and the second's first: lattice by an older
+// spreading; the rule takes the pairs there, and nowhere in this range is either
+// operator slower by the rule than the pairs).
 // Lattice: launches, the planes' cells, the visibilities, and the points that a
 // tile's CTA spreads one after the other where there are few tiles.  The lattice
 // is taken where it promises a tenth or more.

@@ -372,7 +372,7 @@ adj_finish_kernel(const DevProblem* __restrict__ probs, const Plan* __restrict__
         const int t = threadIdx.x % S::EL, e = e0 + t;
         const bool in = e < P.pix.n_pad;
         const int poff = pl.blk_poff[gb], ncon = in ? pl.blk_ncon[gb] : 0;
-        // the step's other loads are issued before the partial sums'
+        // the step's other loads are issued before the partial sums
         const int par = mode == FIN_SOLVE && !P.st->algo ? (P.st->k + 1) & 1 : 0;
         double y0 = 0.0, Io = 0.0;
         int orig = 0;
