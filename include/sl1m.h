@@ -140,8 +140,9 @@ int sl1m_adjoint_dev(sl1m_problem* prob, const double* r_dev, double* img_out_de
 
 /* Forward operator for callers that cannot allocate device memory at the time
  * of the call (device memory owned by a pool or another framework, or a loop
- * that must not enter the allocator).  Same result as sl1m_forward_dev; the
- * paper has no counterpart (this is plumbing, not a step of the method).
+ * that must not enter the allocator).  Same result as sl1m_forward_dev (to
+ * rounding on a lattice, below); the paper has no counterpart (this is
+ * plumbing, not a step of the method).
  *   - Allocates nothing: all of its scratch (descriptor, work-split tables,
  *     input in the library's pixel order, partial sums, output before
  *     reordering) lives in one static device array of 32 MiB that every GPU
@@ -153,6 +154,8 @@ int sl1m_adjoint_dev(sl1m_problem* prob, const double* r_dev, double* img_out_de
  *   - The first call on a device looks up the array's device address (once
  *     per device, with that device current); make that first call before any
  *     stream capture.
+ *   - Always evaluates pairs, also where sl1m_forward_dev would take the
+ *     lattice operator: there the two agree to rounding, not bit for bit.
  *   - All calls share the one array and each leaves its data there: calls
  *     whose work overlaps on the GPU (other streams, other contexts, other
  *     host threads) race and must be serialised by the caller.
@@ -307,7 +310,7 @@ int sl1m_server_info(sl1m_ctx* ctx, sl1m_server_info_t* info);
  * solve); with gains or in FP64 only the grid is tuned.  The choice is kept in the context,
  * keyed by (precision, operator, gains, Gaussian pixels, log2 of the work
  * units); later launches of problems with the same key -- single solves and
- * server batches -- use it.  nst_out, ctas_per_sm_out and npoly_out ([2]:
+ * server batches -- use it (the lattice operator has no tile shape).  nst_out, ctas_per_sm_out and npoly_out ([2]:
  * forward, adjoint) may be NULL.  Synchronous. */
 int sl1m_autotune(sl1m_problem* prob, int precision, int32_t* nst_out, int32_t* ctas_per_sm_out,
                   int32_t* npoly_out);
