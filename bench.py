@@ -287,20 +287,38 @@ def hbm_peak():
         return 6800.0, "of fallback"
 
 
-def lattice_bytes(w):
+def lattice_bytes(w, op="fwd"):
     """What one product of the lattice operator moves on workload w: planes in
     w of 2^lx x 2^ly complex FP32 cells (twice the lattice's sides and more),
     at Delta w = 1 / (4 B) for |n - 1 - nc| <= B over 0 .. max |w|, and 8 planes
-    for the kernel's width; the row pass writes ny rows, the column pass reads
-    them and writes 2^ly, gathering (spreading) reads (writes) those.  An upper
-    bound: tiles that no visibility touches are left out."""
+    for the kernel's width.  Forward: the row pass writes ny rows, the column
+    pass reads those of columns with a visibility and writes the 16 x 16 tiles
+    with one, gathering reads them.  Adjoint: the transpose, whose column pass
+    writes only columns with a visibility."""
     lm, r2 = w.lm, (w.lm ** 2).sum(axis=1)
     nm1 = -r2 / (1 + np.sqrt(1 - r2))
-    aw = np.abs(w.uvw[:, 2])
-    planes = math.ceil((aw.max() - aw.min()) * 2 * (nm1.max() - nm1.min())) + 8
-    n = [len(np.unique(np.round(lm[:, a], 12))) for a in (0, 1)]
-    lx, ly = (max(64, 1 << (2 * k - 1).bit_length()) for k in n)
-    return {"planes": planes, "cells": [lx, ly], "bytes": planes * lx * (2 * n[1] + 2 * ly) * 8}
+    uvw = w.uvw * np.where(w.uvw[:, 2] < 0, -1.0, 1.0)[:, None]      # w < 0: the mirrored point
+    per_w = 2 * (nm1.max() - nm1.min())                              # planes per wavelength
+    w0 = uvw[:, 2].min()
+    planes = math.ceil((uvw[:, 2].max() - w0) * per_w) + 8
+    first = np.clip(np.ceil((uvw[:, 2] - w0) * per_w - 0.5), 0, planes - 8).astype(np.int64)
+    n, side, tiles = [], [], []
+    for a in (0, 1):
+        c = np.unique(np.round(lm[:, a], 12))
+        n.append(len(c))
+        side.append(max(64, 1 << (2 * len(c) - 1).bit_length()))
+        t = uvw[:, a] * ((c[-1] - c[0]) / max(1, len(c) - 1))
+        i = np.ceil((t - np.floor(t)) * side[a] - 4).astype(np.int64)
+        tiles.append([(i % side[a]) // 16, ((i + 7) % side[a]) // 16])
+    act = np.zeros((planes, side[0] // 16, side[1] // 16), bool)     # a point whose first plane this is
+    for tx in tiles[0]:
+        for ty in tiles[1]:
+            act[first, tx, ty] = True
+    act = np.stack([act[max(0, p - 7):p + 1].any(axis=0) for p in range(planes)])
+    col_rows = n[1] * 16 * int(act.any(axis=2).sum())
+    rows = col_rows if op == "adj" else planes * n[1] * side[0]
+    return {"planes": planes, "cells": side, "tiles_with_a_visibility": float(act.mean()),
+            "bytes": 8 * (rows + col_rows + 2 * 256 * int(act.sum()))}
 
 
 def sfu_peak(w, op="fwd"):
@@ -786,13 +804,14 @@ def main():
     roofline["frac_of_measured_sfu"] = achieved / meas["peak"]
     if lattice:
         # bound by the planes' traffic: bytes of a product over its event time
-        by = lattice_bytes(w)
+        by = lattice_bytes(w, op_of(dom))
         hbm, src = hbm_peak()
         sec = pd["ms"] / 1e3 / worked[dom]
         roofline = {"bound": "hbm", "kernel": dom + " (lattice: rows, columns, gather / spread)",
                     "achieved": by["bytes"] / sec / 1e9, "peak": hbm, "unit": "GB/s",
                     "frac": by["bytes"] / sec / 1e9 / hbm, "peak_basis": src, "planes": by["planes"],
-                    "cells": by["cells"], "bytes_per_launch": by["bytes"], "launches": pd["launches"],
+                    "cells": by["cells"], "tiles_with_a_visibility": by["tiles_with_a_visibility"],
+                    "bytes_per_launch": by["bytes"], "launches": pd["launches"],
                     "launches_with_work": worked[dom], "avg_launch_ms": 1e3 * sec, "traffic": None}
     per_kernel = {}
     for k in keys:
