@@ -23,7 +23,7 @@
 // written nor read, and columns without such a tile are not transformed.
 //
 // The interpolation error is 1e-7 of the result's norm and the whole operator
-// in FP32 is 1.6e-7 to 2.4e-7 off FP64 (2-norm, listed sizes below and others),
+// in FP32 is 1.6e-7 to 2.8e-7 off FP64 (2-norm, sizes below and others),
 // where evaluating every pair with the SFU's sine and cosine (sl1m_mixed.cu) is
 // 3.6e-7 to 4.9e-7 off.  The work no longer grows with N_v N_p but with the
 // planes' cells: per plane the kernels move up to (3 2^ly + 2 ny) 2^lx complex
@@ -890,14 +890,13 @@ static cudaError_t raise_limits()
     return cudaFuncSetAttribute(grid_rows_adj_kernel<LOG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 RowShape<LOG>::SMEM);
 }
-cudaError_t grid_prepare_kernels()
+cudaError_t grid_prepare_kernels(int lx, int ly)
 {
-    for (int lg = GR_LOG_MIN; lg <= GR_LOG_MAX; ++lg) {
-        cudaError_t e = cudaSuccess;
-        GRID_DISPATCH(lg, (e = raise_limits<LOG>()));
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
+    cudaError_t e = cudaSuccess;
+    GRID_DISPATCH(lx, (e = raise_limits<LOG>()));
+    if (e != cudaSuccess || lx == ly) return e;
+    GRID_DISPATCH(ly, (e = raise_limits<LOG>()));
+    return e;
 }
 
 }  // namespace sl1m

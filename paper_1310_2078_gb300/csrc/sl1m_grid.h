@@ -71,6 +71,7 @@ cudaError_t grid_forward(const DevProblem* probs, int p, const GridOp& g, int n_
                          cudaStream_t st, long long* n_launch);
 cudaError_t grid_adjoint(const DevProblem* probs, int p, const GridOp& g, int n_pix, int n_pix_pad, double* partial,
                          cudaStream_t st, long long* n_launch);
-cudaError_t grid_prepare_kernels();   // raises the dynamic shared-memory limits (not under capture)
+// raises the dynamic shared-memory limits of the transforms of these lengths (not under capture)
+cudaError_t grid_prepare_kernels(int lx, int ly);
 
 }  // namespace sl1m

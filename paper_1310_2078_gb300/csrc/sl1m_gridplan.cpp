@@ -123,9 +123,8 @@ std::vector<float2> twiddles(int lg)
 //   64^2 x 40,000    110 / 87       66 / 230      500^2 x 3,000          427 / 293     75 / 94
 //   128^2 x 5,000     88 / 68       45 / 54       1024^2 +/-0.3 x 3,000 1609 / 1110   439 / 584
 //   200^2 x 60,000  1185 / 853      98 / 120      1024^2 +/-0.3 x 1,000  629 / 415    291 / 395
-// (the first column's first two rows and the second's first: lattice by an older
-// spreading; the rule takes the pairs there, and nowhere in this range is either
-// operator slower by the rule than the pairs).
+// (64^2 and 256^2 +/-0.5: the rule takes the pairs; lattice measured with a slower
+// spreading kernel.)
 // Lattice: launches, the planes' cells, the visibilities, and the points that a
 // tile's CTA spreads one after the other where there are few tiles.  The lattice
 // is taken where it promises a tenth or more.
@@ -279,13 +278,14 @@ bool grid_build(sl1m_problem& P, cudaStream_t st, size_t budget)
         const int tyn = (1 << g.ly) / GR_TILE;
         std::vector<unsigned char> act((size_t)g.np * tiles, 0), colact((size_t)g.np * txn, 0);
         for (int t = 0; t < tiles; ++t)
-            for (int i = 0; i < ni; ++i) {
+            for (int i = 0, done = 0; i < ni; ++i) {     // planes below `done` are marked
                 const size_t at = (size_t)t * (ni + 1) + i;
                 if (start[at] == start[at + 1]) continue;
-                for (int p = i; p < i + GRW; ++p) {
+                for (int p = std::max(i, done); p < i + GRW; ++p) {
                     act[((size_t)p * txn + t % txn) * tyn + t / txn] = 1;
                     colact[(size_t)p * txn + t % txn] = 1;
                 }
+                done = i + GRW;
             }
         ok = T->start.upload(start.data(), start.size(), st) == cudaSuccess &&
              T->list.upload(list.data(), list.size(), st) == cudaSuccess &&
@@ -310,7 +310,7 @@ bool grid_build(sl1m_problem& P, cudaStream_t st, size_t budget)
     static std::mutex mu;
     {
         std::lock_guard<std::mutex> lk(mu);
-        if (grid_prepare_kernels() != cudaSuccess) {
+        if (grid_prepare_kernels(g.lx, g.ly) != cudaSuccess) {
             cudaGetLastError();
             return false;
         }

@@ -185,17 +185,32 @@ static void sort_baselines(std::vector<int>& order, const std::vector<int>& ant)
         });
 }
 
+// The visibilities sorted by antenna pair, each pair's in the caller's order: two
+// stable counting sorts (comparison sorts of the keys, one for every run length
+// tried, were most of the time that trying the orders took).
+static std::vector<int> sort_by_pair(const std::vector<int32_t>& ant, int n_ant, size_t n)
+{
+    std::vector<int> by(n), next(n);
+    for (size_t k = 0; k < n; ++k) next[k] = (int)k;
+    for (int a = 1; a >= 0; --a) {
+        std::vector<size_t> at((size_t)n_ant + 1, 0);
+        for (size_t k = 0; k < n; ++k) ++at[ant[2 * k + a] + 1];
+        for (int i = 0; i < n_ant; ++i) at[i + 1] += at[i];
+        for (int k : next) by[at[ant[2 * (size_t)k + a]]++] = k;
+        by.swap(next);
+    }
+    return next;
+}
+
 // With gains: an order of the visibilities in which a granule holds few antenna
 // pairs.  Every pair's visibilities are cut, in the caller's order (time, as a
 // rule), into runs of s; granules are 64 / s runs that are neighbours in (u, v)
 // (k-d order of the runs' centres).  What is left over of each pair follows in
-// point order.  keys: the pair of every visibility.
-static std::vector<int> order_by_runs(const std::vector<long long>& keys, const double* uvw, int s)
+// point order.  keys: the pair of every visibility; by: the visibilities sorted by it.
+static std::vector<int> order_by_runs(const std::vector<long long>& keys, const std::vector<int>& by, const double* uvw,
+                                      int s)
 {
     const size_t n = keys.size();
-    std::vector<int> by(n);
-    for (size_t k = 0; k < n; ++k) by[k] = (int)k;
-    std::stable_sort(by.begin(), by.end(), [&](int a, int b) { return keys[a] < keys[b]; });
     std::vector<int> first, rest;               // first member of every run, in `by`
     std::vector<double> centre;                 // (u, v) of every run
     for (size_t i = 0, j; i < n; i = j) {
@@ -760,23 +775,34 @@ int sl1m_problem::rebuild(cudaStream_t st, size_t grid_budget)
         std::vector<int> members(n_vis);
         for (int64_t k = 0; k < n_vis; ++k) members[k] = (int)k;
         std::vector<int> order;
-        kd_append(order, std::move(members), uvw.data(), uvw.data() + 1, 3);
-        if (n_ant > 0) {
+        if (n_ant == 0) {
+            kd_append(order, std::move(members), uvw.data(), uvw.data() + 1, 3);
+        } else {
             // the cheapest of the point order and of runs of 16, 8 and 4 samples
-            // of a pair (tried while the mean pair has that many)
-            std::vector<long long> keys(n_vis), distinct;
+            // of a pair (tried while the mean pair has that many), each made by a
+            // thread of its own
+            std::vector<long long> keys(n_vis);
             for (int64_t k = 0; k < n_vis; ++k) keys[k] = (long long)ant[2 * k] * n_ant + ant[2 * k + 1];
-            distinct = keys;
-            std::sort(distinct.begin(), distinct.end());
-            const double per = (double)n_vis / (double)(std::unique(distinct.begin(), distinct.end()) - distinct.begin());
+            const std::vector<int> by = sort_by_pair(ant, n_ant, n_vis);
+            int64_t distinct = 1;
+            for (int64_t k = 1; k < n_vis; ++k) distinct += keys[by[k]] != keys[by[k - 1]];
+            const double per = (double)n_vis / (double)distinct;
+            using Tried = std::pair<double, std::vector<int>>;
+            std::vector<std::future<Tried>> tried;
+            for (int s = 16; s >= 4; s /= 2)
+                if (per >= 0.75 * s)
+                    tried.push_back(std::async(std::launch::async, [&, s]() -> Tried {
+                        std::vector<int> o = order_by_runs(keys, by, uvw.data(), s);
+                        const double c = gains_order_cost(o, keys, uvw.data(), gext_pix);
+                        return {c, std::move(o)};
+                    }));
+            kd_append(order, std::move(members), uvw.data(), uvw.data() + 1, 3);
             double best = gains_order_cost(order, keys, uvw.data(), gext_pix);
-            for (int s = 16; s >= 4; s /= 2) {
-                if (per < 0.75 * s) continue;
-                std::vector<int> o = order_by_runs(keys, uvw.data(), s);
-                const double c = gains_order_cost(o, keys, uvw.data(), gext_pix);
-                if (c < best) {
-                    best = c;
-                    order.swap(o);
+            for (auto& f : tried) {
+                Tried t = f.get();
+                if (t.first < best) {
+                    best = t.first;
+                    order.swap(t.second);
                 }
             }
         }
@@ -1353,7 +1379,7 @@ static int enqueue_tick(sl1m_ctx* ctx, Batch& B)
     // Under capture the classes are branches of their own: their problems are
     // disjoint, and on small problems one class's finish kernels and tails leave
     // the GPU to the other (four 4096 x 6000 requests, two with gains: 238 ->
-    // 205 us a tick).
+    // 205 us a tick, now 198).
     const bool fork = ctx->use_graphs && !ctx->prof && B.has_class[0] + B.has_class[1] + B.has_class[2] > 1;
     int side = 0;
     bool own = true;                             // the first class stays on the stream
