@@ -4,6 +4,7 @@
 #include "sl1m.h"
 
 #include <algorithm>
+#include <atomic>
 #include <future>
 #include <thread>
 #include <chrono>
@@ -629,6 +630,11 @@ struct ProblemDev {
 
 sl1m_problem::~sl1m_problem() = default;
 
+// Layouts made in this process.  A batch knows its problems by address and by
+// the number of their layout, and a server's batch outlives them: a later
+// problem may have the address of a destroyed one, never its number.
+static std::atomic<uint64_t> g_layouts{0};
+
 int sl1m_problem::rebuild(cudaStream_t st, size_t grid_budget)
 {
     if (!dirty) return SL1M_OK;
@@ -919,7 +925,7 @@ int sl1m_problem::rebuild(cudaStream_t st, size_t grid_budget)
     for (auto& r : ucost_ok) r[0] = r[1] = false;
     solver_ready = false;
     dirty = false;
-    ++gen;
+    gen = ++g_layouts;
     if (grid_build(*this, st, grid_budget))
         ctx->h2d += (long long)(grid->cell.bytes() + grid->list.bytes() + grid->start.bytes());
     return SL1M_OK;

@@ -278,7 +278,7 @@ struct sl1m_problem {
     bool ucost_ok[2][2] = {{false, false}, {false, false}};
     std::unique_ptr<Batch> op_batch[2], solve_batch[2];
     std::unique_ptr<GridTables> grid;         // lattice operator of the mixed path, or null
-    uint64_t gen = 0;                         // counts the layouts
+    uint64_t gen = 0;                         // number of the layout: no two of a process share one
     const UnitCost& unit_cost(int precision, int op);
 
     // grid_budget: device bytes the lattice operator may take, tables and workspace
