@@ -1221,7 +1221,8 @@ int batch_set(sl1m_ctx* ctx, Batch& B, const std::vector<sl1m_problem*>& probs,
     std::vector<uint64_t> gens(np);
     for (int p = 0; p < np; ++p) gens[p] = probs[p]->gen;
     const bool same_set =
-        B.probs == probs && B.precision == precision && B.solver == solver && B.gens == gens;
+        B.ready && B.probs == probs && B.precision == precision && B.solver == solver && B.gens == gens;
+    B.ready = false;                         // until everything below is in place
     B.precision = precision;
     B.solver = solver;
     B.probs = probs;
@@ -1309,6 +1310,7 @@ int batch_set(sl1m_ctx* ctx, Batch& B, const std::vector<sl1m_problem*>& probs,
         B.sc_grid = std::max(1, std::min(ctx->num_sms * 4, np));
     }
     if (!same_set || old_ptrs != baked()) B.graph_ok = false;
+    B.ready = true;
     return SL1M_OK;
 }
 
@@ -1533,7 +1535,7 @@ static int op_prepare(sl1m_problem* prob, int precision, Batch** out)
     d.r = D.r_sorted.p;
     d.fwd_out = D.fwd_sorted.p;
     d.adj_out = D.adj_sorted.p;
-    if (B->probs.empty() || memcmp(&B->hdesc[0], &d, sizeof d) != 0)
+    if (!B->ready || memcmp(&B->hdesc[0], &d, sizeof d) != 0)
         RET(batch_set(ctx, *B, {prob}, {d}, precision, false));
     *out = B.get();
     return SL1M_OK;
@@ -1547,7 +1549,7 @@ static int run_single(sl1m_problem* prob, int precision, int max_ticks, SolveSta
     if (!B) B = std::make_unique<Batch>();
     if (precision == SL1M_FP64) RET(prob->ensure_r64(ctx->stream));
     const DevProblem d = prob->solver_desc();
-    if (B->probs.empty() || memcmp(&B->hdesc[0], &d, sizeof d) != 0)
+    if (!B->ready || memcmp(&B->hdesc[0], &d, sizeof d) != 0)
         RET(batch_set(ctx, *B, {prob}, {d}, precision, true));
     const int check = 8;
     std::vector<int> ph;

@@ -165,6 +165,7 @@ struct Server;
 
 // Device tables of a set of problems run together (one precision).
 struct Batch {
+    bool ready = false;                 // batch_set has succeeded
     int precision = 1;
     bool solver = false;
     std::vector<sl1m_problem*> probs;

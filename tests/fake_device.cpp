@@ -312,10 +312,11 @@ cudaError_t launch_adj_finish(const DevProblem* probs, const Plan* plp, const Pl
     });
     return cudaSuccess;
 }
-cudaError_t launch_phases(const DevProblem*, const int* n, int, int* out, cudaStream_t)
+cudaError_t launch_phases(const DevProblem* probs, const int* n, int, int* out, cudaStream_t)
 {
     launch([=] {
-        for (int i = 0; need(n, 4, "phases") && i < *n; ++i) out[i] = PH_DONE;
+        for (int i = 0; need(n, 4, "phases") && i < *n; ++i)
+            if (need(probs[i].st, sizeof(SolveState), "phases")) out[i] = probs[i].st->phase = PH_DONE;
     });
     return cudaSuccess;
 }

@@ -65,3 +65,19 @@ def test_a_new_problem_at_a_destroyed_ones_address_is_another_problem(sl1m, firs
     assert kinds == ([False, False, True, True] if second is None else [True, True, False, False])
     assert faults(sl1m) == ""
     ctx.close()
+
+
+@pytest.mark.parametrize("call", ["forward", "adjoint", "solve"])
+def test_a_call_after_one_that_ran_out_of_memory_starts_afresh(sl1m, call):
+    """The allocation that fails is that of the partial sums, once the tables are made."""
+    ctx = sl1m.Context(0)
+    P = scattered(ctx)
+    run = {"forward": lambda: P.forward(np.zeros(P.n_pix)), "adjoint": lambda: P.adjoint(np.zeros(P.n_vis, complex)),
+           "solve": lambda: P.solve(1.0, L=1.0, max_iter=3)}[call]
+    sl1m.fake.fake_fail(150_000, 1)
+    with pytest.raises(sl1m.SL1MError) as e:
+        run()
+    assert e.value.status == sl1m.ERR_OOM
+    run()
+    assert faults(sl1m) == ""
+    ctx.close()
