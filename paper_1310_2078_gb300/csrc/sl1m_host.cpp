@@ -1196,9 +1196,59 @@ static int set_grid_plans(sl1m_ctx* ctx, Batch& B, const std::vector<DevProblem>
         }
         H.n_blocks = H.b0[np];
         CK(upload_plan(H, np, BLK, B.plan[op][CLS_GRID], ctx->stream));
-        if (op == 0) CK(ctx->partial_f[CLS_GRID].reserve((size_t)std::max(1, H.n_slots) * BLK, ctx->stream));
-        else CK(ctx->partial_a[CLS_GRID].reserve((size_t)std::max(1, H.n_slots) * BLK, ctx->stream));
+        size_t& need = (op == 0 ? B.need_f : B.need_a)[CLS_GRID];
+        need = (size_t)std::max(1, H.n_slots) * BLK;
+        if (op == 0) CK(ctx->partial_f[CLS_GRID].reserve(need, ctx->stream));
+        else CK(ctx->partial_a[CLS_GRID].reserve(need, ctx->stream));
         B.fin_bytes[op] += (double)H.n_slots * BLK * (op == 0 ? 16.0 : 8.0);
+    }
+    return SL1M_OK;
+}
+
+// Whether the context's scratch, which all its batches share, still covers what
+// this one was set with.
+static bool scratch_covers(const sl1m_ctx* ctx, const Batch& B)
+{
+    bool ok = ctx->grid_ws.n >= B.need_ws;
+    for (int c = 0; c < N_CLS; ++c)
+        ok = ok && ctx->partial_f[c].n >= B.need_f[c] && ctx->partial_a[c].n >= B.need_a[c];
+    return ok;
+}
+
+// The operator class of every problem.  A lattice problem whose workspace
+// cannot be had takes the pair kernels, unless its solve runs already as a
+// lattice's (was_grid): the residual that its last tick left has no polar form,
+// which the pairs' adjoint reads.
+static int set_classes(sl1m_ctx* ctx, Batch& B, const std::vector<char>& was_grid)
+{
+    const size_t np = B.probs.size();
+    B.cls.assign(np, CLS_PAIRS);
+    B.need_ws = 0;
+    size_t most = 0, running = 0;
+    for (size_t p = 0; p < np; ++p) {
+        const sl1m_problem& P = *B.probs[p];
+        if (P.n_ant > 0) B.cls[p] = CLS_GAINS;
+        else if (B.precision != 0 && P.grid) {
+            B.cls[p] = CLS_GRID;
+            most = std::max(most, P.grid->ws_elems);
+            if (was_grid[p]) running = std::max(running, P.grid->ws_elems);
+        }
+    }
+    if (most == 0) return SL1M_OK;
+    const bool all = ctx->grid_ws.reserve(most, ctx->stream) == cudaSuccess;
+    if (!all) {
+        cudaGetLastError();
+        CK(ctx->grid_ws.reserve(running, ctx->stream));
+    }
+    for (size_t p = 0; p < np; ++p) {
+        if (B.cls[p] != CLS_GRID) continue;
+        const size_t need = B.probs[p]->grid->ws_elems;
+        if (all || (need < most && ctx->grid_ws.reserve(need, ctx->stream) == cudaSuccess)) {
+            B.need_ws = std::max(B.need_ws, need);
+        } else {
+            cudaGetLastError();
+            B.cls[p] = CLS_PAIRS;
+        }
     }
     return SL1M_OK;
 }
@@ -1222,6 +1272,12 @@ int batch_set(sl1m_ctx* ctx, Batch& B, const std::vector<sl1m_problem*>& probs,
     for (int p = 0; p < np; ++p) gens[p] = probs[p]->gen;
     const bool same_set =
         B.ready && B.probs == probs && B.precision == precision && B.solver == solver && B.gens == gens;
+    // (solves that run on in this batch)
+    std::vector<char> was_grid(np, 0);
+    if (B.ready && B.solver && solver && B.precision == precision)
+        for (int p = 0; p < np; ++p)
+            for (size_t q = 0; q < B.probs.size(); ++q)
+                if (B.probs[q] == probs[p] && B.gens[q] == gens[p]) was_grid[p] = B.cls[q] == CLS_GRID;
     B.ready = false;                         // until everything below is in place
     B.precision = precision;
     B.solver = solver;
@@ -1240,16 +1296,9 @@ int batch_set(sl1m_ctx* ctx, Batch& B, const std::vector<sl1m_problem*>& probs,
             B.pairs_class[c] = 0;
         }
         B.fin_bytes[0] = B.fin_bytes[1] = 0;
-        // a lattice problem whose workspace cannot be had takes the pair kernels
-        B.cls.assign(np, CLS_PAIRS);
-        for (int p = 0; p < np; ++p) {
-            if (probs[p]->n_ant > 0) {
-                B.cls[p] = CLS_GAINS;
-            } else if (precision != 0 && probs[p]->grid) {
-                if (ctx->grid_ws.reserve(probs[p]->grid->ws_elems, st) == cudaSuccess) B.cls[p] = CLS_GRID;
-                else cudaGetLastError();
-            }
-        }
+        std::fill_n(B.need_f, N_CLS, 0);
+        std::fill_n(B.need_a, N_CLS, 0);
+        RET(set_classes(ctx, B, was_grid));
         if (std::count(B.cls.begin(), B.cls.end(), CLS_GRID)) RET(set_grid_plans(ctx, B, descs));
         for (int c = 0; c < 2; ++c) {
             if (!std::count(B.cls.begin(), B.cls.end(), c)) continue;
@@ -1298,8 +1347,10 @@ int batch_set(sl1m_ctx* ctx, Batch& B, const std::vector<sl1m_problem*>& probs,
             CK(build_plan(nbf, nsf, ctx->num_sms * kf, BLK_GRAN, B.plan[0][c], st, &cf));
             CK(build_plan(nba, nsa, ctx->num_sms * ka, oga, B.plan[1][c], st, &ca));
             const Plan &pf = B.plan[0][c].pl, &pa = B.plan[1][c].pl;
-            CK(ctx->partial_f[c].reserve((size_t)std::max(1, pf.n_slots) * pf.blk_el, st));
-            CK(ctx->partial_a[c].reserve((size_t)std::max(1, pa.n_slots) * pa.blk_el, st));
+            B.need_f[c] = (size_t)std::max(1, pf.n_slots) * pf.blk_el;
+            B.need_a[c] = (size_t)std::max(1, pa.n_slots) * pa.blk_el;
+            CK(ctx->partial_f[c].reserve(B.need_f[c], st));
+            CK(ctx->partial_a[c].reserve(B.need_a[c], st));
             B.fin_bytes[0] += (double)pf.n_slots * pf.blk_el * 16.0;
             B.fin_bytes[1] += (double)pa.n_slots * pa.blk_el * 8.0;
         }
@@ -1437,6 +1488,7 @@ int batch_ticks(sl1m_ctx* ctx, Batch& B, int n)
         B.has_mfista = hm;
         B.graph_ok = false;
     }
+    if (!scratch_covers(ctx, B)) return sl1m_fail(ctx, SL1M_ERR_OOM, "the context's scratch was lost");
     if (!ctx->use_graphs || ctx->prof) {
         for (int i = 0; i < n; ++i) RET(enqueue_tick(ctx, B));
         return SL1M_OK;
@@ -1535,6 +1587,7 @@ static int op_prepare(sl1m_problem* prob, int precision, Batch** out)
     d.r = D.r_sorted.p;
     d.fwd_out = D.fwd_sorted.p;
     d.adj_out = D.adj_sorted.p;
+    if (!scratch_covers(ctx, *B)) B->ready = false;
     if (!B->ready || memcmp(&B->hdesc[0], &d, sizeof d) != 0)
         RET(batch_set(ctx, *B, {prob}, {d}, precision, false));
     *out = B.get();
@@ -1549,6 +1602,7 @@ static int run_single(sl1m_problem* prob, int precision, int max_ticks, SolveSta
     if (!B) B = std::make_unique<Batch>();
     if (precision == SL1M_FP64) RET(prob->ensure_r64(ctx->stream));
     const DevProblem d = prob->solver_desc();
+    if (!scratch_covers(ctx, *B)) B->ready = false;
     if (!B->ready || memcmp(&B->hdesc[0], &d, sizeof d) != 0)
         RET(batch_set(ctx, *B, {prob}, {d}, precision, true));
     const int check = 8;

@@ -43,12 +43,25 @@ struct DBuf {
         n = count;
         return cudaSuccess;
     }
-    // Grow to at least `count` elements (contents are not preserved).
+    // Grow to at least `count` elements (contents are not preserved).  What
+    // cannot grow stays as large as it was (beside the old memory first, then in
+    // its place): others may count on it.
     cudaError_t reserve(size_t count, cudaStream_t st)
     {
         if (count <= n && p) return cudaSuccess;
         cudaStreamSynchronize(st);
-        return alloc(count);
+        T* q = nullptr;
+        cudaError_t e = cudaMalloc((void**)&q, count * sizeof(T));
+        if (e == cudaSuccess) {
+            free();
+            p = q;
+            n = count;
+        } else if (const size_t had = n) {
+            cudaGetLastError();
+            e = alloc(count);
+            if (e != cudaSuccess && alloc(had) != cudaSuccess) cudaGetLastError();   // (n = 0: nothing left)
+        }
+        return e;
     }
     // Allocate exactly `count` and copy from host (zero-fill when `zero`);
     // returns after the copy (the host source may be a temporary).
@@ -178,6 +191,7 @@ struct Batch {
     std::vector<int> cls;               // class of every problem
     std::vector<uint64_t> gens;         // layout of every problem when the plans were made
     std::vector<int> grid_slot[2];      // [op] first partial slot of every lattice problem
+    size_t need_f[N_CLS] = {0, 0, 0}, need_a[N_CLS] = {0, 0, 0}, need_ws = 0;   // of the context's scratch
     int nst[2][2] = {{4, 4}, {4, 4}};   // tile shape per [op][class] (autotuned or default)
     int n_ant_max = 0;
     int sc_grid = 1;

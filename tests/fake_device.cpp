@@ -5,7 +5,8 @@
 // rely on it, that its plan belongs to the problems it is given and that what it
 // reads and writes lies in live allocations, and notes what does not in
 // fake_faults().  A captured graph keeps its launches' checks and runs them again
-// at every launch.  Solves end after their first ticks (every phase reads DONE).
+// at every launch.  Solves end after their first ticks (every phase reads DONE)
+// unless they are held.
 // A new problem takes the lowest free place of a few, so one made after another
 // was destroyed has its address.
 #include <cuda_runtime.h>
@@ -34,6 +35,7 @@ size_t g_fail_min = 0;                             // allocations of this size a
 int g_fail_n = 0;                                  // ... fail this many times
 std::string g_faults;
 long long g_count[5];                              // launches: pairs fwd, adj, lattice fwd, adj; table fills
+bool g_hold = false;                                // solves run on
 thread_local bool t_capturing = false;
 using Check = std::function<void()>;
 std::vector<Check> g_captured;
@@ -130,10 +132,12 @@ void fake_reset()
     LOCK;
     g_faults.clear();
     g_fail_n = 0;
+    g_hold = false;
     g_peak = g_held;
     memset(g_count, 0, sizeof g_count);
 }
 void fake_fail(size_t min_bytes, int n) { LOCK; g_fail_min = min_bytes; g_fail_n = n; }
+void fake_hold(int on) { LOCK; g_hold = on; }
 void fake_total(size_t bytes) { LOCK; g_total = bytes; }
 size_t fake_held() { return g_held; }
 size_t fake_peak() { return g_peak; }
@@ -316,7 +320,7 @@ cudaError_t launch_phases(const DevProblem* probs, const int* n, int, int* out, 
 {
     launch([=] {
         for (int i = 0; need(n, 4, "phases") && i < *n; ++i)
-            if (need(probs[i].st, sizeof(SolveState), "phases")) out[i] = probs[i].st->phase = PH_DONE;
+            if (need(probs[i].st, sizeof(SolveState), "phases")) out[i] = probs[i].st->phase = g_hold ? PH_SOLVE : PH_DONE;
     });
     return cudaSuccess;
 }

@@ -2,6 +2,8 @@
 hoped for: over a CUDA runtime and launchers that run nothing (fake_device.cpp),
 so no device is needed and none can fault.  A launch with another problem's
 tables, or with memory that is not allocated, is noted there."""
+import time
+
 import numpy as np
 import pytest
 
@@ -42,6 +44,13 @@ def scattered(ctx, n_vis=900, n_pix=700, seed=3):
     return P
 
 
+def wait_for(cond, limit_s=60.0):
+    t0 = time.monotonic()
+    while not cond():
+        assert time.monotonic() - t0 < limit_s
+        time.sleep(0.001)
+
+
 def serve(ctx, P):
     t = ctx.server_submit(P, 1.0, L=1.0, max_iter=5)
     return ctx.server_wait(t, P, 60)
@@ -79,5 +88,70 @@ def test_a_call_after_one_that_ran_out_of_memory_starts_afresh(sl1m, call):
         run()
     assert e.value.status == sl1m.ERR_OOM
     run()
+    assert faults(sl1m) == ""
+    ctx.close()
+
+
+# the workspace of the large lattice is above, every other allocation below (but the small one's workspace at 1 MB)
+WORKSPACE = 20_000_000
+
+
+@pytest.mark.parametrize("at_least,times", [(WORKSPACE, 2), (1_000_000, 3)])
+def test_a_workspace_that_cannot_grow_is_left_to_those_who_use_it(sl1m, at_least, times):
+    """... and the problem that asked for more takes the pair kernels.  Three
+    failures: the old workspace is lost, too, and made again by its user."""
+    ctx = sl1m.Context(0)
+    A, B = lattice(ctx), lattice(ctx, 256, 60000)
+    A.forward(np.zeros(A.n_pix))
+    B.forward(np.zeros(B.n_pix), sl1m.FP64)                # laid out; the workspace comes with the first mixed call
+    sl1m.fake.fake_reset()
+    sl1m.fake.fake_fail(at_least, times)
+    B.forward(np.zeros(B.n_pix))
+    assert sl1m.fake.fake_count(0) == 1 and sl1m.fake.fake_count(2) == 0
+    for P in (A, B):
+        P.adjoint(np.zeros(P.n_vis, complex))
+    assert sl1m.fake.fake_count(3) == 1 and sl1m.fake.fake_count(1) == 1
+    assert faults(sl1m) == ""
+    ctx.close()
+
+
+def test_two_lattices_of_a_server_with_room_for_one(sl1m):
+    ctx = sl1m.Context(0)
+    A, B = lattice(ctx), lattice(ctx, 256, 60000)
+    for P in (A, B):
+        P.forward(np.zeros(P.n_pix), sl1m.FP64)
+    sl1m.fake.fake_fail(WORKSPACE, 100)
+    ctx.server_start(max_pairs_per_tick=1e12)
+    sl1m.fake.fake_hold(1)
+    tickets = [ctx.server_submit(P, 1.0, L=1.0, max_iter=5) for P in (A, B)]
+    wait_for(lambda: ctx.server_info()["active"] == 2)
+    sl1m.fake.fake_hold(0)
+    for t, P in zip(tickets, (A, B)):
+        ctx.server_wait(t, P, 60)
+    assert sl1m.fake.fake_count(2) > 0 and faults(sl1m) == ""
+    ctx.close()
+
+
+def test_a_running_lattice_solve_stays_one_when_the_workspace_cannot_grow(sl1m):
+    """Its residual has no polar form, so the pair kernels cannot take it over."""
+    ctx = sl1m.Context(0)
+    A, B = lattice(ctx), lattice(ctx, 256, 60000)
+    B.forward(np.zeros(B.n_pix), sl1m.FP64)
+    ctx.server_start(max_pairs_per_tick=1e12)
+    sl1m.fake.fake_hold(1)
+    tickets = [ctx.server_submit(A, 1.0, L=1.0, max_iter=5)]
+    wait_for(lambda: ctx.server_info()["rounds"] > 3)
+    sl1m.fake.fake_fail(WORKSPACE, 100)
+    tickets.append(ctx.server_submit(B, 1.0, L=1.0, max_iter=5))
+    wait_for(lambda: ctx.server_info()["active"] == 2)
+    r = ctx.server_info()["rounds"]
+    wait_for(lambda: ctx.server_info()["rounds"] > r + 3)
+    before = [sl1m.fake.fake_count(i) for i in range(4)]
+    r = ctx.server_info()["rounds"]
+    wait_for(lambda: ctx.server_info()["rounds"] > r + 3)
+    assert all(sl1m.fake.fake_count(i) > before[i] for i in range(4))      # A lattice, B pairs
+    sl1m.fake.fake_hold(0)
+    for t, P in zip(tickets, (A, B)):
+        ctx.server_wait(t, P, 60)
     assert faults(sl1m) == ""
     ctx.close()
