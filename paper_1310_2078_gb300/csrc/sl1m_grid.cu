@@ -398,11 +398,12 @@ grid_rows_fwd_kernel(const DevProblem* __restrict__ probs, int prob, const GridO
 }
 
 // Adjoint, rows: g1 transformed back along x; Re(exp(+2 pi i w_p nu) z) summed
-// over the CTA's planes (FP32 over GR_PCH planes) into the chunk's partial slots.
+// over the CTA's planes (FP32 over GR_PCH planes) into the chunk's partial slots,
+// which a later pass over the planes adds to.
 template <int LOG>
 __global__ void __launch_bounds__(RowShape<LOG>::THREADS, RowShape<LOG>::CTAS)
-grid_rows_adj_kernel(const DevProblem* __restrict__ probs, int prob, const GridOp g, int p0, int np, int chunk0,
-                     int n_pix, int n_pix_pad, double* __restrict__ partial)
+grid_rows_adj_kernel(const DevProblem* __restrict__ probs, int prob, const GridOp g, int p0, int np, int n_pix,
+                     int n_pix_pad, double* __restrict__ partial)
 {
     using S = RowShape<LOG>;
     constexpr int L = 1 << LOG;
@@ -440,7 +441,6 @@ grid_rows_adj_kernel(const DevProblem* __restrict__ probs, int prob, const GridO
             acc[i] += fmaf(e.x, v[0][cell_q<S::P>(i)].x, e.y * v[0][cell_q<S::P>(i)].y);
         }
     }
-    const int chunk = chunk0 + blockIdx.y;
     if (iy < g.ny) {
 #pragma unroll
         for (int i = 0; i < S::P / 2; ++i) {
@@ -448,14 +448,16 @@ grid_rows_adj_kernel(const DevProblem* __restrict__ probs, int prob, const GridO
             if (ix < 0 || ix >= g.nx) continue;
             const size_t at = (size_t)iy * g.nx + ix;
             const int j = g.cell[at];
-            if (j >= 0)
-                partial[((size_t)(j / BLK) * g.n_chunk + chunk) * BLK + j % BLK] =
-                    (double)acc[i] * ((double)g.amp[at] / (double)g.ascale);
+            if (j >= 0) {
+                double& slot = partial[((size_t)(j / BLK) * g.n_chunk + blockIdx.y) * BLK + j % BLK];
+                const double v = (double)acc[i] * ((double)g.amp[at] / (double)g.ascale);
+                slot = p0 > 0 ? slot + v : v;
+            }
         }
     }
     if (blockIdx.x == 0)                       // padding slots of the last pixel granule
         for (int j = n_pix + threadIdx.x; j < n_pix_pad; j += S::THREADS)
-            partial[((size_t)(j / BLK) * g.n_chunk + chunk) * BLK + j % BLK] = 0.0;
+            partial[((size_t)(j / BLK) * g.n_chunk + blockIdx.y) * BLK + j % BLK] = 0.0;
 }
 
 // Columns: CB adjacent columns of one plane per CTA, so a row of the tile is
@@ -808,12 +810,12 @@ static void rows_fwd(const DevProblem* probs, int p, const GridOp& g, int p0, in
     grid_rows_fwd_kernel<LOG><<<grid, S::THREADS, S::SMEM, st>>>(probs, p, g, p0, np);
 }
 template <int LOG>
-static void rows_adj(const DevProblem* probs, int p, const GridOp& g, int p0, int np, int chunk0, int n_pix,
-                     int n_pix_pad, double* partial, cudaStream_t st)
+static void rows_adj(const DevProblem* probs, int p, const GridOp& g, int p0, int np, int n_pix, int n_pix_pad,
+                     double* partial, cudaStream_t st)
 {
     using S = RowShape<LOG>;
     const dim3 grid((unsigned)((g.ny + S::ROWS - 1) / S::ROWS), (unsigned)((np + GR_PCH - 1) / GR_PCH));
-    grid_rows_adj_kernel<LOG><<<grid, S::THREADS, S::SMEM, st>>>(probs, p, g, p0, np, chunk0, n_pix, n_pix_pad, partial);
+    grid_rows_adj_kernel<LOG><<<grid, S::THREADS, S::SMEM, st>>>(probs, p, g, p0, np, n_pix, n_pix_pad, partial);
 }
 template <int LOG, int SGN>
 static void cols(const DevProblem* probs, int p, const GridOp& g, int p0, int np, cudaStream_t st)
@@ -867,7 +869,7 @@ cudaError_t grid_adjoint(const DevProblem* probs, int p, const GridOp& g, int n_
         const dim3 sg((unsigned)tiles, (unsigned)((np + seg - 1) / seg));
         grid_spread_kernel<<<sg, GR_TILE * GR_TILE, 0, st>>>(probs, p, g, p0, np, seg);
         GRID_DISPATCH(g.ly, (cols<LOG, 1>(probs, p, g, p0, np, st)));
-        GRID_DISPATCH(g.lx, (rows_adj<LOG>(probs, p, g, p0, np, p0 / GR_PCH, n_pix, n_pix_pad, partial, st)));
+        GRID_DISPATCH(g.lx, (rows_adj<LOG>(probs, p, g, p0, np, n_pix, n_pix_pad, partial, st)));
         *n_launch += 3;
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;

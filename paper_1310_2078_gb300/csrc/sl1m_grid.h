@@ -22,7 +22,7 @@ struct GridOp {
     int lx, ly;                 // log2 of the FFT lengths (2^lx >= 2 nx, 2^ly >= 2 ny)
     int np;                     // planes in w
     int np_pass;                // planes the workspace holds at a time
-    int n_chunk;                // adjoint partial slots: chunks of GR_PCH planes, all passes
+    int n_chunk;                // adjoint partial slots: chunks of GR_PCH planes of one pass
     float fscale, ascale;       // powers of two that keep the transforms' sums in range
     const int* cell;            // [ny][nx] sorted pixel index, -1 where the lattice has no pixel
     const float* amp;           // [ny][nx] (1/n) / (kernel transforms), 0 without a pixel
@@ -44,6 +44,11 @@ struct GridOp {
 
 inline size_t grid_plane_elems(const GridOp& g) { return ((size_t)g.ny + ((size_t)1 << g.ly)) << g.lx; }
 inline int grid_tiles(const GridOp& g) { return ((1 << g.lx) / GR_TILE) * ((1 << g.ly) / GR_TILE); }
+// Bytes of its partial sums, forward and adjoint.
+inline size_t grid_sum_bytes(const GridOp& g, int vis_blk, int pix_blk)
+{
+    return ((size_t)vis_blk * 16 + (size_t)pix_blk * 8 * g.n_chunk) * BLK;
+}
 // Radix of a transform of length 2^lg, and of its first pass: 16 where that saves
 // an exchange over radix 8.
 constexpr int grid_radix(int lg) { return lg == 6 || lg == 9 ? 8 : 16; }

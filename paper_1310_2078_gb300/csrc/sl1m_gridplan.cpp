@@ -181,12 +181,13 @@ bool grid_build(sl1m_problem& P, cudaStream_t st, size_t budget)
     const size_t ws_max = std::min({GR_WS_MAX, free_b / 4, budget / 2});
     g.np_pass = (int)std::min<size_t>((size_t)(g.np + GR_PCH - 1) / GR_PCH, ws_max / (plane * GR_PCH)) * GR_PCH;
     if (g.np_pass < GR_PCH) return false;
-    g.n_chunk = (g.np + GR_PCH - 1) / GR_PCH;
+    g.n_chunk = g.np_pass / GR_PCH;
     T->ws_elems = grid_plane_elems(g) * g.np_pass;
     const size_t nv = P.hp.vis.n_pad, cells = (size_t)g.nx * g.ny;
     const int tiles = grid_tiles(g), ni = g.np - GRW + 1;
     const size_t tab = cells * 16 + nv * (16 + 12 * GRW + 8 + 20) + (size_t)tiles * (ni * 5 + 44);
-    if (tab + T->ws_elems * sizeof(float2) > std::min(budget, free_b / 2)) return false;
+    const size_t sums = grid_sum_bytes(g, P.hp.vis.n_blk, P.hp.pix.n_blk);
+    if (tab + sums + T->ws_elems * sizeof(float2) > std::min(budget, free_b / 2)) return false;
     // powers of two that keep a coherent sum of the largest inputs in range
     const auto p2 = [](double n) { return (float)std::exp2(-std::ceil(std::log2(std::max(1.0, n)))); };
     g.fscale = p2((double)P.n_pix);

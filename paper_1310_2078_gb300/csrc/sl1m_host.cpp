@@ -1299,7 +1299,20 @@ int batch_set(sl1m_ctx* ctx, Batch& B, const std::vector<sl1m_problem*>& probs,
         std::fill_n(B.need_f, N_CLS, 0);
         std::fill_n(B.need_a, N_CLS, 0);
         RET(set_classes(ctx, B, was_grid));
-        if (std::count(B.cls.begin(), B.cls.end(), CLS_GRID)) RET(set_grid_plans(ctx, B, descs));
+        if (std::count(B.cls.begin(), B.cls.end(), CLS_GRID)) {
+            const int rc = set_grid_plans(ctx, B, descs);
+            // (no memory for their sums: all of them take the pair kernels, as without a workspace)
+            const bool out = rc == SL1M_ERR_OOM && !std::count(was_grid.begin(), was_grid.end(), 1);
+            if (rc != SL1M_OK && !out) return rc;
+            if (out) {
+                cudaGetLastError();
+                std::replace(B.cls.begin(), B.cls.end(), CLS_GRID, CLS_PAIRS);
+                B.need_ws = B.need_f[CLS_GRID] = B.need_a[CLS_GRID] = 0;
+                B.has_class[CLS_GRID] = false;
+                B.pairs_class[CLS_GRID] = 0;
+                B.fin_bytes[0] = B.fin_bytes[1] = 0;
+            }
+        }
         for (int c = 0; c < 2; ++c) {
             if (!std::count(B.cls.begin(), B.cls.end(), c)) continue;
             std::vector<int> nbf(np), nsf(np), nba(np), nsa(np);

@@ -10,7 +10,9 @@
 // A new problem takes the lowest free place of a few, so one made after another
 // was destroyed has its address.
 #include <cuda_runtime.h>
+#include <dlfcn.h>
 
+#include <atomic>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
@@ -19,6 +21,8 @@
 #include <mutex>
 #include <new>
 #include <string>
+#include <system_error>
+#include <thread>
 #include <vector>
 
 #include "sl1m_host.h"
@@ -27,6 +31,8 @@
 using namespace sl1m;
 
 namespace {
+
+std::atomic<int> g_no_threads{0};                  // threads of the library's cannot be started
 
 std::recursive_mutex g_mu;
 std::map<const char*, size_t> g_live;              // device allocations
@@ -97,6 +103,16 @@ bool g_used[N_PLACES];
 
 }  // namespace
 
+// std::async and std::thread of the library come here (it is linked symbolically).
+void std::thread::_M_start_thread(_State_ptr s, void (*dep)())
+{
+    if (g_no_threads) throw std::system_error(std::make_error_code(std::errc::resource_unavailable_try_again));
+    using Start = void (*)(std::thread*, _State_ptr, void (*)());
+    static const Start next = (Start)dlsym(RTLD_NEXT, "_ZNSt6thread15_M_start_threadESt10unique_ptrINS_6_StateESt14"
+                                                      "default_deleteIS1_EEPFvvE");
+    next(this, std::move(s), dep);
+}
+
 void* operator new(size_t n, const std::nothrow_t&) noexcept
 {
     LOCK;
@@ -133,10 +149,12 @@ void fake_reset()
     g_faults.clear();
     g_fail_n = 0;
     g_hold = false;
+    g_total = (size_t)280 << 30;
     g_peak = g_held;
     memset(g_count, 0, sizeof g_count);
 }
 void fake_fail(size_t min_bytes, int n) { LOCK; g_fail_min = min_bytes; g_fail_n = n; }
+void fake_no_threads(int on) { g_no_threads = on; }
 void fake_hold(int on) { LOCK; g_hold = on; }
 void fake_total(size_t bytes) { LOCK; g_total = bytes; }
 size_t fake_held() { return g_held; }
@@ -279,6 +297,7 @@ cudaError_t grid_adjoint(const DevProblem* probs, int p, const GridOp& g, int n_
     launch([=] {
         check_grid("lattice adjoint", g);
         need(partial, (size_t)n_pix_pad * 8 * g.n_chunk, "lattice adjoint's sums");
+        if (g.n_chunk * GR_PCH > g.np_pass) fault("lattice adjoint: sums of more planes than a pass has");
         if (need(probs, sizeof *probs * (p + 1), "lattice adjoint") && probs[p].pix.n != n_pix)
             fault("lattice adjoint: another problem's tables");
         ++g_count[3];

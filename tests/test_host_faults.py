@@ -2,6 +2,10 @@
 hoped for: over a CUDA runtime and launchers that run nothing (fake_device.cpp),
 so no device is needed and none can fault.  A launch with another problem's
 tables, or with memory that is not allocated, is noted there."""
+import os
+import subprocess
+import sys
+import textwrap
 import time
 
 import numpy as np
@@ -49,6 +53,20 @@ def wait_for(cond, limit_s=60.0):
     while not cond():
         assert time.monotonic() - t0 < limit_s
         time.sleep(0.001)
+
+
+def in_a_child(lib, code):
+    """Runs code in a process of its own, which an exception that crosses the C ABI ends."""
+    pre = f"""
+        import sys
+        sys.path[:0] = {[os.path.dirname(os.path.abspath(__file__)), fake_device.b.ROOT]!r}
+        import numpy as np
+        import fake_device
+        from paper_1310_2078_gb300 import synth
+        sl1m = fake_device.binding({lib!r})
+        """
+    r = subprocess.run([sys.executable, "-c", textwrap.dedent(pre) + textwrap.dedent(code)], capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr[-2000:]
 
 
 def serve(ctx, P):
@@ -154,4 +172,27 @@ def test_a_running_lattice_solve_stays_one_when_the_workspace_cannot_grow(sl1m):
     for t, P in zip(tickets, (A, B)):
         ctx.server_wait(t, P, 60)
     assert faults(sl1m) == ""
+    ctx.close()
+
+
+def test_a_lattice_without_memory_for_its_sums_takes_the_pair_kernels(sl1m):
+    ctx = sl1m.Context(0)
+    A, B = lattice(ctx), lattice(ctx, n_vis=60000)         # one workspace, more sums
+    A.forward(np.zeros(A.n_pix))
+    B.forward(np.zeros(B.n_pix), sl1m.FP64)
+    sl1m.fake.fake_reset()
+    sl1m.fake.fake_fail(900_000, 2)
+    B.forward(np.zeros(B.n_pix))
+    assert sl1m.fake.fake_count(0) == 1 and sl1m.fake.fake_count(2) == 0
+    A.forward(np.zeros(A.n_pix))
+    assert sl1m.fake.fake_count(2) == 1 and faults(sl1m) == ""
+    ctx.close()
+
+
+def test_a_lattice_of_many_passes_holds_the_sums_of_one(sl1m):
+    sl1m.fake.fake_total(400 << 20)                        # 120 of its 648 planes
+    ctx = sl1m.Context(0)
+    P = lattice(ctx, n_vis=60000, w_max=20000.0)
+    P.adjoint(np.zeros(P.n_vis, complex))
+    assert sl1m.fake.fake_count(3) == 1 and faults(sl1m) == ""
     ctx.close()
