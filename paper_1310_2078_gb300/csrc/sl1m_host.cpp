@@ -15,6 +15,7 @@
 #include <map>
 #include <memory>
 #include <string>
+#include <system_error>
 #include <vector>
 
 #include "sl1m_dev.h"
@@ -786,7 +787,7 @@ int sl1m_problem::rebuild(cudaStream_t st, size_t grid_budget)
         } else {
             // the cheapest of the point order and of runs of 16, 8 and 4 samples
             // of a pair (tried while the mean pair has that many), each made by a
-            // thread of its own
+            // thread of its own, or here where none can be had
             std::vector<long long> keys(n_vis);
             for (int64_t k = 0; k < n_vis; ++k) keys[k] = (long long)ant[2 * k] * n_ant + ant[2 * k + 1];
             const std::vector<int> by = sort_by_pair(ant, n_ant, n_vis);
@@ -796,12 +797,18 @@ int sl1m_problem::rebuild(cudaStream_t st, size_t grid_budget)
             using Tried = std::pair<double, std::vector<int>>;
             std::vector<std::future<Tried>> tried;
             for (int s = 16; s >= 4; s /= 2)
-                if (per >= 0.75 * s)
-                    tried.push_back(std::async(std::launch::async, [&, s]() -> Tried {
+                if (per >= 0.75 * s) {
+                    const auto job = [&, s]() -> Tried {
                         std::vector<int> o = order_by_runs(keys, by, uvw.data(), s);
                         const double c = gains_order_cost(o, keys, uvw.data(), gext_pix);
                         return {c, std::move(o)};
-                    }));
+                    };
+                    try {
+                        tried.push_back(std::async(std::launch::async, job));
+                    } catch (const std::system_error&) {
+                        tried.push_back(std::async(std::launch::deferred, job));
+                    }
+                }
             kd_append(order, std::move(members), uvw.data(), uvw.data() + 1, 3);
             double best = gains_order_cost(order, keys, uvw.data(), gext_pix);
             for (auto& f : tried) {

@@ -196,3 +196,25 @@ def test_a_lattice_of_many_passes_holds_the_sums_of_one(sl1m):
     P.adjoint(np.zeros(P.n_vis, complex))
     assert sl1m.fake.fake_count(3) == 1 and faults(sl1m) == ""
     ctx.close()
+
+
+def test_a_gains_layout_where_no_thread_can_be_had(lib):
+    """The orders that threads of their own would try are tried by the caller: the same layout."""
+    in_a_child(lib, """
+        rng = np.random.default_rng(1)
+        uvw, ant = synth.uvw_tracks(synth.antennas(rng, 12, 800.0, 20.0), -30.0, 16)
+        lm = rng.uniform(-0.2, 0.2, (700, 2))
+        shares = []
+        for no_threads in (0, 1):
+            ctx = sl1m.Context(0)
+            P = ctx.problem()
+            P.set_visibilities(uvw, None, None, ant)
+            P.set_pixels(lm)
+            P.set_gains(synth.beam_gains(rng, lm, 12))
+            sl1m.fake.fake_no_threads(no_threads)
+            P.forward(np.zeros(700))
+            assert sl1m.fake.fake_faults() == b""
+            shares.append((P.exact_tile_share(), P.bytes()))
+            ctx.close()
+        assert shares[0] == shares[1]
+        """)
