@@ -28,7 +28,11 @@
  *     one cosine per pair); sums over tiles, norms, step sizes and the
  *     projection stay in FP64.  Dirac pixels on a regular (l, m) lattice
  *     without gains take, where that is faster, an FP32 gridding and FFT
- *     operator instead, whose result is nearer FP64's than the pairs' is.
+ *     operator instead, whose result is nearer FP64's than the pairs' is.  It
+ *     needs tables and a workspace of up to 4 GB, which the problems of a
+ *     context share; whether it is taken, and how many of its planes it works
+ *     on at a time, follows the memory that is free when a problem is laid out,
+ *     so equal calls of two runs can differ by rounding.
  */
 #ifndef SL1M_H
 #define SL1M_H
@@ -246,7 +250,10 @@ int sl1m_solve(sl1m_problem* prob, const sl1m_solve_opts* opts, double* img_out,
 #define SL1M_ADMIT_TWO_LANES 0   /* default: small and large requests in lanes  */
 #define SL1M_ADMIT_ARRIVAL 1     /* one queue, strictly in arrival order         */
 typedef struct {
-    int64_t mem_budget_bytes;   /* 0 = 80% of the device memory free at start   */
+    int64_t mem_budget_bytes;   /* 0 = 80% of the device memory free at start.
+                                   A lattice operator counts too (its workspace
+                                   once for all that run): a solve that is
+                                   admitted without room for it evaluates pairs */
     int32_t max_slots;          /* 0 = 64 concurrent solves                      */
     int32_t ticks_per_round;    /* 0 = 4 steps between admission/retirement     */
     int32_t precision;          /* SL1M_MIXED or SL1M_FP64 for every request     */

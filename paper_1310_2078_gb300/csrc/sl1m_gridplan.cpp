@@ -137,6 +137,8 @@ static double pair_seconds(double pairs) { return 2.8e-5 + pairs / 2.4e12; }
 bool grid_build(sl1m_problem& P, cudaStream_t st, size_t budget)
 {
     P.grid.reset();
+    P.grid_least = 0;
+    P.grid_cut = false;
     if (P.n_ant > 0 || P.has_gauss) return false;
     const double pairs = P.pairs();
     if (0.9 * pair_seconds(pairs) < 4.2e-5) return false;   // launches, not pairs, decide
@@ -179,13 +181,17 @@ bool grid_build(sl1m_problem& P, cudaStream_t st, size_t budget)
     if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return false;
     const size_t plane = grid_plane_elems(g) * sizeof(float2);
     const size_t ws_max = std::min({GR_WS_MAX, free_b / 4, budget / 2});
-    g.np_pass = (int)std::min<size_t>((size_t)(g.np + GR_PCH - 1) / GR_PCH, ws_max / (plane * GR_PCH)) * GR_PCH;
-    if (g.np_pass < GR_PCH) return false;
-    g.n_chunk = g.np_pass / GR_PCH;
-    T->ws_elems = grid_plane_elems(g) * g.np_pass;
     const size_t nv = P.hp.vis.n_pad, cells = (size_t)g.nx * g.ny;
     const int tiles = grid_tiles(g), ni = g.np - GRW + 1;
     const size_t tab = cells * 16 + nv * (16 + 12 * GRW + 8 + 20) + (size_t)tiles * (ni * 5 + 44);
+    const size_t want = (size_t)(g.np + GR_PCH - 1) / GR_PCH, got = ws_max / (plane * GR_PCH);
+    g.np_pass = (int)std::min(want, got) * GR_PCH;
+    g.n_chunk = 1;                                        // (with the fewest planes)
+    P.grid_least = std::max(2 * plane * GR_PCH, tab + grid_sum_bytes(g, P.hp.vis.n_blk, P.hp.pix.n_blk) + plane * GR_PCH);
+    if (g.np_pass < GR_PCH) return false;
+    P.grid_cut = got < std::min(want, GR_WS_MAX / (plane * GR_PCH));
+    g.n_chunk = g.np_pass / GR_PCH;
+    T->ws_elems = grid_plane_elems(g) * g.np_pass;
     const size_t sums = grid_sum_bytes(g, P.hp.vis.n_blk, P.hp.pix.n_blk);
     if (tab + sums + T->ws_elems * sizeof(float2) > std::min(budget, free_b / 2)) return false;
     // powers of two that keep a coherent sum of the largest inputs in range

@@ -636,9 +636,33 @@ sl1m_problem::~sl1m_problem() = default;
 // problem may have the address of a destroyed one, never its number.
 static std::atomic<uint64_t> g_layouts{0};
 
+// The lattice operator of the laid-out problem, as far as grid_budget allows; what
+// was set up for another choice of operator is dropped.
+void sl1m_problem::set_grid(cudaStream_t st, size_t grid_budget)
+{
+    grid.reset();
+    for (auto& b : op_batch) b.reset();
+    for (auto& b : solve_batch) b.reset();
+    gen = ++g_layouts;
+    grid_tried = grid_budget;
+    if (grid_budget == 0) grid_least = std::max<size_t>(1, grid_least);     // (not looked into)
+    else if (grid_build(*this, st, grid_budget))
+        ctx->h2d += (long long)(grid->cell.bytes() + grid->list.bytes() + grid->start.bytes());
+}
+
+size_t sl1m_problem::grid_own_bytes() const
+{
+    return grid ? grid->bytes() + grid_sum_bytes(grid->op, hp.vis.n_blk, hp.pix.n_blk) : 0;
+}
+
 int sl1m_problem::rebuild(cudaStream_t st, size_t grid_budget)
 {
-    if (!dirty) return SL1M_OK;
+    if (!dirty) {
+        // a lattice operator that a server's budget refused, or cut to few planes
+        const bool more = grid ? grid_cut && grid_budget == SIZE_MAX : grid_least > 0 && grid_budget >= grid_least;
+        if (more && grid_budget > grid_tried) set_grid(st, grid_budget);
+        return SL1M_OK;
+    }
     if (n_vis <= 0 || n_pix <= 0)
         return sl1m_fail(ctx, SL1M_ERR_STATE, "problem needs visibilities and pixels");
     if (n_ant > 0 && ant.empty())
@@ -927,14 +951,10 @@ int sl1m_problem::rebuild(cudaStream_t st, size_t grid_budget)
     hp.st = nullptr;
     grid.reset();
     ctx->h2d += (long long)dev_bytes();
-    for (auto& b : op_batch) b.reset();
-    for (auto& b : solve_batch) b.reset();
     for (auto& r : ucost_ok) r[0] = r[1] = false;
     solver_ready = false;
     dirty = false;
-    gen = ++g_layouts;
-    if (grid_build(*this, st, grid_budget))
-        ctx->h2d += (long long)(grid->cell.bytes() + grid->list.bytes() + grid->start.bytes());
+    set_grid(st, grid_budget);
     return SL1M_OK;
 }
 

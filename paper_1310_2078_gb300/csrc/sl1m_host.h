@@ -293,11 +293,19 @@ struct sl1m_problem {
     bool ucost_ok[2][2] = {{false, false}, {false, false}};
     std::unique_ptr<Batch> op_batch[2], solve_batch[2];
     std::unique_ptr<GridTables> grid;         // lattice operator of the mixed path, or null
+    // what the lattice operator was last built or refused with: the budget, the
+    // bytes it takes at least when memory was what it lacked, and whether it got
+    // fewer planes at a time than it could use
+    size_t grid_tried = 0, grid_least = 0;
+    bool grid_cut = false;
     uint64_t gen = 0;                         // number of the layout: no two of a process share one
     const UnitCost& unit_cost(int precision, int op);
 
-    // grid_budget: device bytes the lattice operator may take, tables and workspace
+    // grid_budget: device bytes the lattice operator may take, tables, sums and
+    // workspace (a laid-out problem that had less tries again)
     int rebuild(cudaStream_t st, size_t grid_budget = SIZE_MAX);
+    void set_grid(cudaStream_t st, size_t grid_budget);    // 0: none
+    size_t grid_own_bytes() const;                         // its tables and sums, without the workspace
     int ensure_r64(cudaStream_t st);
     int ensure_solver(cudaStream_t st);
     int init_solve(const sl1m_solve_opts* o, double L, bool power_only, cudaStream_t st);

@@ -19,6 +19,7 @@
 #include <map>
 #include <memory>
 #include <mutex>
+#include <set>
 #include <thread>
 #include <vector>
 
@@ -46,7 +47,8 @@ struct Request {
     bool done = false;
     std::vector<double> img;
     sl1m_solve_stats stats{};
-    size_t bytes = 0;
+    size_t bytes = 0;                            // charged to the budget ...
+    size_t ws = 0;                               // ... beside the lattice workspace it needs
 };
 
 struct Server {
@@ -58,7 +60,11 @@ struct Server {
     std::vector<Request*> active;
     std::map<uint64_t, std::unique_ptr<Request>> reqs;
     uint64_t next_ticket = 1;
+    // in_use: every admitted request's bytes, and the one workspace that the
+    // lattice operators among them share
     size_t budget = 0, in_use = 0;
+    std::multiset<size_t> ws;
+    size_t ws_bytes() const { return ws.empty() ? 0 : *ws.rbegin(); }
     int max_slots = 64, ticks_per_round = 4, precision = SL1M_MIXED;
     int admission = SL1M_ADMIT_TWO_LANES;
     double max_pairs = 4e9;
@@ -94,7 +100,9 @@ static void retire(Server& S, Request* r, int status)
     std::lock_guard<std::mutex> lk(S.mu);
     r->status = status;
     r->done = true;
-    S.in_use -= std::min(S.in_use, r->bytes);
+    const size_t ws = S.ws_bytes();
+    if (r->ws) S.ws.erase(S.ws.find(r->ws));
+    S.in_use -= std::min(S.in_use, r->bytes + ws - S.ws_bytes());
     S.finished += 1;
     S.cv_done.notify_all();
 }
@@ -212,19 +220,28 @@ static void server_loop(Server* Sp)
         std::vector<Request*> joined;
         for (Request* r : admit) {
             sl1m_problem* p = r->prob;
-            // a lattice operator's tables and workspace count against the budget
-            // like the rest, and are only made when they fit what is left of it
-            size_t left;
+            // a lattice operator's tables, sums and workspace count against the
+            // budget like the rest: it is made, or kept, when they fit what is left
+            size_t left, shared;
             {
                 std::lock_guard<std::mutex> lk(S.mu);
+                shared = S.ws_bytes();
                 left = S.budget > S.in_use ? S.budget - S.in_use : 0;
             }
-            int rc = p->rebuild(ctx->upstream, left);
+            const bool mixed = S.precision != SL1M_FP64;         // (FP64 solves have no use for it)
+            int rc = p->rebuild(ctx->upstream, mixed ? left + shared : 0);
             if (rc == SL1M_OK && p->grid) {
-                const size_t extra = p->grid->bytes() + p->grid->ws_elems * sizeof(float2);
-                std::lock_guard<std::mutex> lk(S.mu);
-                r->bytes += extra;
-                S.in_use += extra;
+                const size_t ws = mixed ? p->grid->ws_elems * sizeof(float2) : 0, own = p->grid_own_bytes();
+                const size_t more = own + (ws > shared ? ws - shared : 0);
+                if (more > left) {
+                    p->set_grid(ctx->upstream, 0);
+                } else {
+                    std::lock_guard<std::mutex> lk(S.mu);
+                    r->bytes += own;
+                    r->ws = ws;
+                    if (ws) S.ws.insert(ws);
+                    S.in_use += more;
+                }
             }
             if (rc == SL1M_OK && S.precision == SL1M_FP64) rc = p->ensure_r64(ctx->upstream);
             if (rc == SL1M_OK) rc = p->init_solve(&r->opts, r->opts.L, false, ctx->upstream);

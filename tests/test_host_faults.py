@@ -218,3 +218,48 @@ def test_a_gains_layout_where_no_thread_can_be_had(lib):
             ctx.close()
         assert shares[0] == shares[1]
         """)
+
+
+LATTICE_WS = 8 * (128 + 256) * 256 * 16                    # of lattice()'s 16 planes
+
+
+def held(ctx, sl1m, problems, budget=0):
+    """The server's info while it runs the problems' solves, which then end."""
+    ctx.server_start(mem_budget_bytes=budget, max_pairs_per_tick=1e12)
+    sl1m.fake.fake_hold(1)
+    tickets = [ctx.server_submit(P, 1.0, L=1.0, max_iter=5) for P in problems]
+    wait_for(lambda: ctx.server_info()["active"] == len(problems))
+    info = ctx.server_info()
+    sl1m.fake.fake_hold(0)
+    for t, P in zip(tickets, problems):
+        ctx.server_wait(t, P, 60)
+    assert ctx.server_info()["bytes_in_use"] == 0 and faults(sl1m) == ""
+    ctx.server_stop()
+    return info
+
+
+@pytest.mark.parametrize("first", ["laid out before", "laid out by the server"])
+def test_a_lattice_operator_counts_against_the_servers_budget(sl1m, first):
+    """Without room for it the solve takes the pair kernels, there only."""
+    ctx = sl1m.Context(0)
+    P = lattice(ctx)
+    if first == "laid out before":
+        P.forward(np.zeros(P.n_pix))
+        assert sl1m.fake.fake_count(2) == 1
+    sl1m.fake.fake_reset()
+    budget = 16 << 20                                      # the solve's 11 MB, not its lattice's 17, or 10 by halves
+    info = held(ctx, sl1m, [P], budget)
+    assert sl1m.fake.fake_count(0) > 0 and sl1m.fake.fake_count(2) == 0
+    assert 0 < info["bytes_in_use"] <= budget
+    sl1m.fake.fake_reset()
+    P.forward(np.zeros(P.n_pix))
+    assert sl1m.fake.fake_count(2) == 1 and faults(sl1m) == ""
+    ctx.close()
+
+
+def test_lattice_solves_of_a_server_share_one_workspace(sl1m):
+    ctx = sl1m.Context(0)
+    A, B = lattice(ctx), lattice(ctx)
+    one, two = (held(ctx, sl1m, ps)["bytes_in_use"] for ps in ([A], [A, B]))
+    assert two - LATTICE_WS == 2 * (one - LATTICE_WS) > 0
+    ctx.close()
