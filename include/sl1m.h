@@ -30,7 +30,8 @@
  *     without gains take, where that is faster, an FP32 gridding and FFT
  *     operator instead, whose result is nearer FP64's than the pairs' is.  It
  *     needs tables and a workspace of up to 4 GB, which the problems of a
- *     context share; whether it is taken, and how many of its planes it works
+ *     context share until the last of them on a lattice, or the context, is
+ *     destroyed; whether it is taken, and how many of its planes it works
  *     on at a time, follows the memory that is free when a problem is laid out,
  *     so equal calls of two runs can differ by rounding.
  */

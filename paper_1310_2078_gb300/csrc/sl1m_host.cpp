@@ -1768,6 +1768,9 @@ int sl1m_problem_destroy(sl1m_problem* prob)
     cudaStreamSynchronize(ctx->stream);
     ctx->problems.erase(std::remove(ctx->problems.begin(), ctx->problems.end(), prob), ctx->problems.end());
     delete prob;
+    // the lattice workspace goes with the last lattice problem (a server's loop may be growing it)
+    const auto on_lattice = [](const sl1m_problem* p) { return p->grid != nullptr; };
+    if (!ctx->server && std::none_of(ctx->problems.begin(), ctx->problems.end(), on_lattice)) ctx->grid_ws.free();
     return SL1M_OK;
 }
 

@@ -263,3 +263,19 @@ def test_lattice_solves_of_a_server_share_one_workspace(sl1m):
     one, two = (held(ctx, sl1m, ps)["bytes_in_use"] for ps in ([A], [A, B]))
     assert two - LATTICE_WS == 2 * (one - LATTICE_WS) > 0
     ctx.close()
+
+
+def test_the_lattice_workspace_goes_with_the_last_lattice_problem(sl1m):
+    ctx = sl1m.Context(0)
+    A, B, S = lattice(ctx), lattice(ctx), scattered(ctx)
+    for P in (S, A, B):
+        P.forward(np.zeros(P.n_pix))
+    A.close()
+    before = sl1m.fake.fake_held()
+    B.close()
+    assert before - sl1m.fake.fake_held() > LATTICE_WS
+    C = lattice(ctx)
+    for P in (S, C):
+        P.forward(np.zeros(P.n_pix))
+    assert sl1m.fake.fake_count(2) == 3 and faults(sl1m) == ""
+    ctx.close()
