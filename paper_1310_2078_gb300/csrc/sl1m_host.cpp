@@ -1027,8 +1027,9 @@ const UnitCost& sl1m_problem::unit_cost(int precision, int op)
 }
 
 // Device bytes a problem will hold once laid out with solver buffers
-// (admission estimate; padded sizes, ~100 B per element and side).
-size_t sl1m_problem::estimate_bytes() const
+// (admission estimate; padded sizes, ~100 B per element and side), without a
+// lattice operator's.
+size_t sl1m_problem::estimate_bytes(int precision) const
 {
     const size_t nv = (size_t)((n_vis + G - 1) / G) * G, np = (size_t)((n_pix + G - 1) / G) * G;
     size_t b = nv * (4 * 16 + 32 + 4 + 8 + 16) + np * (4 * 16 + 32 + 4 + 16 + 32);
@@ -1038,6 +1039,8 @@ size_t sl1m_problem::estimate_bytes() const
     }
     b += np * 8 * 4 + nv * 16 * 3;                 // solver vectors
     b += nv * (16 + 8);                            // the adjoint's FP32 Gaussian terms and residual
+    if (any_gauss) b += np * 16 + (np / G) * 4 + nv * 16 * GCLS_MAX;   // pixel offsets, constants per scale
+    if (precision == SL1M_FP64 && n_ant == 0) b += nv * 16;                // the FP64 adjoint's residual
     b += (nv + np) * 16 * 3;                       // operator scratch
     return b + (1 << 16);
 }
@@ -1872,6 +1875,7 @@ int sl1m_set_pixels(sl1m_problem* prob, int64_t n_pix, const double* lm, const d
         prob->kind.clear();
         prob->sigma.clear();
     }
+    prob->any_gauss = std::any_of(prob->kind.begin(), prob->kind.end(), [](int k) { return k != 0; });
     if (prob->n_ant > 0 && (int64_t)prob->gains.size() != 2 * n_pix * prob->n_ant) {
         prob->n_ant = 0;
         prob->gains.clear();

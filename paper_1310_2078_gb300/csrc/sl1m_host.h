@@ -274,6 +274,7 @@ struct sl1m_problem {
     int n_ant = 0;
     std::vector<double> uvw, vis, weights, lm, sigma, gains;
     std::vector<int> ant, kind;
+    bool any_gauss = false;                    // a pixel of a Gaussian kind
     // device layout
     bool dirty = true;
     bool has_gauss = false;
@@ -314,7 +315,7 @@ struct sl1m_problem {
     sl1m::DevProblem solver_desc() const;
     double pairs() const;
     size_t dev_bytes() const;
-    size_t estimate_bytes() const;
+    size_t estimate_bytes(int precision) const;
     ~sl1m_problem();
 };
 

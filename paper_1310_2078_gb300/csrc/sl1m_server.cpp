@@ -119,7 +119,7 @@ static void admit_in_arrival_order(Server& S, std::vector<Request*>& admit)
     for (Request* r : S.active) work += r->prob->pairs();
     while (!S.pending.empty() && (int)(S.active.size() + admit.size()) < S.max_slots) {
         Request* r = S.pending.front();
-        const size_t need = r->prob->estimate_bytes();
+        const size_t need = r->prob->estimate_bytes(S.precision);
         const bool first = S.active.empty() && admit.empty();
         if (S.in_use + need > S.budget && !first) break;
         if (work + r->prob->pairs() > S.max_pairs && !first) break;
@@ -166,7 +166,7 @@ static void admit_two_lanes(Server& S, std::vector<Request*>& admit)
             ++it;
             continue;
         }
-        const size_t need = r->prob->estimate_bytes();
+        const size_t need = r->prob->estimate_bytes(S.precision);
         const bool first = S.active.empty() && admit.empty();
         const bool mem_ok = S.in_use + need <= S.budget || first;
         const bool work_ok = small ? (work_small + w <= small_budget || first)
@@ -359,7 +359,7 @@ int sl1m_server_submit(sl1m_ctx* ctx, sl1m_problem* prob, const sl1m_solve_opts*
     if (prob->n_vis <= 0 || prob->n_pix <= 0) return sl1m_fail(ctx, SL1M_ERR_STATE, "problem incomplete");
     if (!(o->lambda >= 0) || !(o->L >= 0) || o->max_iter < 0 || !(o->rel_tol >= 0))
         return sl1m_fail(ctx, SL1M_ERR_ARG, "bad solver options");
-    if (prob->estimate_bytes() > S->budget)
+    if (prob->estimate_bytes(S->precision) > S->budget)
         return sl1m_fail(ctx, SL1M_ERR_BUSY, "problem exceeds the server memory budget");
     auto r = std::make_unique<Request>();
     r->prob = prob;

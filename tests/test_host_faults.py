@@ -279,3 +279,31 @@ def test_the_lattice_workspace_goes_with_the_last_lattice_problem(sl1m):
         P.forward(np.zeros(P.n_pix))
     assert sl1m.fake.fake_count(2) == 3 and faults(sl1m) == ""
     ctx.close()
+
+
+@pytest.mark.parametrize("gains", [False, True])
+@pytest.mark.parametrize("scales", [1, 4])
+def test_admission_counts_what_a_laid_out_problem_holds(sl1m, scales, gains):
+    """Gaussian pixels of few scales, every buffer there is, in FP64."""
+    rng = np.random.default_rng(2)
+    uvw, ant = synth.uvw_tracks(synth.antennas(rng, 24, 800.0, 20.0), -30.0, 10)
+    lm = rng.uniform(-0.2, 0.2, (1024, 2))
+    ctx = sl1m.Context(0)
+    P = ctx.problem()
+    P.set_visibilities(uvw, None, None, ant)
+    P.set_pixels(lm, np.resize(1e-3 * np.arange(1, scales + 1), 1024), np.full(1024, 2, np.int32))
+    if gains:
+        P.set_gains(synth.beam_gains(rng, lm, 24))
+    for prec in (sl1m.FP64, sl1m.MIXED):
+        P.forward(np.zeros(1024), prec)
+        P.adjoint(np.zeros(len(uvw), complex), prec)
+    P.solve(1.0, L=1.0, max_iter=1)
+    ctx.server_start(precision=sl1m.FP64)
+    sl1m.fake.fake_hold(1)
+    t = ctx.server_submit(P, 1.0, L=1.0, max_iter=5)
+    wait_for(lambda: ctx.server_info()["active"] == 1)
+    in_use, holds = ctx.server_info()["bytes_in_use"], P.bytes()
+    sl1m.fake.fake_hold(0)
+    ctx.server_wait(t, P, 60)
+    assert in_use >= holds
+    ctx.close()
