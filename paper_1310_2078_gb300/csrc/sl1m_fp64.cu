@@ -35,7 +35,7 @@ namespace sl1m {
 constexpr int CIRC = (int)R64_TURN;                 // table points of the circle, and of [1, 2) for 2^x
 static_assert(FP64_SUB == G, "a unit streams one element");
 
-// e^{2 pi i k / CIRC} and 2^(k / CIRC), filled once per device (fp64_init_tables).
+// e^{2 pi i k / CIRC} and 2^(k / CIRC), filled for a device's first context (fp64_init_tables).
 __device__ double2 g_circ[CIRC];
 __device__ double g_exp2[CIRC];
 

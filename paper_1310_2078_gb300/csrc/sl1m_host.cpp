@@ -583,9 +583,36 @@ void sl1m_ctx::drain_profile()
     pending.clear();
 }
 
+// The FP64 kernels' tables, which all contexts of a device read: written for the
+// first of them, before any kernel of theirs, and again only when none is left
+// (the device may have been reset since).
+static std::mutex g_tables_mu;
+static std::map<int, int>& g_tables_users = *new std::map<int, int>;   // contexts by device (outlives them all)
+
+static cudaError_t fp64_tables_acquire(sl1m_ctx* c)
+{
+    std::lock_guard<std::mutex> lk(g_tables_mu);
+    int& users = g_tables_users[c->device];
+    if (users == 0) {
+        cudaError_t e = fp64_init_tables(c->upstream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(c->upstream);
+        if (e != cudaSuccess) return e;
+    }
+    ++users;
+    c->has_tables = true;
+    return cudaSuccess;
+}
+static void fp64_tables_release(sl1m_ctx* c)
+{
+    if (!c->has_tables) return;
+    std::lock_guard<std::mutex> lk(g_tables_mu);
+    --g_tables_users[c->device];
+}
+
 sl1m_ctx::~sl1m_ctx()
 {
     cudaSetDevice(device);
+    fp64_tables_release(this);
     drain_profile();
     for (auto e : ev_pool) cudaEventDestroy(e);
     if (upstream) cudaStreamDestroy(upstream);
@@ -1705,7 +1732,7 @@ int sl1m_create(sl1m_ctx** out, int device, void* cuda_stream)
         c->own_stream = true;
     }
     if (cudaStreamCreateWithFlags(&c->upstream, cudaStreamNonBlocking) != cudaSuccess ||
-        fp64_init_tables(c->stream) != cudaSuccess) {
+        fp64_tables_acquire(c) != cudaSuccess) {
         delete c;
         return SL1M_ERR_CUDA;
     }

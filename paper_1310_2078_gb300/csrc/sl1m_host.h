@@ -220,6 +220,7 @@ struct sl1m_ctx {
     cudaStream_t stream = nullptr;
     cudaStream_t upstream = nullptr;     // uploads of problems joining a running server
     bool own_stream = false;
+    bool has_tables = false;             // counts among the users of the device's FP64 tables
     int num_sms = 1;
     std::string err;                     // last error message, guarded by err_mu: a running
     mutable std::mutex err_mu;           // server thread reports failures here too

@@ -31,7 +31,7 @@ cudaError_t launch_adjoint(int precision, bool gains, int n_ant, const DevProble
 // which: 0 fwd fp64, 1 adj fp64, 2 fwd mixed, 3 adj mixed
 int occupancy(int which, bool gains, int n_ant, int nst = NST_DEFAULT);
 int fwd_smem_bytes(int n_ant, bool gains, int nst);
-// The FP64 kernels' tables on the current device; called by every new context.
+// Writes the FP64 kernels' tables on the current device; called for its first context.
 cudaError_t fp64_init_tables(cudaStream_t st);
 // Owned granules per block of a plan.  A CTA of the mixed gains adjoint works on
 // one pixel granule at a time with all its warps, so its blocks are granules:

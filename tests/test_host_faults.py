@@ -307,3 +307,18 @@ def test_admission_counts_what_a_laid_out_problem_holds(sl1m, scales, gains):
     ctx.server_wait(t, P, 60)
     assert in_use >= holds
     ctx.close()
+
+
+def test_the_fp64_tables_are_written_for_the_first_context(sl1m):
+    """Another context's kernels may be reading them."""
+    fills = lambda: sl1m.fake.fake_count(4)  # noqa: E731
+    a, b = sl1m.Context(0), sl1m.Context(0)
+    assert fills() == 1
+    a.close()
+    c = sl1m.Context(0)
+    assert fills() == 1
+    b.close()
+    c.close()
+    d = sl1m.Context(0)
+    assert fills() == 2
+    d.close()
