@@ -672,9 +672,16 @@ void sl1m_problem::set_grid(cudaStream_t st, size_t grid_budget)
     for (auto& b : solve_batch) b.reset();
     gen = ++g_layouts;
     grid_tried = grid_budget;
-    if (grid_budget == 0) grid_least = std::max<size_t>(1, grid_least);     // (not looked into)
-    else if (grid_build(*this, st, grid_budget))
-        ctx->h2d += (long long)(grid->cell.bytes() + grid->list.bytes() + grid->start.bytes());
+    if (grid_budget == 0) {
+        grid_least = std::max<size_t>(1, grid_least);                       // (not looked into)
+        return;
+    }
+    try {
+        if (grid_build(*this, st, grid_budget))
+            ctx->h2d += (long long)(grid->cell.bytes() + grid->list.bytes() + grid->start.bytes());
+    } catch (const std::bad_alloc&) {                                       // (host memory: the pair kernels need none)
+        cudaStreamSynchronize(st);
+    }
 }
 
 size_t sl1m_problem::grid_own_bytes() const

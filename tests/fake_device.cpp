@@ -33,6 +33,7 @@ using namespace sl1m;
 namespace {
 
 std::atomic<int> g_no_threads{0};                  // threads of the library's cannot be started
+std::atomic<size_t> g_host_limit{SIZE_MAX};        // host allocations above this throw
 
 std::recursive_mutex g_mu;
 std::map<const char*, size_t> g_live;              // device allocations
@@ -125,7 +126,8 @@ void* operator new(size_t n, const std::nothrow_t&) noexcept
 }
 void* operator new(size_t n)
 {
-    if (void* p = malloc(n)) return p;
+    void* p = n > g_host_limit ? nullptr : malloc(n);
+    if (p) return p;
     throw std::bad_alloc();
 }
 void operator delete(void* p) noexcept
@@ -155,6 +157,7 @@ void fake_reset()
 }
 void fake_fail(size_t min_bytes, int n) { LOCK; g_fail_min = min_bytes; g_fail_n = n; }
 void fake_no_threads(int on) { g_no_threads = on; }
+void fake_host_limit(size_t n) { g_host_limit = n; }
 void fake_hold(int on) { LOCK; g_hold = on; }
 void fake_total(size_t bytes) { LOCK; g_total = bytes; }
 size_t fake_held() { return g_held; }

@@ -48,7 +48,7 @@ def binding(lib):
     m.fake = m.load()
     for f, args, res in (("fake_faults", [], C.c_char_p), ("fake_reset", [], None),
                          ("fake_fail", [C.c_size_t, C.c_int], None), ("fake_total", [C.c_size_t], None), ("fake_hold", [C.c_int], None),
-                         ("fake_no_threads", [C.c_int], None),
+                         ("fake_no_threads", [C.c_int], None), ("fake_host_limit", [C.c_size_t], None),
                          ("fake_held", [], C.c_size_t), ("fake_peak", [], C.c_size_t),
                          ("fake_count", [C.c_int], C.c_longlong)):
         fn = getattr(m.fake, f)

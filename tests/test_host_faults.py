@@ -322,3 +322,23 @@ def test_the_fp64_tables_are_written_for_the_first_context(sl1m):
     d = sl1m.Context(0)
     assert fills() == 2
     d.close()
+
+
+def test_a_lattice_whose_tables_do_not_fit_host_memory_takes_the_pair_kernels(lib):
+    """4,096 tiles by 1,600 planes of offsets, 25 MB; everything else is below 20."""
+    in_a_child(lib, """
+        rng = np.random.default_rng(1)
+        for limit in (0, 20_000_000):
+            ctx = sl1m.Context(0)
+            P = ctx.problem()
+            P.set_visibilities(rng.uniform(-1, 1, (200_000, 3)) * [1000.0, 1000.0, 12000.0])
+            P.set_pixels(synth.regular_grid(512, 0.25))
+            sl1m.fake.fake_reset()
+            if limit:
+                sl1m.fake.fake_host_limit(limit)
+            P.forward(np.zeros(P.n_pix))
+            sl1m.fake.fake_host_limit(1 << 60)
+            assert (sl1m.fake.fake_count(0), sl1m.fake.fake_count(2)) == ((1, 0) if limit else (0, 1))
+            assert sl1m.fake.fake_faults() == b""
+            ctx.close()
+        """)
