@@ -107,10 +107,20 @@ extern "C" int sl1m_forward_noalloc(sl1m_problem* prob, const double* x_dev, dou
     }
     const DevProblem& lay = prob->hp;
     const bool gains = prob->n_ant > 0;
-    // work split of this single problem (host tables)
+    // work split of this single problem (host tables).  FP64 units are single
+    // pixels, so its CTAs end inside blocks and a block has more partial slots than
+    // a split by granules gives it; where these would not fit, CTAs take whole
+    // blocks, one slot each.
     HostPlan H;
     const int which = precision == SL1M_FP64 ? 0 : 2;
-    plan_host({lay.vis.n_blk}, {stream_units(precision == SL1M_FP64 ? 0 : 1, lay.pix.n_gran)}, ctx->num_sms * occupancy(which, gains, std::max(1, prob->n_ant)), H);
+    const std::vector<int> units = {stream_units(precision == SL1M_FP64 ? 0 : 1, lay.pix.n_gran)};
+    plan_host({lay.vis.n_blk}, units, ctx->num_sms * occupancy(which, gains, std::max(1, prob->n_ant)), H);
+    const auto slot_bytes = [&] { return sizeof(double2) * (size_t)std::max(1, H.n_slots) * BLK; };
+    const size_t others = sizeof(double) * lay.pix.n_pad + sizeof(double2) * lay.vis.n_pad + 16384 + 16 * (size_t)lay.vis.n_blk;
+    if (precision == SL1M_FP64 && others + slot_bytes() > SCRATCH_BYTES) {
+        H = HostPlan();
+        plan_host({lay.vis.n_blk}, units, lay.vis.n_blk, H);
+    }
     // carve the static scratch
     size_t off = 0;
     auto take = [&](size_t bytes) {
@@ -127,7 +137,7 @@ extern "C" int sl1m_forward_noalloc(sl1m_problem* prob, const double* x_dev, dou
     int* d_ncon = (int*)take(sizeof(int) * std::max<size_t>(1, H.ncon.size()));
     double* d_x = (double*)take(sizeof(double) * lay.pix.n_pad);
     double2* d_out = (double2*)take(sizeof(double2) * lay.vis.n_pad);
-    double2* d_part = (double2*)take(sizeof(double2) * (size_t)std::max(1, H.n_slots) * BLK);
+    double2* d_part = (double2*)take(slot_bytes());
     if (off > SCRATCH_BYTES)
         return sl1m_fail(ctx, SL1M_ERR_ARG,
                          "problem needs %zu bytes of scratch; sl1m_forward_noalloc holds %zu (32 MiB)", off,
