@@ -145,14 +145,16 @@ struct DevProblem {
     const double2* V;         // [vis.n_pad] measured visibilities (sorted)
     const float4* pgauss;     // [pix.n_pad] {l, m, (l^2+m^2)/2, nu = n-1+(l^2+m^2)/2}
     const float4* pgoff;      // [pix.n_pad] {dl, dm, dn, q}: offsets from the granule's centre, q that of
-                              // r^2/2 (centre_q); without Gaussian pixels: pgauss (not read)
+                              // r^2/2 (centre_q); paraxial granules: the offset of nu in place of dn;
+                              // without Gaussian pixels: pgauss (not read)
     const d4* pgauss64;       // pgauss in FP64
     const float* gsig;        // [pix.n_gran] sigma per pixel granule (FP32 path)
     const double* gsig64;     // [pix.n_gran] sigma per pixel granule (FP64 path)
     const int* gkind;         // [pix.n_gran] kind per pixel granule
     const int* gclass;        // [pix.n_gran] the granule's scale in gcls, -1 if none, or null
     const float4* gcls;       // [scales][vis.n_pad] constants of (visibility, Gaussian scale), or null
-    const float4* pghdr;      // [pix.n_gran][4] centre hi, centre lo, extent, {sigma, kind, nu at the centre, scale in gcls or -1}
+    const float4* pghdr;      // [pix.n_gran][4] centre hi, centre lo, extent (w: lo of nu at the centre),
+                              // {sigma, kind, hi of nu at the centre, scale in gcls or -1}
     const float4* vgabs;      // [vis.n_pad] {u, v, -2 w, u^2 + v^2} in FP32 (the adjoint's Gaussian terms)
     float2* r32;              // [vis.n_pad] the mixed adjoint's input residual in polar form,
                               // {|r|, arg r in turns} in FP32

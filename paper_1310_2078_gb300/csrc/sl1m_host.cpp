@@ -795,13 +795,18 @@ int sl1m_problem::rebuild(cudaStream_t st, size_t grid_budget)
             hdr[4 * (size_t)g] = H.cen_hi[g];
             hdr[4 * (size_t)g + 1] = H.cen_lo[g];
             hdr[4 * (size_t)g + 2] = H.ext[g];
-            const double cl = (double)H.cen_hi[g].x + H.cen_lo[g].x, cm = (double)H.cen_hi[g].y + H.cen_lo[g].y,
-                         cn = (double)H.cen_hi[g].z + H.cen_lo[g].z;
+            // nu at the centre: that of its n - 1 and of the q's zero, so that the
+            // offsets of nu are those of n - 1 and q together
+            const double cn = (double)H.cen_hi[g].z + H.cen_lo[g].z;
             const float qc = 0.5f * std::fmaf(H.cen_hi[g].x, H.cen_hi[g].x, H.cen_hi[g].y * H.cen_hi[g].y);
-            hdr[4 * (size_t)g + 3] = make_float4(gs[g], (float)gk[g], (float)(cn + 0.5 * (cl * cl + cm * cm)), -1.f);
+            const double nuc = cn + (double)qc;
+            hdr[4 * (size_t)g + 2].w = f32lo(nuc);
+            hdr[4 * (size_t)g + 3] = make_float4(gs[g], (float)gk[g], f32hi(nuc), -1.f);
             if (has_gauss)
                 for (int t = g * G; t < (g + 1) * G; ++t)
-                    pgo[t] = make_float4(H.off[t].x, H.off[t].y, H.off[t].z, (float)(pg64[t].z - (double)qc));
+                    pgo[t] = make_float4(H.off[t].x, H.off[t].y,
+                                         gk[g] == PARAXIAL ? (float)(pg64[t].w - nuc) : H.off[t].z,
+                                         (float)(pg64[t].z - (double)qc));
         }
         D.pgoff.free();
         if (has_gauss) CK(D.pgoff.upload(pgo.data(), pgo.size(), st));

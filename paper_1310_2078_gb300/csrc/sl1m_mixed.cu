@@ -122,22 +122,25 @@ __device__ __forceinline__ float4 gauss_class(const float4 uvw, float sigma)
 // streamed pixel's offsets y = (dl, dm, dn, q), q = r^2/2 - qc, from its granule's
 // centre (t = u l + v m - w r^2/2 = tc + u dl + v dm - w q), so a lane holds their
 // coefficients for the tile,
-//   phase  p = {2 pi du - gam u, 2 pi dv - gam v, 2 pi dw, gam w} (radians;
-//          paraxial: - 2 pi w on the last two)
+//   phase  p = {2 pi du - gam u, 2 pi dv - gam v, 2 pi dw, gam w} (radians)
 //   exponent e = {k1 u, k1 v, - k1 w, k0 + k1 tc}
 // and what belongs to the centre (gam tc, the constant phase, paraxial w nu_c) is
 // in its C term: 7 FFMA a pair and one 16-byte load, where t, its products and
 // the offset phase took 3 + 3 + 2 and two loads.  EXACT: p without the product
 // of the offsets, which is reduced exactly.
+// Paraxial pixels add - w nu, nu = n - 1 + r^2/2, which dn and q nearly cancel to:
+// w times either, rounded, was up to 30 times the operator's error (w 900, 0.5 off
+// the centre).  They hold the offset of nu instead of dn = dnu - q, so p3 =
+// 2 pi (dw - w), p4 = gam w - 2 pi dw.
 struct GaussTile {
     float4 p, e;
     float beta, id;
 };
 // x = {u, v, w}, dx: its offset (radians; zero when EXACT); yc: the streamed
-// granule's centre, nuc = nu at it.  C (turns) gains the centre's share.  cls:
+// granule's centre, nuc = nu at it (hi and lo).  C (turns) gains the centre's share.  cls:
 // the visibility's constants of the scale (gauss_class, which has the factor id
 // (1 + i beta) in it), or null: formed here, and the factor left to the caller.
-__device__ __forceinline__ GaussTile gauss_tile(const float4 x, const float4 dx, const float4 yc, float nuc, float sigma,
+__device__ __forceinline__ GaussTile gauss_tile(const float4 x, const float4 dx, const float4 yc, float2 nuc, float sigma,
                                                 bool par, const float4* cls, float& C)
 {
     GaussTile g;
@@ -156,9 +159,9 @@ __device__ __forceinline__ GaussTile gauss_tile(const float4 x, const float4 dx,
     const float tc = fmaf(x.x, yc.x, fmaf(x.y, yc.y, -x.z * qc));
     C = frac_turns(C + k.w);
     C = frac_turns(fmaf(-k.x * INV_TWO_PI_F, tc, C));
-    if (par) C = frac_turns(fmaf(-x.z, nuc, C));
-    const float wp = par ? -TWO_PI_F * x.z : 0.f;
-    g.p = make_float4(fmaf(-k.x, x.x, dx.x), fmaf(-k.x, x.y, dx.y), dx.z + wp, fmaf(k.x, x.z, wp));
+    if (par) C = frac_turns(C - tp_frac(x.z, 0.f, nuc.x, nuc.y));
+    g.p = make_float4(fmaf(-k.x, x.x, dx.x), fmaf(-k.x, x.y, dx.y), par ? fmaf(-TWO_PI_F, x.z, dx.z) : dx.z,
+                      par ? fmaf(k.x, x.z, -dx.z) : k.x * x.z);
     g.e = make_float4(k.y * x.x, k.y * x.y, -k.y * x.z, fmaf(k.y, tc, k.z));
     return g;
 }
@@ -544,12 +547,13 @@ fwd_mixed_kernel(const DevProblem* __restrict__ probs, const Plan* __restrict__ 
                     }
                 } else {
                     const bool par = (kind == PARAXIAL);
+                    const float2 nuc = make_float2(meta.z, s_hdr[4 * q + 2].w);
                     GaussTile gt[2];
                     const int scale = (int)meta.w;                       // -1: no table
                     const float4* const cls = scale >= 0 ? P.gcls + (size_t)scale * P.vis.n_pad + e0 : nullptr;
 #pragma unroll
                     for (int r = 0; r < 2; ++r)
-                        gt[r] = gauss_tile(xh[r], exact ? z4 : dx[r], yc_h, meta.z, meta.x, par,
+                        gt[r] = gauss_tile(xh[r], exact ? z4 : dx[r], yc_h, nuc, meta.x, par,
                                            cls ? cls + 32 * r : nullptr, C[r]);
                     if (exact) {
                         const float4 dxt[2] = {P.vis.off[e0], P.vis.off[e0 + 32]},
@@ -1118,7 +1122,8 @@ adj_mixed_gains_kernel(const DevProblem* __restrict__ probs, const Plan* __restr
         const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
         float4 xh[2], dx[2], y[2] = {z4, z4};
         // the granule's centre, which the Gaussian terms are taken from
-        const float qc = centre_q(ch.x, ch.y), nuc = P.pghdr[4 * (size_t)pgi + 3].z;
+        const float qc = centre_q(ch.x, ch.y), nuh = P.pghdr[4 * (size_t)pgi + 3].z,
+                    nul = P.pghdr[4 * (size_t)pgi + 2].w;
         const float4* const cls = gauss && P.gclass && P.gclass[pgi] >= 0
                                       ? P.gcls + (size_t)P.gclass[pgi] * P.vis.n_pad : nullptr;
 #pragma unroll
@@ -1153,11 +1158,11 @@ adj_mixed_gains_kernel(const DevProblem* __restrict__ probs, const Plan* __restr
                     const float tc = fmaf(x.x, ch.x, fmaf(x.y, ch.y, -x.z * qc));
                     b = frac_turns(b + gc.w);
                     b = frac_turns(fmaf(-gc.x * INV_TWO_PI_F, tc, b + rp.y));
-                    if (par) b = frac_turns(fmaf(-x.z, nuc, b));
-                    const float wp = par ? -TWO_PI_F * x.z : 0.f;
+                    if (par) b = frac_turns(b - tp_frac(x.z, 0.f, nuh, nul));
                     o = exact ? z4 : to_rad(o);
-                    s_off[warp][k] = make_float4(fmaf(-gc.x, x.x, o.x), fmaf(-gc.x, x.y, o.y), o.z + wp,
-                                                 fmaf(gc.x, x.z, wp));
+                    s_off[warp][k] = make_float4(fmaf(-gc.x, x.x, o.x), fmaf(-gc.x, x.y, o.y),
+                                                 par ? fmaf(-TWO_PI_F, x.z, o.z) : o.z,
+                                                 par ? fmaf(gc.x, x.z, -o.z) : gc.x * x.z);
                     s_va[warp][k] = make_float4(gc.y * x.x, gc.y * x.y, -gc.y * x.z, fmaf(gc.y, tc, gc.z) + __log2f(rp.x));
                     kr.y = b * TWO_PI_F;
                 } else {
