@@ -153,8 +153,8 @@ struct DevProblem {
     const int* gkind;         // [pix.n_gran] kind per pixel granule
     const int* gclass;        // [pix.n_gran] the granule's scale in gcls, -1 if none, or null
     const float4* gcls;       // [scales][vis.n_pad] constants of (visibility, Gaussian scale), or null
-    const float4* pghdr;      // [pix.n_gran][4] centre hi, centre lo, extent (w: lo of nu at the centre),
-                              // {sigma, kind, hi of nu at the centre, scale in gcls or -1}
+    const float4* pghdr;      // [pix.n_gran][4] centre hi, centre lo (w: kappa), extent (w: lo of nu's middle),
+                              // {sigma, kind, hi of nu's middle, scale in gcls or -1}
     const float4* vgabs;      // [vis.n_pad] {u, v, -2 w, u^2 + v^2} in FP32 (the adjoint's Gaussian terms)
     float2* r32;              // [vis.n_pad] the mixed adjoint's input residual in polar form,
                               // {|r|, arg r in turns} in FP32

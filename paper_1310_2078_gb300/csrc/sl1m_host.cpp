@@ -795,11 +795,18 @@ int sl1m_problem::rebuild(cudaStream_t st, size_t grid_budget)
             hdr[4 * (size_t)g] = H.cen_hi[g];
             hdr[4 * (size_t)g + 1] = H.cen_lo[g];
             hdr[4 * (size_t)g + 2] = H.ext[g];
-            // nu at the centre: that of its n - 1 and of the q's zero, so that the
-            // offsets of nu are those of n - 1 and q together
+            // nu in the middle of the granule's, and how far that is from the n - 1 and
+            // the r^2/2 that the offsets dn and q are taken from (a box's middle is not
+            // on the sphere): dn = dnu - q + kappa
             const double cn = (double)H.cen_hi[g].z + H.cen_lo[g].z;
             const float qc = 0.5f * std::fmaf(H.cen_hi[g].x, H.cen_hi[g].x, H.cen_hi[g].y * H.cen_hi[g].y);
-            const double nuc = cn + (double)qc;
+            double nu0 = 1e300, nu1 = -1e300;
+            for (int t = g * G; t < (g + 1) * G; ++t) {
+                nu0 = std::min(nu0, pg64[t].w);
+                nu1 = std::max(nu1, pg64[t].w);
+            }
+            const double nuc = 0.5 * (nu0 + nu1);
+            hdr[4 * (size_t)g + 1].w = (float)(nuc - cn - (double)qc);
             hdr[4 * (size_t)g + 2].w = f32lo(nuc);
             hdr[4 * (size_t)g + 3] = make_float4(gs[g], (float)gk[g], f32hi(nuc), -1.f);
             if (has_gauss)

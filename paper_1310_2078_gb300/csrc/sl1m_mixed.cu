@@ -130,17 +130,17 @@ __device__ __forceinline__ float4 gauss_class(const float4 uvw, float sigma)
 // of the offsets, which is reduced exactly.
 // Paraxial pixels add - w nu, nu = n - 1 + r^2/2, which dn and q nearly cancel to:
 // w times either, rounded, was up to 30 times the operator's error (w 900, 0.5 off
-// the centre).  They hold the offset of nu instead of dn = dnu - q, so p3 =
-// 2 pi (dw - w), p4 = gam w - 2 pi dw.
+// the centre).  They hold the offset of nu instead of dn = dnu - q + kappa, so p3 =
+// 2 pi (dw - w), p4 = gam w - 2 pi dw, and C gains dw kappa - w nu's middle.
 struct GaussTile {
     float4 p, e;
     float beta, id;
 };
 // x = {u, v, w}, dx: its offset (radians; zero when EXACT); yc: the streamed
-// granule's centre, nuc = nu at it (hi and lo).  C (turns) gains the centre's share.  cls:
+// granule's centre, nuc = {nu's middle hi, lo, kappa}.  C (turns) gains the centre's share.  cls:
 // the visibility's constants of the scale (gauss_class, which has the factor id
 // (1 + i beta) in it), or null: formed here, and the factor left to the caller.
-__device__ __forceinline__ GaussTile gauss_tile(const float4 x, const float4 dx, const float4 yc, float2 nuc, float sigma,
+__device__ __forceinline__ GaussTile gauss_tile(const float4 x, const float4 dx, const float4 yc, float3 nuc, float sigma,
                                                 bool par, const float4* cls, float& C)
 {
     GaussTile g;
@@ -160,6 +160,7 @@ __device__ __forceinline__ GaussTile gauss_tile(const float4 x, const float4 dx,
     C = frac_turns(C + k.w);
     C = frac_turns(fmaf(-k.x * INV_TWO_PI_F, tc, C));
     if (par) C = frac_turns(C - tp_frac(x.z, 0.f, nuc.x, nuc.y));
+    if (par) C = frac_turns(fmaf(dx.z * INV_TWO_PI_F, nuc.z, C));
     g.p = make_float4(fmaf(-k.x, x.x, dx.x), fmaf(-k.x, x.y, dx.y), par ? fmaf(-TWO_PI_F, x.z, dx.z) : dx.z,
                       par ? fmaf(k.x, x.z, -dx.z) : k.x * x.z);
     g.e = make_float4(k.y * x.x, k.y * x.y, -k.y * x.z, fmaf(k.y, tc, k.z));
@@ -326,7 +327,7 @@ __device__ __forceinline__ void fwd_gauss_tile_pt(const float4* __restrict__ s_o
 // Forward stage buffers in dynamic shared memory: two of them, each holding
 // NST streamed pixel granules as they sit in HBM -- offsets {dl, dm, dn, 1/n},
 // offset residuals, Gaussian data {dl, dm, dn, q}, x (FP64) and the granule
-// headers {centre hi, centre lo, extent, {sigma, kind, nu at the centre, scale}} -- filled by bulk (TMA)
+// headers {centre hi, centre lo, extent, {sigma, kind, hi of nu's middle, scale}} -- filled by bulk (TMA)
 // copies that complete on one mbarrier per buffer.  The copies of stage s + 1
 // are issued when stage s starts, so they land while stage s is computed.
 template <int NST>
@@ -502,7 +503,7 @@ fwd_mixed_kernel(const DevProblem* __restrict__ probs, const Plan* __restrict__ 
             }
             __syncwarp();
             for (int q = 0; q < ns; ++q) {
-                const float4 meta = s_hdr[4 * q + 3];                    // {sigma, kind, nu at the centre, scale}
+                const float4 meta = s_hdr[4 * q + 3];                    // {sigma, kind, hi of nu's middle, scale}
                 const int kind = (int)meta.y;
                 const float4 yc_h = s_hdr[4 * q], yc_l = s_hdr[4 * q + 1];
                 const bool exact = dot3(ext, s_hdr[4 * q + 2]) > D_MAX;  // warp-uniform
@@ -547,7 +548,7 @@ fwd_mixed_kernel(const DevProblem* __restrict__ probs, const Plan* __restrict__ 
                     }
                 } else {
                     const bool par = (kind == PARAXIAL);
-                    const float2 nuc = make_float2(meta.z, s_hdr[4 * q + 2].w);
+                    const float3 nuc = make_float3(meta.z, s_hdr[4 * q + 2].w, yc_l.w);
                     GaussTile gt[2];
                     const int scale = (int)meta.w;                       // -1: no table
                     const float4* const cls = scale >= 0 ? P.gcls + (size_t)scale * P.vis.n_pad + e0 : nullptr;
@@ -1123,7 +1124,7 @@ adj_mixed_gains_kernel(const DevProblem* __restrict__ probs, const Plan* __restr
         float4 xh[2], dx[2], y[2] = {z4, z4};
         // the granule's centre, which the Gaussian terms are taken from
         const float qc = centre_q(ch.x, ch.y), nuh = P.pghdr[4 * (size_t)pgi + 3].z,
-                    nul = P.pghdr[4 * (size_t)pgi + 2].w;
+                    nul = P.pghdr[4 * (size_t)pgi + 2].w, kappa = P.pghdr[4 * (size_t)pgi + 1].w;
         const float4* const cls = gauss && P.gclass && P.gclass[pgi] >= 0
                                       ? P.gcls + (size_t)P.gclass[pgi] * P.vis.n_pad : nullptr;
 #pragma unroll
@@ -1159,6 +1160,7 @@ adj_mixed_gains_kernel(const DevProblem* __restrict__ probs, const Plan* __restr
                     b = frac_turns(b + gc.w);
                     b = frac_turns(fmaf(-gc.x * INV_TWO_PI_F, tc, b + rp.y));
                     if (par) b = frac_turns(b - tp_frac(x.z, 0.f, nuh, nul));
+                    if (par && !exact) b = frac_turns(fmaf(o.z, kappa, b));
                     o = exact ? z4 : to_rad(o);
                     s_off[warp][k] = make_float4(fmaf(-gc.x, x.x, o.x), fmaf(-gc.x, x.y, o.y),
                                                  par ? fmaf(-TWO_PI_F, x.z, o.z) : o.z,
