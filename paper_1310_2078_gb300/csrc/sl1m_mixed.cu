@@ -126,8 +126,11 @@ __device__ __forceinline__ float4 gauss_class(const float4 uvw, float sigma)
 //   exponent e = {k1 u, k1 v, - k1 w, k0 + k1 tc}
 // and what belongs to the centre (gam tc, the constant phase, paraxial w nu_c) is
 // in its C term: 7 FFMA a pair and one 16-byte load, where t, its products and
-// the offset phase took 3 + 3 + 2 and two loads.  EXACT: p without the product
-// of the offsets, which is reduced exactly.
+// the offset phase took 3 + 3 + 2 and two loads.  EXACT: the product of the offsets
+// is reduced exactly, and what is left of p is - gam, of e k1, times t - tc, so a
+// lane forms that (3 FFMA) and takes both from it: p = {u, v, - w, gam / 2 pi}, e.w
+// as above, e.x = k1 (a linear p and e without the offsets are 4 + 3: the forward of
+// 133,956 multiscale pixels x 16,557 visibilities took 1.5% longer so).
 // Paraxial pixels add - w nu, nu = n - 1 + r^2/2, which dn and q nearly cancel to:
 // w times either, rounded, was up to 30 times the operator's error (w 900, 0.5 off
 // the centre).  They hold the offset of nu instead of dn = dnu - q + kappa, so p3 =
@@ -136,12 +139,12 @@ struct GaussTile {
     float4 p, e;
     float beta, id;
 };
-// x = {u, v, w}, dx: its offset (radians; zero when EXACT); yc: the streamed
+// x = {u, v, w}, dx: its offset (radians; not read when exact); yc: the streamed
 // granule's centre, nuc = {nu's middle hi, lo, kappa}.  C (turns) gains the centre's share.  cls:
 // the visibility's constants of the scale (gauss_class, which has the factor id
 // (1 + i beta) in it), or null: formed here, and the factor left to the caller.
 __device__ __forceinline__ GaussTile gauss_tile(const float4 x, const float4 dx, const float4 yc, float3 nuc, float sigma,
-                                                bool par, const float4* cls, float& C)
+                                                bool par, bool exact, const float4* cls, float& C)
 {
     GaussTile g;
     float4 k;                                        // gam (radians), k1, k0, constant phase (turns)
@@ -160,10 +163,14 @@ __device__ __forceinline__ GaussTile gauss_tile(const float4 x, const float4 dx,
     C = frac_turns(C + k.w);
     C = frac_turns(fmaf(-k.x * INV_TWO_PI_F, tc, C));
     if (par) C = frac_turns(C - tp_frac(x.z, 0.f, nuc.x, nuc.y));
-    if (par) C = frac_turns(fmaf(dx.z * INV_TWO_PI_F, nuc.z, C));
+    if (par && !exact) C = frac_turns(fmaf(dx.z * INV_TWO_PI_F, nuc.z, C));
     g.p = make_float4(fmaf(-k.x, x.x, dx.x), fmaf(-k.x, x.y, dx.y), par ? fmaf(-TWO_PI_F, x.z, dx.z) : dx.z,
                       par ? fmaf(k.x, x.z, -dx.z) : k.x * x.z);
     g.e = make_float4(k.y * x.x, k.y * x.y, -k.y * x.z, fmaf(k.y, tc, k.z));
+    if (exact) {
+        g.p = make_float4(x.x, x.y, -x.z, k.x * INV_TWO_PI_F);
+        g.e.x = k.y;
+    }
     return g;
 }
 __device__ __forceinline__ float lin4(const float4 a, const float4 y, float s)
@@ -174,8 +181,16 @@ __device__ __forceinline__ float lin3(const float4 e, const float4 y, float s)  
 {
     return fmaf(e.z, y.w, fmaf(e.y, y.y, fmaf(e.x, y.x, s)));
 }
+// EXACT: t - tc, and the phase (turns) with the offsets' product d; PAR: - w nu too.
+template <bool PAR>
+__device__ __forceinline__ float exact_phase(const float4 p, const float4 y, float t, float b, float d)
+{
+    float ph = fmaf(-p.w, t, fmaf(b, INV_TWO_PI_F, d));
+    if (PAR) ph = fmaf(p.z, y.z, ph);
+    return frac_turns(ph);
+}
 
-template <bool GAINS, bool EXACT>
+template <bool GAINS, bool EXACT, bool PAR>
 __device__ __forceinline__ void fwd_gauss_tile(const float4* __restrict__ s_off,
                                                const float4* __restrict__ s_lo,
                                                const float4* __restrict__ s_pg,
@@ -187,7 +202,7 @@ __device__ __forceinline__ void fwd_gauss_tile(const float4* __restrict__ s_off,
 {
     const float2* ga_row[2] = {s_gain + ant[0].x * GP, s_gain + ant[1].x * GP};   // GAINS only
     const float2* gb_row[2] = {s_gain + ant[0].y * GP, s_gain + ant[1].y * GP};
-#pragma unroll(GAINS ? 1 : 4)   // the gains variant stays within its registers
+#pragma unroll(GAINS ? 1 : EXACT ? 2 : 4)   // (within the registers)
     for (int j = 0; j < G; ++j) {
         const float4 y = s_pg[j];              // {dl, dm, dn, q}
         const float2 ba = sBa[j];
@@ -199,12 +214,18 @@ __device__ __forceinline__ void fwd_gauss_tile(const float4* __restrict__ s_off,
                 gb = gb_row[r][j];
             }
             const float b0 = GAINS ? fmaf(gb.y - ga.y, TWO_PI_F, ba.x) : ba.x;
-            float ph = lin4(gt[r].p, y, b0);                 // radians
-            if (EXACT)
-                ph = frac_turns(fmaf(ph, INV_TWO_PI_F, frac_dot3(dx[r], dxl[r], s_off[j], s_lo[j]))) * TWO_PI_F;
+            float ph, ex;                                    // radians; exponent of two
+            if (EXACT) {
+                const float t = lin3(gt[r].p, y, 0.f);
+                ph = exact_phase<PAR>(gt[r].p, y, t, b0, frac_dot3(dx[r], dxl[r], s_off[j], s_lo[j])) * TWO_PI_F;
+                ex = fmaf(gt[r].e.x, t, gt[r].e.w);
+            } else {
+                ph = lin4(gt[r].p, y, b0);
+                ex = lin3(gt[r].e, y, gt[r].e.w);
+            }
             float sn, cs;
             __sincosf(ph, &sn, &cs);
-            float amp = ba.y * ex2_approx(lin3(gt[r].e, y, gt[r].e.w));   // (x/n) e^{Re(qc)}
+            float amp = ba.y * ex2_approx(ex);               // (x/n) e^{Re(qc)}
             if (GAINS) amp *= ga.x * gb.x;
             sr[r] = fmaf(amp, cs, sr[r]);
             si[r] = fmaf(-amp, sn, si[r]);
@@ -286,7 +307,7 @@ __device__ __forceinline__ void fwd_dirac_tile_pt(const float4* __restrict__ s_o
     }
 }
 
-template <bool EXACT>
+template <bool EXACT, bool PAR>
 __device__ __forceinline__ void fwd_gauss_tile_pt(const float4* __restrict__ s_off,
                                                   const float4* __restrict__ s_lo,
                                                   const float4* __restrict__ s_pg,
@@ -310,12 +331,18 @@ __device__ __forceinline__ void fwd_gauss_tile_pt(const float4* __restrict__ s_o
 #pragma unroll
             for (int r = 0; r < 2; ++r) {
                 const float2 tv = T[toff[r] + jj];                     // {B - arg, log2 |a g|}
-                float ph = lin4(gt[r].p, y, tv.x);
-                if (EXACT)
-                    ph = frac_turns(fmaf(ph, INV_TWO_PI_F, frac_dot3(dx[r], dxl[r], s_off[j], s_lo[j]))) * TWO_PI_F;
+                float ph, ex;                                          // radians; exponent of two
+                if (EXACT) {
+                    const float t = lin3(gt[r].p, y, 0.f);
+                    ph = exact_phase<PAR>(gt[r].p, y, t, tv.x, frac_dot3(dx[r], dxl[r], s_off[j], s_lo[j])) * TWO_PI_F;
+                    ex = fmaf(gt[r].e.x, t, gt[r].e.w + tv.y);
+                } else {
+                    ph = lin4(gt[r].p, y, tv.x);
+                    ex = lin3(gt[r].e, y, gt[r].e.w + tv.y);
+                }
                 float sn, cs;
                 __sincosf(ph, &sn, &cs);
-                const float amp = ex2_approx(lin3(gt[r].e, y, gt[r].e.w + tv.y));   // |a g| e^{Re(qc)}
+                const float amp = ex2_approx(ex);                      // |a g| e^{Re(qc)}
                 sr[r] = fmaf(amp, cs, sr[r]);
                 si[r] = fmaf(-amp, sn, si[r]);
             }
@@ -516,7 +543,7 @@ fwd_mixed_kernel(const DevProblem* __restrict__ probs, const Plan* __restrict__ 
                 for (int r = 0; r < 2; ++r) {
                     if (GAUSS) {                                         // (not held across granules)
                         xh[r] = reload4(P.vis.hi + e0 + 32 * r);
-                        dx[r] = to_rad(reload4(P.vis.off + e0 + 32 * r));
+                        if (!exact) dx[r] = to_rad(reload4(P.vis.off + e0 + 32 * r));
                     }
                     C[r] = frac_dot3(xh[r], P.vis.lo[e0 + 32 * r], yc_h, yc_l);
                 }
@@ -550,25 +577,30 @@ fwd_mixed_kernel(const DevProblem* __restrict__ probs, const Plan* __restrict__ 
                     const bool par = (kind == PARAXIAL);
                     const float3 nuc = make_float3(meta.z, s_hdr[4 * q + 2].w, yc_l.w);
                     GaussTile gt[2];
-                    const int scale = (int)meta.w;                       // -1: no table
+                    const int scale = exact ? -1 : (int)meta.w;          // -1: no table (an exact tile is long)
                     const float4* const cls = scale >= 0 ? P.gcls + (size_t)scale * P.vis.n_pad + e0 : nullptr;
 #pragma unroll
                     for (int r = 0; r < 2; ++r)
-                        gt[r] = gauss_tile(xh[r], exact ? z4 : dx[r], yc_h, nuc, meta.x, par,
+                        gt[r] = gauss_tile(xh[r], dx[r], yc_h, nuc, meta.x, par, exact,
                                            cls ? cls + 32 * r : nullptr, C[r]);
                     if (exact) {
                         const float4 dxt[2] = {P.vis.off[e0], P.vis.off[e0 + 32]},
                                      dxl[2] = {P.vis.offlo[e0], P.vis.offlo[e0 + 32]};
-                        if (GAINS && nb > 0)
-                            fwd_gauss_tile_pt<true>(q_off, q_lo, q_pg, q_Ba, gtab, s_pt[warp], s_bl[warp], nb, lch, toff, gt,
-                                                    dxt, dxl, lane, sr, si);
-                        else
-                            fwd_gauss_tile<GAINS, true>(q_off, q_lo, q_pg, q_Ba, gtab, gt, dxt, dxl, ant, sr, si);
+                        if (GAINS && nb > 0) {
+                            if (par) fwd_gauss_tile_pt<true, true>(q_off, q_lo, q_pg, q_Ba, gtab, s_pt[warp], s_bl[warp], nb,
+                                                                   lch, toff, gt, dxt, dxl, lane, sr, si);
+                            else fwd_gauss_tile_pt<true, false>(q_off, q_lo, q_pg, q_Ba, gtab, s_pt[warp], s_bl[warp], nb,
+                                                                lch, toff, gt, dxt, dxl, lane, sr, si);
+                        } else if (par) {
+                            fwd_gauss_tile<GAINS, true, true>(q_off, q_lo, q_pg, q_Ba, gtab, gt, dxt, dxl, ant, sr, si);
+                        } else {
+                            fwd_gauss_tile<GAINS, true, false>(q_off, q_lo, q_pg, q_Ba, gtab, gt, dxt, dxl, ant, sr, si);
+                        }
                     } else if (GAINS && nb > 0) {
-                        fwd_gauss_tile_pt<false>(q_off, q_lo, q_pg, q_Ba, gtab, s_pt[warp], s_bl[warp], nb, lch, toff, gt,
+                        fwd_gauss_tile_pt<false, false>(q_off, q_lo, q_pg, q_Ba, gtab, s_pt[warp], s_bl[warp], nb, lch, toff, gt,
                                                  dx, dx, lane, sr, si);
                     } else {
-                        fwd_gauss_tile<GAINS, false>(q_off, q_lo, q_pg, q_Ba, gtab, gt, dx, dx, ant, sr, si);
+                        fwd_gauss_tile<GAINS, false, false>(q_off, q_lo, q_pg, q_Ba, gtab, gt, dx, dx, ant, sr, si);
                     }
 #pragma unroll
                     for (int r = 0; r < 2; ++r) {
@@ -966,8 +998,8 @@ __device__ __forceinline__ void adjg_dirac_tile(const float4* __restrict__ s_off
 }
 
 // g_off, g_lo, dx, dxl (EXACT): the offsets of either side and their residuals
-// in turns, the coefficients then leave the product of the offsets out.
-template <bool EXACT, bool AL4, class GF>
+// in turns; p and e are then as gauss_tile's.
+template <bool EXACT, bool AL4, bool PAR, class GF>
 __device__ __forceinline__ void adjg_gauss_tile(const float4* __restrict__ s_p, const float4* __restrict__ s_e,
                                                 const float2* __restrict__ s_kr, const float4* __restrict__ g_off,
                                                 const float4* __restrict__ g_lo, const GF& gain,
@@ -986,11 +1018,16 @@ __device__ __forceinline__ void adjg_gauss_tile(const float4* __restrict__ s_p, 
         if (!AL4 || kk == 0) adjg_next_run<EXACT>(__float_as_int(kr.x), cur, gain, Ct, M, Phi, z, acc);
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
-            float ph = EXACT ? 0.f : kr.y + Phi[r];    // radians
-            ph = fmaf(p.w, y[r].w, fmaf(p.z, y[r].z, fmaf(p.y, y[r].y, fmaf(p.x, y[r].x, ph))));
-            if (EXACT)
-                ph = frac_turns(fmaf(ph + kr.y, INV_TWO_PI_F, Phi[r]) + frac_dot3(dx[r], dxl[r], g_off[k], g_lo[k])) * TWO_PI_F;
-            const float amp = ex2_approx(fmaf(e.z, y[r].w, fmaf(e.y, y[r].y, fmaf(e.x, y[r].x, e.w))));   // |r'| e^{Re(qc)}
+            float ph, ex;                              // radians; exponent of two
+            if (EXACT) {
+                const float t = lin3(p, y[r], 0.f);
+                ph = exact_phase<PAR>(p, y[r], t, kr.y, Phi[r] + frac_dot3(dx[r], dxl[r], g_off[k], g_lo[k])) * TWO_PI_F;
+                ex = fmaf(e.x, t, e.w);
+            } else {
+                ph = lin4(p, y[r], kr.y + Phi[r]);
+                ex = lin3(e, y[r], e.w);
+            }
+            const float amp = ex2_approx(ex);          // |r'| e^{Re(qc)}
             z[r] = fmaf((kk & 1) ? -amp : amp, __cosf(ph), z[r]);      // odd k: -cos(theta + pi)
         }
     }
@@ -1161,11 +1198,13 @@ adj_mixed_gains_kernel(const DevProblem* __restrict__ probs, const Plan* __restr
                     b = frac_turns(fmaf(-gc.x * INV_TWO_PI_F, tc, b + rp.y));
                     if (par) b = frac_turns(b - tp_frac(x.z, 0.f, nuh, nul));
                     if (par && !exact) b = frac_turns(fmaf(o.z, kappa, b));
-                    o = exact ? z4 : to_rad(o);
-                    s_off[warp][k] = make_float4(fmaf(-gc.x, x.x, o.x), fmaf(-gc.x, x.y, o.y),
-                                                 par ? fmaf(-TWO_PI_F, x.z, o.z) : o.z,
-                                                 par ? fmaf(gc.x, x.z, -o.z) : gc.x * x.z);
-                    s_va[warp][k] = make_float4(gc.y * x.x, gc.y * x.y, -gc.y * x.z, fmaf(gc.y, tc, gc.z) + __log2f(rp.x));
+                    o = to_rad(o);
+                    s_off[warp][k] = exact ? make_float4(x.x, x.y, -x.z, gc.x * INV_TWO_PI_F)
+                                           : make_float4(fmaf(-gc.x, x.x, o.x), fmaf(-gc.x, x.y, o.y),
+                                                         par ? fmaf(-TWO_PI_F, x.z, o.z) : o.z,
+                                                         par ? fmaf(gc.x, x.z, -o.z) : gc.x * x.z);
+                    s_va[warp][k] = make_float4(exact ? gc.y : gc.y * x.x, gc.y * x.y, -gc.y * x.z,
+                                                fmaf(gc.y, tc, gc.z) + __log2f(rp.x));
                     kr.y = b * TWO_PI_F;
                 } else {
                     o.w = frac_turns(b + rp.y) * TWO_PI_F;
@@ -1191,11 +1230,13 @@ adj_mixed_gains_kernel(const DevProblem* __restrict__ probs, const Plan* __restr
             if (exact) {
                 const float4 dxt[2] = {P.pix.off[eidx[0]], P.pix.off[eidx[1]]},
                              dxl[2] = {P.pix.offlo[eidx[0]], P.pix.offlo[eidx[1]]};
-                if (gauss) adjg_gauss_tile<true, false>(s_off[warp], s_va[warp], s_kr[warp], P.vis.off + (size_t)g * G, g_lo, sg, Ct, y, dxt, dxl, acc);
+                const float4* g_off = P.vis.off + (size_t)g * G;
+                if (gauss && par) adjg_gauss_tile<true, false, true>(s_off[warp], s_va[warp], s_kr[warp], g_off, g_lo, sg, Ct, y, dxt, dxl, acc);
+                else if (gauss) adjg_gauss_tile<true, false, false>(s_off[warp], s_va[warp], s_kr[warp], g_off, g_lo, sg, Ct, y, dxt, dxl, acc);
                 else adjg_dirac_tile<true, false>(s_off[warp], g_lo, s_kr[warp], sg, Ct, dxt, dxl, acc);
             } else if (gauss) {
-                if (al4) adjg_gauss_tile<false, true>(s_off[warp], s_va[warp], s_kr[warp], g_lo, g_lo, sg, Ct, y, dx, dx, acc);
-                else adjg_gauss_tile<false, false>(s_off[warp], s_va[warp], s_kr[warp], g_lo, g_lo, sg, Ct, y, dx, dx, acc);
+                if (al4) adjg_gauss_tile<false, true, false>(s_off[warp], s_va[warp], s_kr[warp], g_lo, g_lo, sg, Ct, y, dx, dx, acc);
+                else adjg_gauss_tile<false, false, false>(s_off[warp], s_va[warp], s_kr[warp], g_lo, g_lo, sg, Ct, y, dx, dx, acc);
             } else {
                 if (al4) adjg_dirac_tile<false, true>(s_off[warp], g_lo, s_kr[warp], sg, Ct, dx, dx, acc);
                 else adjg_dirac_tile<false, false>(s_off[warp], g_lo, s_kr[warp], sg, Ct, dx, dx, acc);
