@@ -43,54 +43,80 @@ struct Axis {
     int kmin = 0, n = 1;
 };
 
-// The spacing is the smallest distance from the first pixel, refined over the
-// whole span; every pixel then has to sit on its lattice point to within
-// `tol` (a phase error of 1e-8 turn at the longest baseline).  A lattice whose
-// first pixel has no neighbour one step away is not recognised.
-Axis find_axis(const double* c, int64_t n, double tol)
+// Loops over the pixels, cut into NT chunks, on as many threads as pay (one takes
+// tens of us to start).
+constexpr size_t NT = 16;
+template <class F>
+void pixel_chunks(int64_t n, const F& fn)
 {
-    Axis A;
-    A.x0 = c[0];
-    const size_t nt = 64;                               // chunks of the reductions
-    std::vector<double> near(nt, 1e300), lo(nt, 1e300), hi(nt, -1e300);
-    const auto chunk = [&](size_t t) { return std::make_pair((size_t)n * t / nt, (size_t)n * (t + 1) / nt); };
-    parallel_chunks(nt, (size_t)std::max<int64_t>(1, 65536 / std::max<int64_t>(1, n / (int64_t)nt)),
-                    [&](size_t t0, size_t t1) {
-        for (size_t t = t0; t < t1; ++t) {
-            const auto r = chunk(t);
-            for (size_t i = r.first; i < r.second; ++i) {
-                const double v = c[2 * i], d = std::fabs(v - A.x0);
-                if (d > tol) near[t] = std::min(near[t], d);
-                lo[t] = std::min(lo[t], v);
-                hi[t] = std::max(hi[t], v);
-            }
-        }
+    parallel_chunks(NT, (size_t)std::max<int64_t>(1, 65536 * (int64_t)NT / std::max<int64_t>(1, n)), [&](size_t t0, size_t t1) {
+        for (size_t t = t0; t < t1; ++t) fn(t, (size_t)n * t / NT, (size_t)n * (t + 1) / NT);
     });
-    const double dmin = *std::min_element(near.begin(), near.end());
-    const double xl = *std::min_element(lo.begin(), lo.end()), xh = *std::max_element(hi.begin(), hi.end());
-    if (dmin > 1e299) {                                 // one value
-        A.ok = true;
-        return A;
+}
+
+// Both axes, and the range of n - 1.  The spacing is the smallest distance from
+// the first pixel, refined over the whole span; every pixel then has to sit on its
+// lattice point to within `tol` (a phase error of 1e-8 turn at the longest
+// baseline).  A lattice whose first pixel has no neighbour one step away is not
+// recognised.
+void find_axes(const double* lm, int64_t n, const double (&tol)[2], Axis (&A)[2], double& n0, double& n1)
+{
+    struct Part {
+        double near[2] = {1e300, 1e300}, lo[2] = {1e300, 1e300}, hi[2] = {-1e300, -1e300}, n0 = 1e300, n1 = -1e300;
+        bool off[2] = {false, false};
+    };
+    std::vector<Part> part(NT);
+    for (int a = 0; a < 2; ++a) A[a].x0 = lm[a];
+    pixel_chunks(n, [&](size_t t, size_t i0, size_t i1) {
+        Part p;
+        for (size_t i = i0; i < i1; ++i) {
+            for (int a = 0; a < 2; ++a) {
+                const double v = lm[2 * i + a], d = std::fabs(v - A[a].x0);
+                if (d > tol[a]) p.near[a] = std::min(p.near[a], d);
+                p.lo[a] = std::min(p.lo[a], v);
+                p.hi[a] = std::max(p.hi[a], v);
+            }
+            const double r2 = lm[2 * i] * lm[2 * i] + lm[2 * i + 1] * lm[2 * i + 1];
+            const double v = -r2 / (1.0 + std::sqrt(1.0 - r2));
+            p.n0 = std::min(p.n0, v);
+            p.n1 = std::max(p.n1, v);
+        }
+        part[t] = p;
+    });
+    Part all;
+    for (const Part& p : part) {
+        for (int a = 0; a < 2; ++a) {
+            all.near[a] = std::min(all.near[a], p.near[a]);
+            all.lo[a] = std::min(all.lo[a], p.lo[a]);
+            all.hi[a] = std::max(all.hi[a], p.hi[a]);
+        }
+        all.n0 = std::min(all.n0, p.n0);
+        all.n1 = std::max(all.n1, p.n1);
     }
-    const double span = xh - A.x0 > A.x0 - xl ? xh - A.x0 : A.x0 - xl;
-    const double steps = std::rint(span / dmin);
-    if (!(steps >= 1.0) || steps > 8192.0) return A;
-    A.step = span / steps;
-    A.kmin = (int)std::rint((xl - A.x0) / A.step);
-    A.n = (int)std::rint((xh - A.x0) / A.step) - A.kmin + 1;
-    std::vector<char> bad(nt, 0);
-    parallel_chunks(nt, (size_t)std::max<int64_t>(1, 65536 / std::max<int64_t>(1, n / (int64_t)nt)),
-                    [&](size_t t0, size_t t1) {
-        for (size_t t = t0; t < t1; ++t) {
-            const auto r = chunk(t);
-            for (size_t i = r.first; i < r.second; ++i) {
-                const double d = c[2 * i] - A.x0;
-                if (std::fabs(d - std::rint(d / A.step) * A.step) > tol) bad[t] = 1;
+    n0 = all.n0;
+    n1 = all.n1;
+    for (int a = 0; a < 2; ++a) {
+        if (all.near[a] > 1e299) continue;              // one value
+        const double up = all.hi[a] - A[a].x0, down = A[a].x0 - all.lo[a], span = up > down ? up : down;
+        const double steps = std::rint(span / all.near[a]);
+        if (!(steps >= 1.0) || steps > 8192.0) return;
+        A[a].step = span / steps;
+        A[a].kmin = (int)std::rint((all.lo[a] - A[a].x0) / A[a].step);
+        A[a].n = (int)std::rint((all.hi[a] - A[a].x0) / A[a].step) - A[a].kmin + 1;
+    }
+    pixel_chunks(n, [&](size_t t, size_t i0, size_t i1) {
+        bool off[2] = {false, false};
+        for (int a = 0; a < 2; ++a) {
+            if (A[a].n == 1) continue;
+            for (size_t i = i0; i < i1; ++i) {
+                const double d = lm[2 * i + a] - A[a].x0;
+                off[a] |= std::fabs(d - std::rint(d / A[a].step) * A[a].step) > tol[a];
             }
         }
+        std::copy(off, off + 2, part[t].off);
     });
-    A.ok = std::count(bad.begin(), bad.end(), 1) == 0;
-    return A;
+    for (int a = 0; a < 2; ++a)
+        A[a].ok = std::none_of(part.begin(), part.end(), [a](const Part& p) { return p.off[a]; });
 }
 
 int log2_at_least(int n)
@@ -151,16 +177,10 @@ bool grid_build(sl1m_problem& P, cudaStream_t st, size_t budget)
         w0 = std::min(w0, w);
         w1 = std::max(w1, w);
     }
-    const Axis ax = find_axis(P.lm.data(), P.n_pix, 1e-8 / std::max(1.0, um));
-    if (!ax.ok) return false;
-    const Axis ay = find_axis(P.lm.data() + 1, P.n_pix, 1e-8 / std::max(1.0, vm));
-    if (!ay.ok) return false;
-    for (int64_t j = 0; j < P.n_pix; ++j) {
-        const double l = P.lm[2 * j], m = P.lm[2 * j + 1], r2 = l * l + m * m;
-        const double v = -r2 / (1.0 + std::sqrt(1.0 - r2));
-        n0 = std::min(n0, v);
-        n1 = std::max(n1, v);
-    }
+    Axis axes[2];
+    find_axes(P.lm.data(), P.n_pix, {1e-8 / std::max(1.0, um), 1e-8 / std::max(1.0, vm)}, axes, n0, n1);
+    const Axis &ax = axes[0], &ay = axes[1];
+    if (!ax.ok || !ay.ok) return false;
     auto T = std::make_unique<GridTables>();
     GridOp& g = T->op;
     g.nx = ax.n;
@@ -194,6 +214,13 @@ bool grid_build(sl1m_problem& P, cudaStream_t st, size_t budget)
     T->ws_elems = grid_plane_elems(g) * g.np_pass;
     const size_t sums = grid_sum_bytes(g, P.hp.vis.n_blk, P.hp.pix.n_blk);
     if (tab + sums + T->ws_elems * sizeof(float2) > std::min(budget, free_b / 2)) return false;
+    const double wp0 = w0 - (0.5 * GRW - 0.5) * dw;
+    // any failure below (memory, above all) leaves the pair operator in place.  The
+    // set-up kernels run while the host makes the tables and the lists.
+    bool ok = T->pos.alloc(nv) == cudaSuccess && T->wts.alloc(nv * 3 * GRW) == cudaSuccess && T->rot.alloc(nv) == cudaSuccess &&
+              grid_setup_vis(P.hp.vis.d, (int)nv, g, ax.step, ay.step, ax.x0 + (ax.kmin + g.nx / 2) * ax.step,
+                             ay.x0 + (ay.kmin + g.ny / 2) * ay.step, nc, wp0, dw, T->pos.p, T->wts.p, T->rot.p,
+                             st) == cudaSuccess;
     // powers of two that keep a coherent sum of the largest inputs in range
     const auto p2 = [](double n) { return (float)std::exp2(-std::ceil(std::log2(std::max(1.0, n)))); };
     g.fscale = p2((double)P.n_pix);
@@ -222,20 +249,22 @@ bool grid_build(sl1m_problem& P, cudaStream_t st, size_t budget)
         for (int q = 0; q < GR_NQ; ++q) s += quad[GR_NQ + q] * std::cos(2.0 * M_PI * xi * quad[q]);
         return 0.5 / s;
     };
-    for (int i = 0; i < g.nx; ++i) cxy[i] = inv_hat((double)(i - g.cx) / (1 << g.lx));
-    for (int i = 0; i < g.ny; ++i) cxy[g.nx + i] = inv_hat((double)(i - g.cy) / (1 << g.ly));
-    const double wp0 = w0 - (0.5 * GRW - 0.5) * dw;
+    const auto hats = [&](int n, int c, int lg, double* out) {        // (even in i - c)
+        for (int i = 0; i <= c; ++i) out[i] = inv_hat((double)(i - c) / (1 << lg));
+        for (int i = c + 1; i < n; ++i) out[i] = 2 * c - i >= 0 ? out[2 * c - i] : inv_hat((double)(i - c) / (1 << lg));
+    };
+    hats(g.nx, g.cx, g.lx, cxy.data());
+    if (g.ny == g.nx && g.ly == g.lx) std::copy(cxy.begin(), cxy.begin() + g.nx, cxy.begin() + g.nx);
+    else hats(g.ny, g.cy, g.ly, cxy.data() + g.nx);
     std::vector<float2> wp(g.np);
     for (int p = 0; p < g.np; ++p) {
         const double w = wp0 + p * dw;
         wp[p] = make_float2((float)w, (float)(w - (double)(float)w));
     }
     const std::vector<float2> tx = twiddles(g.lx), ty = twiddles(g.ly);
-    // any failure below (memory, above all) leaves the pair operator in place
-    bool ok = T->cell.upload(cell.data(), cells, st) == cudaSuccess && T->wp.upload(wp.data(), wp.size(), st) == cudaSuccess &&
-              T->twx.upload(tx.data(), tx.size(), st) == cudaSuccess && T->twy.upload(ty.data(), ty.size(), st) == cudaSuccess &&
-              T->amp.alloc(cells) == cudaSuccess && T->nu.alloc(cells) == cudaSuccess && T->pos.alloc(nv) == cudaSuccess &&
-              T->wts.alloc(nv * 3 * GRW) == cudaSuccess && T->rot.alloc(nv) == cudaSuccess;
+    ok = ok && T->cell.upload(cell.data(), cells, st) == cudaSuccess && T->wp.upload(wp.data(), wp.size(), st) == cudaSuccess &&
+         T->twx.upload(tx.data(), tx.size(), st) == cudaSuccess && T->twy.upload(ty.data(), ty.size(), st) == cudaSuccess &&
+         T->amp.alloc(cells) == cudaSuccess && T->nu.alloc(cells) == cudaSuccess;
     DBuf<double> dq, dc;
     ok = ok && dq.upload(quad.data(), quad.size(), st) == cudaSuccess && dc.upload(cxy.data(), cxy.size(), st) == cudaSuccess;
     std::vector<int4> pos(nv);
@@ -244,59 +273,124 @@ bool grid_build(sl1m_problem& P, cudaStream_t st, size_t budget)
         g.wp = T->wp.p;
         g.twx = T->twx.p;
         g.twy = T->twy.p;
-        ok = grid_setup_cells(P.hp.pix.d, g, dc.p, dq.p, nc, dw, T->amp.p, T->nu.p, st) == cudaSuccess &&
-             grid_setup_vis(P.hp.vis.d, (int)nv, g, ax.step, ay.step, ax.x0 + (ax.kmin + g.cx) * ax.step,
-                            ay.x0 + (ay.kmin + g.cy) * ay.step, nc, wp0, dw, T->pos.p, T->wts.p, T->rot.p,
-                            st) == cudaSuccess &&
-             cudaMemcpyAsync(pos.data(), T->pos.p, nv * sizeof(int4), cudaMemcpyDeviceToHost, st) == cudaSuccess &&
-             cudaStreamSynchronize(st) == cudaSuccess;
+        ok = cudaMemcpyAsync(pos.data(), T->pos.p, nv * sizeof(int4), cudaMemcpyDeviceToHost, st) == cudaSuccess &&
+             cudaStreamSynchronize(st) == cudaSuccess &&
+             grid_setup_cells(P.hp.pix.d, g, dc.p, dq.p, nc, dw, T->amp.p, T->nu.p, st) == cudaSuccess;
     }
     // visibilities per tile (at most two tiles per axis), by first plane, in the
-    // library's order: a counting sort
+    // library's order: counting sorts by tile and then, within each, by plane;
+    // on threads of their own by rows of tiles where there are many
     std::vector<int> start, list, order;
     if (ok) {
-        const int txn = (1 << g.lx) / GR_TILE, mx = (1 << g.lx) - 1, my = (1 << g.ly) - 1;
-        start.assign((size_t)tiles * (ni + 1) + 1, 0);
-        const auto each = [&](const auto& f) {
-            for (size_t k = 0; k < nv; ++k) {
-                if (P.vis_orig[k] < 0) continue;
-                const int xa = pos[k].x / GR_TILE, xb = ((pos[k].x + GRW - 1) & mx) / GR_TILE;
-                const int ya = pos[k].y / GR_TILE, yb = ((pos[k].y + GRW - 1) & my) / GR_TILE;
-                for (int y = 0; y < (ya == yb ? 1 : 2); ++y)
-                    for (int x = 0; x < (xa == xb ? 1 : 2); ++x)
-                        f(k, ((size_t)(y ? yb : ya) * txn + (x ? xb : xa)) * (ni + 1) + pos[k].z);
-            }
+        const int txn = (1 << g.lx) / GR_TILE, tyn = (1 << g.ly) / GR_TILE, mx = (1 << g.lx) - 1, my = (1 << g.ly) - 1;
+        struct Part {
+            int y0, y1, n_list = 0, n_order = 0;
+            std::vector<int> at, by_tile;                    // tile's first in by_tile; visibilities by tile
         };
-        each([&](size_t, size_t at) { ++start[at + 1]; });
-        for (size_t i = 1; i < start.size(); ++i) start[i] += start[i - 1];
-        list.resize(std::max(1, start.back()));
-        std::vector<int> fill(start.begin(), start.end() - 1);
-        each([&](size_t k, size_t at) { list[fill[at]++] = (int)k; });
-        // each visibility once, at its first tile; then the padding slots
-        order.reserve(nv);
-        for (int t = 0; t < tiles; ++t)
-            for (int i = start[(size_t)t * (ni + 1)]; i < start[(size_t)(t + 1) * (ni + 1)]; ++i) {
-                const int4 q = pos[list[i]];
-                if ((q.y / GR_TILE) * txn + q.x / GR_TILE == t) order.push_back(list[i]);
-            }
-        for (size_t k = 0; k < nv; ++k)
-            if (P.vis_orig[k] < 0) order.push_back((int)k);
-        // which tiles of each plane have a visibility
-        const int tyn = (1 << g.ly) / GR_TILE;
-        std::vector<unsigned char> act((size_t)g.np * tiles, 0), colact((size_t)g.np * txn, 0);
-        for (int t = 0; t < tiles; ++t)
-            for (int i = 0, done = 0; i < ni; ++i) {     // planes below `done` are marked
-                const size_t at = (size_t)t * (ni + 1) + i;
-                if (start[at] == start[at + 1]) continue;
-                for (int p = std::max(i, done); p < i + GRW; ++p) {
-                    act[((size_t)p * txn + t % txn) * tyn + t / txn] = 1;
-                    colact[(size_t)p * txn + t % txn] = 1;
+        std::vector<Part> part(nv + (size_t)tiles * ni < ((size_t)1 << 20) ? 1 : std::min<size_t>(8, (size_t)tyn));
+        for (size_t t = 0; t < part.size(); ++t) {
+            part[t].y0 = (int)(tyn * t / part.size());
+            part[t].y1 = (int)(tyn * (t + 1) / part.size());
+        }
+        const auto parts = [&](const auto& fn) {
+            parallel_chunks(part.size(), 1, [&](size_t t0, size_t t1) {
+                for (size_t t = t0; t < t1; ++t) fn(t, part[t]);
+            });
+        };
+        parts([&](size_t, Part& p) {
+            // f(visibility, tile, whether it counts) over a visibility's four tiles: a
+            // test per tile would be guessed wrong half the time, so they all run
+            const auto each = [&](const auto& f) {
+                const int y0 = p.y0, rows = p.y1 - p.y0;
+                for (size_t k = 0; k < nv; ++k) {
+                    const int4 q = pos[k];
+                    const unsigned xa = (unsigned)q.x / GR_TILE, xb = (unsigned)((q.x + GRW - 1) & mx) / GR_TILE;
+                    const unsigned ya = (unsigned)q.y / GR_TILE - y0, yb = (unsigned)((q.y + GRW - 1) & my) / GR_TILE - y0;
+                    const bool in = P.vis_orig[k] >= 0, a = in & (ya < (unsigned)rows), b = in & (yb < (unsigned)rows) & (yb != ya);
+                    if (rows < tyn && !a && !b) continue;
+                    const unsigned ra = a ? ya * txn : 0, rb = b ? yb * txn : 0;
+                    f((int)k, ra + xa, a);
+                    f((int)k, ra + xb, a & (xb != xa));
+                    f((int)k, rb + xa, b);
+                    f((int)k, rb + xb, b & (xb != xa));
+                    p.n_order += a;
                 }
-                done = i + GRW;
+            };
+            // (a place more per tile: what does not count is written there, too)
+            const int n = (p.y1 - p.y0) * txn;
+            p.at.assign((size_t)n + 1, 0);
+            each([&](int, unsigned t, bool in) { p.at[t + 1] += in; });
+            for (int t = 0; t < n; ++t) {
+                p.n_list += p.at[t + 1];
+                p.at[t + 1] += p.at[t] + 1;
             }
+            p.by_tile.resize(p.at.back());
+            std::vector<int> fill(p.at.begin(), p.at.end() - 1);
+            p.n_order = 0;
+            each([&](int k, unsigned t, bool in) {
+                p.by_tile[fill[t]] = k;
+                fill[t] += in;
+            });
+        });
+        std::vector<int> list0(part.size() + 1, 0), order0(part.size() + 1, 0);
+        for (size_t t = 0; t < part.size(); ++t) {
+            list0[t + 1] = list0[t] + part[t].n_list;
+            order0[t + 1] = order0[t] + part[t].n_order;
+        }
+        start.resize((size_t)tiles * (ni + 1) + 1);
+        start[0] = 0;
+        list.resize(std::max(1, list0.back()));
+        order.resize(nv);
+        std::vector<unsigned char> act((size_t)g.np * tiles, 0), colact((size_t)g.np * txn, 0);
+        parts([&](size_t n, Part& p) {
+            std::vector<int> mine(p.n_order + 1);                    // (a place more: written before it is known to count)
+            int* out = mine.data();
+            std::vector<int> fill(ni);
+            int sum = list0[n];
+            for (int t = 0; t < (p.y1 - p.y0) * txn; ++t) {
+                const int* k0 = p.by_tile.data() + p.at[t];
+                const int* k1 = p.by_tile.data() + p.at[t + 1] - 1;
+                const int tile = p.y0 * txn + t, first = sum;
+                int* st = start.data() + (size_t)tile * (ni + 1) + 1;       // ends of the planes; st[-1]: the tile before
+                std::fill(fill.begin(), fill.end(), 0);
+                for (const int* k = k0; k < k1; ++k) ++fill[pos[*k].z];
+                for (int z = 0; z < ni; ++z) {
+                    st[z] = sum + fill[z];
+                    fill[z] = sum;
+                    sum = st[z];
+                }
+                st[ni] = sum;
+                for (const int* k = k0; k < k1; ++k) list[fill[pos[*k].z]++] = *k;
+                // each visibility once, at its first tile
+                for (int i = first; i < sum; ++i) {
+                    const int4 q = pos[list[i]];
+                    *out = list[i];
+                    out += (q.y / GR_TILE) * txn + q.x / GR_TILE == tile;
+                }
+            }
+            std::copy(mine.data(), out, order.data() + order0[n]);
+        });
+        // which planes of a tile have a visibility (a column of tiles after the other: its
+        // planes' bytes are neighbours); those below `done` are marked
+        parts([&](size_t n, Part& p) {
+            for (int x = 0; x < txn; ++x)
+                for (int y = p.y0; y < p.y1; ++y) {
+                    const int* st = start.data() + ((size_t)y * txn + x) * (ni + 1) + 1;
+                    int from = y == p.y0 && x == 0 ? list0[n] : st[-1];
+                    for (int z = 0, done = 0; z < ni; from = st[z], ++z) {
+                        if (st[z] == from) continue;
+                        for (int d = std::max(z, done); d < z + GRW; ++d) act[((size_t)d * txn + x) * tyn + y] = 1;
+                        done = z + GRW;
+                    }
+                }
+        });
+        for (size_t c = 0; c < colact.size(); ++c) colact[c] = std::memchr(act.data() + c * tyn, 1, tyn) != nullptr;
+        size_t at = order0.back();                           // then the padding slots
+        for (size_t k = 0; k < nv; ++k)
+            if (P.vis_orig[k] < 0) order[at++] = (int)k;
         ok = T->start.upload(start.data(), start.size(), st) == cudaSuccess &&
              T->list.upload(list.data(), list.size(), st) == cudaSuccess &&
-             T->order.upload(order.data(), order.size(), st) == cudaSuccess &&
+             T->order.upload(order.data(), nv, st) == cudaSuccess &&
              T->act.upload(act.data(), act.size(), st) == cudaSuccess &&
              T->colact.upload(colact.data(), colact.size(), st) == cudaSuccess;
     }

@@ -408,15 +408,21 @@ void plan_host(const std::vector<int>& nb, const std::vector<int>& ns, int Cmax,
     if (costs && U > 0) {
         // cumulative cost per problem; boundaries at multiples of total / C
         std::vector<double> W(np + 1, 0.0);
+        // of the problems with a cost per unit, the sum before every STEP-th: the
+        // sums between are formed again, in the same order, where a boundary lies
+        constexpr long long STEP = 64;
+        std::vector<std::vector<double>> sums(np);
         for (int p = 0; p < np; ++p) {
             const UnitCost* uc = (*costs)[p];
             const long long up = H.u0[p + 1] - H.u0[p];
-            double w = 0.0;
+            double w = (uc ? uc->uniform : 1.0) * (double)up;
             if (uc && !uc->unit.empty() && (long long)uc->unit.size() * uc->sub == up) {
-                for (float f : uc->unit) w += f;
-                w *= uc->sub;
-            } else {
-                w = (uc ? uc->uniform : 1.0) * (double)up;
+                const long long nu = (long long)uc->unit.size();
+                w = 0.0;
+                for (long long k = 0; k < nu; ++k) {
+                    if (k % STEP == 0) sums[p].push_back(w);
+                    w += (double)uc->unit[k] * uc->sub;
+                }
             }
             W[p + 1] = W[p] + w;
         }
@@ -424,25 +430,25 @@ void plan_host(const std::vector<int>& nb, const std::vector<int>& ns, int Cmax,
         H.cta_u0.assign(C + 1, 0);
         H.cta_u0[C] = U;
         int p = 0;
-        std::vector<double> pref;
-        int pref_of = -1;
         for (int c = 1; c < C; ++c) {
             const double t = T * (double)c / (double)C;
             while (p < np - 1 && W[p + 1] < t) ++p;
             const UnitCost* uc = (*costs)[p];
             const long long up = H.u0[p + 1] - H.u0[p];
             long long i;
-            if (uc && !uc->unit.empty() && (long long)uc->unit.size() * uc->sub == up) {
+            if (!sums[p].empty()) {
+                // the first i whose sum of i units reaches t, and the sum of i - 1
                 const long long nu = (long long)uc->unit.size();
-                if (pref_of != p) {
-                    pref.assign(nu + 1, 0.0);
-                    for (long long k = 0; k < nu; ++k) pref[k + 1] = pref[k] + (double)uc->unit[k] * uc->sub;
-                    pref_of = p;
+                const auto step = std::lower_bound(sums[p].begin(), sums[p].end(), t - W[p]) - sums[p].begin();
+                i = std::max<long long>(0, step - 1) * STEP;
+                double sum = sums[p][i / STEP], before = 0.0;
+                while (i <= nu && sum < t - W[p]) {
+                    before = sum;
+                    if (i < nu) sum += (double)uc->unit[i] * uc->sub;
+                    ++i;
                 }
-                i = std::lower_bound(pref.begin(), pref.end(), t - W[p]) - pref.begin();
                 if (uc->sub > 1 && i > 0)        // within the run of equal units that ends there
-                    i = (i - 1) * uc->sub +
-                        (long long)std::ceil((t - W[p] - pref[i - 1]) / uc->unit[std::min(i, nu) - 1] - 1e-9);
+                    i = (i - 1) * uc->sub + (long long)std::ceil((t - W[p] - before) / uc->unit[std::min(i, nu) - 1] - 1e-9);
             } else {
                 const double w = (uc ? uc->uniform : 1.0);
                 i = (long long)std::ceil((t - W[p]) / w - 1e-9);
@@ -1050,7 +1056,8 @@ const UnitCost& sl1m_problem::unit_cost(int precision, int op)
     const int bg = own_granules(precision, op, n_ant > 0), nblk = own_blocks(precision, op, n_ant > 0, ng_own);
     uc.sub = stream_units(precision, 1);               // units per streamed granule
     uc.unit.resize((size_t)nblk * ng_str);
-    for (int b = 0; b < nblk; ++b) {
+    parallel_chunks((size_t)nblk, std::max<size_t>(1, 131072 / std::max(1, ng_str)), [&](size_t b0, size_t b1) {
+    for (int b = (int)b0; b < (int)b1; ++b) {
         const int w1 = std::min(ng_own, (b + 1) * bg);
         double kb = 1.0, own_pairs = 0.0;
         if (op == 0 && by_pairs)
@@ -1069,6 +1076,7 @@ const UnitCost& sl1m_problem::unit_cost(int precision, int op)
                 (float)((kbase * (ex ? 3.0 : 1.0) + (op == 0 ? own_pairs : by_pairs ? pair_cost(g) : 0.0)) * gfac);
         }
     }
+    });
     return uc;
 }
 

@@ -20,6 +20,7 @@
 #include <map>
 #include <mutex>
 #include <new>
+#include <set>
 #include <string>
 #include <system_error>
 #include <thread>
@@ -42,6 +43,7 @@ size_t g_fail_min = 0;                             // allocations of this size a
 int g_fail_n = 0;                                  // ... fail this many times
 std::string g_faults;
 long long g_count[5];                              // launches: pairs fwd, adj, lattice fwd, adj; table fills
+std::set<const void*> g_checked;                    // lattices whose lists were compared
 bool g_hold = false;                                // solves run on
 thread_local bool t_capturing = false;
 using Check = std::function<void()>;
@@ -102,6 +104,52 @@ constexpr int N_PLACES = 8;
 alignas(64) char g_place[N_PLACES][sizeof(sl1m_problem)];
 bool g_used[N_PLACES];
 
+// The lattice's lists, restated from its definition: positions as grid_setup_vis
+// (below) made them, padding slots as in P.vis.orig.
+void check_lists(const DevProblem& P, const GridOp& g)
+{
+    const int txn = (1 << g.lx) / GR_TILE, tyn = (1 << g.ly) / GR_TILE, tiles = txn * tyn, ni = g.np - GRW + 1;
+    const int nv = P.vis.n_pad, mx = (1 << g.lx) - 1, my = (1 << g.ly) - 1;
+    if (!need(g.pos, (size_t)nv * 16, "positions") || !need(P.vis.orig, (size_t)nv * 4, "slots")) return;
+    std::vector<std::vector<int>> by((size_t)tiles * ni);
+    std::vector<unsigned char> act((size_t)g.np * tiles, 0), colact((size_t)g.np * txn, 0);
+    for (int k = 0; k < nv; ++k) {
+        if (P.vis.orig[k] < 0) continue;
+        bool seen[4] = {};
+        const int4 q = g.pos[k];
+        int at[4];
+        for (int c = 0; c < 4; ++c) {
+            const int x = (c & 1 ? (q.x + GRW - 1) & mx : q.x) / GR_TILE, y = (c & 2 ? (q.y + GRW - 1) & my : q.y) / GR_TILE;
+            at[c] = y * txn + x;
+            for (int d = 0; d < c; ++d) seen[c] |= at[d] == at[c];
+            if (seen[c]) continue;
+            by[(size_t)at[c] * ni + q.z].push_back(k);
+            for (int z = q.z; z < q.z + GRW; ++z) act[((size_t)z * txn + x) * tyn + y] = colact[(size_t)z * txn + x] = 1;
+        }
+    }
+    std::vector<int> start = {0}, list, order;
+    for (int t = 0; t < tiles; ++t) {
+        for (int z = 0; z < ni; ++z) {
+            for (int k : by[(size_t)t * ni + z]) {
+                list.push_back(k);
+                if ((g.pos[k].y / GR_TILE) * txn + g.pos[k].x / GR_TILE == t) order.push_back(k);
+            }
+            start.push_back((int)list.size());
+        }
+        start.push_back((int)list.size());
+    }
+    for (int k = 0; k < nv; ++k)
+        if (P.vis.orig[k] < 0) order.push_back(k);
+    const auto same = [](const auto& v, const auto* p, const char* what) {
+        if (!need(p, v.size() * sizeof v[0], what) || memcmp(p, v.data(), v.size() * sizeof v[0])) fault("lattice: %s differs", what);
+    };
+    same(start, g.start, "start");
+    same(list, g.list, "list");
+    same(order, g.order, "order");
+    same(act, g.act, "act");
+    same(colact, g.colact, "colact");
+}
+
 }  // namespace
 
 // std::async and std::thread of the library come here (it is linked symbolically).
@@ -151,6 +199,7 @@ void fake_reset()
     g_faults.clear();
     g_fail_n = 0;
     g_hold = false;
+    g_checked.clear();
     g_total = (size_t)280 << 30;
     g_peak = g_held;
     memset(g_count, 0, sizeof g_count);
@@ -289,6 +338,7 @@ cudaError_t grid_forward(const DevProblem* probs, int p, const GridOp& g, int n_
         if (need(probs, sizeof *probs * (p + 1), "lattice forward") &&
             (probs[p].vis.n_pad != n_vis_pad || !need(g.order, (size_t)n_vis_pad * 4, "lattice forward's order")))
             fault("lattice forward: another problem's tables");
+        if (g_checked.insert(g.start).second) check_lists(probs[p], g);
         ++g_count[2];
     });
     *n += 3;
@@ -313,10 +363,14 @@ cudaError_t grid_setup_cells(const d4*, GridOp, const double*, const double*, do
 {
     return cudaSuccess;
 }
-cudaError_t grid_setup_vis(const d4*, int n, GridOp, double, double, double, double, double, double, double, int4* pos,
+cudaError_t grid_setup_vis(const d4*, int n, GridOp g, double, double, double, double, double, double, double, int4* pos,
                            float*, float2*, cudaStream_t)
 {
-    if (need(pos, (size_t)n * 16, "positions")) memset(pos, 0, (size_t)n * 16);
+    unsigned r = 12345;                                // (any positions; half of them in a few tiles)
+    const auto next = [&](int m) { return (int)((r = r * 1664525u + 1013904223u) >> 8) % m; };
+    for (int k = 0; need(pos, (size_t)n * 16, "positions") && k < n; ++k)
+        pos[k] = k % 2 ? make_int4(next(1 << g.lx), next(1 << g.ly), next(g.np - GRW + 1), 0)
+                       : make_int4(next(40), (1 << g.ly) - 1 - next(9), next(g.np - GRW + 1) / 3, 1);
     return cudaSuccess;
 }
 cudaError_t fp64_init_tables(cudaStream_t) { LOCK; ++g_count[4]; return cudaSuccess; }
