@@ -199,7 +199,7 @@ __device__ __forceinline__ double2 zero_of(double2) { return make_double2(0.0, 0
 // FP64, 2 CTAs summing 228 slots, took 108 us of a 280 us step.
 template <int SL>
 struct FinShape {
-    static constexpr int THREADS = SL >= 16 ? 1024 : 256;
+    static constexpr int THREADS = SL >= 8 ? 512 : 256;
     static constexpr int EL = THREADS / SL;             // elements per CTA: 64 or 256
     static constexpr int NG = EL / G;                   // granules per CTA
 };
@@ -633,11 +633,15 @@ __global__ void phases_kernel(const DevProblem* __restrict__ probs, const int* _
 
 // Threads per element by the mean number of slots of a block (the kernels'
 // loads are 8 deep): up to 2 slots one thread has them in flight anyway; above
-// 48, 16 threads take at most a few rounds each.
+// 48, 8 threads take a few rounds each.  16 of them made CTAs of 1,024 threads and
+// 64 registers, which start only on an empty SM: behind another stream's
+// operator they waited for whole SMs and kept its CTAs off them meanwhile
+// (35,344 multiscale pixels x 2,702 visibilities forward, three streams in turn: 163
+// us a call; 151 with 8, and a 30-tick FP64 solve 5.71 -> 5.69 ms).
 static int slot_threads(const Plan& pl)
 {
     const double mean = (double)pl.n_slots / (pl.n_blocks > 0 ? pl.n_blocks : 1);
-    return mean <= 2.0 && pl.blk_el >= 256 ? 1 : mean <= 48.0 ? 4 : 16;
+    return mean <= 2.0 && pl.blk_el >= 256 ? 1 : mean <= 48.0 ? 4 : 8;
 }
 template <int SL>
 static int fin_grid(const Plan& pl, int num_sms)
@@ -653,8 +657,7 @@ cudaError_t launch_fwd_finish(const DevProblem* probs, const Plan* plp, const Pl
     switch (slot_threads(pl)) {
     case 1: fwd_finish_kernel<1><<<fin_grid<1>(pl, num_sms), 256, 0, st>>>(probs, plp, partial, polar, user_out); break;
     case 4: fwd_finish_kernel<4><<<fin_grid<4>(pl, num_sms), 256, 0, st>>>(probs, plp, partial, polar, user_out); break;
-    default:
-        fwd_finish_kernel<16><<<fin_grid<16>(pl, num_sms), 1024, 0, st>>>(probs, plp, partial, polar, user_out);
+    default: fwd_finish_kernel<8><<<fin_grid<8>(pl, num_sms), 512, 0, st>>>(probs, plp, partial, polar, user_out);
     }
     return cudaGetLastError();
 }
@@ -665,7 +668,7 @@ cudaError_t launch_adj_finish(const DevProblem* probs, const Plan* plp, const Pl
     switch (slot_threads(pl)) {
     case 1: adj_finish_kernel<1><<<fin_grid<1>(pl, num_sms), 256, 0, st>>>(probs, plp, partial, user_out); break;
     case 4: adj_finish_kernel<4><<<fin_grid<4>(pl, num_sms), 256, 0, st>>>(probs, plp, partial, user_out); break;
-    default: adj_finish_kernel<16><<<fin_grid<16>(pl, num_sms), 1024, 0, st>>>(probs, plp, partial, user_out);
+    default: adj_finish_kernel<8><<<fin_grid<8>(pl, num_sms), 512, 0, st>>>(probs, plp, partial, user_out);
     }
     return cudaGetLastError();
 }
