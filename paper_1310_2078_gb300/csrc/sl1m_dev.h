@@ -158,6 +158,9 @@ struct DevProblem {
     const float4* vgabs;      // [vis.n_pad] {u, v, -2 w, u^2 + v^2} in FP32 (the adjoint's Gaussian terms)
     float2* r32;              // [vis.n_pad] the mixed adjoint's input residual in polar form,
                               // {|r|, arg r in turns} in FP32
+    int* huge;                // lattice problems: [3] an input of 2^40 or more in this step's forward, in the
+                              // coming adjoint, in I_0 (whatever writes an input marks it, the finish
+                              // kernel that ends the operator clears the first two); or null
     double2* r64;             // [vis.n_pad] the FP64 adjoint's, {arg r in 1/R64_TURN turns, |r|}
     const float2* gpol32;     // [pix.n_gran][gain_rows(n_ant)][GP] {|G|, arg G in turns} or null
     const double2* gains64;   // [pix.n_pad][n_ant] or null

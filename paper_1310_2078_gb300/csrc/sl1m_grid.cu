@@ -325,6 +325,15 @@ __device__ __forceinline__ int cell_of(int e, int lg, int c0)
     return (e < (1 << (lg - 1)) ? e : e - (1 << lg)) + c0;
 }
 
+// The scale of an operator's input (which: 0 forward, 1 adjoint; both marks are
+// read at once, a chain of loads less).
+__device__ __forceinline__ float in_scale(const DevProblem& P, int which, float huge_scale)
+{
+    const int now = P.huge[which], first = which == 0 ? P.huge[2] : 0;
+    const bool init = which == 0 && P.st && P.st->phase == PH_SINIT;
+    return (init ? first : now) ? huge_scale : GR_SCALE;
+}
+
 // exp(-2 pi i w nu) with both factors split in FP32 halves.
 __device__ __forceinline__ float2 plane_phase(float2 w, float2 nu)
 {
@@ -361,6 +370,7 @@ grid_rows_fwd_kernel(const DevProblem* __restrict__ probs, int prob, const GridO
     const int rb = threadIdx.x / S::T;
     const int gi[1] = {(int)threadIdx.x % S::T};
     const int iy = blockIdx.x * S::ROWS + rb;
+    const float scale = in_scale(probs[prob], 0, g.fscale);
     float a[S::P / 2];
     float2 nu[S::P / 2];
 #pragma unroll
@@ -372,7 +382,7 @@ grid_rows_fwd_kernel(const DevProblem* __restrict__ probs, int prob, const GridO
             const size_t at = (size_t)iy * g.nx + ix;
             const int j = g.cell[at];
             if (j >= 0) {
-                a[i] = __double2float_rn(X[j]) * g.amp[at] * g.fscale;
+                a[i] = __double2float_rn(X[j]) * scale * g.amp[at];
                 nu[i] = g.nu[at];
             }
         }
@@ -413,6 +423,7 @@ grid_rows_adj_kernel(const DevProblem* __restrict__ probs, int prob, const GridO
     const int rb = threadIdx.x / S::T;
     const int gi[1] = {(int)threadIdx.x % S::T};
     const int iy = blockIdx.x * S::ROWS + rb;
+    const float unscale = __frcp_rn(in_scale(probs[prob], 1, g.ascale));     // (a power of two)
     float acc[S::P / 2];
     float2 nu[S::P / 2];
 #pragma unroll
@@ -450,7 +461,7 @@ grid_rows_adj_kernel(const DevProblem* __restrict__ probs, int prob, const GridO
             const int j = g.cell[at];
             if (j >= 0) {
                 double& slot = partial[((size_t)(j / BLK) * g.n_chunk + blockIdx.y) * BLK + j % BLK];
-                const double v = (double)acc[i] * ((double)g.amp[at] / (double)g.ascale);
+                const double v = (double)acc[i] * ((double)g.amp[at] * (double)unscale);
                 slot = p0 > 0 ? slot + v : v;
             }
         }
@@ -547,6 +558,7 @@ grid_gather_kernel(const DevProblem* __restrict__ probs, int prob, const GridOp 
     const int i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (i >= n_vis_pad) return;
     const int k = g.order[i];
+    const float unscale = __frcp_rn(in_scale(probs[prob], 0, g.fscale));     // (a power of two)
     const int4 ps = g.pos[k];
     if (!ALL && (ps.z >= p0 + np || ps.z + GRW <= p0) && p0 > 0) return;     // nothing to add
     const float* wt = g.wts + (size_t)k * (3 * GRW);
@@ -588,7 +600,7 @@ grid_gather_kernel(const DevProblem* __restrict__ probs, int prob, const GridOp 
     }
     if (lane == 0) {
         const float2 e = g.rot[k];
-        const double inv = 1.0 / (double)g.fscale;
+        const double inv = (double)unscale;
         double2 v = make_double2((double)fmaf(e.x, sr, -e.y * si) * inv, (double)fmaf(e.x, si, e.y * sr) * inv);
         if (ps.w) v.y = -v.y;                  // taken at the mirrored point
         if (!ALL && p0 > 0) {                  // a later pass over the planes
@@ -638,6 +650,7 @@ grid_spread_kernel(const DevProblem* __restrict__ probs, int prob, const GridOp 
         s_act[threadIdx.x] = g.act[((size_t)(ta + threadIdx.x) * tiles_x + tile % tiles_x) * (Ly / GR_TILE) + tile / tiles_x];
     // this thread's part of the staging: point si, weights sf of each axis
     const int si = threadIdx.x >> 3, sf = threadIdx.x & 7;
+    const float scale = in_scale(probs[prob], 1, g.ascale);
     float lwx = 0.f, lwy = 0.f, lww = 0.f;
     float4 lpt = make_float4(0.f, 0.f, 0.f, 0.f);
     int lip = 0;
@@ -653,7 +666,7 @@ grid_spread_kernel(const DevProblem* __restrict__ probs, int prob, const GridOp 
         if (sf == 0) {
             const float2 o = g.rot[k];
             const double2 r = R[k];
-            const float rr = (float)r.x * g.ascale, ri = (float)(ps.w ? -r.y : r.y) * g.ascale;
+            const float rr = (float)r.x * scale, ri = (float)(ps.w ? -r.y : r.y) * scale;
             lpt = make_float4(fmaf(o.x, rr, o.y * ri), fmaf(o.x, ri, -o.y * rr), __int_as_float(ps.x),
                               __int_as_float(ps.y));
         }

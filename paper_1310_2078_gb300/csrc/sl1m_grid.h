@@ -13,6 +13,12 @@ constexpr int GR_PCH = 8;       // planes a CTA of the row kernels takes
 constexpr int GR_LOG_MIN = 6, GR_LOG_MAX = 12;   // FFT lengths 64 .. 4096
 // The exponential-of-semicircle kernel phi(z) = exp(GR_BETA (sqrt(1 - (2z/GRW)^2) - 1)).
 constexpr double GR_BETA = 2.30 * GRW;
+// Inputs are scaled by GR_SCALE, so that small ones stay clear of FP32's
+// denormals, unless one is GR_HUGE or more (DevProblem::huge): then by 1 / the
+// number of them, so that a coherent sum of the largest stays in range.  Powers of
+// two: in between the results are the same.
+constexpr double GR_HUGE = 1099511627776.0;            // 2^40
+constexpr float GR_SCALE = 1099511627776.0f;
 constexpr int GR_NQ = 32;       // Gauss-Legendre nodes on half the kernel's support
 
 // One problem's lattice operator (pointers into device memory).
@@ -23,7 +29,7 @@ struct GridOp {
     int np;                     // planes in w
     int np_pass;                // planes the workspace holds at a time
     int n_chunk;                // adjoint partial slots: chunks of GR_PCH planes of one pass
-    float fscale, ascale;       // powers of two that keep the transforms' sums in range
+    float fscale, ascale;       // powers of two that keep the transforms' sums of huge inputs in range
     const int* cell;            // [ny][nx] sorted pixel index, -1 where the lattice has no pixel
     const float* amp;           // [ny][nx] (1/n) / (kernel transforms), 0 without a pixel
     const float2* nu;           // [ny][nx] n - 1 - nc, FP32 hi and lo

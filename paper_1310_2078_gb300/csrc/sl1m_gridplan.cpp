@@ -264,7 +264,8 @@ bool grid_build(sl1m_problem& P, cudaStream_t st, size_t budget)
     const std::vector<float2> tx = twiddles(g.lx), ty = twiddles(g.ly);
     ok = ok && T->cell.upload(cell.data(), cells, st) == cudaSuccess && T->wp.upload(wp.data(), wp.size(), st) == cudaSuccess &&
          T->twx.upload(tx.data(), tx.size(), st) == cudaSuccess && T->twy.upload(ty.data(), ty.size(), st) == cudaSuccess &&
-         T->amp.alloc(cells) == cudaSuccess && T->nu.alloc(cells) == cudaSuccess;
+         T->amp.alloc(cells) == cudaSuccess && T->nu.alloc(cells) == cudaSuccess &&
+         T->huge.upload(nullptr, 3, st, true) == cudaSuccess;
     DBuf<double> dq, dc;
     ok = ok && dq.upload(quad.data(), quad.size(), st) == cudaSuccess && dc.upload(cxy.data(), cxy.size(), st) == cudaSuccess;
     std::vector<int4> pos(nv);

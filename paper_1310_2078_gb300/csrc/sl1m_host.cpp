@@ -674,6 +674,7 @@ static std::atomic<uint64_t> g_layouts{0};
 void sl1m_problem::set_grid(cudaStream_t st, size_t grid_budget)
 {
     grid.reset();
+    hp.huge = nullptr;
     for (auto& b : op_batch) b.reset();
     for (auto& b : solve_batch) b.reset();
     gen = ++g_layouts;
@@ -683,8 +684,10 @@ void sl1m_problem::set_grid(cudaStream_t st, size_t grid_budget)
         return;
     }
     try {
-        if (grid_build(*this, st, grid_budget))
+        if (grid_build(*this, st, grid_budget)) {
             ctx->h2d += (long long)(grid->cell.bytes() + grid->list.bytes() + grid->start.bytes());
+            hp.huge = grid->huge.p;
+        }
     } catch (const std::bad_alloc&) {                                       // (host memory: the pair kernels need none)
         cudaStreamSynchronize(st);
     }
@@ -1155,10 +1158,11 @@ int sl1m_problem::init_solve(const sl1m_solve_opts* o, double L, bool power_only
     ProblemDev& D = *dev;
     double l1_0 = 0.0;
     const size_t np = hp.pix.n_pad;
+    if (hp.huge) CK(cudaMemsetAsync(hp.huge, 0, 3 * sizeof(int), st));
     if (o && o->x0) {
         CK(D.x_user.reserve(n_pix, st));
         CK(cudaMemcpyAsync(D.x_user.p, o->x0, sizeof(double) * n_pix, cudaMemcpyHostToDevice, st));
-        CKL(launch_gather_real(D.x_user.p, D.I0.p, hp.pix.orig, hp.pix.n_pad, 1.0, st));
+        CKL(launch_gather_real(D.x_user.p, D.I0.p, hp.pix.orig, hp.pix.n_pad, 1.0, hp.huge ? hp.huge + 2 : nullptr, st));
         for (int64_t j = 0; j < n_pix; ++j) l1_0 += o->x0[j];
         ctx->h2d += (long long)sizeof(double) * n_pix;
     } else {
@@ -1977,7 +1981,7 @@ int sl1m_forward_dev(sl1m_problem* prob, const double* x_dev, double* vis_out_de
     Batch* B;
     RET(op_prepare(prob, precision, &B));
     ProblemDev& D = *prob->dev;
-    CKL(launch_gather_real(x_dev, D.x_sorted.p, prob->hp.pix.orig, prob->hp.pix.n_pad, 1.0, ctx->stream));
+    CKL(launch_gather_real(x_dev, D.x_sorted.p, prob->hp.pix.orig, prob->hp.pix.n_pad, 1.0, prob->hp.huge, ctx->stream));
     return batch_op(ctx, *B, 0, vis_out_dev);
 }
 

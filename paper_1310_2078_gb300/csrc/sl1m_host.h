@@ -144,7 +144,7 @@ cudaError_t upload_plan(const HostPlan& H, int n_probs, int blk_el, DevPlan& D, 
 struct GridTables {
     sl1m::GridOp op{};
     size_t ws_elems = 0;                 // float2 of workspace
-    DBuf<int> cell, list, start, order;
+    DBuf<int> cell, list, start, order, huge;
     DBuf<float> amp, wts;
     DBuf<float2> nu, wp, twx, twy, rot;
     DBuf<int4> pos;

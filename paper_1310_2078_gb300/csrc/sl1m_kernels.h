@@ -66,8 +66,9 @@ cudaError_t launch_wait_selftest(unsigned long long* waited_ns, int n_blocks, cu
 unsigned long long wait_limit_ns();
 
 // solver kernels (sl1m_solver.cu)
+// huge (may be null): set where a value is GR_HUGE or more (sl1m_grid.h).
 cudaError_t launch_gather_real(const double* src, double* dst, const int* orig, int n_pad,
-                               double scale, cudaStream_t st);
+                               double scale, int* huge, cudaStream_t st);
 // P: the problem's descriptor on the device.
 cudaError_t launch_gather_resid(const double2* src, const DevProblem* P, int n_pad, int polar, double2* dst,
                                 cudaStream_t st);

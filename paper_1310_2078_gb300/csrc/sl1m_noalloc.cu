@@ -150,6 +150,7 @@ extern "C" int sl1m_forward_noalloc(sl1m_problem* prob, const double* x_dev, dou
     d.r = nullptr;
     d.fwd_out = d_out;
     d.adj_out = nullptr;
+    d.huge = nullptr;
     Plan pl{};
     pl.n_probs = 1;
     pl.C = H.C;
@@ -188,7 +189,7 @@ extern "C" int sl1m_forward_noalloc(sl1m_problem* prob, const double* x_dev, dou
     CKN(stage_to_device(base, img.data(), head, st, &ctx->n_launch));
     // every partial slot the finish reads is written by exactly one CTA of this
     // launch, so nothing in the scratch needs clearing
-    CKN(launch_gather_real(x_dev, d_x, lay.pix.orig, lay.pix.n_pad, 1.0, st));
+    CKN(launch_gather_real(x_dev, d_x, lay.pix.orig, lay.pix.n_pad, 1.0, nullptr, st));
     CKN(launch_forward(precision == SL1M_FP64 ? 0 : 1, gains, prob->n_ant, d_desc, d_plan, H.C, d_part, st));
     CKN(launch_fwd_finish(d_desc, d_plan, pl, ctx->num_sms, d_part, 0, nullptr, st));
     CKN(launch_scatter_cplx(d_out, (double2*)vis_out_dev, lay.vis.orig, lay.vis.n_pad, st));

@@ -8,18 +8,32 @@
 #include <math.h>
 
 #include "sl1m_dev.h"
+#include "sl1m_grid.h"
 #include "sl1m_kernels.h"
 
 namespace sl1m {
 
+// Marks an input of a lattice operator that needs the other scale (sl1m_grid.h).
+__device__ __forceinline__ void mark_huge(int* flag, double v)
+{
+    if (flag && !(fabs(v) < GR_HUGE)) *flag = 1;
+}
+__device__ __forceinline__ void mark_huge(int* flag, double2 v)
+{
+    mark_huge(flag, v.x);
+    mark_huge(flag, v.y);
+}
+
 // ---------------------------------------------------------- permutations
 
 __global__ void gather_real_kernel(const double* __restrict__ src, double* __restrict__ dst,
-                                   const int* __restrict__ orig, int n_pad, double scale)
+                                   const int* __restrict__ orig, int n_pad, double scale, int* huge)
 {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_pad; i += gridDim.x * blockDim.x) {
         const int o = orig[i];
-        dst[i] = o >= 0 ? src[o] * scale : 0.0;
+        const double v = o >= 0 ? src[o] * scale : 0.0;
+        dst[i] = v;
+        mark_huge(huge, v);
     }
 }
 
@@ -34,6 +48,7 @@ __global__ void gather_resid_kernel(const double2* __restrict__ src, const DevPr
         const double2 v = o >= 0 ? src[o] : make_double2(0.0, 0.0);
         dst[i] = v;
         write_polar(*P, polar, i, v);
+        mark_huge(P->huge ? P->huge + 1 : nullptr, v);
     }
 }
 
@@ -71,15 +86,16 @@ __global__ void weighted_vis_kernel(const DevProblem* __restrict__ P, int polar,
         const double2 v = make_double2(w * P->V[i].x, w * P->V[i].y);
         r[i] = v;
         write_polar(*P, polar, i, v);
+        mark_huge(P->huge ? P->huge + 1 : nullptr, v);
     }
 }
 
 static int grid_for(int n) { return n <= 0 ? 1 : (n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096; }
 
 cudaError_t launch_gather_real(const double* src, double* dst, const int* orig, int n_pad,
-                               double scale, cudaStream_t st)
+                               double scale, int* huge, cudaStream_t st)
 {
-    gather_real_kernel<<<grid_for(n_pad), 256, 0, st>>>(src, dst, orig, n_pad, scale);
+    gather_real_kernel<<<grid_for(n_pad), 256, 0, st>>>(src, dst, orig, n_pad, scale, huge);
     return cudaGetLastError();
 }
 cudaError_t launch_gather_resid(const double2* src, const DevProblem* P, int n_pad, int polar, double2* dst,
@@ -282,6 +298,7 @@ fwd_finish_kernel(const DevProblem* __restrict__ probs, const Plan* __restrict__
         const DevProblem& P = probs[p];
         const int mode = fwd_finish_mode(P);
         if (mode < 0) continue;
+        if (P.huge && e0 == 0 && threadIdx.x == 0) P.huge[0] = 0;      // (the operator is done with it)
         const int t = threadIdx.x % S::EL, e = e0 + t;
         const bool in = e < P.vis.n_pad;
         const int poff = pl.blk_poff[gb], ncon = in ? pl.blk_ncon[gb] : 0;
@@ -299,6 +316,7 @@ fwd_finish_kernel(const DevProblem* __restrict__ probs, const Plan* __restrict__
                 const double2 r = make_double2(W * s.x, W * s.y);
                 B.r[e] = r;
                 write_polar(P, polar, e, r);
+                mark_huge(P.huge ? P.huge + 1 : nullptr, r);
             } else {
                 const double W = P.vis.d[e].w;
                 const double2 V = P.V[e];
@@ -323,6 +341,7 @@ fwd_finish_kernel(const DevProblem* __restrict__ probs, const Plan* __restrict__
                 if (mode == FIN_INIT || !S2.algo) {
                     B.r[e] = r;
                     write_polar(P, polar, e, r);
+                    mark_huge(P.huge ? P.huge + 1 : nullptr, r);
                 }
             }
         }
@@ -369,6 +388,7 @@ adj_finish_kernel(const DevProblem* __restrict__ probs, const Plan* __restrict__
         const DevProblem& P = probs[p];
         const int mode = adj_finish_mode(P);
         if (mode < 0) continue;
+        if (P.huge && e0 == 0 && threadIdx.x == 0) P.huge[1] = 0;      // (the operator is done with it)
         const int t = threadIdx.x % S::EL, e = e0 + t;
         const bool in = e < P.pix.n_pad;
         const int poff = pl.blk_poff[gb], ncon = in ? pl.blk_ncon[gb] : 0;
@@ -393,6 +413,7 @@ adj_finish_kernel(const DevProblem* __restrict__ probs, const Plan* __restrict__
             } else if (mode == FIN_POWER) {
                 const double z = s * P.st->inv_mu;
                 B.xv[e] = z;
+                mark_huge(P.huge, z);
                 acc = z * z;
             } else {
                 const SolveState& S2 = *P.st;
@@ -400,6 +421,7 @@ adj_finish_kernel(const DevProblem* __restrict__ probs, const Plan* __restrict__
                 const double v = y0 - s * inv_L;
                 double In = v > thr ? v - thr : 0.0;
                 if (orig < 0) In = 0.0;
+                mark_huge(P.huge, In);
                 if (S2.algo) {
                     B.I[1][e] = In;                 // z_k; y is formed by the mix kernel
                 } else {
@@ -611,6 +633,7 @@ mfista_mix_kernel(const DevProblem* __restrict__ probs, const Plan* __restrict__
                 const double2 r = make_double2(W * (ayr - V.x), W * (ayi - V.y));
                 B.r[e] = r;
                 write_polar(P, polar, e, r);
+                mark_huge(P.huge ? P.huge + 1 : nullptr, r);
                 if (take) B.AI[0][e] = az;
             } else {
                 if (e >= P.pix.n_pad) continue;

@@ -405,7 +405,7 @@ cudaError_t wait_fault_clear(cudaStream_t) { return cudaSuccess; }
 cudaError_t launch_wait_selftest(unsigned long long*, int, cudaStream_t) { return cudaSuccess; }
 unsigned long long wait_limit_ns() { return 1; }
 int occupancy(int, bool, int, int) { return 4; }
-cudaError_t launch_gather_real(const double*, double*, const int*, int, double, cudaStream_t) { return cudaSuccess; }
+cudaError_t launch_gather_real(const double*, double*, const int*, int, double, int*, cudaStream_t) { return cudaSuccess; }
 cudaError_t launch_gather_resid(const double2*, const DevProblem*, int, int, double2*, cudaStream_t) { return cudaSuccess; }
 cudaError_t launch_scatter_real(const double*, double*, const int*, int, cudaStream_t) { return cudaSuccess; }
 cudaError_t launch_scatter_cplx(const double2*, double2*, const int*, int, cudaStream_t) { return cudaSuccess; }
