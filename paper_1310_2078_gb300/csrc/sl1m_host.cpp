@@ -1431,10 +1431,8 @@ int batch_set(sl1m_ctx* ctx, Batch& B, const std::vector<sl1m_problem*>& probs,
             const auto ta = ctx->tune.find(tune_key(precision, 1, c == 1, gauss, ua));
             if (tf != ctx->tune.end()) { B.nst[0][c] = tf->second.first; kf = tf->second.second; }
             if (ta != ctx->tune.end()) { B.nst[1][c] = ta->second.first; ka = ta->second.second; }
-            if (precision == 0 || c == 0) {         // no Gaussian pixels: the Dirac-only instances
-                B.nst[0][c] = shape_for(B.nst[0][c], gauss);
-                B.nst[1][c] = shape_for(B.nst[1][c], gauss);
-            }
+            B.nst[0][c] = shape_for(B.nst[0][c], gauss);    // no Gaussian pixels: the Dirac-only instances
+            B.nst[1][c] = shape_for(B.nst[1][c], gauss);
             const int occf = occupancy(precision == 0 ? 0 : 2, c == 1, std::max(1, B.n_ant_max), B.nst[0][c]);
             const int occa = occupancy(precision == 0 ? 1 : 3, c == 1, std::max(1, B.n_ant_max), B.nst[1][c]);
             kf = kf > 0 ? std::min(kf, occf) : occf;
@@ -2162,7 +2160,7 @@ int sl1m_autotune(sl1m_problem* prob, int precision, int32_t* nst_out, int32_t* 
         float best = 1e30f;
         int bcode = NST_DEFAULT, bk = 0;
         const auto time_shape = [&](int code, int k) -> float {
-            if (mixed_plain) code = shape_for(code, prob->has_gauss);
+            if (precision == SL1M_MIXED) code = shape_for(code, prob->has_gauss);
             DevPlan P;
             if (build_plan(nb, ns, ctx->num_sms * k, own_granules(precision, op, gains), P, st, &uc) != cudaSuccess) { rc = SL1M_ERR_CUDA; return 0.f; }
             const size_t need = (size_t)std::max(1, P.pl.n_slots) * P.pl.blk_el;
@@ -2196,7 +2194,7 @@ int sl1m_autotune(sl1m_problem* prob, int precision, int32_t* nst_out, int32_t* 
         for (size_t ci = 0; ci < cands.size(); ++ci) {
             const int nst = cands[ci];
             const int occ = occupancy((precision == SL1M_FP64 ? 0 : 2) + op, gains, std::max(1, prob->n_ant),
-                                      mixed_plain ? shape_for(nst, prob->has_gauss) : nst);
+                                      precision == SL1M_MIXED ? shape_for(nst, prob->has_gauss) : nst);
             float bn = 1e30f;
             for (int k = 1; k <= occ && rc == SL1M_OK; ++k) {
                 const float ms = time_shape(nst, k);

@@ -1360,6 +1360,15 @@ static FwdKernel fwd_kernel_of(int code)
     const int nst = shape_nst(code), np = shape_npoly(code);
     return shape_dirac_only(code) ? fwd_kernel_gs<false>(nst, np) : fwd_kernel_gs<true>(nst, np);
 }
+// With gains: without Gaussian pixels in the batch, an instance that holds its
+// visibilities' coordinates across granules, where the other reloads them to make
+// room for the Gaussian tiles (43,264 pixels x 38,676 visibilities, 48 antennas, 974 ->
+// 945 us; in the shared one such sets had become up to 4% slower than before it
+// took the linear tiles).
+static FwdKernel fwd_gains_kernel_of(int code)
+{
+    return shape_dirac_only(code) ? fwd_mixed_kernel<true, 1, 0, false> : fwd_mixed_kernel<true, 1, 0, true>;
+}
 // The no-gains adjoint stages 2 or 4 granules (with 8, its stage buffers and
 // per-warp records would leave room for 1 CTA per SM).
 static AdjKernel adj_kernel_of(int code)
@@ -1375,7 +1384,7 @@ cudaError_t launch_forward_mixed(bool gains, int n_ant, int nst, const DevProble
     // the dynamic shared-memory limits were raised by occupancy_mixed() when
     // the batch was built (not here: this may run under capture)
     if (gains)
-        fwd_mixed_kernel<true, 1><<<C, NTHREADS, fwd_smem_bytes(n_ant, true, 1), st>>>(probs, plp, partial);
+        fwd_gains_kernel_of(nst)<<<C, NTHREADS, fwd_smem_bytes(n_ant, true, 1), st>>>(probs, plp, partial);
     else
         fwd_kernel_of(nst)<<<C, NTHREADS, fwd_smem_bytes(0, false, nst), st>>>(probs, plp, partial);
     return cudaGetLastError();
@@ -1391,15 +1400,16 @@ cudaError_t launch_adjoint_mixed(bool gains, int n_ant, int nst, const DevProble
 
 int occupancy_mixed(int op, bool gains, int n_ant, int nst)
 {
-    static int fwd_smem_limit = 0, adj_smem_limit = 0;   // only ever raised
+    static int fwd_smem_limit[2] = {0, 0}, adj_smem_limit = 0;   // only ever raised
     if (op == 0) {
         if (gains) {
             const int sm = fwd_smem_bytes(n_ant, true, 1);
-            if (sm > fwd_smem_limit) {
-                cudaFuncSetAttribute(fwd_mixed_kernel<true, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-                fwd_smem_limit = sm;
+            int& limit = fwd_smem_limit[shape_dirac_only(nst)];
+            if (sm > limit) {
+                cudaFuncSetAttribute(fwd_gains_kernel_of(nst), cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+                limit = sm;
             }
-            return occ_of(fwd_mixed_kernel<true, 1>, sm);
+            return occ_of(fwd_gains_kernel_of(nst), sm);
         }
         const int sm = fwd_smem_bytes(0, false, nst);      // fixed per tile shape
         cudaFuncSetAttribute(fwd_kernel_of(nst), cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
