@@ -51,6 +51,16 @@ __host__ __device__ inline int gain_rows(int n_ant) { return (n_ant + 1) & ~1; }
 constexpr int NB_MAX = 28;
 constexpr int BT_CH = 16;             // pixels per chunk of that table
 constexpr int BT_P = BT_CH + 1;       // its padded row (rows start in different banks)
+// A granule of runs with up to OWN_MAX antenna pairs measures its offsets from each
+// pair's own centre (DevProblem::gcen; `ext` bounds those): a run of one pair's samples
+// is a short track, but the granule of several is wide, and the phase of the offsets
+// is rounded, and handed to the SFU, with an error that grows with it.  65,536
+// multiscale pixels x 32,000 visibilities, errors (mean of three draws) forward /
+// adjoint: granules of neighbours 3.70e-7 / 3.56e-7, of runs 4.05e-7 / 3.90e-7 from
+// one centre and 3.69e-7 / 3.58e-7 from their own, in 1,869 us instead of 1,931 and 1,510
+// instead of 1,411.  Slot of a visibility's pair: w of its offset residual (an int's
+// bits).
+constexpr int OWN_MAX = 8, GNB_OWN = 256;
 constexpr int BLK_GRAN = 8;           // owned granules per CTA (one per warp)
 constexpr int BLK = G * BLK_GRAN;     // owned elements per CTA block
 constexpr int NTHREADS = 256;         // 8 warps
@@ -141,7 +151,11 @@ struct DevProblem {
     const int2* ant;          // [vis.n_pad] antenna pair (a, b)
     const int* vslot;         // gains: [vis.n_pad] slot of the visibility's pair in its granule's list
     const int2* gbl;          // gains: [vis.n_gran][NB_MAX] the granule's distinct pairs, sorted
-    const int* gnb;           // gains: [vis.n_gran] number of pairs, 0 if more than NB_MAX
+    const int* gnb;           // gains: [vis.n_gran] number of pairs, 0 if more than NB_MAX; GNB_OWN added
+                              // where the pairs have centres of their own
+    const float4* vown;       // gains: [vis.n_pad] offset from the own centre of the visibility's pair, or of its granule
+    const float4* gcen;       // gains: [vis.n_gran][OWN_MAX] offset of each pair's centre from the granule's;
+                              // w of the first: 1 where the pairs have them
     const double2* V;         // [vis.n_pad] measured visibilities (sorted)
     const float4* pgauss;     // [pix.n_pad] {l, m, (l^2+m^2)/2, nu = n-1+(l^2+m^2)/2}
     const float4* pgoff;      // [pix.n_pad] {dl, dm, dn, q}: offsets from the granule's centre, q that of

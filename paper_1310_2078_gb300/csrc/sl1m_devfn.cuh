@@ -49,6 +49,22 @@ __device__ __forceinline__ float tp_frac(float ah, float al, float bh, float bl)
     return __fadd_rn(f, lo);
 }
 
+// e . (x, y, z) in turns up to a whole number: the remainders of the first two
+// products, each rounded once; the third, of n - 1, is small.
+__device__ __forceinline__ float turns_of(const float4 e, float x, float y, float z)
+{
+    const float M = 12582912.0f;
+    const float a = __fmaf_rn(e.x, x, -__fsub_rn(__fmaf_rn(e.x, x, M), M));
+    const float b = __fmaf_rn(e.y, y, -__fsub_rn(__fmaf_rn(e.y, y, M), M));
+    return __fmaf_rn(e.z, z, __fadd_rn(a, b));
+}
+// A visibility's offset (o, residual lo) from its own pair's centre (sl1m_dev.h: OWN_MAX).
+__device__ __forceinline__ float4 own_offset(const float4 o, const float4 lo, const float4* cen)
+{
+    const float4 e = cen[__float_as_int(lo.w)];
+    return make_float4(__fadd_rn(o.x - e.x, lo.x), __fadd_rn(o.y - e.y, lo.y), __fadd_rn(o.z - e.z, lo.z), o.w);
+}
+
 // frac(a . b) over x, y, z in turns, result in [-0.5, 0.5].
 __device__ __forceinline__ float frac_dot3(const float4 ah, const float4 al,
                                            const float4 bh, const float4 bl)
@@ -56,6 +72,13 @@ __device__ __forceinline__ float frac_dot3(const float4 ah, const float4 al,
     float s = __fadd_rn(tp_frac(ah.x, al.x, bh.x, bl.x), tp_frac(ah.y, al.y, bh.y, bl.y));
     s = __fadd_rn(s, tp_frac(ah.z, al.z, bh.z, bl.z));
     return frac_turns(s);
+}
+
+// frac_dot3 with a rounding less at a turn and more (for a term that a whole tile shares).
+__device__ __forceinline__ float frac_dot3_near(const float4 ah, const float4 al, const float4 bh, const float4 bl)
+{
+    const float s = frac_turns(__fadd_rn(tp_frac(ah.x, al.x, bh.x, bl.x), tp_frac(ah.y, al.y, bh.y, bl.y)));
+    return frac_turns(__fadd_rn(s, tp_frac(ah.z, al.z, bh.z, bl.z)));
 }
 
 // sin and cos of ph (radians, |ph| < 2^22 turns) on the FMA pipe, for a share

@@ -4,6 +4,7 @@
 #include "sl1m.h"
 
 #include <algorithm>
+#include <array>
 #include <atomic>
 #include <future>
 #include <thread>
@@ -126,6 +127,75 @@ static void kd_append(std::vector<int>& order, std::vector<int> members, const d
     while (order.size() % G) order.push_back(-1);
 }
 
+// Pairs' own centres are worth their work (41 instructions a table row, not 28) where
+// they make a granule's offsets this much shorter, and these bound a phase of so many
+// turns in the mean pixel granule: the terms that do not depend on the order are
+// up to half a turn themselves.
+constexpr double OWN_GAIN = 0.75, OWN_FROM = 0.5;
+
+// Mean half extents of the pixel granules.
+static std::array<double, 3> mean_extent(const std::vector<float4>& pext)
+{
+    std::array<double, 3> m = {0, 0, 0};
+    for (const float4& p : pext) {
+        m[0] += p.x;
+        m[1] += p.y;
+        m[2] += p.z;
+    }
+    for (double& v : m) v /= (double)std::max<size_t>(1, pext.size());
+    return m;
+}
+
+// Half extents of a granule's offsets as the kernels bound them: of its members or,
+// in an order of runs (keys: the pair of every visibility), where the granule has no more
+// than OWN_MAX pairs and it pays, of each pair's members about the pair's own centre.
+struct Reach {
+    float e[3];
+    int n_pairs = 0;                             // OWN_MAX + 1: more (without keys: 0)
+    bool own = false;
+};
+static Reach granule_reach(const int* members, const double* uvw, const long long* keys, const std::array<double, 3>& pmean)
+{
+    struct Box {
+        long long key;
+        double mn[3], mx[3];
+        void add(const double* x)
+        {
+            for (int a = 0; a < 3; ++a) {
+                mn[a] = std::min(mn[a], x[a]);
+                mx[a] = std::max(mx[a], x[a]);
+            }
+        }
+    };
+    const Box none = {0, {1e300, 1e300, 1e300}, {-1e300, -1e300, -1e300}};
+    Box all = none, of[OWN_MAX];
+    Reach r;
+    int& n = r.n_pairs;
+    for (int i = 0; i < G; ++i) {
+        const int o = members[i];
+        if (o < 0) continue;
+        const double* x = uvw + 3 * (size_t)o;
+        all.add(x);
+        if (!keys || n > OWN_MAX) continue;
+        int s = 0;
+        while (s < n && of[s].key != keys[o]) ++s;
+        if (s == n && n++ < OWN_MAX) {
+            of[s] = none;
+            of[s].key = keys[o];
+        }
+        if (s < OWN_MAX) of[s].add(x);
+    }
+    double wa[3], wo[3] = {0, 0, 0};
+    for (int a = 0; a < 3; ++a) {
+        wa[a] = std::max(0.0, all.mx[a] - all.mn[a]);
+        for (int s = 0; s < n && n <= OWN_MAX; ++s) wo[a] = std::max(wo[a], of[s].mx[a] - of[s].mn[a]);
+    }
+    r.own = keys && n <= OWN_MAX && wo[0] + wo[1] + wo[2] <= OWN_GAIN * (wa[0] + wa[1] + wa[2]) &&
+            0.5 * (wa[0] * pmean[0] + wa[1] * pmean[1] + wa[2] * pmean[2]) >= OWN_FROM;
+    for (int a = 0; a < 3; ++a) r.e[a] = (float)(0.5 * (r.own ? wo[a] : wa[a]));
+    return r;
+}
+
 // Reorder whole visibility granules (members unchanged) by the share of
 // (visibility granule, pixel granule) tiles whose extents bound the phase
 // product term above D_MAX turns, which the mixed kernels evaluate on the
@@ -134,27 +204,20 @@ static void kd_append(std::vector<int>& order, std::vector<int> members, const d
 // granule costs: a wide granule among narrow ones leaves 7 warps idle.  A
 // stable sort by that share (most granules: 0, kept in k-d order) groups the
 // wide ones into the same blocks.  The share is taken against up to 1,024
-// pixel granules (every ceil(n/1024)-th), with the extents as half the
-// bounding box, as layout_side computes them.
-static void group_by_exact_share(std::vector<int>& order, const double* uvw, const std::vector<float4>& pext)
+// pixel granules (every ceil(n/1024)-th), with the extents as the layout
+// computes them (granule_reach).
+static void group_by_exact_share(std::vector<int>& order, const double* uvw, const long long* keys,
+                                 const std::vector<float4>& pext)
 {
     const size_t ng = order.size() / G;
     if (ng < 2 || pext.empty()) return;
     const size_t step = (pext.size() + 1023) / 1024;
+    const std::array<double, 3> pmean = mean_extent(pext);
     std::vector<std::pair<float, int>> key(ng);
     parallel_chunks(ng, 256, [&](size_t g0, size_t g1) {
         for (size_t g = g0; g < g1; ++g) {
-            double mn[3] = {1e300, 1e300, 1e300}, mx[3] = {-1e300, -1e300, -1e300};
-            for (size_t i = g * G; i < (g + 1) * G; ++i) {
-                const int o = order[i];
-                if (o < 0) continue;
-                for (int a = 0; a < 3; ++a) {
-                    mn[a] = std::min(mn[a], uvw[3 * (size_t)o + a]);
-                    mx[a] = std::max(mx[a], uvw[3 * (size_t)o + a]);
-                }
-            }
-            const float e[3] = {(float)(0.5 * (mx[0] - mn[0])), (float)(0.5 * (mx[1] - mn[1])),
-                                (float)(0.5 * (mx[2] - mn[2]))};
+            const Reach reach = granule_reach(order.data() + g * G, uvw, keys, pmean);
+            const float* e = reach.e;
             int n_ex = 0, n = 0;
             for (size_t p = 0; p < pext.size(); p += step, ++n)
                 n_ex += e[0] * pext[p].x + e[1] * pext[p].y + e[2] * pext[p].z > D_MAX;
@@ -243,37 +306,48 @@ static std::vector<int> order_by_runs(const std::vector<long long>& keys, const 
 // Relative cost of the gains kernels' tiles over all granules of an order: a
 // pair takes about 15 instructions (three times that on the exact phase path),
 // and every distinct antenna pair of a granule about 28 per streamed pixel
-// (the pair table); a granule with more than NB_MAX pairs takes gathers, about
-// 10 more a pair.
-static double gains_order_cost(const std::vector<int>& order, const std::vector<long long>& keys, const double* uvw,
-                               const std::vector<float4>& pext)
+// (the pair table; 41 with a centre of its own); a granule with more than NB_MAX
+// pairs takes gathers, about 10 more a pair.  runs: as granule_reach takes own centres.
+struct OrderCost {
+    double cost = 0.0;
+    double spread2 = 0.0;                         // mean square of the phase bound of the offsets' product, over tiles
+};
+static OrderCost gains_order_cost(const std::vector<int>& order, const std::vector<long long>& keys, bool runs,
+                                  const double* uvw, const std::vector<float4>& pext)
 {
     const size_t ng = order.size() / G, step = (pext.size() + 255) / 256;
-    std::vector<double> cost(ng, 0.0);
+    const std::array<double, 3> pmean = mean_extent(pext);
+    std::vector<OrderCost> cost(ng);
     parallel_chunks(ng, 64, [&](size_t g0, size_t g1) {
         std::vector<long long> ks;
         for (size_t g = g0; g < g1; ++g) {
-            double mn[3] = {1e300, 1e300, 1e300}, mx[3] = {-1e300, -1e300, -1e300};
-            ks.clear();
-            for (size_t i = g * G; i < (g + 1) * G; ++i) {
-                const int o = order[i];
-                if (o < 0) continue;
-                ks.push_back(keys[o]);
-                for (int a = 0; a < 3; ++a) {
-                    mn[a] = std::min(mn[a], uvw[3 * (size_t)o + a]);
-                    mx[a] = std::max(mx[a], uvw[3 * (size_t)o + a]);
-                }
+            const Reach reach = granule_reach(order.data() + g * G, uvw, runs ? keys.data() : nullptr, pmean);
+            const float* e = reach.e;
+            int nb = runs ? reach.n_pairs : OWN_MAX + 1;
+            const double row = reach.own ? 41.0 : 28.0;
+            if (nb > OWN_MAX) {
+                ks.clear();
+                for (size_t i = g * G; i < (g + 1) * G; ++i)
+                    if (order[i] >= 0) ks.push_back(keys[order[i]]);
+                std::sort(ks.begin(), ks.end());
+                nb = (int)(std::unique(ks.begin(), ks.end()) - ks.begin());
             }
-            std::sort(ks.begin(), ks.end());
-            const int nb = (int)(std::unique(ks.begin(), ks.end()) - ks.begin());
             int n_ex = 0, n = 0;
-            for (size_t p = 0; p < pext.size(); p += step, ++n)
-                n_ex += 0.5 * ((mx[0] - mn[0]) * pext[p].x + (mx[1] - mn[1]) * pext[p].y + (mx[2] - mn[2]) * pext[p].z) > D_MAX;
-            cost[g] = G * (15.0 + 30.0 * n_ex / std::max(1, n)) + (nb <= NB_MAX ? 28.0 * nb : 10.0 * G);
+            double d2 = 0.0;
+            for (size_t p = 0; p < pext.size(); p += step, ++n) {
+                const float d = e[0] * pext[p].x + e[1] * pext[p].y + e[2] * pext[p].z;
+                n_ex += d > D_MAX;
+                d2 += d > D_MAX ? 0.0 : (double)d * d;
+            }
+            cost[g].cost = G * (15.0 + 30.0 * n_ex / std::max(1, n)) + (nb <= NB_MAX ? row * nb : 10.0 * G);
+            cost[g].spread2 = d2 / std::max(1, n) / (double)ng;
         }
     });
-    double t = 0;
-    for (double c : cost) t += c;
+    OrderCost t;
+    for (const OrderCost& c : cost) {
+        t.cost += c.cost;
+        t.spread2 += c.spread2;
+    }
     return t;
 }
 
@@ -364,6 +438,53 @@ static void layout_side(const std::vector<int>& order, const std::vector<d4>& xy
         }
     }
     });
+}
+
+// The offsets of granule g from its pairs' own centres (slots vslot, nb of them),
+// where that pays (false: left as it is): centres relative to the granule's, in FP32
+// (w of the first: 1), the slot beside every offset's residual, and the granule's
+// extent as these offsets bound it.
+static bool own_centres(HostSide& H, int g, const int* vslot, int nb, const std::array<double, 3>& pmean, float4* cen,
+                        float4* own)
+{
+    double mn[OWN_MAX][3], mx[OWN_MAX][3], far[3] = {0, 0, 0};
+    std::fill(&mn[0][0], &mn[0][0] + 3 * OWN_MAX, 1e300);
+    std::fill(&mx[0][0], &mx[0][0] + 3 * OWN_MAX, -1e300);
+    const auto offset = [&](int i, double d[3]) {
+        d[0] = (double)H.off[i].x + H.offlo[i].x;
+        d[1] = (double)H.off[i].y + H.offlo[i].y;
+        d[2] = (double)H.off[i].z + H.offlo[i].z;
+    };
+    double d[3];
+    for (int i = g * G; i < (g + 1) * G; ++i) {
+        offset(i, d);
+        const int s = vslot[i];
+        for (int a = 0; a < 3; ++a) {
+            mn[s][a] = std::min(mn[s][a], d[a]);
+            mx[s][a] = std::max(mx[s][a], d[a]);
+        }
+    }
+    double w[3] = {0, 0, 0};
+    for (int s = 0; s < nb; ++s)
+        for (int a = 0; a < 3; ++a) w[a] = std::max(w[a], 0.5 * (mx[s][a] - mn[s][a]));
+    const float4 all = H.ext[g];
+    if (w[0] + w[1] + w[2] > OWN_GAIN * ((double)all.x + all.y + all.z) ||
+        all.x * pmean[0] + all.y * pmean[1] + all.z * pmean[2] < OWN_FROM)
+        return false;
+    for (int s = 0; s < nb; ++s)
+        cen[s] = make_float4((float)(0.5 * (mn[s][0] + mx[s][0])), (float)(0.5 * (mn[s][1] + mx[s][1])),
+                             (float)(0.5 * (mn[s][2] + mx[s][2])), s == 0 ? 1.f : 0.f);
+    for (int i = g * G; i < (g + 1) * G; ++i) {
+        offset(i, d);
+        const float4 c = cen[vslot[i]];
+        std::memcpy(&H.offlo[i].w, &vslot[i], sizeof(float));
+        far[0] = std::max(far[0], std::fabs(d[0] - c.x));
+        far[1] = std::max(far[1], std::fabs(d[1] - c.y));
+        far[2] = std::max(far[2], std::fabs(d[2] - c.z));
+        own[i] = make_float4((float)(d[0] - c.x), (float)(d[1] - c.y), (float)(d[2] - c.z), H.off[i].w);
+    }
+    H.ext[g] = make_float4((float)(far[0] * 1.0000002), (float)(far[1] * 1.0000002), (float)(far[2] * 1.0000002), 0.f);
+    return true;
 }
 
 // ============================================================ device buffers
@@ -643,6 +764,7 @@ struct ProblemDev {
     DBuf<double2> r64;               // made by the first FP64 call
     DBuf<int> vslot, gnb;
     DBuf<int2> gbl;
+    DBuf<float4> gcen, vown;
     DBuf<double2> V;
     DBuf<float4> pgauss, pgoff;
     DBuf<d4> pgauss64;
@@ -861,25 +983,29 @@ int sl1m_problem::rebuild(cudaStream_t st, size_t grid_budget)
         std::vector<int> members(n_vis);
         for (int64_t k = 0; k < n_vis; ++k) members[k] = (int)k;
         std::vector<int> order;
+        std::vector<long long> keys;
+        bool runs = false;                       // with gains: an order of runs was taken
         if (n_ant == 0) {
             kd_append(order, std::move(members), uvw.data(), uvw.data() + 1, 3);
         } else {
-            // the cheapest of the point order and of runs of 16, 8 and 4 samples
-            // of a pair (tried while the mean pair has that many), each made by a
-            // thread of its own, or here where none can be had
-            std::vector<long long> keys(n_vis);
+            // the cheapest of the point order and of runs of 16, 8 and 4 samples of a
+            // pair (tried while the mean pair has that many), each made by a thread of
+            // its own, or here where none can be had.  Runs count only where their offsets
+            // are in the mean square no longer than the point order's: a phase is rounded
+            // with an error that grows with them.
+            keys.resize(n_vis);
             for (int64_t k = 0; k < n_vis; ++k) keys[k] = (long long)ant[2 * k] * n_ant + ant[2 * k + 1];
             const std::vector<int> by = sort_by_pair(ant, n_ant, n_vis);
             int64_t distinct = 1;
             for (int64_t k = 1; k < n_vis; ++k) distinct += keys[by[k]] != keys[by[k - 1]];
             const double per = (double)n_vis / (double)distinct;
-            using Tried = std::pair<double, std::vector<int>>;
+            using Tried = std::pair<OrderCost, std::vector<int>>;
             std::vector<std::future<Tried>> tried;
             for (int s = 16; s >= 4; s /= 2)
                 if (per >= 0.75 * s) {
                     const auto job = [&, s]() -> Tried {
                         std::vector<int> o = order_by_runs(keys, by, uvw.data(), s);
-                        const double c = gains_order_cost(o, keys, uvw.data(), gext_pix);
+                        const OrderCost c = gains_order_cost(o, keys, true, uvw.data(), gext_pix);
                         return {c, std::move(o)};
                     };
                     try {
@@ -889,24 +1015,24 @@ int sl1m_problem::rebuild(cudaStream_t st, size_t grid_budget)
                     }
                 }
             kd_append(order, std::move(members), uvw.data(), uvw.data() + 1, 3);
-            double best = gains_order_cost(order, keys, uvw.data(), gext_pix);
+            const OrderCost point = gains_order_cost(order, keys, false, uvw.data(), gext_pix);
+            double best = point.cost;
             for (auto& f : tried) {
                 Tried t = f.get();
-                if (t.first < best) {
-                    best = t.first;
+                if (t.first.cost < best && t.first.spread2 <= point.spread2) {
+                    best = t.first.cost;
+                    runs = true;
                     order.swap(t.second);
                 }
             }
         }
-        group_by_exact_share(order, uvw.data(), gext_pix);
+        group_by_exact_share(order, uvw.data(), runs ? keys.data() : nullptr, gext_pix);
         if (n_ant > 0) sort_baselines(order, ant);
         std::vector<d4> xyz(n_vis);
         for (int64_t k = 0; k < n_vis; ++k)
             xyz[k] = make_d4(uvw[3 * k], uvw[3 * k + 1], uvw[3 * k + 2], weights.empty() ? 1.0 : weights[k]);
         HostSide H;
         layout_side(order, xyz, (int)n_vis, H);
-        CK(upload_side(H, D.vis, hp.vis, st));
-        gext_vis = H.ext;
         std::vector<int2> a(H.n_pad, make_int2(0, 0));
         std::vector<double2> Vs(H.n_pad, make_double2(0.0, 0.0));
         for (int i = 0; i < H.n_pad; ++i) {
@@ -915,22 +1041,15 @@ int sl1m_problem::rebuild(cudaStream_t st, size_t grid_budget)
             if (!ant.empty()) a[i] = make_int2(ant[2 * o], ant[2 * o + 1]);
             Vs[i] = make_double2(vis[2 * o], vis[2 * o + 1]);
         }
-        CK(D.ant.upload(a.data(), a.size(), st));
-        CK(D.V.upload(Vs.data(), Vs.size(), st));
-        // {u, v, -2 w, u^2 + v^2} in FP32, as the adjoint's Gaussian terms take it
-        std::vector<float4> ga(H.n_pad);
-        for (int i = 0; i < H.n_pad; ++i) {
-            const float4 h = H.hi[i];
-            ga[i] = make_float4(h.x, h.y, -2.0f * h.z, std::fmaf(h.x, h.x, h.y * h.y));
-        }
-        CK(D.vgabs.upload(ga.data(), ga.size(), st));
-        CK(D.r32.upload(nullptr, H.n_pad, st, true));
-        vis_orig = H.orig;
         if (n_ant > 0) {
             // each granule's distinct antenna pairs (adjacent after sort_baselines)
             gpairs_vis.assign(H.n_gran, 0);
+            gown_vis.assign(H.n_gran, 0);
+            const std::array<double, 3> pmean = mean_extent(gext_pix);
             std::vector<int> vslot(H.n_pad, 0), gnb(H.n_gran, 0);
             std::vector<int2> gbl((size_t)H.n_gran * NB_MAX, make_int2(0, 0));
+            std::vector<float4> gcen((size_t)H.n_gran * OWN_MAX, make_float4(0.f, 0.f, 0.f, 0.f));
+            std::vector<float4> vown(H.off.begin(), H.off.end());
             for (int g = 0; g < H.n_gran; ++g) {
                 int nb = 0;
                 bool over = false;
@@ -944,17 +1063,38 @@ int sl1m_problem::rebuild(cudaStream_t st, size_t grid_budget)
                     vslot[i] = nb - 1;
                 }
                 gnb[g] = over ? 0 : nb;
+                if (runs && !over && nb <= OWN_MAX &&
+                    own_centres(H, g, vslot.data(), nb, pmean, gcen.data() + (size_t)g * OWN_MAX, vown.data()))
+                    gnb[g] += GNB_OWN;
+                gown_vis[g] = gnb[g] >= GNB_OWN;
                 for (int i = g * G; i < (g + 1) * G; ++i)
                     gpairs_vis[g] += i == g * G || a[i].x != a[i - 1].x || a[i].y != a[i - 1].y;
             }
             CK(D.vslot.upload(vslot.data(), vslot.size(), st));
             CK(D.gbl.upload(gbl.data(), gbl.size(), st));
             CK(D.gnb.upload(gnb.data(), gnb.size(), st));
+            CK(D.gcen.upload(gcen.data(), gcen.size(), st));
+            CK(D.vown.upload(vown.data(), vown.size(), st));
         } else {
             D.vslot.free();
             D.gbl.free();
             D.gnb.free();
+            D.gcen.free();
+            D.vown.free();
         }
+        CK(upload_side(H, D.vis, hp.vis, st));
+        gext_vis = H.ext;
+        CK(D.ant.upload(a.data(), a.size(), st));
+        CK(D.V.upload(Vs.data(), Vs.size(), st));
+        // {u, v, -2 w, u^2 + v^2} in FP32, as the adjoint's Gaussian terms take it
+        std::vector<float4> ga(H.n_pad);
+        for (int i = 0; i < H.n_pad; ++i) {
+            const float4 h = H.hi[i];
+            ga[i] = make_float4(h.x, h.y, -2.0f * h.z, std::fmaf(h.x, h.x, h.y * h.y));
+        }
+        CK(D.vgabs.upload(ga.data(), ga.size(), st));
+        CK(D.r32.upload(nullptr, H.n_pad, st, true));
+        vis_orig = H.orig;
     }
     // constants per (visibility, Gaussian scale), for few scales; the pixel
     // granules' headers name the scale too
@@ -988,6 +1128,8 @@ int sl1m_problem::rebuild(cudaStream_t st, size_t grid_budget)
     hp.vslot = n_ant > 0 ? D.vslot.p : nullptr;
     hp.gbl = n_ant > 0 ? D.gbl.p : nullptr;
     hp.gnb = n_ant > 0 ? D.gnb.p : nullptr;
+    hp.gcen = n_ant > 0 ? D.gcen.p : nullptr;
+    hp.vown = n_ant > 0 ? D.vown.p : nullptr;
     hp.V = D.V.p;
     hp.pgauss = D.pgauss.p;
     hp.pgoff = has_gauss ? D.pgoff.p : D.pgauss.p;
@@ -1047,11 +1189,12 @@ const UnitCost& sl1m_problem::unit_cost(int precision, int op)
     const bool any_exact = precision == 1 && (mo.x * ms.x + mo.y * ms.y + mo.z * ms.z) > D_MAX;
     // gains: a tile's own cost of the antenna pairs of its visibility granule, in
     // units of its pairs' (instructions of a tile of 64 x 64: forward 2,414 + 70 per
-    // pair table row, or 640 more with gathers; adjoint 2,180 + 30 per run)
+    // pair table row, or 640 more with gathers; adjoint 2,180 + 30 per run; 28 and 26
+    // more where pairs have centres of their own)
     const bool by_pairs = n_ant > 0 && precision == 1 && !gpairs_vis.empty();
     const auto pair_cost = [&](int g) {
-        const int nb = gpairs_vis[g];
-        return op == 0 ? (nb <= NB_MAX ? 70.0 * nb : 640.0 * 2) / 2414.0 : 30.0 * nb / 2180.0;
+        const int nb = gpairs_vis[g], own = gown_vis[g];
+        return op == 0 ? (nb <= NB_MAX ? (70.0 + 28.0 * own) * nb : 640.0 * 2) / 2414.0 : (30.0 + 26.0 * own) * nb / 2180.0;
     };
     uc.uniform = base(k0) * gfac;
     if (one_kind && !any_exact && !by_pairs) return uc;
@@ -1092,7 +1235,7 @@ size_t sl1m_problem::estimate_bytes(int precision) const
     size_t b = nv * (4 * 16 + 32 + 4 + 8 + 16) + np * (4 * 16 + 32 + 4 + 16 + 32);
     if (n_ant > 0) {
         b += (size_t)gain_rows(n_ant) * GP * (np / G) * 8 + (size_t)n_ant * np * 16;   // FP32 + FP64
-        b += nv * 4 + (nv / G) * (NB_MAX * 8 + 4);                                     // pair lists
+        b += nv * (4 + 16) + (nv / G) * (NB_MAX * 8 + 4 + OWN_MAX * 16);                // pair lists, own centres
     }
     b += np * 8 * 4 + nv * 16 * 3;                 // solver vectors
     b += nv * (16 + 8);                            // the adjoint's FP32 Gaussian terms and residual
@@ -1228,7 +1371,7 @@ size_t sl1m_problem::dev_bytes() const
     };
     side(D.vis);
     side(D.pix);
-    b += D.ant.bytes() + D.vgabs.bytes() + D.gcls.bytes() + D.gclass.bytes() + D.r32.bytes() + D.r64.bytes() + D.vslot.bytes() + D.gbl.bytes() + D.gnb.bytes() + D.V.bytes() + D.pgauss.bytes() + D.pgoff.bytes() + D.pgauss64.bytes() + D.gsig.bytes() +
+    b += D.ant.bytes() + D.vgabs.bytes() + D.gcls.bytes() + D.gclass.bytes() + D.r32.bytes() + D.r64.bytes() + D.vslot.bytes() + D.gbl.bytes() + D.gnb.bytes() + D.gcen.bytes() + D.vown.bytes() + D.V.bytes() + D.pgauss.bytes() + D.pgoff.bytes() + D.pgauss64.bytes() + D.gsig.bytes() +
          D.gsig64.bytes() + D.gkind.bytes() + D.pghdr.bytes() + D.gpol32.bytes() + D.gains64.bytes();
     b += D.x_user.bytes() + D.x_sorted.bytes() + D.adj_sorted.bytes() + D.img_user.bytes() +
          D.r_user.bytes() + D.r_sorted.bytes() + D.fwd_sorted.bytes() + D.vis_user.bytes();

@@ -291,6 +291,7 @@ struct sl1m_problem {
     std::vector<int> gkind_pix;               // pixel granule kinds
     std::vector<double> gsig_pix;             // and scales
     std::vector<int> gpairs_vis;              // gains: runs of equal antenna pairs per visibility granule
+    std::vector<char> gown_vis;               // gains: whether its pairs have centres of their own
     UnitCost ucost[2][2];                      // [precision][0 forward / 1 adjoint]
     bool ucost_ok[2][2] = {{false, false}, {false, false}};
     std::unique_ptr<Batch> op_batch[2], solve_batch[2];

@@ -246,19 +246,40 @@ __device__ __forceinline__ void fwd_gauss_tile(const float4* __restrict__ s_off,
 // Pixels per chunk: as many of the granule's 64 as the table holds rows for
 // (lch: their log2), since building a chunk is a chain of shared loads, a
 // logarithm and a store that only its 32 entries at a time overlap.
+// cen: the pairs' own centres, or null.  Their products with the pixels' offsets s_off
+// are equal for all samples of a pair, so they belong to the entries: a lane takes a
+// pixel for all pairs and reads its offset once.
 __device__ __forceinline__ int pair_chunk_log2(int nb)
 {
     return nb * (64 + 1) <= NB_MAX * BT_P ? 6 : nb * (32 + 1) <= NB_MAX * BT_P ? 5 : 4;
 }
 template <bool LOG>
 __device__ __forceinline__ void build_pair_table(float2* __restrict__ T, const int2* __restrict__ bl, int nb,
-                                                 const float2* __restrict__ sBa,
-                                                 const float2* __restrict__ gtab, int c0, int lch, int lane)
+                                                 const float2* __restrict__ sBa, const float4* __restrict__ s_off,
+                                                 const float4* __restrict__ cen, const float2* __restrict__ gtab,
+                                                 int c0, int lch, int lane)
 {
     const int n = nb << lch, row = (1 << lch) + 1;
-#pragma unroll 3
-    for (int e = lane; e < n; e += 32) {
-        const int s = e >> lch, jj = e & ((1 << lch) - 1), j = c0 + jj;
+    if (cen) {                                    // (few pairs: chunks of 32 pixels or more)
+        for (int jj = lane; jj < 1 << lch; jj += 32) {
+            const int j = c0 + jj;
+            const float2 ba = sBa[j];
+            const float4 o = s_off[j];
+            const float b0 = fmaf(ba.x, INV_TWO_PI_F, ba.y < 0.f ? -0.5f : 0.f), a0 = fabsf(ba.y);
+#pragma unroll 4
+            for (int s = 0; s < nb; ++s) {
+                const int2 ab = bl[s];
+                const float2 ga = gtab[ab.x * GP + j], gb = gtab[ab.y * GP + j];
+                const float ph = frac_turns(frac_turns(b0 - (ga.y - gb.y)) + turns_of(cen[s], o.x, o.y, o.z)) * TWO_PI_F;
+                const float m = a0 * (ga.x * gb.x);
+                T[s * row + jj] = make_float2(ph, LOG ? __log2f(m) : m);
+            }
+        }
+        return;
+    }
+    // (most pairs: chunks of BT_CH pixels, the places at constant strides)
+    const auto entry = [&](int s, int jj, int at) {
+        const int j = c0 + jj;
         const int2 ab = bl[s];
         const float2 ga = gtab[ab.x * GP + j], gb = gtab[ab.y * GP + j];
         const float2 ba = sBa[j];                                    // {B_j (radians), a_j}
@@ -266,7 +287,17 @@ __device__ __forceinline__ void build_pair_table(float2* __restrict__ T, const i
         const float arg = (ga.y - gb.y) + (ba.y < 0.f ? 0.5f : 0.f);
         const float ph = frac_turns(fmaf(ba.x, INV_TWO_PI_F, -arg)) * TWO_PI_F;
         const float m = fabsf(ba.y) * (ga.x * gb.x);
-        T[s * row + jj] = make_float2(ph, LOG ? __log2f(m) : m);   // log2(0) = -inf: amplitude 0
+        T[at] = make_float2(ph, LOG ? __log2f(m) : m);              // log2(0) = -inf: amplitude 0
+    };
+    if (1 << lch == BT_CH) {
+#pragma unroll 3
+        for (int e = lane; e < n; e += 32) entry(e / BT_CH, e % BT_CH, e / BT_CH * BT_P + e % BT_CH);
+    } else {
+#pragma unroll 3
+        for (int e = lane; e < n; e += 32) {
+            const int s = e >> lch, jj = e & ((1 << lch) - 1);
+            entry(s, jj, s * row + jj);
+        }
     }
 }
 
@@ -275,13 +306,13 @@ __device__ __forceinline__ void fwd_dirac_tile_pt(const float4* __restrict__ s_o
                                                   const float4* __restrict__ s_lo,
                                                   const float2* __restrict__ sBa,
                                                   const float2* __restrict__ gtab, float2* __restrict__ T,
-                                                  const int2* __restrict__ bl, int nb, int lch, const int (&toff)[2],
-                                                  const float4 (&dx)[2], const float4 (&dxl)[2], int lane,
-                                                  float (&sr)[2], float (&si)[2])
+                                                  const int2* __restrict__ bl, const float4* __restrict__ cen, int nb,
+                                                  int lch, const int (&toff)[2], const float4 (&dx)[2],
+                                                  const float4 (&dxl)[2], int lane, float (&sr)[2], float (&si)[2])
 {
 #pragma unroll 1
     for (int c0 = 0; c0 < G; c0 += 1 << lch) {
-        build_pair_table<false>(T, bl, nb, sBa, gtab, c0, lch, lane);
+        build_pair_table<false>(T, bl, nb, sBa, s_off, cen, gtab, c0, lch, lane);
         __syncwarp();
 #pragma unroll 1
         for (int j8 = 0; j8 < 1 << lch; j8 += 8)
@@ -313,13 +344,13 @@ __device__ __forceinline__ void fwd_gauss_tile_pt(const float4* __restrict__ s_o
                                                   const float4* __restrict__ s_pg,
                                                   const float2* __restrict__ sBa,
                                                   const float2* __restrict__ gtab, float2* __restrict__ T,
-                                                  const int2* __restrict__ bl, int nb, int lch, const int (&toff)[2],
-                                                  const GaussTile (&gt)[2], const float4 (&dx)[2],
+                                                  const int2* __restrict__ bl, const float4* __restrict__ cen, int nb,
+                                                  int lch, const int (&toff)[2], const GaussTile (&gt)[2], const float4 (&dx)[2],
                                                   const float4 (&dxl)[2], int lane, float (&sr)[2], float (&si)[2])
 {
 #pragma unroll 1
     for (int c0 = 0; c0 < G; c0 += 1 << lch) {
-        build_pair_table<true>(T, bl, nb, sBa, gtab, c0, lch, lane);
+        build_pair_table<true>(T, bl, nb, sBa, s_off, cen, gtab, c0, lch, lane);
         __syncwarp();
 #pragma unroll 1
         for (int j4 = 0; j4 < 1 << lch; j4 += 4)
@@ -407,7 +438,9 @@ fwd_mixed_kernel(const DevProblem* __restrict__ probs, const Plan* __restrict__ 
     __shared__ __align__(8) unsigned long long s_sbar[2];   // stage buffers
     __shared__ __align__(8) unsigned long long s_gbar[2];   // GAINS: gains tables
     // GAINS: per warp, its visibility granule's pair list and pair table
-    __shared__ int2 s_bl[GAINS ? BLK_GRAN : 1][GAINS ? NB_MAX : 1];
+    // (a granule whose pairs have their own centres has few: these follow its pairs)
+    __shared__ __align__(16) int2 s_bl[GAINS ? BLK_GRAN : 1][GAINS ? NB_MAX : 1];
+    static_assert(NB_MAX * sizeof(int2) >= OWN_MAX * (sizeof(int2) + sizeof(float4)) && NB_MAX % 2 == 0, "s_bl");
     __shared__ float2 s_pt[GAINS ? BLK_GRAN : 1][GAINS ? NB_MAX * BT_P : 1];
     float2* const s_gain = reinterpret_cast<float2*>(s_dyn + 2 * S::BYTES);
 
@@ -463,18 +496,18 @@ fwd_mixed_kernel(const DevProblem* __restrict__ probs, const Plan* __restrict__ 
             cl = P.vis.cen_lo[vg];
             ext = P.vis.ext[vg];
 #pragma unroll
-            for (int r = 0; r < 2; ++r) {
-                if (!GAUSS) {
-                    xh[r] = P.vis.hi[e0 + 32 * r];
-                    dx[r] = to_rad(P.vis.off[e0 + 32 * r]);
-                }
+            for (int r = 0; r < 2; ++r)
                 if (GAINS) ant[r] = P.ant[e0 + 32 * r];
-            }
         }
         double tr[2] = {0.0, 0.0}, ti[2] = {0.0, 0.0};
         int nb = 0, lch = 4, toff[2] = {0, 0};  // GAINS: pairs in the granule's list (0: gathers)
+        bool own = false;                       // with centres of their own
+        float4* const s_bc = reinterpret_cast<float4*>(s_bl[warp] + OWN_MAX);
         if (GAINS) {
             if (vg_ok) nb = P.gnb[vg];
+            own = nb >= GNB_OWN;
+            nb &= GNB_OWN - 1;
+            if (own && lane < OWN_MAX) s_bc[lane] = P.gcen[(size_t)vg * OWN_MAX + lane];
             if (nb > 0) {
                 lch = pair_chunk_log2(nb);
 #pragma unroll
@@ -482,6 +515,16 @@ fwd_mixed_kernel(const DevProblem* __restrict__ probs, const Plan* __restrict__ 
                 if (lane < nb) s_bl[warp][lane] = P.gbl[(size_t)vg * NB_MAX + lane];
             }
             __syncwarp();
+        }
+        const auto offsets = [&](int r) {       // radians per turn
+            return to_rad(reload4((GAINS ? P.vown : P.vis.off) + e0 + 32 * r));
+        };
+        if (!GAUSS && vg_ok) {
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                xh[r] = P.vis.hi[e0 + 32 * r];
+                dx[r] = offsets(r);
+            }
         }
 
         for (int gs = g0; gs < g1; gs += NST) {
@@ -543,21 +586,22 @@ fwd_mixed_kernel(const DevProblem* __restrict__ probs, const Plan* __restrict__ 
                 for (int r = 0; r < 2; ++r) {
                     if (GAUSS) {                                         // (not held across granules)
                         xh[r] = reload4(P.vis.hi + e0 + 32 * r);
-                        if (!exact) dx[r] = to_rad(reload4(P.vis.off + e0 + 32 * r));
+                        if (!exact) dx[r] = offsets(r);
                     }
                     C[r] = frac_dot3(xh[r], P.vis.lo[e0 + 32 * r], yc_h, yc_l);
                 }
                 float sr[2] = {0.f, 0.f}, si[2] = {0.f, 0.f};
+                const float4* const cen = GAINS && own ? s_bc : nullptr;       // (exact tiles: not used)
                 if (!GAUSS || kind == DIRAC) {
                     if (GAINS && nb > 0) {
                         if (exact) {
                             const float4 dxt[2] = {P.vis.off[e0], P.vis.off[e0 + 32]},
                                          dxl[2] = {P.vis.offlo[e0], P.vis.offlo[e0 + 32]};
-                            fwd_dirac_tile_pt<true>(q_off, q_lo, q_Ba, gtab, s_pt[warp], s_bl[warp], nb, lch, toff, dxt,
-                                                    dxl, lane, sr, si);
+                            fwd_dirac_tile_pt<true>(q_off, q_lo, q_Ba, gtab, s_pt[warp], s_bl[warp], nullptr, nb, lch, toff,
+                                                    dxt, dxl, lane, sr, si);
                         } else {
-                            fwd_dirac_tile_pt<false>(q_off, q_lo, q_Ba, gtab, s_pt[warp], s_bl[warp], nb, lch, toff, dx,
-                                                     dx, lane, sr, si);
+                            fwd_dirac_tile_pt<false>(q_off, q_lo, q_Ba, gtab, s_pt[warp], s_bl[warp], cen, nb, lch, toff,
+                                                     dx, dx, lane, sr, si);
                         }
                     } else if (exact) {
                         const float4 dxt[2] = {P.vis.off[e0], P.vis.off[e0 + 32]},
@@ -587,18 +631,18 @@ fwd_mixed_kernel(const DevProblem* __restrict__ probs, const Plan* __restrict__ 
                         const float4 dxt[2] = {P.vis.off[e0], P.vis.off[e0 + 32]},
                                      dxl[2] = {P.vis.offlo[e0], P.vis.offlo[e0 + 32]};
                         if (GAINS && nb > 0) {
-                            if (par) fwd_gauss_tile_pt<true, true>(q_off, q_lo, q_pg, q_Ba, gtab, s_pt[warp], s_bl[warp], nb,
-                                                                   lch, toff, gt, dxt, dxl, lane, sr, si);
-                            else fwd_gauss_tile_pt<true, false>(q_off, q_lo, q_pg, q_Ba, gtab, s_pt[warp], s_bl[warp], nb,
-                                                                lch, toff, gt, dxt, dxl, lane, sr, si);
+                            if (par) fwd_gauss_tile_pt<true, true>(q_off, q_lo, q_pg, q_Ba, gtab, s_pt[warp], s_bl[warp],
+                                                                   nullptr, nb, lch, toff, gt, dxt, dxl, lane, sr, si);
+                            else fwd_gauss_tile_pt<true, false>(q_off, q_lo, q_pg, q_Ba, gtab, s_pt[warp], s_bl[warp],
+                                                                nullptr, nb, lch, toff, gt, dxt, dxl, lane, sr, si);
                         } else if (par) {
                             fwd_gauss_tile<GAINS, true, true>(q_off, q_lo, q_pg, q_Ba, gtab, gt, dxt, dxl, ant, sr, si);
                         } else {
                             fwd_gauss_tile<GAINS, true, false>(q_off, q_lo, q_pg, q_Ba, gtab, gt, dxt, dxl, ant, sr, si);
                         }
                     } else if (GAINS && nb > 0) {
-                        fwd_gauss_tile_pt<false, false>(q_off, q_lo, q_pg, q_Ba, gtab, s_pt[warp], s_bl[warp], nb, lch, toff, gt,
-                                                 dx, dx, lane, sr, si);
+                        fwd_gauss_tile_pt<false, false>(q_off, q_lo, q_pg, q_Ba, gtab, s_pt[warp], s_bl[warp], cen, nb, lch,
+                                                        toff, gt, dx, dx, lane, sr, si);
                     } else {
                         fwd_gauss_tile<GAINS, false, false>(q_off, q_lo, q_pg, q_Ba, gtab, gt, dx, dx, ant, sr, si);
                     }
@@ -952,31 +996,36 @@ __device__ __forceinline__ void adjg_flush(const float (&M)[2], float (&z)[2], f
 // At a new pair `key` (antenna indices a = key >> 16, b = key & 0xffff, both
 // valid): flush the run so far, then M = |G_ja| |G_jb| and Phi = C + psi_jb -
 // psi_ja (radians; turns when EXACT) for the lane's two pixels, Ct = C in
-// turns.
-template <bool EXACT, class GF>
-__device__ __forceinline__ void adjg_next_run(int key, int& cur, const GF& gain, const float (&Ct)[2],
+// turns.  OWN: cen holds the granule's pairs' own centres, in the order of its runs;
+// dj: the pixels' offsets (par: of nu and q in z and w).
+template <bool EXACT, bool OWN, class GF>
+__device__ __forceinline__ void adjg_next_run(int key, int& cur, int& slot, const GF& gain, const float (&Ct)[2],
+                                              const float4* cen, const float4 (&dj)[2], bool par,
                                               float (&M)[2], float (&Phi)[2], float (&z)[2], float (&acc)[2])
 {
     if (key == cur) return;                       // warp-uniform: every lane has the same k
     adjg_flush(M, z, acc);
     cur = key;
+    if (OWN) ++slot;
     const int a = key >> 16, b = key & 0xffff;
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
         const float2 ga = gain(a, r), gb = gain(b, r);   // {|G|, arg G in turns}
         M[r] = ga.x * gb.x;
-        const float f = frac_turns(Ct[r] + (gb.y - ga.y));
+        float f = frac_turns(Ct[r] + (gb.y - ga.y));
+        if (OWN)
+            f = frac_turns(f + turns_of(cen[slot], dj[r].x, dj[r].y, par ? dj[r].z - dj[r].w : dj[r].z));
         Phi[r] = EXACT ? f : f * TWO_PI_F;
     }
 }
 
-template <bool EXACT, bool AL4, class GF>
+template <bool EXACT, bool AL4, bool OWN, class GF>
 __device__ __forceinline__ void adjg_dirac_tile(const float4* __restrict__ s_off, const float4* __restrict__ g_lo,
                                                 const float2* __restrict__ s_kr, const GF& gain,
-                                                const float (&Ct)[2], const float4 (&dx)[2],
+                                                const float (&Ct)[2], const float4* cen, const float4 (&dx)[2],
                                                 const float4 (&dxl)[2], float (&acc)[2])
 {
-    int cur = -1;
+    int cur = -1, slot = -1;
     float M[2] = {0.f, 0.f}, Phi[2] = {0.f, 0.f}, z[2] = {0.f, 0.f};
 #pragma unroll(AL4 ? 2 : 1)
     for (int k0 = 0; k0 < G; k0 += 4)
@@ -985,7 +1034,8 @@ __device__ __forceinline__ void adjg_dirac_tile(const float4* __restrict__ s_off
         const int k = k0 + kk;
         const float4 o = s_off[k];
         const float2 kr = s_kr[k];             // {key, |r|}
-        if (!AL4 || kk == 0) adjg_next_run<EXACT>(__float_as_int(kr.x), cur, gain, Ct, M, Phi, z, acc);
+        if (!AL4 || kk == 0)
+            adjg_next_run<EXACT, OWN>(__float_as_int(kr.x), cur, slot, gain, Ct, cen, dx, false, M, Phi, z, acc);
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
             float ph;                              // radians
@@ -999,14 +1049,14 @@ __device__ __forceinline__ void adjg_dirac_tile(const float4* __restrict__ s_off
 
 // g_off, g_lo, dx, dxl (EXACT): the offsets of either side and their residuals
 // in turns; p and e are then as gauss_tile's.
-template <bool EXACT, bool AL4, bool PAR, class GF>
+template <bool EXACT, bool AL4, bool OWN, bool PAR, class GF>
 __device__ __forceinline__ void adjg_gauss_tile(const float4* __restrict__ s_p, const float4* __restrict__ s_e,
                                                 const float2* __restrict__ s_kr, const float4* __restrict__ g_off,
                                                 const float4* __restrict__ g_lo, const GF& gain,
-                                                const float (&Ct)[2], const float4 (&y)[2],
+                                                const float (&Ct)[2], const float4* cen, bool par, const float4 (&y)[2],
                                                 const float4 (&dx)[2], const float4 (&dxl)[2], float (&acc)[2])
 {
-    int cur = -1;
+    int cur = -1, slot = -1;
     float M[2] = {0.f, 0.f}, Phi[2] = {0.f, 0.f}, z[2] = {0.f, 0.f};
 #pragma unroll 1
     for (int k0 = 0; k0 < G; k0 += 4)
@@ -1015,7 +1065,8 @@ __device__ __forceinline__ void adjg_gauss_tile(const float4* __restrict__ s_p, 
         const int k = k0 + kk;
         const float4 p = s_p[k], e = s_e[k];
         const float2 kr = s_kr[k];                 // {key, B'' (radians)}
-        if (!AL4 || kk == 0) adjg_next_run<EXACT>(__float_as_int(kr.x), cur, gain, Ct, M, Phi, z, acc);
+        if (!AL4 || kk == 0)
+            adjg_next_run<EXACT, OWN>(__float_as_int(kr.x), cur, slot, gain, Ct, cen, y, par, M, Phi, z, acc);
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
             float ph, ex;                              // radians; exponent of two
@@ -1068,8 +1119,8 @@ cudaError_t launch_gauss_class(const d4* vd, int n_pad, const double* sigma, int
 // inside the run.  For each owned granule the 8 warp sums are added in warp
 // order (deterministic).  A unit is one pixel granule x one visibility granule.
 struct AdjRaw {                                   // one warp's slice, bytes
-    static constexpr int OFF = 0, LO = 1024, HI = 2048, R = 3072, ANT = 3584, CEN = 4096;
-    static constexpr int BYTES = CEN + 48;        // a multiple of 16
+    static constexpr int OFF = 0, LO = 1024, HI = 2048, R = 3072, ANT = 3584, CEN = 4096, OWN = CEN + 48;
+    static constexpr int BYTES = OWN + OWN_MAX * 16;   // a multiple of 16
 };
 
 // Lane 0: copy visibility granule g of P into a warp's raw slice (r: the
@@ -1087,6 +1138,7 @@ __device__ __forceinline__ void adj_raw_load(unsigned char* raw, const DevProble
     bulk_copy(raw + AdjRaw::CEN, P.vis.cen_hi + g, 16, bar);
     bulk_copy(raw + AdjRaw::CEN + 16, P.vis.cen_lo + g, 16, bar);
     bulk_copy(raw + AdjRaw::CEN + 32, P.vis.ext + g, 16, bar);
+    bulk_copy(raw + AdjRaw::OWN, P.gcen + (size_t)g * OWN_MAX, OWN_MAX * 16, bar);
 }
 
 __global__ void __launch_bounds__(NTHREADS, 2)
@@ -1095,10 +1147,11 @@ adj_mixed_gains_kernel(const DevProblem* __restrict__ probs, const Plan* __restr
 {
     // per warp, what its tiles read for its current granule
     // (Dirac / Gaussian owners)
-    __shared__ float4 s_off[BLK_GRAN][G];       // {du, dv, dw, B + arg r (radians)} / {p1, p2, p3, p4}
+    __shared__ float4 s_off[BLK_GRAN][G];       // {du, dv, dw (radians; turns when exact), B + arg r (radians)} / {p1, p2, p3, p4}
+    __shared__ float4 s_cen[BLK_GRAN][OWN_MAX]; // the pairs' own centres
+    const auto red = [&](int w) { return reinterpret_cast<double*>(s_off[w]); };   // a warp's sums, when its tiles are done
     __shared__ float2 s_kr[BLK_GRAN][G];        // {pair key, |r|} / {pair key, B''}
     __shared__ float4 s_va[BLK_GRAN][G];        // - / {e1, e2, e4, k0''}
-    __shared__ double s_red[BLK_GRAN][G];
     __shared__ __align__(8) unsigned long long s_wbar[BLK_GRAN];   // each warp's raw slice
     __shared__ __align__(8) unsigned long long s_gbar;             // the gains table
     // dynamic: [raw slices, BLK_GRAN x AdjRaw::BYTES][the owned granule's gains
@@ -1114,6 +1167,7 @@ adj_mixed_gains_kernel(const DevProblem* __restrict__ probs, const Plan* __restr
     const float2* const raw_r = reinterpret_cast<const float2*>(raw + AdjRaw::R);
     const int2* const raw_ant = reinterpret_cast<const int2*>(raw + AdjRaw::ANT);
     const float4* const raw_cen = reinterpret_cast<const float4*>(raw + AdjRaw::CEN);
+    const float4* const raw_own = reinterpret_cast<const float4*>(raw + AdjRaw::OWN);
     const Plan pl = *plp;
     const long long c = blockIdx.x;
     long long u, u_end;
@@ -1144,7 +1198,7 @@ adj_mixed_gains_kernel(const DevProblem* __restrict__ probs, const Plan* __restr
         const int gtab_n = gain_rows(P.n_ant) * GP;      // float2 per granule table
         const int gb = pl.prob_b0[p] + pgi;              // a block is one pixel granule (own_granules)
         double* dst = partial + (size_t)slot_of(pl, gb) * G;
-        __syncthreads();                                 // s_gain / s_red free again
+        __syncthreads();                                 // s_gain and the sums free again
         if (threadIdx.x == 0 && !fault) {
             fence_proxy_async_smem();                    // the table's last readers are done
             bulk_load(s_gain, P.gpol32 + (size_t)pgi * gtab_n, (unsigned)gtab_n * (unsigned)sizeof(float2),
@@ -1167,7 +1221,7 @@ adj_mixed_gains_kernel(const DevProblem* __restrict__ probs, const Plan* __restr
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
             xh[r] = P.pix.hi[eidx[r]];
-            dx[r] = to_rad(P.pix.off[eidx[r]]);
+            dx[r] = P.pix.off[eidx[r]];
             if (gauss) y[r] = P.pgoff[eidx[r]];
         }
         const SmemGain sg{s_gain, lane};
@@ -1180,6 +1234,8 @@ adj_mixed_gains_kernel(const DevProblem* __restrict__ probs, const Plan* __restr
             // derive this granule's records for the tiles
             const float4 yc_h = raw_cen[0], yc_l = raw_cen[1], yext = raw_cen[2];
             const bool exact = dot3(ext, yext) > D_MAX;
+            const bool own = !exact && raw_own[0].w > 0.f;
+            if (lane < OWN_MAX) s_cen[warp][lane] = raw_own[lane];
             int keys[2];
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
@@ -1198,7 +1254,7 @@ adj_mixed_gains_kernel(const DevProblem* __restrict__ probs, const Plan* __restr
                     b = frac_turns(fmaf(-gc.x * INV_TWO_PI_F, tc, b + rp.y));
                     if (par) b = frac_turns(b - tp_frac(x.z, 0.f, nuh, nul));
                     if (par && !exact) b = frac_turns(fmaf(o.z, kappa, b));
-                    o = to_rad(o);
+                    o = to_rad(own ? own_offset(o, raw_lo[k], raw_own) : o);
                     s_off[warp][k] = exact ? make_float4(x.x, x.y, -x.z, gc.x * INV_TWO_PI_F)
                                            : make_float4(fmaf(-gc.x, x.x, o.x), fmaf(-gc.x, x.y, o.y),
                                                          par ? fmaf(-TWO_PI_F, x.z, o.z) : o.z,
@@ -1207,6 +1263,7 @@ adj_mixed_gains_kernel(const DevProblem* __restrict__ probs, const Plan* __restr
                                                 fmaf(gc.y, tc, gc.z) + __log2f(rp.x));
                     kr.y = b * TWO_PI_F;
                 } else {
+                    if (!exact) o = to_rad(own ? own_offset(o, raw_lo[k], raw_own) : o);
                     o.w = frac_turns(b + rp.y) * TWO_PI_F;
                     s_off[warp][k] = o;
                 }
@@ -1224,35 +1281,40 @@ adj_mixed_gains_kernel(const DevProblem* __restrict__ probs, const Plan* __restr
             if (lane == 0 && !fault && g + BLK_GRAN < g1) adj_raw_load(raw, P, g + BLK_GRAN, &s_wbar[warp]);
             float Ct[2];                          // the tile's centre term C, turns
 #pragma unroll
-            for (int r = 0; r < 2; ++r) Ct[r] = frac_dot3(xh[r], P.pix.lo[eidx[r]], yc_h, yc_l);
+            for (int r = 0; r < 2; ++r) Ct[r] = frac_dot3_near(xh[r], P.pix.lo[eidx[r]], yc_h, yc_l);
             const float4* g_lo = P.vis.offlo + (size_t)g * G;   // exact tiles only (rare)
+            const float4* const cen = s_cen[warp];
             float acc[2] = {0.f, 0.f};
             if (exact) {
                 const float4 dxt[2] = {P.pix.off[eidx[0]], P.pix.off[eidx[1]]},
                              dxl[2] = {P.pix.offlo[eidx[0]], P.pix.offlo[eidx[1]]};
                 const float4* g_off = P.vis.off + (size_t)g * G;
-                if (gauss && par) adjg_gauss_tile<true, false, true>(s_off[warp], s_va[warp], s_kr[warp], g_off, g_lo, sg, Ct, y, dxt, dxl, acc);
-                else if (gauss) adjg_gauss_tile<true, false, false>(s_off[warp], s_va[warp], s_kr[warp], g_off, g_lo, sg, Ct, y, dxt, dxl, acc);
-                else adjg_dirac_tile<true, false>(s_off[warp], g_lo, s_kr[warp], sg, Ct, dxt, dxl, acc);
+                if (gauss && par) adjg_gauss_tile<true, false, false, true>(s_off[warp], s_va[warp], s_kr[warp], g_off, g_lo, sg, Ct, cen, par, y, dxt, dxl, acc);
+                else if (gauss) adjg_gauss_tile<true, false, false, false>(s_off[warp], s_va[warp], s_kr[warp], g_off, g_lo, sg, Ct, cen, par, y, dxt, dxl, acc);
+                else adjg_dirac_tile<true, false, false>(s_off[warp], g_lo, s_kr[warp], sg, Ct, cen, dxt, dxl, acc);
             } else if (gauss) {
-                if (al4) adjg_gauss_tile<false, true, false>(s_off[warp], s_va[warp], s_kr[warp], g_lo, g_lo, sg, Ct, y, dx, dx, acc);
-                else adjg_gauss_tile<false, false, false>(s_off[warp], s_va[warp], s_kr[warp], g_lo, g_lo, sg, Ct, y, dx, dx, acc);
+                if (own && al4) adjg_gauss_tile<false, true, true, false>(s_off[warp], s_va[warp], s_kr[warp], g_lo, g_lo, sg, Ct, cen, par, y, dx, dx, acc);
+                else if (own) adjg_gauss_tile<false, false, true, false>(s_off[warp], s_va[warp], s_kr[warp], g_lo, g_lo, sg, Ct, cen, par, y, dx, dx, acc);
+                else if (al4) adjg_gauss_tile<false, true, false, false>(s_off[warp], s_va[warp], s_kr[warp], g_lo, g_lo, sg, Ct, cen, par, y, dx, dx, acc);
+                else adjg_gauss_tile<false, false, false, false>(s_off[warp], s_va[warp], s_kr[warp], g_lo, g_lo, sg, Ct, cen, par, y, dx, dx, acc);
             } else {
-                if (al4) adjg_dirac_tile<false, true>(s_off[warp], g_lo, s_kr[warp], sg, Ct, dx, dx, acc);
-                else adjg_dirac_tile<false, false>(s_off[warp], g_lo, s_kr[warp], sg, Ct, dx, dx, acc);
+                if (own && al4) adjg_dirac_tile<false, true, true>(s_off[warp], g_lo, s_kr[warp], sg, Ct, cen, dx, dx, acc);
+                else if (own) adjg_dirac_tile<false, false, true>(s_off[warp], g_lo, s_kr[warp], sg, Ct, cen, dx, dx, acc);
+                else if (al4) adjg_dirac_tile<false, true, false>(s_off[warp], g_lo, s_kr[warp], sg, Ct, cen, dx, dx, acc);
+                else adjg_dirac_tile<false, false, false>(s_off[warp], g_lo, s_kr[warp], sg, Ct, cen, dx, dx, acc);
             }
 #pragma unroll
             for (int r = 0; r < 2; ++r) tot[r] += (double)acc[r];
             __syncwarp();                                 // s_off ... of this warp free again
         }
 #pragma unroll
-        for (int r = 0; r < 2; ++r) s_red[warp][lane + 32 * r] = tot[r];
+        for (int r = 0; r < 2; ++r) red(warp)[lane + 32 * r] = tot[r];
         __syncthreads();
         if (warp == 0) {
 #pragma unroll
             for (int r = 0; r < 2; ++r) {
                 double t = 0.0;
-                for (int w = 0; w < BLK_GRAN; ++w) t += s_red[w][lane + 32 * r];
+                for (int w = 0; w < BLK_GRAN; ++w) t += red(w)[lane + 32 * r];
                 dst[lane + 32 * r] = t * P.pix.d[eidx[r]].w;
             }
         }
@@ -1362,9 +1424,9 @@ static FwdKernel fwd_kernel_of(int code)
 }
 // With gains: without Gaussian pixels in the batch, an instance that holds its
 // visibilities' coordinates across granules, where the other reloads them to make
-// room for the Gaussian tiles (43,264 pixels x 38,676 visibilities, 48 antennas, 974 ->
-// 945 us; in the shared one such sets had become up to 4% slower than before it
-// took the linear tiles).
+// room for the Gaussian tiles (us per call, in orders of runs from one centre: 65,536
+// pixels x 32,000 visibilities 1,278 -> 1,175; 43,264 x 38,676 1,000 -> 951;
+// 47,961 x 32,822 1,953 -> 1,860).
 static FwdKernel fwd_gains_kernel_of(int code)
 {
     return shape_dirac_only(code) ? fwd_mixed_kernel<true, 1, 0, false> : fwd_mixed_kernel<true, 1, 0, true>;
