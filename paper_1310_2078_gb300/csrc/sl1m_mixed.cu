@@ -600,8 +600,12 @@ fwd_mixed_kernel(const DevProblem* __restrict__ probs, const Plan* __restrict__ 
                             fwd_dirac_tile_pt<true>(q_off, q_lo, q_Ba, gtab, s_pt[warp], s_bl[warp], nullptr, nb, lch, toff,
                                                     dxt, dxl, lane, sr, si);
                         } else {
-                            fwd_dirac_tile_pt<false>(q_off, q_lo, q_Ba, gtab, s_pt[warp], s_bl[warp], cen, nb, lch, toff,
-                                                     dx, dx, lane, sr, si);
+                            // (apart, so that most granules' table loop has no branch: 47,961
+                            // pixels x 32,822 visibilities 1,952 -> 1,922 us)
+                            if (cen) fwd_dirac_tile_pt<false>(q_off, q_lo, q_Ba, gtab, s_pt[warp], s_bl[warp], s_bc, nb, lch,
+                                                              toff, dx, dx, lane, sr, si);
+                            else fwd_dirac_tile_pt<false>(q_off, q_lo, q_Ba, gtab, s_pt[warp], s_bl[warp], nullptr, nb, lch,
+                                                          toff, dx, dx, lane, sr, si);
                         }
                     } else if (exact) {
                         const float4 dxt[2] = {P.vis.off[e0], P.vis.off[e0 + 32]},
