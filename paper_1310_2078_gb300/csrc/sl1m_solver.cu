@@ -656,7 +656,10 @@ __global__ void phases_kernel(const DevProblem* __restrict__ probs, const int* _
 
 // Threads per element by the mean number of slots of a block (the kernels'
 // loads are 8 deep): up to 2 slots one thread has them in flight anyway; above
-// 48, 8 threads take a few rounds each.  16 of them made CTAs of 1,024 threads and
+// 96, 8 threads take a few rounds each.  (Between 48 and 96 slots CTAs of 256 threads start
+// sooner behind another stream's operator: 3,001 Dirac pixels x 129,891 visibilities
+// adjoint, 76 slots, three streams in turn: 135.9 us a call with 8 threads, 132.4
+// with 4.)  16 of them made CTAs of 1,024 threads and
 // 64 registers, which start only on an empty SM: behind another stream's
 // operator they waited for whole SMs and kept its CTAs off them meanwhile
 // (35,344 multiscale pixels x 2,702 visibilities forward, three streams in turn: 163
@@ -664,7 +667,7 @@ __global__ void phases_kernel(const DevProblem* __restrict__ probs, const int* _
 static int slot_threads(const Plan& pl)
 {
     const double mean = (double)pl.n_slots / (pl.n_blocks > 0 ? pl.n_blocks : 1);
-    return mean <= 2.0 && pl.blk_el >= 256 ? 1 : mean <= 48.0 ? 4 : 8;
+    return mean <= 2.0 && pl.blk_el >= 256 ? 1 : mean <= 96.0 ? 4 : 8;
 }
 template <int SL>
 static int fin_grid(const Plan& pl, int num_sms)
