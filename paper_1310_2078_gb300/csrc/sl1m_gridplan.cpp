@@ -154,6 +154,12 @@ std::vector<float2> twiddles(int lg)
 // Lattice: launches, the planes' cells, the visibilities, and the points that a
 // tile's CTA spreads one after the other where there are few tiles.  The lattice
 // is taken where it promises a tenth or more.
+// The fit is older than the ring-buffer spreading and the radix-16 transforms and puts
+// the lattice about a third too high (256^2 +/-0.5 x 40,320: 400 us, measured 300;
+// 1024^2 x 406,400: 1,444, measured 1,055); pairs on the exact path, three times as dear,
+// are not in pair_seconds (256^2 +/-0.5 x 5,000: 165 us, measured 270).  Both err
+// towards the pairs, and both directions take one operator: 64^2 x 40,000 would want
+// the lattice forward and the pair adjoint.
 static double grid_seconds(const GridOp& g, double n_vis)
 {
     return 4.2e-5 + 2.8e-12 * (double)g.np * grid_plane_elems(g) + 1.05e-9 * n_vis + 2.7e-7 * n_vis / grid_tiles(g);

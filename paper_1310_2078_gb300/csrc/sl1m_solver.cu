@@ -659,11 +659,11 @@ __global__ void phases_kernel(const DevProblem* __restrict__ probs, const int* _
 // 96, 8 threads take a few rounds each.  (Between 48 and 96 slots CTAs of 256 threads start
 // sooner behind another stream's operator: 3,001 Dirac pixels x 129,891 visibilities
 // adjoint, 76 slots, three streams in turn: 135.9 us a call with 8 threads, 132.4
-// with 4.)  16 of them made CTAs of 1,024 threads and
-// 64 registers, which start only on an empty SM: behind another stream's
-// operator they waited for whole SMs and kept its CTAs off them meanwhile
-// (35,344 multiscale pixels x 2,702 visibilities forward, three streams in turn: 163
-// us a call; 151 with 8, and a 30-tick FP64 solve 5.71 -> 5.69 ms).
+// with 4.)  16 of them made CTAs of 1,024 threads and 64 registers, which start
+// only on an empty SM: behind another stream's operator they waited for whole SMs
+// and kept its CTAs off them meanwhile (35,344 multiscale pixels x 2,702
+// visibilities forward, three streams in turn: 163 us a call; 151 with 8, and a
+// 30-tick FP64 solve 5.71 -> 5.69 ms).
 static int slot_threads(const Plan& pl)
 {
     const double mean = (double)pl.n_slots / (pl.n_blocks > 0 ? pl.n_blocks : 1);
