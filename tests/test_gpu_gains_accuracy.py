@@ -9,6 +9,7 @@ Granules of runs that measure their offsets from one centre made it 1.06 to 1.14
 import numpy as np
 import pytest
 
+import oracle
 from paper_1310_2078_gb300 import synth
 
 pytestmark = pytest.mark.gpu
@@ -40,3 +41,30 @@ def test_runs_of_a_pair_are_as_accurate_as_neighbours(gpu_lib, seed):
     ratio = np.array(err[0]) / np.array(err[1])
     print("errors", err, "ratio", ratio)
     assert np.all(ratio <= 1.04), ratio
+
+
+@pytest.mark.parametrize("n_times", [16, 13, 9])              # runs that all begin at multiples of 4, and others
+@pytest.mark.parametrize("kinds,tol", [((0,), 6e-7), ((2,), 6e-7), ((0, 2), 6e-7), ((1,), 3e-6)])
+def test_own_centres_of_every_pixel_kind(gpu_lib, n_times, kinds, tol):
+    """Layouts most of whose granules measure from their pairs' own centres (24 antennas,
+    small pixel granules), against the oracle.  A pair's phase is rounded to about 2e-7
+    rad rms and its sine and cosine to as much again: 6e-7 of the 2-norm; paraxial
+    pixels add w nu of their granule's offsets.  A wrong centre is an error of order 1."""
+    rng = synth.rng_for(n_times)
+    uvw, ant = synth.uvw_tracks(synth.antennas(rng, 24, 1000.0, 20.0), -30.0, n_times)
+    lm = synth.regular_grid(64, 0.25)
+    lm = lm + rng.uniform(-0.002, 0.002, lm.shape)
+    kind = np.resize(np.array(kinds, np.int32), len(lm))
+    sigma = np.where(kind == 0, 0.0, 1e-3)
+    gains = synth.beam_gains(rng, lm, 24, theta=(0.3, 0.5), ramp=0.5)
+    O = oracle.Problem(uvw, lm, sigma, kind, None, ant, gains, threads=8)
+    ctx = gpu_lib.Context(0)
+    P = ctx.problem()
+    P.set_visibilities(uvw, None, None, ant)
+    P.set_pixels(lm, sigma, kind)
+    P.set_gains(gains)
+    x = rng.normal(size=len(lm))
+    r = rng.normal(size=len(uvw)) + 1j * rng.normal(size=len(uvw))
+    for got, want in ((P.forward(x), oracle.forward(O, x)), (P.adjoint(r), oracle.adjoint(O, r))):
+        assert np.linalg.norm(got - want) <= tol * np.linalg.norm(want)
+    ctx.close()
